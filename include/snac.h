@@ -84,7 +84,12 @@ typedef struct {
 
 typedef enum { SNAC_FP64 = 0, SNAC_MIXED = 1 } snac_precision;
 
-/* Solver options; pass NULL to snac_plan_create for the defaults shown. */
+/* Solver options; pass NULL to snac_plan_create for the defaults shown.
+ * With the default schedule (nu1, nu2, max_cycles, max_coarse, fused, inner_reduction, onchip and
+ * bottom_cells as shown) a layout whose blocks assemble into a rectangle with one uniform plane axis (an
+ * even number of cells, half or all of it a product of 2, 3, 5 and 7; the other axis not periodic) solves the
+ * reduced equations directly -- a transform along that axis (Table 1) and tridiagonal systems along the
+ * other -- in place of V-cycles; setting any of these options asks for the multigrid. */
 typedef struct {
   int32_t precision;   /* SNAC_FP64 (default): every stage in FP64. SNAC_MIXED: transforms and
                           multigrid in FP32 inside the FP64 defect-correction loop; the outer
@@ -126,7 +131,8 @@ typedef struct {
 typedef struct {
   int32_t status;        /* status of the last solve                                                */
   int32_t outer_iters;   /* defect-correction iterations performed                                  */
-  int32_t total_cycles;  /* V-cycles summed over wavenumbers and outer iterations                    */
+  int32_t total_cycles;  /* V-cycles summed over wavenumbers and outer iterations (a direct solve of
+                            a wavenumber counts as one)                                             */
   int32_t max_mode_cycles; /* largest number of V-cycles of one wavenumber in one outer iteration   */
   int32_t levels;        /* multigrid levels (1 = direct solve of the plane)                         */
   int32_t n_modes;       /* n_z                                                                      */

@@ -1,0 +1,370 @@
+// Separable solve of the reduced equations (Eq. 9) on an assembled rectangle: device code.
+//
+// When the blocks of a plan assemble into a full rectangle, the reduced operator of every wavenumber
+// is A_x + A_y + sigma_q with one-dimensional A_x, A_y. If one of the two plane axes is uniform, the
+// real-to-real transform of its boundary pair diagonalises it (the same Table 1 kinds as along the
+// homogeneous axis), and what is left is one tridiagonal system along the other axis per
+// (wavenumber, transform slot): an exact solve of about 40 operations per cell in place of several
+// V-cycles. "m" numbers cells along the transformed axis (M of them), "n" along the tridiagonal one
+// (N); spectral slot kappa stands for one eigenvector of the transformed axis.
+//
+// Transforms work on complex columns of a shared-memory buffer (fft_dev.cuh):
+//   pair kinds (PP, NN, DD): column c holds lines 2c and 2c+1 as real and imaginary part of one
+//       length-M FFT; with Z_k = A_k + i B_k the two spectra separate by additions. PP is kept at twice
+//       its usual scale; NN uses Makhoul's order v_t = x_2t | x_2(M-1-t)+1 and DD is NN of (-1)^m x_m
+//       with its slots in the NN numbering (slot kappa = DST-II index M-1-kappa).
+//   DCT-IV kinds (ND; DN = ND of (-1)^m x_m, slots reversed likewise): column c holds line c as a
+//       half-length sequence t_j = (x_2j + i x_M-1-2j) e^{-i pi (4j+1)/4M}.
+// Forward then inverse multiplies by 2 M for every kind; the tridiagonal solve divides by it.
+//
+// Tridiagonal systems: (lo + hi + tau) u_n - lo u_{n-1} - hi u_{n+1} = -f_n / 2M with couplings lo, hi
+// >= 0 and tau = -lambda_kappa - sigma_q + (Dirichlet face terms) >= 0. Elimination carries the row
+// sums (tau) instead of the diagonal, so that every operation adds or multiplies non-negative numbers:
+// no cancellation, the factors are accurate to a few units in the last place of the working type even
+// where the system is nearly singular, and an exactly singular one (all tau = 0) ends in an exactly zero
+// pivot, whose unknown is set to zero (the caller fixes the mean).
+#pragma once
+
+#include "fft_dev.cuh"
+
+namespace snac {
+namespace {
+
+enum { LINES_PAIR = 0, LINES_DCT4 = 1 };
+
+// One row of the tridiagonal axis: couplings, face term, and lo / hi (0 where hi = 0).
+template <typename T>
+struct alignas(4 * sizeof(T)) TriRow {
+  T lo, hi, tau, ratio;
+};
+
+template <typename T>
+struct DirectArgs {
+  FftTab F;
+  int M, N, cls, kind;
+  int nq;                  // wavenumbers held
+  const Cpl<T>* tw;        // e^{-2 pi i k / F.n}
+  const Cpl<T>* w2n;       // e^{-i pi k / 2M}, k = 0..M (pair kinds)
+  const Cpl<T>* t4a;       // e^{-i pi (4j+1) / 4M} (DCT-IV kinds)
+  const Cpl<T>* t4b;       // e^{-i pi k / M}
+  const int* perm;         // row of frequency k
+  const T* lam;            // eigenvalue of slot kappa (<= 0), times cscale
+  const TriRow<T>* tri;    // [N], times cscale
+  const T* sigma;          // per wavenumber
+  const unsigned* cellmn;  // per plane cell: m | n << 16
+  long long ncell;
+  T cscale;                // power of two that brings the couplings of tri (and lam) to about 1
+  T scale;                 // cscale / 2M
+  // plane offset of (m, n): base[n nbm + mblk[m]] + m mstr[n]
+  const int* base;
+  const int* mblk;
+  const int* mstr;
+  int nbm, xl, vec;        // xl: the transformed axis is the contiguous one; vec: pairs may be loaded as vectors
+};
+
+template <typename T>
+inline DirectArgs<T> direct_args(const snac_plan* P) {
+  const DirectTab& D = P->direct;
+  DirectArgs<T> A{};
+  A.F = D.fft;
+  A.M = D.M;
+  A.N = D.N;
+  A.cls = D.cls;
+  A.kind = D.kind;
+  A.nq = P->nz;
+  A.tw = (const Cpl<T>*)D.d_tw;
+  A.w2n = A.tw + D.w2n;
+  A.t4a = A.tw + D.t4a;
+  A.t4b = A.tw + D.t4b;
+  A.perm = D.d_perm;
+  A.lam = (const T*)D.d_lam;
+  A.tri = (const TriRow<T>*)D.d_tri;
+  if constexpr (sizeof(T) == 8) A.sigma = P->d_sigma64;
+  else A.sigma = P->d_sigma32;
+  A.cellmn = D.d_cellmn;
+  A.ncell = P->lev[0].ncell;
+  A.cscale = (T)D.cscale;
+  A.scale = (T)(D.cscale / (2.0 * D.M));
+  A.base = D.d_base;
+  A.mblk = D.d_mblk;
+  A.mstr = D.d_mstr;
+  A.nbm = D.nbm;
+  A.xl = D.xl;
+  A.vec = D.vec;
+  return A;
+}
+
+// Two spectra from one pair column: z1 = Z_k, z2 = Z_{M-k}; slots k -> y1 (line a, line b), M-k -> y2.
+template <typename T>
+__device__ __forceinline__ void pair_post(int kind, Cpl<T> w, Cpl<T> z1, Cpl<T> z2, Cpl<T>& y1, Cpl<T>& y2) {
+  const T ar = z1.re + z2.re, ai = z1.im - z2.im, br = z1.im + z2.im, bi = z2.re - z1.re;
+  if (kind == KIND_PP) {
+    y1 = {ar, br};
+    y2 = {ai, bi};
+  } else {
+    y1 = {w.re * ar - w.im * ai, w.re * br - w.im * bi};
+    y2 = {-(w.im * ar + w.re * ai), -(w.im * br + w.re * bi)};
+  }
+}
+
+// The inverse: slots k, M-k of both lines -> Z_k, Z_{M-k} (k = 0: x2 is taken as zero by the caller).
+template <typename T>
+__device__ __forceinline__ void pair_pre(int kind, Cpl<T> w, Cpl<T> x1, Cpl<T> x2, Cpl<T>& z1, Cpl<T>& z2) {
+  T ar = x1.re, ai = x2.re, br = x1.im, bi = x2.im;
+  if (kind != KIND_PP) {
+    ar = w.re * x1.re - w.im * x2.re;
+    ai = -(w.re * x2.re + w.im * x1.re);
+    br = w.re * x1.im - w.im * x2.im;
+    bi = -(w.re * x2.im + w.im * x1.im);
+  }
+  z1 = {ar - bi, ai + br};
+  z2 = {ar + bi, br - ai};
+}
+
+// Natural row of cell m of a pair column.
+__device__ __forceinline__ int pair_pos(int kind, int m, int M) {
+  return kind == KIND_PP ? m : ((m & 1) ? M - 1 - (m >> 1) : m >> 1);
+}
+__device__ __forceinline__ bool flip_kind(int kind) { return kind == KIND_DD || kind == KIND_DN; }
+
+__device__ __forceinline__ float tri_recip(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ double tri_recip(double x) { return recip(x); }
+
+// R consecutive rows of a tridiagonal system per thread, P threads per system (segments; the first
+// segment is padded in front by identity rows, so the last one ends at row N - 1). Each thread
+// eliminates its rows to u_r = D_r + c_r u_{r+1} + a_r u_{-1} (u_{-1}: the previous segment's last
+// unknown), the segments' last unknowns form a tridiagonal system of P rows that the first segment's
+// thread solves, and each thread substitutes back. load(n) gives the right-hand side, store(n, u)
+// takes the solution; ex: 7 x P x kg values, this system's column kk. Every thread of the CTA calls it
+// (three barriers). tq = -lambda - sigma >= 0.
+// `act` is false for threads past the last segment, which only take part in the barriers; `live`
+// for those with a system to solve.
+template <typename T, int R, typename Load, typename Store>
+__device__ __forceinline__ void tri_segment(const TriRow<T>* __restrict__ tri, int N, int P, int seg, int kk, int kg,
+                                            bool act, bool live, T tq, T scale, T* __restrict__ ex, Load&& load,
+                                            Store&& store) {
+  const int n0 = seg * R - (P * R - N);
+  T D[R], c[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) D[r] = live && n0 + r >= 0 ? load(n0 + r) : (T)0;
+  T a = 1, sl = 0, dp = 0, pi = 1, F = 0, H = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    TriRow<T> w{0, 0, 1, 0};
+    if (n0 + r >= 0) {
+      w = tri[n0 + r];
+      w.tau += tq;
+    }
+    const T la = w.lo * a, ls = fma(w.lo, sl, w.tau);
+    const T den = la + ls + w.hi;
+    const T inv = den > (T)0 ? tri_recip(den) : (T)0;
+    c[r] = w.hi * inv;
+    a = la * inv;
+    sl = ls * inv;
+    dp = fma(w.lo, dp, -scale * D[r]) * inv;
+    D[r] = dp;
+    if (r < R - 1) {
+      F = fma(pi, dp, F);
+      H = fma(pi, sl, H);
+      pi *= c[r];
+    }
+  }
+  const int st = P * kg;
+  T* e = ex + seg * kg + kk;
+  if (act) {
+    e[0] = dp;
+    e[st] = c[R - 1];
+    e[2 * st] = a;
+    e[3 * st] = sl;
+    e[4 * st] = F;
+    e[5 * st] = pi;
+    e[6 * st] = H;
+  }
+  __syncthreads();
+  if (act && seg == 0) {
+    T* z = ex + kk;
+    T g = 0, y = 0;
+    for (int s = 0; s < P; ++s) {
+      const int o = s * kg;
+      const bool more = s + 1 < P;
+      const T cs = z[o + st];
+      const T lo = z[o + 2 * st];
+      const T hi = more ? cs * z[o + kg + 5 * st] : (T)0;
+      const T tau = more ? fma(cs, z[o + kg + 6 * st], z[o + 3 * st]) : z[o + 3 * st];
+      const T d = more ? fma(cs, z[o + kg + 4 * st], z[o]) : z[o];
+      const T sum = fma(lo, g, tau);
+      const T den = sum + hi;
+      const T inv = den > (T)0 ? tri_recip(den) : (T)0;
+      g = sum * inv;
+      y = fma(lo, y, d) * inv;
+      z[o] = y;
+      z[o + st] = hi * inv;
+    }
+    for (int s = P - 2; s >= 0; --s) {
+      const int o = s * kg;
+      y = fma(z[o + st], y, z[o]);
+      z[o] = y;
+    }
+  }
+  __syncthreads();
+  T x = act ? e[0] : (T)0;
+  T aa = act && seg > 0 ? e[-kg] : (T)0;
+  __syncthreads();  // ex is free for the next round
+#pragma unroll
+  for (int r = 0; r < R - 1; ++r) {
+    const T ra = n0 + r >= 0 ? tri[n0 + r].ratio : (T)0;
+    aa *= ra * c[r];
+    D[r] += aa;
+  }
+  if (live && n0 + R - 1 >= 0) store(n0 + R - 1, x);
+#pragma unroll
+  for (int r = R - 2; r >= 0; --r) {
+    x = fma(c[r], x, D[r]);
+    if (live && n0 + r >= 0) store(n0 + r, x);
+  }
+}
+
+// Shared memory of a whole-plane solve: the buffer, then the exchange of the tridiagonal segments.
+constexpr int PLANE_R = 8;  // rows per thread of the tridiagonal phase
+
+struct PlaneShape {
+  int cols, rp, s1;
+  size_t buf, bytes;  // elements of the buffer (real), bytes in all
+};
+__host__ __device__ inline PlaneShape plane_shape(const FftTab& F, int M, int N, int cls, size_t w, int nt) {
+  PlaneShape s;
+  s.cols = cls == LINES_PAIR ? (N + 1) / 2 : N;
+  s.rp = s.cols | 1;
+  s.s1 = F.l1 * s.rp;
+  s.s1 += (1 - s.s1) & 15;  // consecutive slots of the first radix on different banks
+  s.buf = 2 * (size_t)(F.n / F.l1) * s.s1;
+  s.bytes = (s.buf + 7 * (size_t)nt) * w;
+  return s;
+}
+
+// One wavenumber's solve by one CTA of nt threads, the whole plane in shared memory: f -> u (global
+// plane of this wavenumber, caller cell order).
+template <typename T>
+__device__ void plane_direct(const DirectArgs<T>& A, int q, const T* __restrict__ f, T* __restrict__ u,
+                             unsigned char* smem, int nt) {
+  const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls, sizeof(T), nt);
+  Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
+  T* bt = reinterpret_cast<T*>(smem);
+  T* ex = bt + S.buf;
+  const ColsAny cm{S.cols, S.rp};
+  const int M = A.M, N = A.N, kind = A.kind, l1 = A.F.l1;
+  const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
+  const int ncell = (int)A.ncell;
+  if (pair && (N & 1)) {  // the last column's missing line
+    for (int m = threadIdx.x; m < M; m += nt) bt[2 * (fft_row(m, l1, S.s1, S.rp) + S.cols - 1) + 1] = 0;
+  }
+  for (int c = threadIdx.x; c < ncell; c += nt) {
+    const unsigned mn = A.cellmn[c];
+    const int m = mn & 0xffffu, n = mn >> 16;
+    T v = f[c];
+    if (flip && (m & 1)) v = -v;
+    int o;
+    if (pair) o = 2 * (fft_row(pair_pos(kind, m, M), l1, S.s1, S.rp) + (n >> 1)) + (n & 1);
+    else o = 2 * (fft_row((m & 1) ? (M - 1 - m) >> 1 : m >> 1, l1, S.s1, S.rp) + n) + (m & 1);
+    bt[o] = v;
+  }
+  __syncthreads();
+  if (!pair) {
+    for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
+      int j, c;
+      cm.split(t, j, c);
+      const int o = fft_row(j, l1, S.s1, S.rp) + c;
+      buf[o] = cx_mul(buf[o], A.t4a[j]);
+    }
+    __syncthreads();
+  }
+  fft_all<false>(buf, A.F, S.s1, cm, A.tw, nt);
+  if (pair) {
+    for (int t = threadIdx.x; t < (M / 2 + 1) * S.cols; t += nt) {
+      int k, c;
+      cm.split(t, k, c);
+      const int o1 = fft_row(A.perm[k], l1, S.s1, S.rp) + c;
+      const int o2 = k == 0 ? o1 : fft_row(A.perm[M - k], l1, S.s1, S.rp) + c;
+      Cpl<T> y1, y2;
+      pair_post(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], buf[o1], buf[o2], y1, y2);
+      if (o2 != o1) buf[o2] = y2;
+      buf[o1] = y1;
+    }
+  } else {
+    for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
+      int k, c;
+      cm.split(t, k, c);
+      const int o = fft_row(A.perm[k], l1, S.s1, S.rp) + c;
+      const Cpl<T> v = cx_mul(buf[o], A.t4b[k]);
+      buf[o] = Cpl<T>{(T)2 * v.re, (T)-2 * v.im};
+    }
+  }
+  __syncthreads();
+  {
+    const int P = (N + PLANE_R - 1) / PLANE_R, kg = nt / P;
+    const int seg = quot16(threadIdx.x, kg), kk = threadIdx.x - seg * kg;
+    const bool mine = seg < P;
+    const T sg = A.sigma[q];
+    for (int k0 = 0; k0 < M; k0 += kg) {
+      const int kap = k0 + kk;
+      const bool live = mine && kap < M;
+      int o = 0, ns = 1;
+      T tq = 0;
+      if (live) {
+        tq = -fma(sg, A.cscale, A.lam[kap]);
+        if (pair) {
+          o = 2 * fft_row(A.perm[kap], l1, S.s1, S.rp);
+        } else {
+          ns = 2;
+          o = 2 * fft_row(A.perm[(kap & 1) ? (M - 1 - kap) >> 1 : kap >> 1], l1, S.s1, S.rp) + (kap & 1);
+        }
+      }
+      tri_segment<T, PLANE_R>(A.tri, N, P, mine ? seg : 0, kk, kg, mine, live, tq, A.scale, ex,
+                              [&](int n) { return bt[o + n * ns]; }, [&](int n, T v) { bt[o + n * ns] = v; });
+    }
+  }
+  __syncthreads();
+  if (pair) {
+    for (int t = threadIdx.x; t < (M / 2 + 1) * S.cols; t += nt) {
+      int k, c;
+      cm.split(t, k, c);
+      const int o1 = fft_row(A.perm[k], l1, S.s1, S.rp) + c;
+      const int o2 = k == 0 ? o1 : fft_row(A.perm[M - k], l1, S.s1, S.rp) + c;
+      const Cpl<T> x1 = buf[o1];
+      const Cpl<T> x2 = k == 0 || (kind == KIND_PP && 2 * k == M) ? Cpl<T>{0, 0} : buf[o2];
+      Cpl<T> z1, z2;
+      pair_pre(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], x1, x2, z1, z2);
+      if (o2 != o1) buf[o2] = z2;
+      buf[o1] = z1;
+    }
+  } else {
+    for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
+      int j, c;
+      cm.split(t, j, c);
+      const int o = fft_row(A.perm[j], l1, S.s1, S.rp) + c;
+      const Cpl<T> v = cx_mul(buf[o], A.t4a[j]);
+      buf[o] = Cpl<T>{v.re, -v.im};
+    }
+  }
+  __syncthreads();
+  fft_all<true>(buf, A.F, S.s1, cm, A.tw, nt);
+  for (int c = threadIdx.x; c < ncell; c += nt) {
+    const unsigned mn = A.cellmn[c];
+    const int m = mn & 0xffffu, n = mn >> 16;
+    T v;
+    if (pair) {
+      v = bt[2 * (fft_row(pair_pos(kind, m, M), l1, S.s1, S.rp) + (n >> 1)) + (n & 1)];
+    } else {
+      const int k = (m & 1) ? (M - 1 - m) >> 1 : m >> 1;
+      const Cpl<T> z = buf[fft_row(k, l1, S.s1, S.rp) + n];
+      const Cpl<T> y = cx_mul(Cpl<T>{z.re, -z.im}, A.t4b[k]);
+      v = (m & 1) ? (T)-2 * y.im : (T)2 * y.re;
+    }
+    if (flip && (m & 1)) v = -v;
+    u[c] = v;
+  }
+  __syncthreads();  // the shared memory is free for the next wavenumber
+}
+
+}  // namespace
+}  // namespace snac

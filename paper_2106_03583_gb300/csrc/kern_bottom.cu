@@ -13,8 +13,10 @@
 // coarsest plane solved through the eigen-decomposition of its symmetrised operator. From the zero
 // iterate of each level, the first colour-0 half-sweep is u = f / diag, which is written directly.
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
+#include "direct_dev.cuh"
 #include "kern_common.cuh"
 #include "snac_impl.h"
 #include "transform_dev.cuh"
@@ -413,12 +415,23 @@ struct OnchipArgs {
   int max_cycles;
   int* cycles;              // per wavenumber: V-cycles run
   double* norm2;            // per wavenumber: ||r_q||^2 on return
+  int direct;               // separable plans: the direct solve (direct_dev.cuh) in place of the V-cycles
+  DirectArgs<T> D;
 };
 
 // One wavenumber's solve, from a zero iterate, by one CTA.
 template <typename T>
 __device__ void onchip_mode(const OnchipArgs<T>& O, int q, unsigned char* smem_raw) {
   const BottomArgs<T>& A = O.B;
+  if (O.direct) {
+    const long long o = (long long)q * O.D.ncell;
+    plane_direct<T>(O.D, q, A.f_top + o, A.u_top + o, smem_raw, BT);
+    if (threadIdx.x == 0) {
+      O.cycles[q] = 1;
+      O.norm2[q] = 0.0;
+    }
+    return;
+  }
   const int nl = A.nlev;
   double* b = reinterpret_cast<double*>(smem_raw + A.coarse_off);
   double* y = b + MAX_COARSE;
@@ -690,11 +703,21 @@ OnchipArgs<T> onchip_args(snac_plan* P, double target) {
   O.max_cycles = P->max_cycles;
   O.cycles = P->dh_cycles;
   O.norm2 = P->dh_mode_norm2;
+  O.direct = P->direct.on ? 1 : 0;
+  if (P->direct.on) O.D = direct_args<T>(P);
   return O;
+}
+
+// Dynamic shared memory of one wavenumber's on-chip solve.
+template <typename T>
+size_t onchip_smem(const snac_plan* P) {
+  const DirectTab& D = P->direct;
+  return D.on ? plane_shape(D.fft, D.M, D.N, D.cls, sizeof(T), BT).bytes : bottom_layout(P, 0, sizeof(T)).bytes;
 }
 
 // algorithmic bytes and flops of one on-chip V-cycle of one wavenumber, and of its load and store
 double onchip_cycle_flops(const snac_plan* P) {
+  if (P->direct.on) return (5.0 * std::log2((double)P->direct.M) + 28.0) * P->lev[0].ncell / 4.0;  // one direct solve
   double fl = 0.0;
   const int L = (int)P->lev.size() - 1;
   for (int l = 0; l < L; ++l) fl += (double)P->lev[l].ncell * (12.0 * (P->nu1 + P->nu2) + 15.0 + 8.0);
@@ -704,12 +727,11 @@ double onchip_cycle_flops(const snac_plan* P) {
 template <typename T>
 cudaError_t onchip_t(snac_plan* P, int nact, double target, cudaStream_t s) {
   const OnchipArgs<T> O = onchip_args<T>(P, target);
-  const BottomLayout lay = bottom_layout(P, 0, sizeof(T));
   cudaFuncSetAttribute(k_onchip<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, BOTTOM_MAX_SMEM);
   const double w = sizeof(T);
   // per wavenumber: f in, u out; the flops of an assumed 4 cycles (the kernel decides how many run)
   LaunchScope ls(P, K_ONCHIP, 2.0 * w * (double)P->lev[0].ncell * nact, 4.0 * onchip_cycle_flops(P) * nact, s);
-  k_onchip<T><<<nact, BT, lay.bytes, s>>>(O);
+  k_onchip<T><<<nact, BT, onchip_smem<T>(P), s>>>(O);
   return cudaGetLastError();
 }
 
@@ -822,7 +844,7 @@ constexpr int fused_tc() {
 template <typename T>
 size_t fused_smem(const snac_plan* P) {
   const size_t fft = 2 * (size_t)(P->nzt / 2) * fused_tc<T>() * sizeof(Cx<T>);
-  return std::max(fft, bottom_layout(P, 0, sizeof(T)).bytes);
+  return std::max(fft, onchip_smem<T>(P));
 }
 
 template <typename T>
@@ -945,7 +967,7 @@ cudaError_t onchip_batch_t(snac_plan* const* plans, const double* targets, int n
   size_t smem = 0;
   for (int k = 0; k < nplans; ++k) {
     args[k] = onchip_args<T>(plans[k], targets[k]);
-    smem = std::max(smem, bottom_layout(plans[k], 0, sizeof(T)).bytes);
+    smem = std::max(smem, onchip_smem<T>(plans[k]));
   }
   char* base = static_cast<char*>(d_scratch);
   OnchipArgs<T>* d_args = reinterpret_cast<OnchipArgs<T>*>(base);

@@ -1,0 +1,507 @@
+// Separable solve of the reduced equations (Eq. 9) for planes too large for one CTA's shared memory:
+// three passes over the mode-space field, each reading and writing it once --
+//   k_lines_fwd  transform along the uniform plane axis, planes -> spectral [q][n][kappa]
+//   k_tri        one tridiagonal system per (q, kappa) along the other axis, in place
+//   k_lines_bwd  inverse transform, spectral -> planes
+// and the plan-side tables of the method (see direct_dev.cuh for the transforms and the systems).
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "direct_dev.cuh"
+
+namespace snac {
+namespace {
+
+constexpr int LNT = 256;  // threads of a line-transform CTA
+
+// Shared memory of a line-transform CTA: C = 2^lc complex columns of F.n rows.
+__host__ __device__ inline int line_s1(const FftTab& F, int lc) { return (F.l1 << lc) + 4; }
+__host__ __device__ inline size_t line_smem(const FftTab& F, int lc, size_t w) {
+  return 2 * w * (size_t)(F.n / F.l1) * line_s1(F, lc);
+}
+
+struct ColsShift {
+  int lc;
+  __device__ __forceinline__ int cols() const { return 1 << lc; }
+  __device__ __forceinline__ int pitch() const { return 1 << lc; }
+  __device__ __forceinline__ void split(int t, int& idx, int& c) const {
+    idx = t >> lc;
+    c = t & ((1 << lc) - 1);
+  }
+  // a warp covers 4 columns x 8 indices (32-byte segments of 8 lines' contiguous data)
+  __device__ __forceinline__ void split8(int t, int& idx, int& c) const {
+    const int cl = lc < 2 ? lc : 2;
+    const int lo = t & ((1 << cl) - 1), kk = (t >> cl) & 7, hi = t >> (cl + 3);
+    const int ch = lc - cl;
+    c = ((hi & ((1 << ch) - 1)) << cl) | lo;
+    idx = ((hi >> ch) << 3) | kk;
+  }
+  __device__ __forceinline__ int total8(int rows) const { return ((rows + 7) & ~7) << lc; }
+};
+
+// Lines of one CTA: global line number g = q N + n; per line the plane base of q and n.
+struct LineSet {
+  long long* plane;  // q ncell, or -1 past the last line
+  int* n;
+};
+
+template <typename T>
+__device__ __forceinline__ long long line_off(const DirectArgs<T>& A, const LineSet& S, int l, int m) {
+  const int n = S.n[l];
+  const int b = A.nbm == 1 ? 0 : A.mblk[m];
+  return S.plane[l] + A.base[n * A.nbm + b] + (long long)m * A.mstr[n];
+}
+
+template <typename T>
+__device__ __forceinline__ int line_setup(const DirectArgs<T>& A, int lines, long long* plane, int* ln) {
+  const int g0 = blockIdx.x * lines;
+  const int total = A.nq * A.N;
+  for (int l = threadIdx.x; l < lines; l += LNT) {
+    const int g = g0 + l;
+    const int q = g / A.N;
+    plane[l] = g < total ? (long long)q * A.ncell : -1;
+    ln[l] = g < total ? g - q * A.N : 0;
+  }
+  __syncthreads();
+  return g0;
+}
+
+constexpr int MAX_LINES = 64;
+constexpr int LB = 4;  // loads of a batch in flight per thread
+
+template <typename T>
+__global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_fwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
+                                                                         T* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ long long plane[MAX_LINES];
+  __shared__ int ln[MAX_LINES];
+  Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
+  T* bt = reinterpret_cast<T*>(smem);
+  const ColsShift cm{lc};
+  const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
+  const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
+  const int lines = pair ? 2 * C : C;
+  const int g0 = line_setup(A, lines, plane, ln);
+  const LineSet S{plane, ln};
+  const int nlive = min(lines, A.nq * A.N - g0);
+  if (pair) {
+    if (A.xl) {  // items: two consecutive cells of both lines of a column
+      const int total = cm.total8(M / 2);
+      for (int t0 = threadIdx.x; t0 < total; t0 += LB * LNT) {
+        Cpl<T> a[LB], b[LB];
+#pragma unroll
+        for (int u = 0; u < LB; ++u) {
+          int h, c;
+          cm.split8(t0 + u * LNT, h, c);
+          a[u] = b[u] = Cpl<T>{0, 0};
+          if (t0 + u * LNT < total && 2 * h < M) {
+            const int m = 2 * h;
+            if (A.vec) {
+              if (2 * c < nlive) a[u] = *reinterpret_cast<const Cpl<T>*>(in + line_off(A, S, 2 * c, m));
+              if (2 * c + 1 < nlive) b[u] = *reinterpret_cast<const Cpl<T>*>(in + line_off(A, S, 2 * c + 1, m));
+            } else {
+              if (2 * c < nlive) a[u] = Cpl<T>{in[line_off(A, S, 2 * c, m)], in[line_off(A, S, 2 * c, m + 1)]};
+              if (2 * c + 1 < nlive) b[u] = Cpl<T>{in[line_off(A, S, 2 * c + 1, m)], in[line_off(A, S, 2 * c + 1, m + 1)]};
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < LB; ++u) {
+          int h, c;
+          cm.split8(t0 + u * LNT, h, c);
+          if (t0 + u * LNT >= total || 2 * h >= M) continue;
+          if (flip) a[u].im = -a[u].im, b[u].im = -b[u].im;
+          buf[fft_row(pair_pos(kind, 2 * h, M), l1, s1, C) + c] = Cpl<T>{a[u].re, b[u].re};
+          buf[fft_row(pair_pos(kind, 2 * h + 1, M), l1, s1, C) + c] = Cpl<T>{a[u].im, b[u].im};
+        }
+      }
+    } else {  // the lines are adjacent in memory: one element of both lines of a column
+      const int total = M << lc;
+      for (int t0 = threadIdx.x; t0 < total; t0 += 2 * LB * LNT) {
+        Cpl<T> v[2 * LB];
+#pragma unroll
+        for (int u = 0; u < 2 * LB; ++u) {
+          int m, c;
+          cm.split(t0 + u * LNT, m, c);
+          v[u] = Cpl<T>{0, 0};
+          if (t0 + u * LNT < total) {
+            if (A.vec) {
+              if (2 * c < nlive) v[u] = *reinterpret_cast<const Cpl<T>*>(in + line_off(A, S, 2 * c, m));
+            } else {
+              if (2 * c < nlive) v[u].re = in[line_off(A, S, 2 * c, m)];
+              if (2 * c + 1 < nlive) v[u].im = in[line_off(A, S, 2 * c + 1, m)];
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 2 * LB; ++u) {
+          int m, c;
+          cm.split(t0 + u * LNT, m, c);
+          if (t0 + u * LNT >= total) continue;
+          if (flip && (m & 1)) v[u] = Cpl<T>{-v[u].re, -v[u].im};
+          buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c] = v[u];
+        }
+      }
+    }
+  } else {
+    // t_j and t_j' (j' = M/2 - 1 - j) from cells 2j, 2j+1, 2j', 2j'+1 of the column's line
+    const int h = M / 2, items = (h + 1) / 2, total = A.xl ? cm.total8(items) : items << lc;
+    for (int t = threadIdx.x; t < total; t += LNT) {
+      int j, c;
+      if (A.xl) cm.split8(t, j, c);
+      else cm.split(t, j, c);
+      if (j >= items) continue;
+      const int jj = h - 1 - j;
+      Cpl<T> p{0, 0}, r{0, 0};
+      if (c < nlive) {
+        p = Cpl<T>{in[line_off(A, S, c, 2 * j)], in[line_off(A, S, c, 2 * j + 1)]};
+        r = Cpl<T>{in[line_off(A, S, c, 2 * jj)], in[line_off(A, S, c, 2 * jj + 1)]};
+      }
+      if (flip) p.im = -p.im, r.im = -r.im;
+      buf[fft_row(j, l1, s1, C) + c] = cx_mul(Cpl<T>{p.re, r.im}, A.t4a[j]);
+      buf[fft_row(jj, l1, s1, C) + c] = cx_mul(Cpl<T>{r.re, p.im}, A.t4a[jj]);
+    }
+  }
+  __syncthreads();
+  fft_all<false>(buf, A.F, s1, cm, A.tw, LNT);
+  // spectra: line g of the CTA at out[g M + kappa]
+  T* o0 = out + (long long)g0 * M;
+  if (pair) {
+    const int total = cm.total8(M / 2 + 1);
+    for (int t = threadIdx.x; t < total; t += LNT) {
+      int k, c;
+      cm.split8(t, k, c);
+      if (2 * k > M) continue;
+      const Cpl<T> z1 = buf[fft_row(A.perm[k], l1, s1, C) + c];
+      const Cpl<T> z2 = k == 0 ? z1 : buf[fft_row(A.perm[M - k], l1, s1, C) + c];
+      Cpl<T> y1, y2;
+      pair_post(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], z1, z2, y1, y2);
+      T* oa = o0 + (long long)(2 * c) * M;
+      const bool mirror = k > 0 && 2 * k < M;
+      if (2 * c < nlive) {
+        oa[k] = y1.re;
+        if (mirror) oa[M - k] = y2.re;
+      }
+      if (2 * c + 1 < nlive) {
+        oa[M + k] = y1.im;
+        if (mirror) oa[M + M - k] = y2.im;
+      }
+    }
+  } else {
+    const int h = M / 2, items = (h + 1) / 2, total = cm.total8(items);
+    for (int t = threadIdx.x; t < total; t += LNT) {
+      int k, c;
+      cm.split8(t, k, c);
+      if (k >= items || c >= nlive) continue;
+      const int kk = h - 1 - k;
+      const Cpl<T> v = cx_mul(buf[fft_row(A.perm[k], l1, s1, C) + c], A.t4b[k]);
+      const Cpl<T> w = cx_mul(buf[fft_row(A.perm[kk], l1, s1, C) + c], A.t4b[kk]);
+      T* o = o0 + (long long)c * M;
+      o[2 * k] = (T)2 * v.re;
+      o[2 * k + 1] = (T)-2 * w.im;
+      o[2 * kk] = (T)2 * w.re;
+      o[2 * kk + 1] = (T)-2 * v.im;
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_bwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
+                                                                         T* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ long long plane[MAX_LINES];
+  __shared__ int ln[MAX_LINES];
+  Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
+  const ColsShift cm{lc};
+  const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
+  const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
+  const int lines = pair ? 2 * C : C;
+  const int g0 = line_setup(A, lines, plane, ln);
+  const LineSet S{plane, ln};
+  const int nlive = min(lines, A.nq * A.N - g0);
+  const T* i0 = in + (long long)g0 * M;
+  if (pair) {
+    const int total = cm.total8(M / 2 + 1);
+    for (int t0 = threadIdx.x; t0 < total; t0 += LB * LNT) {
+      Cpl<T> x1[LB], x2[LB];
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        int k, c;
+        cm.split8(t0 + u * LNT, k, c);
+        x1[u] = x2[u] = Cpl<T>{0, 0};
+        if (t0 + u * LNT < total && 2 * k <= M) {
+          const T* ia = i0 + (long long)(2 * c) * M;
+          const bool two = k > 0 && !(kind == KIND_PP && 2 * k == M);
+          if (2 * c < nlive) {
+            x1[u].re = ia[k];
+            if (two) x2[u].re = ia[M - k];
+          }
+          if (2 * c + 1 < nlive) {
+            x1[u].im = ia[M + k];
+            if (two) x2[u].im = ia[M + M - k];
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        int k, c;
+        cm.split8(t0 + u * LNT, k, c);
+        if (t0 + u * LNT >= total || 2 * k > M) continue;
+        Cpl<T> z1, z2;
+        pair_pre(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], x1[u], x2[u], z1, z2);
+        buf[fft_row(A.perm[k], l1, s1, C) + c] = z1;
+        if (k > 0 && 2 * k < M) buf[fft_row(A.perm[M - k], l1, s1, C) + c] = z2;
+      }
+    }
+  } else {
+    const int h = M / 2, items = (h + 1) / 2, total = cm.total8(items);
+    for (int t = threadIdx.x; t < total; t += LNT) {
+      int j, c;
+      cm.split8(t, j, c);
+      if (j >= items) continue;
+      const int jj = h - 1 - j;
+      Cpl<T> p{0, 0}, r{0, 0};
+      if (c < nlive) {
+        const T* i = i0 + (long long)c * M;
+        p = Cpl<T>{i[2 * j], i[2 * j + 1]};
+        r = Cpl<T>{i[2 * jj], i[2 * jj + 1]};
+      }
+      const Cpl<T> v = cx_mul(Cpl<T>{p.re, r.im}, A.t4a[j]), w = cx_mul(Cpl<T>{r.re, p.im}, A.t4a[jj]);
+      buf[fft_row(A.perm[j], l1, s1, C) + c] = Cpl<T>{v.re, -v.im};  // forward = conj(inverse(conj))
+      buf[fft_row(A.perm[jj], l1, s1, C) + c] = Cpl<T>{w.re, -w.im};
+    }
+  }
+  __syncthreads();
+  fft_all<true>(buf, A.F, s1, cm, A.tw, LNT);
+  if (pair) {
+    if (A.xl) {
+      const int total = cm.total8(M / 2);
+      for (int t = threadIdx.x; t < total; t += LNT) {
+        int h, c;
+        cm.split8(t, h, c);
+        const int m = 2 * h;
+        if (m >= M) continue;
+        const Cpl<T> e = buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c];
+        Cpl<T> o = buf[fft_row(pair_pos(kind, m + 1, M), l1, s1, C) + c];
+        if (flip) o = Cpl<T>{-o.re, -o.im};
+        if (A.vec) {
+          if (2 * c < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c, m)) = Cpl<T>{e.re, o.re};
+          if (2 * c + 1 < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c + 1, m)) = Cpl<T>{e.im, o.im};
+        } else {
+          if (2 * c < nlive) {
+            out[line_off(A, S, 2 * c, m)] = e.re;
+            out[line_off(A, S, 2 * c, m + 1)] = o.re;
+          }
+          if (2 * c + 1 < nlive) {
+            out[line_off(A, S, 2 * c + 1, m)] = e.im;
+            out[line_off(A, S, 2 * c + 1, m + 1)] = o.im;
+          }
+        }
+      }
+    } else {
+      const int total = M << lc;
+      for (int t = threadIdx.x; t < total; t += LNT) {
+        int m, c;
+        cm.split(t, m, c);
+        Cpl<T> v = buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c];
+        if (flip && (m & 1)) v = Cpl<T>{-v.re, -v.im};
+        if (A.vec) {
+          if (2 * c < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c, m)) = v;
+        } else {
+          if (2 * c < nlive) out[line_off(A, S, 2 * c, m)] = v.re;
+          if (2 * c + 1 < nlive) out[line_off(A, S, 2 * c + 1, m)] = v.im;
+        }
+      }
+    }
+  } else {
+    const int h = M / 2, items = (h + 1) / 2, total = A.xl ? cm.total8(items) : items << lc;
+    for (int t = threadIdx.x; t < total; t += LNT) {
+      int k, c;
+      if (A.xl) cm.split8(t, k, c);
+      else cm.split(t, k, c);
+      if (k >= items || c >= nlive) continue;
+      const int kk = h - 1 - k;
+      const Cpl<T> z = buf[fft_row(k, l1, s1, C) + c], y = buf[fft_row(kk, l1, s1, C) + c];
+      const Cpl<T> v = cx_mul(Cpl<T>{z.re, -z.im}, A.t4b[k]), w = cx_mul(Cpl<T>{y.re, -y.im}, A.t4b[kk]);
+      const T sg = flip ? (T)2 : (T)-2;  // cells 2k + 1 carry -2 Im, sign-flipped for DN
+      out[line_off(A, S, c, 2 * k)] = (T)2 * v.re;
+      out[line_off(A, S, c, 2 * k + 1)] = sg * w.im;
+      out[line_off(A, S, c, 2 * kk)] = (T)2 * w.re;
+      out[line_off(A, S, c, 2 * kk + 1)] = sg * v.im;
+    }
+  }
+}
+
+// FP32: KG systems x P segments of TRI_R rows per CTA, the rows in registers: the field is read and
+// written once (a sequential sweep per system would write and re-read both factors).
+constexpr int TRI_R = 16;
+
+template <typename T, int KG>
+__global__ void __launch_bounds__(1024, 1) k_tri_seg(const DirectArgs<T> A, int P, const unsigned char* __restrict__ low,
+                                                   T* __restrict__ x) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int kk = threadIdx.x % KG, seg = threadIdx.x / KG;
+  const long long sys = (long long)blockIdx.x * KG + kk;
+  const bool live = sys < (long long)A.nq * A.M && !low[sys];  // (k_tri_low solves the others)
+  const int q = live ? (int)(sys / A.M) : 0, kap = live ? (int)(sys - (long long)q * A.M) : 0;
+  T* col = x + (long long)q * A.N * A.M + kap;
+  const T tq = live ? -fma(A.sigma[q], A.cscale, A.lam[kap]) : (T)1;
+  tri_segment<T, TRI_R>(A.tri, A.N, P, seg, kk, KG, true, live, tq, A.scale, reinterpret_cast<T*>(smem),
+                        [&](int n) { return col[(long long)n * A.M]; },
+                        [&](int n, T v) { col[(long long)n * A.M] = v; });
+}
+
+// The smoothest systems of an FP32 plan in FP64 arithmetic (FP32 right-hand side and solution). A
+// rounded elimination leaves errors that differ from row to row, relative to the solution; the outer
+// residual sees them times the row coupling (1e6 and more on a stretched axis), and the solution is
+// largest where lambda + sigma is smallest. These few systems (list) therefore set the residual a
+// correction step can reach: with all of them in FP32 the second step on the 1024 x 512 x 512 channel ends
+// at 0.9-1.5e-10 relative residual, with the list in FP64 at 5e-11.
+constexpr int LOW_KG = 8, LOW_R = 8;
+__global__ void __launch_bounds__(512, 1) k_tri_low(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
+                                                  const double* __restrict__ sigma, double cscale, double scale,
+                                                  const int* __restrict__ list, int nlist, int M, int N, int P,
+                                                  float* __restrict__ x) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int kk = threadIdx.x % LOW_KG, seg = threadIdx.x / LOW_KG;
+  const int k = blockIdx.x * LOW_KG + kk;
+  const bool live = k < nlist;
+  const int sys = live ? list[k] : 0;
+  const int q = sys / M, kap = sys - q * M;
+  float* col = x + (long long)q * N * M + kap;
+  const double tq = live ? -fma(sigma[q], cscale, lam[kap]) : 1.0;
+  tri_segment<double, LOW_R>(tri, N, P, seg, kk, LOW_KG, true, live, tq, scale, reinterpret_cast<double*>(smem),
+                             [&](int n) { return (double)col[(long long)n * M]; },
+                             [&](int n, double v) { col[(long long)n * M] = (float)v; });
+}
+
+// One thread per system, rows in order: fewest operations per row (the FP64 plans are bound by the
+// FP64 pipe, not by the extra pass over the factors c, kept in the plan's other mode buffer). S: the
+// arithmetic's type.
+template <typename T, typename S>
+__global__ void __launch_bounds__(128) k_tri_seq(const TriRow<S>* __restrict__ tri, const S* __restrict__ lam,
+                                               const S* __restrict__ sigma, S cscale, S scale, int nq, int M, int N,
+                                               T* __restrict__ x, S* __restrict__ cw) {
+  const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (sys >= (long long)nq * M) return;
+  const int q = (int)(sys / M), kap = (int)(sys - (long long)q * M);
+  const long long o = (long long)q * N * M + kap;
+  x += o;
+  cw += o;
+  const S tq = -fma(sigma[q], cscale, lam[kap]);
+  constexpr int U = 8;
+  S g = 0, d = 0;
+  for (int n0 = 0; n0 < N; n0 += U) {
+    T v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = n0 + u < N ? x[(long long)(n0 + u) * M] : (T)0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (n0 + u >= N) break;
+      const TriRow<S> w = tri[n0 + u];
+      const S s = fma(w.lo, g, w.tau + tq);
+      const S den = s + w.hi;
+      const S inv = den > (S)0 ? tri_recip(den) : (S)0;
+      g = s * inv;
+      d = fma(w.lo, d, -scale * (S)v[u]) * inv;
+      x[(long long)(n0 + u) * M] = (T)d;
+      cw[(long long)(n0 + u) * M] = w.hi * inv;
+    }
+  }
+  S y = 0;
+  for (int n0 = (N - 1) / U * U; n0 >= 0; n0 -= U) {
+    T v[U];
+    S c[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool in = n0 + u < N;
+      v[u] = in ? x[(long long)(n0 + u) * M] : (T)0;
+      c[u] = in ? cw[(long long)(n0 + u) * M] : (S)0;
+    }
+#pragma unroll
+    for (int u = U - 1; u >= 0; --u) {
+      if (n0 + u >= N) continue;
+      y = fma(c[u], y, (S)v[u]);
+      x[(long long)(n0 + u) * M] = (T)y;
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_nonfinite(const T* __restrict__ v, long long n, int* __restrict__ flag) {
+  bool bad = false;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    bad = bad || !isfinite(v[i]);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
+}
+
+template <typename T>
+cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
+  const DirectArgs<T> A = direct_args<T>(P);
+  const double cells = (double)P->nz * P->lev[0].ncell, w = sizeof(T);
+  // complex columns per line CTA: about 32 KB of shared memory, 2 to 16 columns
+  int lc = 1;
+  while (lc < 4 && ((size_t)A.F.n << (lc + 1)) * 2 * w <= 36 * 1024) ++lc;
+  const int lines = A.cls == LINES_PAIR ? 2 << lc : 1 << lc;
+  const long long total = (long long)A.nq * A.N;
+  const unsigned grid = (unsigned)((total + lines - 1) / lines);
+  const size_t smem = line_smem(A.F, lc, w);
+  T* f = (T*)P->lev[0].d_f;
+  T* u = (T*)P->lev[0].d_u;
+  const double fl = (2.5 * std::log2((double)A.M) + 4.0) * cells;
+  constexpr int kMax = 160 * 1024;  // the largest need (4096-point FP64 lines): function-wide, never lowered
+  {
+    LaunchScope ls(P, K_LINES_FWD, 2.0 * w * cells, fl, s);
+    cudaFuncSetAttribute(k_lines_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    k_lines_fwd<T><<<grid, LNT, smem, s>>>(A, lc, f, u);
+  }
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  {
+    LaunchScope ls(P, K_TRI, 2.0 * w * cells, 20.0 * cells, s);
+    const long long sys = (long long)A.nq * A.M;
+    const int segs = (A.N + TRI_R - 1) / TRI_R;
+    if constexpr (sizeof(T) == 4) {
+      const DirectTab& D = P->direct;
+      const int lsegs = (A.N + LOW_R - 1) / LOW_R;
+      if (D.nlow)
+        k_tri_low<<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
+            (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / (2.0 * A.M), D.d_lowlist,
+            D.nlow, A.M, A.N, lsegs, u);
+      if (segs <= 32) {
+        k_tri_seg<T, 32><<<(unsigned)((sys + 31) / 32), 32 * segs, 7 * sizeof(T) * 32 * segs, s>>>(A, segs, D.d_low, u);
+      } else if (segs <= 64) {
+        k_tri_seg<T, 16><<<(unsigned)((sys + 15) / 16), 16 * segs, 7 * sizeof(T) * 16 * segs, s>>>(A, segs, D.d_low, u);
+      } else {
+        k_tri_seq<T, T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A.tri, A.lam, A.sigma, A.cscale, A.scale, A.nq,
+                                                                      A.M, A.N, u, f);
+      }
+    } else {
+      k_tri_seq<T, T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A.tri, A.lam, A.sigma, A.cscale, A.scale, A.nq,
+                                                                      A.M, A.N, u, f);
+    }
+  }
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  {
+    LaunchScope ls(P, K_LINES_BWD, 2.0 * w * cells, fl, s);
+    cudaFuncSetAttribute(k_lines_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    k_lines_bwd<T><<<grid, LNT, smem, s>>>(A, lc, u, f);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStream_t s) {
+  *P->h_wait = 0;
+  if (P->precision == SNAC_FP64) k_nonfinite<double><<<4 * P->sms, 256, 0, s>>>((const double*)v, n, P->dh_wait);
+  else k_nonfinite<float><<<4 * P->sms, 256, 0, s>>>((const float*)v, n, P->dh_wait);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_direct(snac_plan* P, cudaStream_t s) {
+  return P->precision == SNAC_FP64 ? direct_t<double>(P, s) : direct_t<float>(P, s);
+}
+
+}  // namespace snac

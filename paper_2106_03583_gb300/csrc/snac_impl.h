@@ -159,10 +159,45 @@ struct TwiddleOffsets {
   int fft, twn, tw2n, tw4a, tw4b, total;
 };
 
+// Passes of an in-place shared-memory FFT of length n (fft_dev.cuh): pass s splits spans of span[s]
+// points by rad[s]; l1 = n / rad[0].
+constexpr int FFT_MAX_PASS = 12;
+struct FftTab {
+  int n, np, l1;
+  int rad[FFT_MAX_PASS], span[FFT_MAX_PASS];
+};
+
+// Separable plans (the blocks assemble into a rectangle with a uniform plane axis): the reduced
+// equations are solved by a transform along that axis and tridiagonal systems along the other
+// (direct_dev.cuh). Tables in the plan's inner type.
+struct DirectTab {
+  bool on = false;
+  int M = 0, N = 0;        // cells along the transformed / the tridiagonal axis
+  int cls = 0, kind = 0;   // LINES_PAIR / LINES_DCT4; boundary pair of the transformed axis
+  int xl = 0, vec = 0, nbm = 1;
+  FftTab fft{};
+  int w2n = 0, t4a = 0, t4b = 0;  // offsets in the twiddle table
+  double cscale = 1.0;
+  int nlow = 0;                      // mixed plans: systems solved in FP64 arithmetic (k_tri_low)
+  int* d_lowlist = nullptr;          // their numbers q M + kappa
+  unsigned char* d_low = nullptr;    // per system: 1 if listed
+  void* d_tw = nullptr;
+  int* d_perm = nullptr;
+  void* d_lam = nullptr;
+  void* d_tri = nullptr;
+  double* d_lam64 = nullptr;  // the same in FP64 (mixed plans; FP64 plans: the tables above)
+  double* d_tri64 = nullptr;
+  unsigned* d_cellmn = nullptr;
+  int* d_base = nullptr;
+  int* d_mblk = nullptr;
+  int* d_mstr = nullptr;
+};
+
 // Kernel kinds counted by the tracing facility.
 enum KernelKind {
   K_FIELD3D = 0, K_REDUCE, K_FIX_MEAN, K_SHIFT, K_FORWARD, K_BACKWARD, K_SMOOTH, K_RESTRICT, K_PROLONG,
-  K_COARSE, K_MODE_RESID, K_MODE_REDUCE, K_MODE_APPLY, K_FDOWN, K_FUP, K_BOTTOM, K_FIELD3D_FF, K_ONCHIP, K_FWD_ONCHIP, K_COUNT
+  K_COARSE, K_MODE_RESID, K_MODE_REDUCE, K_MODE_APPLY, K_FDOWN, K_FUP, K_BOTTOM, K_FIELD3D_FF, K_ONCHIP, K_FWD_ONCHIP,
+  K_LINES_FWD, K_TRI, K_LINES_BWD, K_COUNT
 };
 
 struct KernelStat {
@@ -196,6 +231,7 @@ struct snac_plan {
   int onchip_opt = 0;         // snac_options.onchip
   int bottom_cells = 0;       // snac_options.bottom_cells
   void* d_onchip = nullptr;   // BottomLevel<inner type> table from level 0
+  snac::DirectTab direct;     // separable plans: direct solves of the reduced equations
   double* d_pweight = nullptr;
   int* h_cycles = nullptr;    // per wavenumber: V-cycles of the last on-chip solve (mapped pinned)
   int* dh_cycles = nullptr;
@@ -393,6 +429,16 @@ struct BottomLayout {
   size_t bytes;
 };
 BottomLayout bottom_layout(const snac_plan* P, int lb, size_t w);
+// Separable plans: every wavenumber's solution of the reduced equations for the right-hand sides in
+// lev[0].d_f (plain order), into mode_solution(P).
+cudaError_t launch_direct(snac_plan* P, cudaStream_t s);
+// *h_wait = 1 if any of the n values (inner type) is NaN or Inf, else 0.
+cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStream_t s);
+// Where a solve leaves the mode-space solution: the level-0 iterate, or (direct solves of planes too
+// large for one CTA, whose last pass goes back to the planes' order) the level-0 right-hand side.
+inline void* mode_solution(const snac_plan* P) {
+  return P->direct.on && !P->onchip ? P->lev[0].d_f : P->lev[0].d_u;
+}
 // Small transfers through mapped pinned memory, done by one-CTA kernels (no copy engine).
 cudaError_t launch_to_host(const double* d_src, double* dh_dst, int n, cudaStream_t s);
 cudaError_t launch_from_host(const int* dh_src, int* d_dst, int n, cudaStream_t s);

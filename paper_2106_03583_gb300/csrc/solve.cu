@@ -301,7 +301,26 @@ void mode_solves_many(const std::vector<ModeRun*>& runs, Wait&& wait) {
     if (r->st == SNAC_OK) r->finish();
 }
 
+// A direct solve counts as one cycle of every wavenumber.
+void direct_results(snac_plan* P, int* cycles_out) {
+  std::fill(cycles_out, cycles_out + P->nz, 1);
+  P->info.total_cycles += P->nz;
+}
+
 int mode_solves(snac_plan* P, double target, cudaStream_t s, int* cycles_out) {
+  if (P->direct.on) {  // (the V-cycle paths see a non-finite right-hand side in its norms)
+    CK(launch_nonfinite(P, P->lev[0].d_f, (long long)P->nz * P->lev[0].ncell, s));
+    CK(cudaStreamSynchronize(s));
+    if (*P->h_wait) {
+      *P->h_wait = 0;
+      return SNAC_ERR_NONFINITE;
+    }
+    if (!P->onchip) {
+      CK(launch_direct(P, s));
+      direct_results(P, cycles_out);
+      return SNAC_OK;
+    }
+  }
   if (P->onchip) {  // every wavenumber's whole solve in one CTA; convergence decided on the device
     const int st = set_active_all(P, s);
     if (st) return st;
@@ -425,7 +444,9 @@ cudaError_t job_resid_read(Job& J, cudaStream_t s) {
   if (J.k == 0 && J.p_zero) return cudaSuccess;
   if (J.ff && !J.redo) {
     J.rn = std::sqrt(P->h_sums[0]);
-    J.r32 = !(J.rn <= 2.0 * J.tol * J.fn);  // (NaN stays: reported by the decision)
+    // (NaN stays: reported by the decision). Direct plans take another step anyway above half the
+    // tolerance, where the float-float value decides as well
+    J.r32 = !(J.rn <= (P->direct.on && J.k < P->max_outer ? 0.5 : 2.0) * J.tol * J.fn);
     if (J.r32) return cudaSuccess;
     J.redo = true;
     const bool need_vp = P->singular;
@@ -460,7 +481,12 @@ int job_decide(Job& J, cudaStream_t s) {
   }
   const double rel = rn / fn;
   P->info.rel_res = rel;
-  const bool done = rel <= J.tol;
+  // Direct solves in FP32 stop at half the tolerance where they can: what is left after such a step lies
+  // in the smoothest modes, where a residual just under the tolerance still means several times as much
+  // error in p, and one more step takes it away (measured on the 2.7e8-cell channel at 1e-10: residual
+  // 5-9e-11 and error 3-6e-10 after two steps, 2.5e-13 and below 1e-14 after three)
+  const bool margin = P->direct.on && P->precision == SNAC_MIXED && J.k > 0 && J.k < P->max_outer;
+  const bool done = rel <= (margin ? 0.5 * J.tol : J.tol);
   // a correction that did not lower the residual: the inner solve has reached the floating-point
   // floor of the outer residual (or diverged); more steps would not help
   const bool stalled = J.updated && rel >= J.prev_rel;
@@ -474,12 +500,12 @@ int job_decide(Job& J, cudaStream_t s) {
     if (stalled) {
       // return the better iterate: take the last correction back (its modes are still in the
       // level-0 iterate) and report the residual of what is returned, re-evaluated
-      CK(launch_backward_update(P, P->lev[0].d_u, J.p, s, true));
+      CK(launch_backward_update(P, mode_solution(P), J.p, s, true));
       CK(launch_field3d(P, 0, J.f, J.p, P->d_r3, J.fshift, false, false, s));
       if ((st = read_sums(P, s))) return st;
       P->info.rel_res = std::sqrt(P->h_sums[0]) / fn;
     }
-    J.finish(done ? SNAC_OK : SNAC_ERR_NOT_CONVERGED);
+    J.finish(done || P->info.rel_res <= J.tol ? SNAC_OK : SNAC_ERR_NOT_CONVERGED);
     return SNAC_OK;
   }
   J.prev_rel = rel;
@@ -489,15 +515,22 @@ int job_decide(Job& J, cudaStream_t s) {
   J.target = 0.5 * J.tol * fn;
   if (P->precision == SNAC_MIXED && P->inner_reduction * rn > J.tol * fn) J.target = P->inner_reduction * rn;
   J.aim_final = J.target <= 0.5 * J.tol * fn;
+  if (P->direct.on && P->precision == SNAC_MIXED) {
+    // a direct step reduces the residual to the FP32 floor whatever the target: by 1e-4 or so from f, by
+    // about 3e-7 from the rough residual that such a step leaves. The FP64 pass comes directly where
+    // that reaches the tolerance (with the margin above)
+    J.aim_final = J.k > 0 && 3e-7 * rel <= 0.5 * J.tol;
+  }
   J.fused = fused_ready(P);
   if (J.fused) {  // the forward transform goes into the same launch as the wavenumber solves
     if (J.k == 0 && J.p_zero) J.fin = FusedInput{J.f, false, J.fshift};
     else J.fin = FusedInput{P->d_r3, J.r32, 0.0};
     return SNAC_OK;
   }
-  if (J.k == 0 && J.p_zero) CK(launch_forward(P, J.f, P->lev[0].d_f, J.fshift, P->scaled_f, s));
+  const bool split = P->scaled_f && !P->direct.on;
+  if (J.k == 0 && J.p_zero) CK(launch_forward(P, J.f, P->lev[0].d_f, J.fshift, split, s));
   else if (J.r32) CK(launch_forward_f32(P, reinterpret_cast<const float*>(P->d_r3), P->lev[0].d_f, s));
-  else CK(launch_forward(P, P->d_r3, P->lev[0].d_f, 0.0, P->scaled_f, s));
+  else CK(launch_forward(P, P->d_r3, P->lev[0].d_f, 0.0, split, s));
   return SNAC_OK;
 }
 
@@ -509,8 +542,8 @@ cudaError_t job_update(Job& J, cudaStream_t s) {
     P->info.max_mode_cycles = std::max(P->info.max_mode_cycles, J.cyc[q]);
   }
   cudaError_t e = cudaSuccess;
-  if (P->singular) e = launch_fix_mean(P, P->lev[0].d_u, s);
-  if (e == cudaSuccess) e = launch_backward_update(P, P->lev[0].d_u, J.p, s);
+  if (P->singular) e = launch_fix_mean(P, mode_solution(P), s);
+  if (e == cudaSuccess) e = launch_backward_update(P, mode_solution(P), J.p, s);
   J.updated = true;
   ++J.k;
   return e;
@@ -686,11 +719,15 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
         for (Job* J : chip[g]) job_cuda(*J, e, "on-chip wavenumber solves");
     }
     if (status) break;
+    for (Job& J : jobs)  // direct solves of separable plans: launches only, nothing to wait for
+      if (!J.finished && J.P->direct.on && !J.P->onchip) {
+        if (job_cuda(J, launch_direct(J.P, js(J)), "direct wavenumber solves") == SNAC_OK) direct_results(J.P, J.cyc.data());
+      }
     {  // the level-by-level plans' wavenumber solves, in lock-step with one another
       std::vector<ModeRun> runs;
       std::vector<Job*> owners;
       for (Job& J : jobs)
-        if (!J.finished && !J.P->onchip) {
+        if (!J.finished && !J.P->onchip && !J.P->direct.on) {
           ModeRun r;
           r.P = J.P;
           r.s = js(J);
@@ -868,7 +905,7 @@ int snac_mode_solve(snac_plan* plan, const void* d_rhs, void* d_sol, double targ
   cudaStream_t s = (cudaStream_t)stream;
   const size_t bytes = (size_t)P->nz * P->lev[0].ncell * plan_inner_size(P);
   // the right-hand side into the level-0 buffer, in the order the cycles read it
-  if (P->scaled_f) CK(launch_to_split(P, (const double*)d_rhs, (double*)P->lev[0].d_f, s));
+  if (P->scaled_f && !P->direct.on) CK(launch_to_split(P, (const double*)d_rhs, (double*)P->lev[0].d_f, s));
   else CK(cudaMemcpyAsync(P->lev[0].d_f, d_rhs, bytes, cudaMemcpyDeviceToDevice, s));
   P->info = snac_solve_info{};
   P->info.levels = (int)P->lev.size();
@@ -882,7 +919,7 @@ int snac_mode_solve(snac_plan* plan, const void* d_rhs, void* d_sol, double targ
     P->mode_cycles[q] = cyc[q];
     P->info.max_mode_cycles = std::max(P->info.max_mode_cycles, cyc[q]);
   }
-  CK(cudaMemcpyAsync(d_sol, P->lev[0].d_u, bytes, cudaMemcpyDeviceToDevice, s));
+  CK(cudaMemcpyAsync(d_sol, mode_solution(P), bytes, cudaMemcpyDeviceToDevice, s));
   CK(cudaStreamSynchronize(s));
   profile_resolve(P);
   return SNAC_OK;
