@@ -103,7 +103,7 @@ __device__ __forceinline__ void pair_post(int kind, Cpl<T> w, Cpl<T> z1, Cpl<T> 
     y2 = {ai, bi};
   } else {
     y1 = {w.re * ar - w.im * ai, w.re * br - w.im * bi};
-    y2 = {-(w.im * ar + w.re * ai), -(w.im * br + w.re * bi)};
+    y2 = {-w.im * ar - w.re * ai, -w.im * br - w.re * bi};
   }
 }
 
@@ -113,9 +113,9 @@ __device__ __forceinline__ void pair_pre(int kind, Cpl<T> w, Cpl<T> x1, Cpl<T> x
   T ar = x1.re, ai = x2.re, br = x1.im, bi = x2.im;
   if (kind != KIND_PP) {
     ar = w.re * x1.re - w.im * x2.re;
-    ai = -(w.re * x2.re + w.im * x1.re);
+    ai = -w.re * x2.re - w.im * x1.re;
     br = w.re * x1.im - w.im * x2.im;
-    bi = -(w.re * x2.im + w.im * x1.im);
+    bi = -w.re * x2.im - w.im * x1.im;
   }
   z1 = {ar - bi, ai + br};
   z2 = {ar + bi, br - ai};
@@ -261,8 +261,7 @@ __device__ void plane_direct(const DirectArgs<T>& A, int q, const T* __restrict_
   for (int c = threadIdx.x; c < ncell; c += nt) {
     const unsigned mn = A.cellmn[c];
     const int m = mn & 0xffffu, n = mn >> 16;
-    T v = f[c];
-    if (flip && (m & 1)) v = -v;
+    const T v = neg_if(flip && (m & 1), f[c]);
     int o;
     if (pair) o = 2 * (fft_row(pair_pos(kind, m, M), l1, S.s1, S.rp) + (n >> 1)) + (n & 1);
     else o = 2 * (fft_row((m & 1) ? (M - 1 - m) >> 1 : m >> 1, l1, S.s1, S.rp) + n) + (m & 1);
@@ -360,8 +359,7 @@ __device__ void plane_direct(const DirectArgs<T>& A, int q, const T* __restrict_
       const Cpl<T> y = cx_mul(Cpl<T>{z.re, -z.im}, A.t4b[k]);
       v = (m & 1) ? (T)-2 * y.im : (T)2 * y.re;
     }
-    if (flip && (m & 1)) v = -v;
-    u[c] = v;
+    u[c] = neg_if(flip && (m & 1), v);
   }
   __syncthreads();  // the shared memory is free for the next wavenumber
 }

@@ -43,6 +43,12 @@ template <typename T>
 __device__ __forceinline__ Cpl<T> cx_mulc(Cpl<T> a, Cpl<T> b) {
   return {a.re * b.re + a.im * b.im, a.im * b.re - a.re * b.im};
 }
+// x with its sign flipped if f, on the integer pipe (a selected negation would go to the FP64 pipe)
+__device__ __forceinline__ double neg_if(bool f, double x) {
+  return __hiloint2double(__double2hiint(x) ^ (f ? (int)0x80000000 : 0), __double2loint(x));
+}
+__device__ __forceinline__ float neg_if(bool f, float x) { return f ? -x : x; }
+
 // multiplication by -i (forward) or +i (inverse)
 template <bool INV, typename T>
 __device__ __forceinline__ Cpl<T> rot(Cpl<T> a) {
@@ -161,13 +167,13 @@ __device__ __forceinline__ int quot16(int n, int d) {
 }
 
 // The columns of a buffer: item t of a pass is (index t / columns, column t % columns).
-template <int LC>
-struct ColsPow2 {
-  __device__ __forceinline__ int cols() const { return 1 << LC; }
-  __device__ __forceinline__ int pitch() const { return 1 << LC; }
+struct ColsShift {  // 2^lc columns
+  int lc;
+  __device__ __forceinline__ int cols() const { return 1 << lc; }
+  __device__ __forceinline__ int pitch() const { return 1 << lc; }
   __device__ __forceinline__ void split(int t, int& idx, int& c) const {
-    idx = t >> LC;
-    c = t & ((1 << LC) - 1);
+    idx = t >> lc;
+    c = t & ((1 << lc) - 1);
   }
 };
 struct ColsAny {

@@ -20,6 +20,7 @@
 #include "kern_common.cuh"
 #include "snac_impl.h"
 #include "transform_dev.cuh"
+#include "ztrans_dev.cuh"
 
 namespace snac {
 namespace {
@@ -563,6 +564,8 @@ struct FwdArgs {
   T* out;                // level-0 right-hand side, [q][cell]
   long long ncell;
   T sub0;                // F(1) x (mean removed from f), on mode 0 (k = 0 from a zero guess)
+  ZArgs<T> Z;            // smooth lengths (zs): the transform of ztrans_dev.cuh
+  int zs;
   int n, kind, in_f32, nchunks;
   int need;              // chunks a solve item waits for (nchunks; more only in the timeout self-test)
   int* done;             // chunks counted so far (zero at launch)
@@ -584,10 +587,17 @@ __device__ __forceinline__ int load_acquire(const int* p) {
 template <typename T, int TC>
 __device__ void fused_chunk(const FwdArgs<T>& F, int c, unsigned char* smem) {
   const ChunkDev ch = F.chunks[c];
-  const int sel = F.kind * 2 + F.in_f32;
+  const int sel = F.zs ? -1 - F.in_f32 : F.kind * 2 + F.in_f32;
 #define SNAC_FWD(KD, TI)                                                                                   \
   forward_chunk<T, TC, KD, TI, BT>(ch, F.blk, F.cb, F.n, F.tw, static_cast<const TI*>(F.in3), F.out, F.ncell, F.sub0, 0, smem)
   switch (sel) {
+    case -1:
+      z_forward<T, double>(F.Z, ch, F.blk, F.cb, static_cast<const double*>(F.in3), F.out, F.ncell, F.sub0, 0, smem, BT);
+      break;
+    case -2:
+      if constexpr (sizeof(T) == 4)
+        z_forward<T, float>(F.Z, ch, F.blk, F.cb, static_cast<const float*>(F.in3), F.out, F.ncell, F.sub0, 0, smem, BT);
+      break;
     case 2 * KIND_PP: SNAC_FWD(KIND_PP, double); break;
     case 2 * KIND_PP + 1: SNAC_FWD(KIND_PP, float); break;
     case 2 * KIND_NN: SNAC_FWD(KIND_NN, double); break;
@@ -813,14 +823,21 @@ __global__ void k_zero_ints(int* __restrict__ p, int n) {
 }
 
 template <typename T>
+int fwd_chunks(const snac_plan* P) {
+  return (int)(P->zsmooth ? P->zchunks.size() : sizeof(T) == 8 ? P->chunks64.size() : P->chunks32.size());
+}
+
+template <typename T>
 FwdArgs<T> fwd_args(snac_plan* P, const void* in3, bool in_f32, double shift0, int* done, int* status, int extra) {
   FwdArgs<T> F{};
   const bool f64 = sizeof(T) == 8;
-  F.chunks = f64 ? P->d_chunks64 : P->d_chunks32;
+  F.chunks = P->zsmooth ? P->d_zchunks : f64 ? P->d_chunks64 : P->d_chunks32;
   F.blk = P->lev[0].d_blk;
   F.cb = P->d_cblk;
   const Cx<T>* t = reinterpret_cast<const Cx<T>*>(f64 ? (const void*)P->d_tw64 : (const void*)P->d_tw32);
   F.tw = Tw<T>{t + P->tw.fft, t + P->tw.twn, t + P->tw.tw2n, t + P->tw.tw4a, t + P->tw.tw4b};
+  F.zs = P->zsmooth ? 1 : 0;
+  if (P->zsmooth) F.Z = z_args<T>(P, P->ztc);
   F.in3 = in3;
   F.out = (T*)P->lev[0].d_f;
   F.ncell = P->lev[0].ncell;
@@ -829,7 +846,7 @@ FwdArgs<T> fwd_args(snac_plan* P, const void* in3, bool in_f32, double shift0, i
   F.n = P->nzt;
   F.kind = P->kind;
   F.in_f32 = in_f32 ? 1 : 0;
-  F.nchunks = (int)(f64 ? P->chunks64.size() : P->chunks32.size());
+  F.nchunks = fwd_chunks<T>(P);
   F.need = F.nchunks + extra;
   F.done = done;
   F.status = status;
@@ -910,7 +927,7 @@ cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs
   std::vector<int4> items;
   size_t smem = 0;
   for (int k = 0; k < nplans; ++k)
-    for (int c = 0; c < (int)(sizeof(T) == 8 ? plans[k]->chunks64.size() : plans[k]->chunks32.size()); ++c)
+    for (int c = 0; c < fwd_chunks<T>(plans[k]); ++c)
       items.push_back(make_int4(0, k, c, 0));
   for (int k = 0; k < nplans; ++k)
     for (int q = 0; q < plans[k]->nz; ++q) items.push_back(make_int4(1, k, q, 0));

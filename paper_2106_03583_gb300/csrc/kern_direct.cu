@@ -21,15 +21,9 @@ __host__ __device__ inline size_t line_smem(const FftTab& F, int lc, size_t w) {
   return 2 * w * (size_t)(F.n / F.l1) * line_s1(F, lc);
 }
 
-struct ColsShift {
-  int lc;
-  __device__ __forceinline__ int cols() const { return 1 << lc; }
-  __device__ __forceinline__ int pitch() const { return 1 << lc; }
-  __device__ __forceinline__ void split(int t, int& idx, int& c) const {
-    idx = t >> lc;
-    c = t & ((1 << lc) - 1);
-  }
-  // a warp covers 4 columns x 8 indices (32-byte segments of 8 lines' contiguous data)
+// Columns of a line CTA: besides the split of fft_dev.cuh, one in which a warp covers 4 columns x 8
+// indices (32-byte segments of 8 lines' contiguous data).
+struct ColsLine : ColsShift {
   __device__ __forceinline__ void split8(int t, int& idx, int& c) const {
     const int cl = lc < 2 ? lc : 2;
     const int lo = t & ((1 << cl) - 1), kk = (t >> cl) & 7, hi = t >> (cl + 3);
@@ -71,14 +65,14 @@ constexpr int MAX_LINES = 64;
 constexpr int LB = 4;  // loads of a batch in flight per thread
 
 template <typename T>
-__global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_fwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
+__global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
                                                                          T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long plane[MAX_LINES];
   __shared__ int ln[MAX_LINES];
   Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
   T* bt = reinterpret_cast<T*>(smem);
-  const ColsShift cm{lc};
+  const ColsLine cm{{lc}};
   const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
   const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
   const int lines = pair ? 2 * C : C;
@@ -111,7 +105,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_fwd(const
           int h, c;
           cm.split8(t0 + u * LNT, h, c);
           if (t0 + u * LNT >= total || 2 * h >= M) continue;
-          if (flip) a[u].im = -a[u].im, b[u].im = -b[u].im;
+          a[u].im = neg_if(flip, a[u].im), b[u].im = neg_if(flip, b[u].im);
           buf[fft_row(pair_pos(kind, 2 * h, M), l1, s1, C) + c] = Cpl<T>{a[u].re, b[u].re};
           buf[fft_row(pair_pos(kind, 2 * h + 1, M), l1, s1, C) + c] = Cpl<T>{a[u].im, b[u].im};
         }
@@ -139,7 +133,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_fwd(const
           int m, c;
           cm.split(t0 + u * LNT, m, c);
           if (t0 + u * LNT >= total) continue;
-          if (flip && (m & 1)) v[u] = Cpl<T>{-v[u].re, -v[u].im};
+          v[u] = Cpl<T>{neg_if(flip && (m & 1), v[u].re), neg_if(flip && (m & 1), v[u].im)};
           buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c] = v[u];
         }
       }
@@ -158,7 +152,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_fwd(const
         p = Cpl<T>{in[line_off(A, S, c, 2 * j)], in[line_off(A, S, c, 2 * j + 1)]};
         r = Cpl<T>{in[line_off(A, S, c, 2 * jj)], in[line_off(A, S, c, 2 * jj + 1)]};
       }
-      if (flip) p.im = -p.im, r.im = -r.im;
+      p.im = neg_if(flip, p.im), r.im = neg_if(flip, r.im);
       buf[fft_row(j, l1, s1, C) + c] = cx_mul(Cpl<T>{p.re, r.im}, A.t4a[j]);
       buf[fft_row(jj, l1, s1, C) + c] = cx_mul(Cpl<T>{r.re, p.im}, A.t4a[jj]);
     }
@@ -207,13 +201,13 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_fwd(const
 }
 
 template <typename T>
-__global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_bwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
+__global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
                                                                          T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long plane[MAX_LINES];
   __shared__ int ln[MAX_LINES];
   Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
-  const ColsShift cm{lc};
+  const ColsLine cm{{lc}};
   const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
   const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
   const int lines = pair ? 2 * C : C;
@@ -284,7 +278,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_bwd(const
         if (m >= M) continue;
         const Cpl<T> e = buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c];
         Cpl<T> o = buf[fft_row(pair_pos(kind, m + 1, M), l1, s1, C) + c];
-        if (flip) o = Cpl<T>{-o.re, -o.im};
+        o = Cpl<T>{neg_if(flip, o.re), neg_if(flip, o.im)};
         if (A.vec) {
           if (2 * c < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c, m)) = Cpl<T>{e.re, o.re};
           if (2 * c + 1 < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c + 1, m)) = Cpl<T>{e.im, o.im};
@@ -305,7 +299,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 3 : 2) k_lines_bwd(const
         int m, c;
         cm.split(t, m, c);
         Cpl<T> v = buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c];
-        if (flip && (m & 1)) v = Cpl<T>{-v.re, -v.im};
+        v = Cpl<T>{neg_if(flip && (m & 1), v.re), neg_if(flip && (m & 1), v.im)};
         if (A.vec) {
           if (2 * c < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c, m)) = v;
         } else {

@@ -18,6 +18,7 @@
 #include <cmath>
 
 #include "transform_dev.cuh"
+#include "ztrans_dev.cuh"
 
 namespace snac {
 namespace {
@@ -160,6 +161,39 @@ __global__ void __launch_bounds__(TNT, 3) k_backward(const ChunkDev* __restrict_
   }
 }
 
+template <typename T, typename TI>
+__global__ void __launch_bounds__(TNT, sizeof(T) == 4 ? 4 : 3) k_zforward(const ZArgs<T> A, const ChunkDev* __restrict__ chunks,
+                                                                       const BlockDev* __restrict__ blk,
+                                                                       const CallerBlk* __restrict__ cb,
+                                                                       const TI* __restrict__ in3, T* __restrict__ out,
+                                                                       long long ncell, T sub0, int split) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  z_forward<T, TI>(A, chunks[blockIdx.x], blk, cb, in3, out, ncell, sub0, split, smem, blockDim.x);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(TNT, sizeof(T) == 4 ? 4 : 3) k_zbackward(const ZArgs<T> A, const ChunkDev* __restrict__ chunks,
+                                                                        const BlockDev* __restrict__ blk,
+                                                                        const CallerBlk* __restrict__ cb,
+                                                                        const T* __restrict__ modes,
+                                                                        double* __restrict__ p3, long long ncell,
+                                                                        double inv_theta) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  z_backward<T>(A, chunks[blockIdx.x], blk, cb, modes, p3, ncell, inv_theta, smem, blockDim.x);
+}
+
+constexpr int kZSmem = 64 * 1024;  // the plan keeps n_z / 2 x columns x 2 sizeof(T) at or below it
+// One thread per butterfly of the widest radix (16 FP32, 8 FP64), 64 to 256.
+template <typename T>
+int z_threads(const snac_plan* P, int tc) {
+  const int t = P->nzt / 2 * tc / (sizeof(T) == 4 ? 16 : 8);
+  return t >= 256 ? 256 : t >= 128 ? 128 : 64;
+}
+template <typename T>
+size_t z_smem(const snac_plan* P, int tc) {
+  return (size_t)(P->nzt / 2) * tc * sizeof(Cpl<T>);
+}
+
 // Dynamic shared memory of a transform launch: two half-length complex buffers of TC columns. The
 // kernel's maximum is a function-wide attribute shared by every plan and thread, so it is always set
 // to the largest need of any plan that uses this instantiation (128 KB: transform_columns keeps
@@ -182,9 +216,14 @@ struct Geom {
   const CallerBlk* cb;
   long long ncell;
   double n3;
+  const ChunkDev* zch;  // chunks of the smooth-length transforms
+  size_t nz;
+  int ztc;  // their width
 };
 
-Geom plan_geom(const snac_plan* P) { return Geom{P->lev[0].d_blk, P->d_cblk, P->lev[0].ncell, (double)P->n3}; }
+Geom plan_geom(const snac_plan* P) {
+  return Geom{P->lev[0].d_blk, P->d_cblk, P->lev[0].ncell, (double)P->n3, P->d_zchunks, P->zchunks.size(), P->ztc};
+}
 
 template <typename T, int TC, typename TI = double>
 cudaError_t fwd_t(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, const ChunkDev* dch, const void* twb,
@@ -197,6 +236,12 @@ cudaError_t fwd_t(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, 
   const double n3 = G.n3;
   // read the 3-D field, write the modes; FFT model 2.5 log2(n) flops per point plus pre/post-processing
   LaunchScope ls(P, K_FORWARD, (double)(sizeof(TI) + sizeof(T)) * n3, (2.5 * std::log2((double)P->nzt) + 8.0) * n3, s);
+  if (P->zsmooth) {
+    cudaFuncSetAttribute(k_zforward<T, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kZSmem);
+    k_zforward<T, TI><<<(unsigned)G.nz, z_threads<T>(P, G.ztc), z_smem<T>(P, G.ztc), s>>>(z_args<T>(P, G.ztc), G.zch, G.blk, G.cb, in3,
+                                                                         (T*)modes, G.ncell, sub0, split ? 1 : 0);
+    return cudaGetLastError();
+  }
   auto go = [&](auto kern) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem<T, TC>);
     kern<<<(unsigned)ch.size(), TNT, smem, s>>>(dch, G.blk, G.cb, P->nzt, make_tw<T>(P, twb), in3, (T*)modes, G.ncell,
@@ -219,6 +264,12 @@ cudaError_t bwd_t(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, 
   const double n3 = G.n3;
   // read the modes, read and write the FP64 field
   LaunchScope ls(P, K_BACKWARD, (16.0 + sizeof(T)) * n3, (2.5 * std::log2((double)P->nzt) + 10.0) * n3, s);
+  if (P->zsmooth) {
+    cudaFuncSetAttribute(k_zbackward<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kZSmem);
+    k_zbackward<T><<<(unsigned)G.nz, z_threads<T>(P, G.ztc), z_smem<T>(P, G.ztc), s>>>(z_args<T>(P, G.ztc), G.zch, G.blk, G.cb,
+                                                                        (const T*)modes, p3, G.ncell, sign / P->theta);
+    return cudaGetLastError();
+  }
   auto go = [&](auto kern) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem<T, TC>);
     kern<<<(unsigned)ch.size(), TNT, smem, s>>>(dch, G.blk, G.cb, P->nzt, make_tw<T>(P, twb), (const T*)modes, p3,
@@ -298,6 +349,11 @@ static cudaError_t pencil_tables(snac_plan* P, long long ncols) {
   const int t64 = P->tc64, t32 = P->tc32;
   for (long long c0 = 0; c0 < ncols; c0 += t64) P->pen_ch64.push_back({0, (int)c0, (int)std::min<long long>(t64, ncols - c0), 0});
   for (long long c0 = 0; c0 < ncols; c0 += t32) P->pen_ch32.push_back({0, (int)c0, (int)std::min<long long>(t32, ncols - c0), 0});
+  P->pen_zch.clear();
+  P->pen_ztc = z_chunk_columns(P, ncols);
+  if (P->zsmooth)
+    for (long long c0 = 0; c0 < ncols; c0 += P->pen_ztc)
+      P->pen_zch.push_back({0, (int)c0, (int)std::min<long long>(P->pen_ztc, ncols - c0), 0});
   auto put = [&](auto** d, const void* src, size_t bytes) -> cudaError_t {
     cudaError_t e = cudaMalloc((void**)d, bytes);
     if (e != cudaSuccess) return e;
@@ -307,7 +363,9 @@ static cudaError_t pencil_tables(snac_plan* P, long long ncols) {
   cudaError_t e;
   if ((e = put(&P->d_pen_tblk, &b, sizeof b)) != cudaSuccess || (e = put(&P->d_pen_tcb, &c, sizeof c)) != cudaSuccess ||
       (e = put(&P->d_pen_ch64, P->pen_ch64.data(), P->pen_ch64.size() * sizeof(ChunkDev))) != cudaSuccess ||
-      (e = put(&P->d_pen_ch32, P->pen_ch32.data(), P->pen_ch32.size() * sizeof(ChunkDev))) != cudaSuccess)
+      (e = put(&P->d_pen_ch32, P->pen_ch32.data(), P->pen_ch32.size() * sizeof(ChunkDev))) != cudaSuccess ||
+      (P->zsmooth &&
+       (e = put(&P->d_pen_zch, P->pen_zch.data(), P->pen_zch.size() * sizeof(ChunkDev))) != cudaSuccess))
     return e;
   P->pen_tcols = ncols;
   return cudaSuccess;
@@ -316,7 +374,7 @@ static cudaError_t pencil_tables(snac_plan* P, long long ncols) {
 cudaError_t launch_pencil_forward(snac_plan* P, long long ncols, const double* in, void* modes, cudaStream_t s) {
   cudaError_t e = pencil_tables(P, ncols);
   if (e != cudaSuccess) return e;
-  const Geom G{P->d_pen_tblk, P->d_pen_tcb, ncols, (double)ncols * P->nzt};
+  const Geom G{P->d_pen_tblk, P->d_pen_tcb, ncols, (double)ncols * P->nzt, P->d_pen_zch, P->pen_zch.size(), P->pen_ztc};
   if (P->precision == SNAC_FP64)
     return fwd_any<double, double>(P, G, P->pen_ch64, P->d_pen_ch64, P->d_tw64, in, modes, 0.0, false, s);
   return fwd_any<float, double>(P, G, P->pen_ch32, P->d_pen_ch32, P->d_tw32, in, modes, 0.0, false, s);
@@ -325,7 +383,7 @@ cudaError_t launch_pencil_forward(snac_plan* P, long long ncols, const double* i
 cudaError_t launch_pencil_backward(snac_plan* P, long long ncols, const void* modes, double* p, cudaStream_t s) {
   cudaError_t e = pencil_tables(P, ncols);
   if (e != cudaSuccess) return e;
-  const Geom G{P->d_pen_tblk, P->d_pen_tcb, ncols, (double)ncols * P->nzt};
+  const Geom G{P->d_pen_tblk, P->d_pen_tcb, ncols, (double)ncols * P->nzt, P->d_pen_zch, P->pen_zch.size(), P->pen_ztc};
   if (P->precision == SNAC_FP64)
     return bwd_any<double>(P, G, P->pen_ch64, P->d_pen_ch64, P->d_tw64, modes, p, 1.0, s);
   return bwd_any<float>(P, G, P->pen_ch32, P->d_pen_ch32, P->d_tw32, modes, p, 1.0, s);

@@ -395,6 +395,20 @@ bool fft_tab(int n, int max_log2, FftTab& F) {
   return true;
 }
 
+// Row of every frequency after the forward passes (digit-reversed order).
+std::vector<int> fft_perm(const FftTab& F) {
+  std::vector<int> perm(F.n);
+  for (int k = 0; k < F.n; ++k) {
+    int q = k, p = 0;
+    for (int s = 0; s < F.np; ++s) {
+      p += (q % F.rad[s]) * (F.span[s] / F.rad[s]);
+      q /= F.rad[s];
+    }
+    perm[k] = p;
+  }
+  return perm;
+}
+
 // The direct solve of the reduced equations (direct_dev.cuh), where the layout allows it: the blocks
 // tile a rectangle with one cell grid per axis, each outer side has one face kind, one plane axis is
 // uniform with an even length whose half or whole has no prime factor above 7, and the other is not
@@ -503,15 +517,7 @@ int build_direct(snac_plan* P, const std::vector<HBlock>& hb) {
   for (int k = 0; k <= M; ++k) put(D.w2n + k, -M_PI * k / (2.0 * M));
   for (int k = 0; k < M / 2; ++k) put(D.t4a + k, -M_PI * (4.0 * k + 1.0) / (4.0 * M));
   for (int k = 0; k < M / 2; ++k) put(D.t4b + k, -M_PI * k / (double)M);
-  std::vector<int> perm(nf);
-  for (int k = 0; k < nf; ++k) {
-    int q = k, p = 0;
-    for (int s = 0; s < F.np; ++s) {
-      p += (q % F.rad[s]) * (F.span[s] / F.rad[s]);
-      q /= F.rad[s];
-    }
-    perm[k] = p;
-  }
+  const std::vector<int> perm = fft_perm(F);
   // eigenvalues of the slots and the tridiagonal rows, scaled by a power of two to couplings of about 1
   double h = 0.0;
   for (double v : w[ax]) h += v;
@@ -697,6 +703,8 @@ int build_twiddles(snac_plan* P) {
   int st;
   if ((st = upload(P, &P->d_tw64, tw))) return st;
   if ((st = upload(P, &P->d_tw32, to32(tw)))) return st;
+  P->zsmooth = fft_tab(m, P->precision == SNAC_FP64 ? 3 : 4, P->zfft);
+  if (P->zsmooth && (st = upload(P, &P->d_zperm, fft_perm(P->zfft)))) return st;
   return SNAC_OK;
 }
 
@@ -1182,6 +1190,10 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     P->tc32 = transform_columns(P->nzt, false);
     if ((st = build_chunks(P, P->tc64, P->chunks64, &P->d_chunks64))) break;
     if ((st = build_chunks(P, P->tc32, P->chunks32, &P->d_chunks32))) break;
+    if (P->zsmooth) {
+      P->ztc = z_chunk_columns(P, P->lev[0].ncell);
+      if ((st = build_chunks(P, P->ztc, P->zchunks, &P->d_zchunks))) break;
+    }
     {
       const HostLevel& l0 = P->lev[0];
       std::vector<double> area(l0.ncell);

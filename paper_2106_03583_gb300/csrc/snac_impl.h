@@ -277,6 +277,12 @@ struct snac_plan {
   int* d_singular_mode = nullptr;  // per mode: 1 if the reduced system is singular
   // transforms
   snac::TwiddleOffsets tw{};
+  bool zsmooth = false;      // n_z / 2 has no prime factor above 7: the transforms of ztrans_dev.cuh
+  snac::FftTab zfft{};       // their passes (length n_z / 2) and the row of every frequency
+  int* d_zperm = nullptr;
+  int ztc = 0;               // their columns per CTA, and the chunks of that width
+  std::vector<snac::ChunkDev> zchunks;
+  snac::ChunkDev* d_zchunks = nullptr;
   double* d_tw64 = nullptr;  // double2 table
   float* d_tw32 = nullptr;   // float2 table
   int tc64 = 8, tc32 = 16;  // columns per transform CTA (transform_columns)
@@ -311,7 +317,9 @@ struct snac_plan {
   long long pen_tcols = -1;
   snac::BlockDev* d_pen_tblk = nullptr;
   snac::CallerBlk* d_pen_tcb = nullptr;
-  std::vector<snac::ChunkDev> pen_ch64, pen_ch32;
+  std::vector<snac::ChunkDev> pen_ch64, pen_ch32, pen_zch;
+  snac::ChunkDev* d_pen_zch = nullptr;
+  int pen_ztc = 0;
   snac::ChunkDev* d_pen_ch64 = nullptr;
   snac::ChunkDev* d_pen_ch32 = nullptr;
   std::vector<void*> pen_tallocs;
@@ -341,6 +349,17 @@ struct snac_plan {
 };
 
 namespace snac {
+
+// Columns per CTA of the smooth-length transforms on a field of `columns` columns: from 8 (FP64) or 16
+// (FP32: whole 64-byte segments; fewer for axes beyond 1024) up to what gives every thread of a CTA a
+// butterfly of the widest radix (2048 / 4096 points), as long as four CTAs per multiprocessor remain.
+inline int z_chunk_columns(const snac_plan* P, long long columns) {
+  const bool f64 = P->precision == SNAC_FP64;
+  const int m = P->nzt / 2, most = f64 ? 2048 : 4096;
+  int tc = f64 ? P->tc64 : P->tc32;
+  while (tc < 64 && m * tc * 2 <= most && columns / (2 * tc) >= 4LL * P->sms) tc *= 2;
+  return tc;
+}
 
 // ---- launchers (field kernels: 3-D FP64 residual and reductions) ----
 // mode 0: r = (f - fshift) - A p; d_sums = {||r||^2, ||f - fshift||^2 if need_f2, sum V p if need_vp}

@@ -669,7 +669,7 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
         plans.push_back(J->P);
         ins.push_back(J->fin);
         targets.push_back(J->target);
-        nitems += J->P->nz + (int)(J->P->precision == SNAC_FP64 ? J->P->chunks64.size() : J->P->chunks32.size());
+        nitems += J->P->nz + (int)std::max(J->P->chunks64.size(), J->P->chunks32.size());
       }
       const size_t need = fwd_onchip_batch_scratch((int)plans.size(), nitems);
       if (need > scratch_bytes) {
