@@ -370,54 +370,122 @@ __global__ void __launch_bounds__(512, 1) k_tri_low(const TriRow<double>* __rest
                              [&](int n, double v) { col[(long long)n * M] = (float)v; });
 }
 
-// One thread per system, rows in order: fewest operations per row (the FP64 plans are bound by the
-// FP64 pipe, not by the extra pass over the factors c, kept in the plan's other mode buffer). S: the
-// arithmetic's type.
-template <typename T, typename S>
-__global__ void __launch_bounds__(128) k_tri_seq(const TriRow<S>* __restrict__ tri, const S* __restrict__ lam,
-                                               const S* __restrict__ sigma, S cscale, S scale, int nq, int M, int N,
-                                               T* __restrict__ x, S* __restrict__ cw) {
+// Rows in order, one thread per system, for systems too long for the segments of one CTA (FP32; the
+// factors c go to the plan's other mode buffer).
+template <typename T>
+__global__ void __launch_bounds__(128) k_tri_seq(const DirectArgs<T> A, T* __restrict__ x, T* __restrict__ cw) {
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (sys >= (long long)nq * M) return;
-  const int q = (int)(sys / M), kap = (int)(sys - (long long)q * M);
-  const long long o = (long long)q * N * M + kap;
+  if (sys >= (long long)A.nq * A.M) return;
+  const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
+  const long long o = (long long)q * A.N * A.M + kap;
   x += o;
   cw += o;
-  const S tq = -fma(sigma[q], cscale, lam[kap]);
+  const T tq = -fma(A.sigma[q], A.cscale, A.lam[kap]);
   constexpr int U = 8;
-  S g = 0, d = 0;
-  for (int n0 = 0; n0 < N; n0 += U) {
+  T g = 0, d = 0;
+  for (int n0 = 0; n0 < A.N; n0 += U) {
     T v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = n0 + u < N ? x[(long long)(n0 + u) * M] : (T)0;
+    for (int u = 0; u < U; ++u) v[u] = n0 + u < A.N ? x[(long long)(n0 + u) * A.M] : (T)0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (n0 + u >= N) break;
-      const TriRow<S> w = tri[n0 + u];
-      const S s = fma(w.lo, g, w.tau + tq);
-      const S den = s + w.hi;
-      const S inv = den > (S)0 ? tri_recip(den) : (S)0;
+      if (n0 + u >= A.N) break;
+      const TriRow<T> w = A.tri[n0 + u];
+      const T s = fma(w.lo, g, w.tau + tq);
+      const T den = s + w.hi;
+      const T inv = den > (T)0 ? tri_recip(den) : (T)0;
       g = s * inv;
-      d = fma(w.lo, d, -scale * (S)v[u]) * inv;
-      x[(long long)(n0 + u) * M] = (T)d;
-      cw[(long long)(n0 + u) * M] = w.hi * inv;
+      d = fma(w.lo, d, -A.scale * v[u]) * inv;
+      x[(long long)(n0 + u) * A.M] = d;
+      cw[(long long)(n0 + u) * A.M] = w.hi * inv;
     }
   }
-  S y = 0;
-  for (int n0 = (N - 1) / U * U; n0 >= 0; n0 -= U) {
-    T v[U];
-    S c[U];
+  T y = 0;
+  for (int n0 = (A.N - 1) / U * U; n0 >= 0; n0 -= U) {
+    T v[U], c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const bool in = n0 + u < N;
-      v[u] = in ? x[(long long)(n0 + u) * M] : (T)0;
-      c[u] = in ? cw[(long long)(n0 + u) * M] : (S)0;
+      const bool in = n0 + u < A.N;
+      v[u] = in ? x[(long long)(n0 + u) * A.M] : (T)0;
+      c[u] = in ? cw[(long long)(n0 + u) * A.M] : (T)0;
     }
 #pragma unroll
     for (int u = U - 1; u >= 0; --u) {
+      if (n0 + u >= A.N) continue;
+      y = fma(c[u], y, v[u]);
+      x[(long long)(n0 + u) * A.M] = y;
+    }
+  }
+}
+
+// FP64 plans: the elimination is bound by the FP64 pipe (14 operations per row, half of them for the
+// pivot's reciprocal, which depends on the plan only), so the reciprocals are kept: [row of
+// DirectTab::qrow][n][kappa], wavenumbers of equal sigma (q and n - q of the real DFT) sharing one set. The
+// solve is then 5 operations per row at 48 bytes per cell. Measured on 512 x 512 x 256: 1.89 -> 0.71 ms (FP32 plans,
+// kept in FP32: 24 bytes per cell, 0.44 -> 0.36 ms, from 256 systems per multiprocessor on; below that the
+// segments of k_tri_seg have the shorter chain).
+template <typename T>
+__global__ void __launch_bounds__(128) k_tri_factor(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
+                                                  const double* __restrict__ sigma, double cscale, int M, int N,
+                                                  const int* __restrict__ qof, int rows, T* __restrict__ fac) {
+  const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (sys >= (long long)rows * M) return;
+  const int r = (int)(sys / M), kap = (int)(sys - (long long)r * M);
+  const double tq = -fma(sigma[qof[r]], cscale, lam[kap]);
+  T* f = fac + (long long)r * N * M + kap;
+  double g = 0;
+  for (int n = 0; n < N; ++n) {
+    const TriRow<double> w = tri[n];
+    const double s = fma(w.lo, g, w.tau + tq);
+    const double den = s + w.hi;
+    const double inv = den > 0 ? 1.0 / den : 0.0;
+    g = s * inv;
+    f[(long long)n * M] = (T)inv;
+  }
+}
+
+constexpr int TRI_U = 8;  // rows whose loads are in flight per thread
+template <typename T>
+__global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const int* __restrict__ qrow,
+                                                  const unsigned char* __restrict__ low, const T* __restrict__ fac,
+                                                  T* __restrict__ x) {
+  const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (sys >= (long long)A.nq * A.M || (sizeof(T) == 4 && low[sys])) return;
+  const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
+  const int N = A.N, M = A.M;
+  x += (long long)q * N * M + kap;
+  fac += (long long)qrow[q] * N * M + kap;
+  const T sc = -A.scale;
+  T d = 0;
+  for (int n0 = 0; n0 < N; n0 += TRI_U) {
+    T v[TRI_U], f[TRI_U];
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const bool in = n0 + u < N;
+      v[u] = in ? x[(long long)(n0 + u) * M] : (T)0;
+      f[u] = in ? fac[(long long)(n0 + u) * M] : (T)0;
+    }
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      if (n0 + u >= N) break;
+      d = fma(A.tri[n0 + u].lo, d, sc * v[u]) * f[u];
+      x[(long long)(n0 + u) * M] = d;
+    }
+  }
+  T y = 0;
+  for (int n0 = (N - 1) / TRI_U * TRI_U; n0 >= 0; n0 -= TRI_U) {
+    T v[TRI_U], f[TRI_U];
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const bool in = n0 + u < N;
+      v[u] = in ? x[(long long)(n0 + u) * M] : (T)0;
+      f[u] = in ? fac[(long long)(n0 + u) * M] : (T)0;
+    }
+#pragma unroll
+    for (int u = TRI_U - 1; u >= 0; --u) {
       if (n0 + u >= N) continue;
-      y = fma(c[u], y, (S)v[u]);
-      x[(long long)(n0 + u) * M] = (T)y;
+      y = fma(A.tri[n0 + u].hi * f[u], y, v[u]);
+      x[(long long)(n0 + u) * M] = y;
     }
   }
 }
@@ -463,17 +531,17 @@ cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
         k_tri_low<<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
             (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / (2.0 * A.M), D.d_lowlist,
             D.nlow, A.M, A.N, lsegs, u);
-      if (segs <= 32) {
+      if (D.d_fac) {
+        k_tri_pre<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A, D.d_qrow, D.d_low, (const T*)D.d_fac, u);
+      } else if (segs <= 32) {
         k_tri_seg<T, 32><<<(unsigned)((sys + 31) / 32), 32 * segs, 7 * sizeof(T) * 32 * segs, s>>>(A, segs, D.d_low, u);
       } else if (segs <= 64) {
         k_tri_seg<T, 16><<<(unsigned)((sys + 15) / 16), 16 * segs, 7 * sizeof(T) * 16 * segs, s>>>(A, segs, D.d_low, u);
       } else {
-        k_tri_seq<T, T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A.tri, A.lam, A.sigma, A.cscale, A.scale, A.nq,
-                                                                      A.M, A.N, u, f);
+        k_tri_seq<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A, u, f);
       }
     } else {
-      k_tri_seq<T, T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A.tri, A.lam, A.sigma, A.cscale, A.scale, A.nq,
-                                                                      A.M, A.N, u, f);
+      k_tri_pre<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A, P->direct.d_qrow, nullptr, (const T*)P->direct.d_fac, u);
     }
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -491,6 +559,17 @@ cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStrea
   *P->h_wait = 0;
   if (P->precision == SNAC_FP64) k_nonfinite<double><<<4 * P->sms, 256, 0, s>>>((const double*)v, n, P->dh_wait);
   else k_nonfinite<float><<<4 * P->sms, 256, 0, s>>>((const float*)v, n, P->dh_wait);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tri_factor(snac_plan* P, const int* d_qof, int rows, cudaStream_t s) {
+  const DirectTab& D = P->direct;
+  const bool f64 = P->precision == SNAC_FP64;
+  const TriRow<double>* tri = (const TriRow<double>*)(f64 ? D.d_tri : (void*)D.d_tri64);
+  const double* lam = f64 ? (const double*)D.d_lam : D.d_lam64;
+  const unsigned grid = (unsigned)(((long long)rows * D.M + 127) / 128);
+  if (f64) k_tri_factor<double><<<grid, 128, 0, s>>>(tri, lam, P->d_sigma64, D.cscale, D.M, D.N, d_qof, rows, (double*)D.d_fac);
+  else k_tri_factor<float><<<grid, 128, 0, s>>>(tri, lam, P->d_sigma64, D.cscale, D.M, D.N, d_qof, rows, (float*)D.d_fac);
   return cudaGetLastError();
 }
 

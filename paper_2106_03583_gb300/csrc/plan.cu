@@ -1098,6 +1098,28 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     // the automatic inner reduction: an on-chip plan's V-cycles are cheap next to an outer step,
     // so it asks more of each step (measured on c64: 3 outer steps at 1e-4, 2 at 3e-5, 18 % faster)
     if (P->inner_reduction == 0.0) P->inner_reduction = P->onchip ? 3e-5 : 1e-4;
+    if (P->direct.on && !P->onchip && (P->precision == SNAC_FP64 || (long long)P->nz * P->direct.M >= 256LL * P->sms)) {
+      std::vector<int> qrow(P->nz), qof;
+      std::map<int, int> seen;  // wavenumbers q and n - q of the real DFT have one eigenvalue
+      for (int l = 0; l < P->nz; ++l) {
+        const int q = P->q0 + l;
+        const auto it = seen.emplace(P->kind == KIND_PP ? std::min(q, P->nzt - q) : q, (int)qof.size());
+        if (it.second) qof.push_back(l);
+        qrow[l] = it.first->second;
+      }
+      int* d_qof = nullptr;
+      if ((st = upload(P, &P->direct.d_qrow, qrow)) || (st = upload(P, &d_qof, qof)) ||
+          (st = dmalloc(P, (char**)&P->direct.d_fac, qof.size() * (size_t)P->direct.M * P->direct.N * inner)))
+        break;
+      cudaStream_t cs = nullptr;
+      bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
+      ok = ok && launch_tri_factor(P, d_qof, (int)qof.size(), cs) == cudaSuccess && cudaStreamSynchronize(cs) == cudaSuccess;
+      if (cs) cudaStreamDestroy(cs);
+      if (!ok) {
+        st = fail(SNAC_ERR_CUDA, "factoring the tridiagonal systems failed");
+        break;
+      }
+    }
     // fused FP32 tile kernels on the levels whose blocks all keep the halo inside their neighbours
     // (above the bottom sub-cycle; not needed when the whole solve runs on chip)
     const bool want_fused = !P->onchip && (P->fused == 1 || (P->fused < 0 && P->precision == SNAC_MIXED));

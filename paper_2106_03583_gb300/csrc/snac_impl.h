@@ -178,6 +178,8 @@ struct DirectTab {
   FftTab fft{};
   int w2n = 0, t4a = 0, t4b = 0;  // offsets in the twiddle table
   double cscale = 1.0;
+  void* d_fac = nullptr;             // plans not on chip: reciprocal pivots (k_tri_pre), inner type
+  int* d_qrow = nullptr;             // per wavenumber: its set of them
   int nlow = 0;                      // mixed plans: systems solved in FP64 arithmetic (k_tri_low)
   int* d_lowlist = nullptr;          // their numbers q M + kappa
   unsigned char* d_low = nullptr;    // per system: 1 if listed
@@ -451,6 +453,9 @@ BottomLayout bottom_layout(const snac_plan* P, int lb, size_t w);
 // Separable plans: every wavenumber's solution of the reduced equations for the right-hand sides in
 // lev[0].d_f (plain order), into mode_solution(P).
 cudaError_t launch_direct(snac_plan* P, cudaStream_t s);
+// The reciprocal pivots of an FP64 plan's tridiagonal systems, once per plan (d_qof: a wavenumber of
+// every set).
+cudaError_t launch_tri_factor(snac_plan* P, const int* d_qof, int rows, cudaStream_t s);
 // *h_wait = 1 if any of the n values (inner type) is NaN or Inf, else 0.
 cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStream_t s);
 // Where a solve leaves the mode-space solution: the level-0 iterate, or (direct solves of planes too
