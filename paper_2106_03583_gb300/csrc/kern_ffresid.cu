@@ -13,6 +13,7 @@
 //
 // The solve uses this pass for the defect-correction steps whose residual is far above the
 // tolerance, and the FP64 pass of kern_field.cu for the check that decides convergence.
+#include <algorithm>
 #include <cmath>
 
 #include "kern_common.cuh"
@@ -219,7 +220,9 @@ cudaError_t launch_field3d_ff(snac_plan* P, const double* f, const double* p, fl
                               bool need_f2, bool need_vp, cudaStream_t s) {
   if (!P->d_czff || !P->d_cxff) return cudaErrorInvalidValue;
   LevelView<double> L = level_view<double>(P->lev[0]);
-  const int zsplit = std::min(P->nzt, 16);
+  // CTAs per tile: enough to fill the GPU, few partials to reduce (as field_grid of kern_field.cu)
+  const int tiles = (int)P->lev[0].tiles.size();
+  const int zsplit = std::max(1, std::min({P->nzt, 16, (32 * P->sms + tiles - 1) / tiles}));
   const int kchunk = (P->nzt + zsplit - 1) / zsplit;
   const dim3 grid((unsigned)P->lev[0].tiles.size(), (unsigned)((P->nzt + kchunk - 1) / kchunk));
   // squares of r / fscale: fscale is ||f|| / sqrt(n) rounded to a power of two

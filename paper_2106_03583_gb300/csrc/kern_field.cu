@@ -1,6 +1,8 @@
 // FP64 kernels on 3-D fields: the outer residual r = f - A p of the defect-correction loop (Eq. 8),
 // the operator itself, right-hand-side statistics, deterministic reductions, and the mean fix of
 // singular problems.
+#include <algorithm>
+
 #include "snac_impl.h"
 #include "kern_common.cuh"
 
@@ -73,20 +75,21 @@ __global__ void __launch_bounds__(TILE_THREADS) k_field3d(LevelView<double> L, c
       const int kd = k > 0 ? k - 1 : (periodic_z ? nz - 1 : k);
       const int ku = k < nz - 1 ? k + 1 : (periodic_z ? 0 : k);
       const double pc = p[c];
-      // with the shift and no ||f - fshift||^2 wanted, fshift enters the chain: r = f - (fshift + A p)
-      constexpr bool FOLD = MODE == 0 && SHIFT && !NEED_F2;
-      double ap = FOLD ? fma(cx.lo, p[pw + k * sw], fshift) : cx.lo * p[pw + k * sw];
-      ap = fma(cx.hi, p[pe + k * se], ap);
-      ap = fma(cy.lo, p[ps + k * ss], ap);
-      ap = fma(cy.hi, p[pn + k * sn], ap);
-      ap = fma(z.lo, p[base + kd * sc], ap);
-      ap = fma(z.hi, p[base + ku * sc], ap);
-      ap = fma(dg, pc, ap);
+      // the chain starts from f (MODE 1: from the first product), so the residual costs no subtraction
+      // of its own: 7 products and the square, 8 FP64 operations per cell
+      const double fv = MODE == 1 ? 0.0 : SHIFT ? f[c] - fshift : f[c];
+      const double sg = MODE == 1 ? 1.0 : -1.0;
+      double ap = MODE == 1 ? cx.lo * p[pw + k * sw] : fma(-cx.lo, p[pw + k * sw], fv);
+      ap = fma(sg * cx.hi, p[pe + k * se], ap);
+      ap = fma(sg * cy.lo, p[ps + k * ss], ap);
+      ap = fma(sg * cy.hi, p[pn + k * sn], ap);
+      ap = fma(sg * z.lo, p[base + kd * sc], ap);
+      ap = fma(sg * z.hi, p[base + ku * sc], ap);
+      ap = fma(sg * dg, pc, ap);
       if (MODE == 1) {
         r[c] = ap;
       } else {
-        const double fv = SHIFT && !FOLD ? f[c] - fshift : f[c];
-        const double rv = fv - ap;
+        const double rv = ap;
         r[c] = rv;
         acc[0] = fma(rv, rv, acc[0]);
         if (NEED_F2) acc[1] = fma(fv, fv, acc[1]);
@@ -127,13 +130,14 @@ __global__ void __launch_bounds__(TILE_THREADS) k_prepass(LevelView<double> L, c
       const long long c = base + k * sk;
       const double fv = f[c];
       bits |= (unsigned long long)__double_as_longlong(p[c]);
-      if (SING) {
-        acc[0] = fma(va, fv, acc[0]);
-        acc[1] = fma(va, fabs(fv), acc[1]);
+      if (SING) {  // plain sums along the column: its cells have one volume
         acc[3] += fv;
+        acc[1] += fabs(fv);
       }
       acc[2] = fma(fv, fv, acc[2]);
     }
+    acc[0] = va * acc[3];
+    acc[1] *= va;
   }
   block_sum<4>(acc, sh);
   const int any = __syncthreads_or((bits << 1) != 0ull);  // the shift drops the sign bit (-0.0 is zero)
@@ -230,8 +234,13 @@ void residual_t(const LevelView<double>& L, dim3 grid, snac_plan* P, const doubl
   else field3d_t<0, SH, false, false>(L, grid, P, f, p, r, fshift, s);
 }
 
+// The z planes are dealt to as few CTAs per tile as fill the GPU (about four waves of eight CTAs per
+// multiprocessor): every CTA leaves a partial for the one-CTA reduction, which took 23-43 us on the large
+// problems with 16 CTAs per tile.
 dim3 field_grid(const snac_plan* P) {
-  return dim3((unsigned)P->lev[0].tiles.size(), (unsigned)std::min(P->nzt, ZSPLIT));
+  const int tiles = (int)P->lev[0].tiles.size();
+  const int z = (32 * P->sms + tiles - 1) / tiles;
+  return dim3((unsigned)tiles, (unsigned)std::max(1, std::min({P->nzt, ZSPLIT, z})));
 }
 
 }  // namespace
