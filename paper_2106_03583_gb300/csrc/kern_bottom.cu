@@ -569,7 +569,8 @@ struct FwdArgs {
   int n, kind, in_f32, nchunks;
   int need;              // chunks a solve item waits for (nchunks; more only in the timeout self-test)
   int* done;             // chunks counted so far (zero at launch)
-  int* status;           // 1 if a wait of this plan gave up
+  int* status;           // 1 if a wait of this plan gave up (mapped host memory)
+  int* bad;              // the same in device memory, for the update behind the launch
 };
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -627,6 +628,7 @@ __device__ void fused_solve(const FwdArgs<T>& F, const OnchipArgs<T>& O, int q, 
       if (global_ns() - t0 > (unsigned long long)wait_ns) {
         give_up = 1;
         atomicOr(F.status, 1);
+        atomicOr(F.bad, 1);
         break;
       }
       __nanosleep(500);
@@ -651,7 +653,14 @@ __global__ void __launch_bounds__(BT, 1) k_fwd_onchip(const FwdArgs<T> F, const 
     __syncthreads();
     const int k = item;
     __syncthreads();
-    if (k >= nitems) break;
+    if (k >= nitems) {
+      // every CTA's last claim comes after its own items: the last of all resets the counters
+      if (threadIdx.x == 0 && k == nitems + (int)gridDim.x - 1) {
+        *next = 0;
+        *F.done = 0;
+      }
+      break;
+    }
     if (k < F.nchunks) fused_chunk<T, TC>(F, k, smem_raw);
     else fused_solve(F, O, k - F.nchunks, wait_ns, smem_raw, &skip);
   }
@@ -850,6 +859,7 @@ FwdArgs<T> fwd_args(snac_plan* P, const void* in3, bool in_f32, double shift0, i
   F.need = F.nchunks + extra;
   F.done = done;
   F.status = status;
+  F.bad = P->d_fused + 2;
   return F;
 }
 
@@ -864,24 +874,28 @@ size_t fused_smem(const snac_plan* P) {
   return std::max(fft, onchip_smem<T>(P));
 }
 
+// Clears the mark of a launch whose wait gave up (the counters reset themselves).
+cudaError_t fused_reset(snac_plan* P, cudaStream_t s) {
+  if (!*P->h_wait) return cudaSuccess;
+  *P->h_wait = 0;
+  k_zero_ints<<<1, 32, 0, s>>>(P->d_fused + 2, 1);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t fwd_onchip_t(snac_plan* P, const void* in3, bool in_f32, double shift0, double target, double wait_s,
                          int extra, cudaStream_t s) {
   constexpr int TC = fused_tc<T>();
-  *P->h_wait = 0;
-  k_zero_ints<<<1, 32, 0, s>>>(P->d_fused, 2);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = fused_reset(P, s);
   if (e != cudaSuccess) return e;
   const FwdArgs<T> F = fwd_args<T>(P, in3, in_f32, shift0, P->d_fused + 1, P->dh_wait, extra);
   const OnchipArgs<T> O = onchip_args<T>(P, target);
   const size_t smem = fused_smem<T>(P);
   cudaFuncSetAttribute(k_fwd_onchip<T, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, BOTTOM_MAX_SMEM);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fwd_onchip<T, TC>, BT, smem);
   const int nitems = F.nchunks + P->nz;
   // one CTA per multiprocessor: two wavenumber solves never share one (their V-cycles are bound by
   // the SM's own pipes), and the transform chunks still spread over every SM
-  const int grid = std::max(1, std::min(nitems, std::min(std::max(1, per_sm), 1) * P->sms));
+  const int grid = std::max(1, std::min(nitems, P->sms));
   const double w = sizeof(T), n3 = (double)P->n3;
   LaunchScope ls(P, K_FWD_ONCHIP, (in_f32 ? 4.0 : 8.0) * n3 + w * n3 + 2.0 * w * (double)P->lev[0].ncell * P->nz,
                  (2.5 * std::log2((double)P->nzt) + 8.0) * n3 + 4.0 * onchip_cycle_flops(P) * P->nz, s);
@@ -934,7 +948,8 @@ cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs
   int* d_ctr = reinterpret_cast<int*>(reinterpret_cast<char*>(d_items) + up(items.size() * sizeof(int4)));
   for (int k = 0; k < nplans; ++k) {
     snac_plan* P = plans[k];
-    *P->h_wait = 0;
+    const cudaError_t er = fused_reset(P, s);
+    if (er != cudaSuccess) return er;
     fargs[k] = fwd_args<T>(P, inputs[k].in3, inputs[k].in_f32, inputs[k].shift0, d_ctr + 1 + k, P->dh_wait, 0);
     args[k] = onchip_args<T>(P, targets[k]);
     smem = std::max(smem, fused_smem<T>(P));
@@ -952,10 +967,8 @@ cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs
   k_zero_ints<<<1, 256, 0, s>>>(d_ctr, 1 + nplans);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cudaFuncSetAttribute(k_fwd_onchip_batch<T, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, BOTTOM_MAX_SMEM);
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fwd_onchip_batch<T, TC>, BT, smem);
   const int nitems = (int)items.size();
-  const int grid = std::max(1, std::min(nitems, std::min(std::max(1, per_sm), 1) * sms));  // one CTA per SM
+  const int grid = std::max(1, std::min(nitems, sms));  // one CTA per SM
   k_fwd_onchip_batch<T, TC><<<grid, BT, smem, s>>>(d_fargs, d_args, d_items, nitems, d_ctr, (long long)(wait_s * 1e9));
   return cudaGetLastError();
 }

@@ -20,6 +20,66 @@ __device__ __forceinline__ T warp_sum_t(T v) {
   return v;
 }
 
+// Where the sums of a 3-D pass go: the last CTA to leave its partial ([CTA][4]) adds them all up in a fixed
+// order and writes the four sums to device memory (out) and to the mapped host copy (host), so a pass is
+// one launch: no reduction kernel and no copy kernel behind it (each cost 4-6 us of a small solve). ticket
+// is zero before the launch and after it. flag (pre-pass): also out[SUM_NONZERO] = (double)*flag, then 0.
+struct SumOut {
+  double* part;
+  double* out;
+  double* host;
+  int* ticket;
+  int npart;
+  int* flag;
+};
+
+// Called by every thread of the CTA after thread 0 has written the CTA's partial; sh: 4 x 32 doubles.
+__device__ __forceinline__ void finish_sums(const SumOut& S, double* sh) {
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(S.ticket, 1) == S.npart - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  const double2* p = reinterpret_cast<const double2*>(S.part);
+  for (int i = threadIdx.x; i < S.npart; i += blockDim.x) {
+    const double2 a = __ldcg(p + 2 * i), b = __ldcg(p + 2 * i + 1);
+    acc[0] += a.x;
+    acc[1] += a.y;
+    acc[2] += b.x;
+    acc[3] += b.y;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double x = warp_sum(acc[k]);
+    if (lane == 0) sh[k * 32 + warp] = x;
+  }
+  __syncthreads();
+  if (warp < 4) {
+    const double x = warp_sum(lane < nwarp ? sh[warp * 32 + lane] : 0.0);
+    if (lane == 0) {
+      S.out[warp] = x;
+      S.host[warp] = x;
+    }
+  }
+  if (threadIdx.x == 0) {
+    *S.ticket = 0;
+    if (S.flag) {
+      const double f = (double)atomicExch(S.flag, 0);  // ready for the next pre-pass
+      S.out[SUM_NONZERO] = f;
+      S.host[SUM_NONZERO] = f;
+    }
+  }
+}
+
+inline SumOut sum_out(const snac_plan* P, int npart, bool flag = false) {
+  return SumOut{P->d_partial, P->d_sums, P->dh_sums, P->d_flag + 1, npart, flag ? P->d_flag : nullptr};
+}
+
 // The four x-y neighbours of cell (i, j) of block b: (block, index within that block's plane).
 // Inside the block the neighbour is the adjacent cell; across a connected (or periodic) face the
 // facing cell of the connected block (faces coincide, Sec. 3.1); on a physical face the cell itself

@@ -556,9 +556,9 @@ cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStream_t s) {
-  *P->h_wait = 0;
-  if (P->precision == SNAC_FP64) k_nonfinite<double><<<4 * P->sms, 256, 0, s>>>((const double*)v, n, P->dh_wait);
-  else k_nonfinite<float><<<4 * P->sms, 256, 0, s>>>((const float*)v, n, P->dh_wait);
+  P->h_check[0] = 0;
+  if (P->precision == SNAC_FP64) k_nonfinite<double><<<4 * P->sms, 256, 0, s>>>((const double*)v, n, P->dh_check);
+  else k_nonfinite<float><<<4 * P->sms, 256, 0, s>>>((const float*)v, n, P->dh_check);
   return cudaGetLastError();
 }
 

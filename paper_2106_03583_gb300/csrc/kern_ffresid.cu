@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 3)
                  const float4* __restrict__ cyff, const float2* __restrict__ dgff, const float4* __restrict__ czff,
                  int nz, int periodic_z, int kchunk, double dz, const double* __restrict__ f,
                  const double* __restrict__ p, float* __restrict__ r, float2 fsh, float nscale, double inv_nscale2,
-                 double* __restrict__ partial) {
+                 const SumOut S) {
   __shared__ double sh[4 * 32];
   const TileDev t = L.tiles[blockIdx.x];
   const BlockDev B = L.blk[t.b];
@@ -189,12 +189,13 @@ __global__ void __launch_bounds__(TILE_THREADS, 3)
   }
   block_sum_d<3>(acc, sh);
   if (threadIdx.x == 0) {
-    double* o = partial + 4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
+    double* o = S.part + 4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
     o[0] = acc[0];
     o[1] = acc[1];
     o[2] = acc[2];
     o[3] = 0.0;
   }
+  finish_sums(S, sh);
 }
 
 template <bool SH, bool F2, bool VP>
@@ -202,7 +203,7 @@ void ff_t(const LevelView<double>& L, dim3 grid, int kchunk, snac_plan* P, const
           float2 fsh, float nscale, double inv_nscale2, cudaStream_t s) {
   k_field3d_ff<SH, F2, VP><<<grid, TILE_THREADS, 0, s>>>(L, P->d_cblk, P->d_cxff, P->d_cyff, P->d_dgff, P->d_czff,
                                                           P->nzt, P->kind == KIND_PP, kchunk, P->dz, f, p, r, fsh,
-                                                          nscale, inv_nscale2, P->d_partial);
+                                                          nscale, inv_nscale2, sum_out(P, (int)(grid.x * grid.y)));
 }
 
 template <bool SH>
@@ -239,9 +240,7 @@ cudaError_t launch_field3d_ff(snac_plan* P, const double* f, const double* p, fl
     if (fshift != 0.0) ff_sel<true>(L, grid, kchunk, P, f, p, r, fsh, need_f2, need_vp, nscale, inv2, s);
     else ff_sel<false>(L, grid, kchunk, P, f, p, r, fsh, need_f2, need_vp, nscale, inv2, s);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_reduce_partials(P, (int)(grid.x * grid.y), P->d_sums, s);
+  return cudaGetLastError();
 }
 
 }  // namespace snac

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(TILE_THREADS) k_field3d(LevelView<double> L, c
                                                            const Coef<double>* __restrict__ cz, int nz, int periodic_z,
                                                            double zd, double dz, const double* __restrict__ f,
                                                            const double* __restrict__ p, double* __restrict__ r,
-                                                           double fshift, double* __restrict__ partial) {
+                                                           double fshift, const SumOut S) {
   __shared__ double sh[4 * 32];
   const TileDev t = L.tiles[blockIdx.x];
   const BlockDev B = L.blk[t.b];
@@ -100,22 +100,22 @@ __global__ void __launch_bounds__(TILE_THREADS) k_field3d(LevelView<double> L, c
   if (MODE == 1) return;
   block_sum<3>(acc, sh);
   if (threadIdx.x == 0) {
-    double* o = partial + 4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
+    double* o = S.part + 4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
     o[0] = acc[0];
     o[1] = acc[1];
     o[2] = acc[2];
     o[3] = 0.0;
   }
+  finish_sums(S, sh);
 }
 
 // Before the first residual: statistics of the right-hand side and whether the initial guess is
 // zero. partial {sum V f, sum V |f|, ||f||^2, sum f} (the first two and the last only for singular
-// problems); *nonzero = 1 if any p has a bit set other than its sign.
+// problems); *S.flag = 1 if any p has a bit set other than its sign.
 template <bool SING>
 __global__ void __launch_bounds__(TILE_THREADS) k_prepass(LevelView<double> L, const CallerBlk* __restrict__ cb, int nz,
                                                            double dz, const double* __restrict__ f,
-                                                           const double* __restrict__ p, double* __restrict__ partial,
-                                                           int* __restrict__ nonzero) {
+                                                           const double* __restrict__ p, const SumOut S) {
   __shared__ double sh[4 * 32];
   const TileDev t = L.tiles[blockIdx.x];
   const BlockDev B = L.blk[t.b];
@@ -142,19 +142,18 @@ __global__ void __launch_bounds__(TILE_THREADS) k_prepass(LevelView<double> L, c
   block_sum<4>(acc, sh);
   const int any = __syncthreads_or((bits << 1) != 0ull);  // the shift drops the sign bit (-0.0 is zero)
   if (threadIdx.x == 0) {
-    double* o = partial + 4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
+    double* o = S.part + 4 * ((long long)blockIdx.y * gridDim.x + blockIdx.x);
     o[0] = acc[0];
     o[1] = acc[1];
     o[2] = acc[2];
     o[3] = acc[3];
-    if (any) atomicOr(nonzero, 1);
+    if (any) atomicOr(S.flag, 1);
   }
+  finish_sums(S, sh);
 }
 
 // Deterministic sum of npart x 4 partials into out[4] (one CTA, fixed order).
-// With `flag`, also out_flag = (double)*flag (read after the kernels that set it), and *flag = 0.
-__global__ void __launch_bounds__(1024) k_reduce4(const double* __restrict__ part, int npart, double* __restrict__ out,
-                                                  int* __restrict__ flag, double* __restrict__ out_flag) {
+__global__ void __launch_bounds__(1024) k_reduce4(const double* __restrict__ part, int npart, double* __restrict__ out) {
   __shared__ double sh[4 * 32];
   double acc[4] = {0, 0, 0, 0};
   for (int i = threadIdx.x; i < npart; i += blockDim.x) {
@@ -162,13 +161,8 @@ __global__ void __launch_bounds__(1024) k_reduce4(const double* __restrict__ par
     for (int k = 0; k < 4; ++k) acc[k] += part[4 * (long long)i + k];
   }
   block_sum<4>(acc, sh);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0)
     for (int k = 0; k < 4; ++k) out[k] = acc[k];
-    if (flag) {
-      *out_flag = (double)*flag;
-      *flag = 0;  // ready for the next pre-pass
-    }
-  }
 }
 
 // Control data between device memory and mapped pinned host memory (one CTA; n is small).
@@ -209,6 +203,21 @@ __global__ void __launch_bounds__(256) k_fix_apply(T* __restrict__ u0, long long
     u0[c] = (T)((double)u0[c] + kappa);
 }
 
+// The same in one CTA for planes of at most FIX_ONE cells (three launches in one).
+constexpr long long FIX_ONE = 16384;
+template <typename T>
+__global__ void __launch_bounds__(1024) k_fix_one(T* __restrict__ u0, const double* __restrict__ area, long long ncell,
+                                                  const double* __restrict__ sums, double alpha, double area_total) {
+  __shared__ double sh[32];
+  __shared__ double kap;
+  double acc[1] = {0.0};
+  for (long long c = threadIdx.x; c < ncell; c += blockDim.x) acc[0] = fma(area[c], (double)u0[c], acc[0]);
+  block_sum<1>(acc, sh);
+  if (threadIdx.x == 0) kap = -(sums[2] + alpha * acc[0]) / (alpha * area_total);
+  __syncthreads();
+  for (long long c = threadIdx.x; c < ncell; c += blockDim.x) u0[c] = (T)((double)u0[c] + kap);
+}
+
 __global__ void k_shift(double* __restrict__ p, long long n, const double* __restrict__ c) {
   const double s = *c;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -222,7 +231,7 @@ template <int MODE, bool SH, bool F2, bool VP>
 void field3d_t(const LevelView<double>& L, dim3 grid, snac_plan* P, const double* f, const double* p, double* r,
                double fshift, cudaStream_t s) {
   k_field3d<MODE, SH, F2, VP><<<grid, TILE_THREADS, 0, s>>>(L, P->d_cblk, P->d_cz, P->nzt, P->kind == KIND_PP, P->cz[0].d,
-                                                             P->dz, f, p, r, fshift, P->d_partial);
+                                                             P->dz, f, p, r, fshift, sum_out(P, (int)(grid.x * grid.y)));
 }
 
 template <bool SH>
@@ -259,34 +268,24 @@ cudaError_t launch_field3d(snac_plan* P, int mode, const double* f, const double
     else if (fshift != 0.0) residual_t<true>(L, grid, P, f, p, r, fshift, need_f2, need_vp, s);
     else residual_t<false>(L, grid, P, f, p, r, fshift, need_f2, need_vp, s);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || mode == 1) return e;
-  return launch_reduce_partials(P, (int)(grid.x * grid.y), P->d_sums, s);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_prepass(snac_plan* P, const double* f, const double* p, cudaStream_t s) {
   LevelView<double> L = level_view<double>(P->lev[0]);
   const dim3 grid = field_grid(P);
   const double n3 = (double)P->n3;
-  cudaError_t e;
-  {
-    // read f and p (the flag is zero: set at plan creation, reset by the reduction that reads it)
-    LaunchScope ls(P, K_FIELD3D, 16.0 * n3, (P->singular ? 7.0 : 2.0) * n3, s);
-    if (P->singular)
-      k_prepass<true><<<grid, TILE_THREADS, 0, s>>>(L, P->d_cblk, P->nzt, P->dz, f, p, P->d_partial, P->d_flag);
-    else
-      k_prepass<false><<<grid, TILE_THREADS, 0, s>>>(L, P->d_cblk, P->nzt, P->dz, f, p, P->d_partial, P->d_flag);
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const int npart = (int)(grid.x * grid.y);
-  LaunchScope ls(P, K_REDUCE, 32.0 * npart, 4.0 * npart, s);
-  k_reduce4<<<1, 1024, 0, s>>>(P->d_partial, npart, P->d_sums, P->d_flag, P->d_sums + SUM_NONZERO);
+  // read f and p (the flag is zero: set at plan creation, reset by the sums that read it)
+  const SumOut S = sum_out(P, (int)(grid.x * grid.y), true);
+  LaunchScope ls(P, K_FIELD3D, 16.0 * n3, (P->singular ? 7.0 : 2.0) * n3, s);
+  if (P->singular) k_prepass<true><<<grid, TILE_THREADS, 0, s>>>(L, P->d_cblk, P->nzt, P->dz, f, p, S);
+  else k_prepass<false><<<grid, TILE_THREADS, 0, s>>>(L, P->d_cblk, P->nzt, P->dz, f, p, S);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce_partials(snac_plan* P, int npart, double* out, cudaStream_t s) {
   LaunchScope ls(P, K_REDUCE, 32.0 * npart, 4.0 * npart, s);
-  k_reduce4<<<1, 1024, 0, s>>>(P->d_partial, npart, out, nullptr, nullptr);
+  k_reduce4<<<1, 1024, 0, s>>>(P->d_partial, npart, out);
   return cudaGetLastError();
 }
 
@@ -312,6 +311,12 @@ cudaError_t launch_fix_mean(snac_plan* P, void* u0, cudaStream_t s) {
   const double alpha = P->dz * P->nzt / P->theta;
   const long long n = P->lev[0].ncell;
   const int w = plan_inner_size(P);
+  if (n <= FIX_ONE) {
+    LaunchScope ls(P, K_FIX_MEAN, (double)n * (8.0 + 2.0 * w), 3.0 * n, s);
+    if (w == 8) k_fix_one<double><<<1, 1024, 0, s>>>((double*)u0, P->d_area0, n, P->d_sums, alpha, P->area_total);
+    else k_fix_one<float><<<1, 1024, 0, s>>>((float*)u0, P->d_area0, n, P->d_sums, alpha, P->area_total);
+    return cudaGetLastError();
+  }
   const int ctas = std::min(MEAN_CTAS, P->npartial);  // one partial per CTA, d_partial holds npartial
   {
     LaunchScope ls(P, K_FIX_MEAN, (double)n * (8.0 + w), 2.0 * n, s);

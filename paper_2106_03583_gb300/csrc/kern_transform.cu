@@ -177,8 +177,9 @@ __global__ void __launch_bounds__(TNT, sizeof(T) == 4 ? 4 : 3) k_zbackward(const
                                                                         const CallerBlk* __restrict__ cb,
                                                                         const T* __restrict__ modes,
                                                                         double* __restrict__ p3, long long ncell,
-                                                                        double inv_theta) {
+                                                                        double inv_theta, const int* __restrict__ skip) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (skip != nullptr && *skip) return;
   z_backward<T>(A, chunks[blockIdx.x], blk, cb, modes, p3, ncell, inv_theta, smem, blockDim.x);
 }
 
@@ -259,7 +260,7 @@ cudaError_t fwd_t(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, 
 
 template <typename T, int TC>
 cudaError_t bwd_t(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, const ChunkDev* dch, const void* twb,
-                  const void* modes, double* p3, double sign, cudaStream_t s) {
+                  const void* modes, double* p3, double sign, cudaStream_t s, const int* skip) {
   const size_t smem = 2 * (size_t)(P->nzt / 2) * TC * sizeof(Cx<T>);
   const double n3 = G.n3;
   // read the modes, read and write the FP64 field
@@ -267,7 +268,7 @@ cudaError_t bwd_t(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, 
   if (P->zsmooth) {
     cudaFuncSetAttribute(k_zbackward<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kZSmem);
     k_zbackward<T><<<(unsigned)G.nz, z_threads<T>(P, G.ztc), z_smem<T>(P, G.ztc), s>>>(z_args<T>(P, G.ztc), G.zch, G.blk, G.cb,
-                                                                        (const T*)modes, p3, G.ncell, sign / P->theta);
+                                                                        (const T*)modes, p3, G.ncell, sign / P->theta, skip);
     return cudaGetLastError();
   }
   auto go = [&](auto kern) {
@@ -301,12 +302,12 @@ cudaError_t fwd_any(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch
 
 template <typename T>
 cudaError_t bwd_any(snac_plan* P, const Geom& G, const std::vector<ChunkDev>& ch, const ChunkDev* dch, const void* twb,
-                    const void* modes, double* p3, double sign, cudaStream_t s) {
+                    const void* modes, double* p3, double sign, cudaStream_t s, const int* skip = nullptr) {
   const int tc = sizeof(T) == 8 ? P->tc64 : P->tc32;
   constexpr int B = sizeof(T) == 8 ? 8 : 16;
-  if (tc == B) return bwd_t<T, B>(P, G, ch, dch, twb, modes, p3, sign, s);
-  if (tc == B / 2) return bwd_t<T, B / 2>(P, G, ch, dch, twb, modes, p3, sign, s);
-  if (tc == B / 4) return bwd_t<T, B / 4>(P, G, ch, dch, twb, modes, p3, sign, s);
+  if (tc == B) return bwd_t<T, B>(P, G, ch, dch, twb, modes, p3, sign, s, skip);
+  if (tc == B / 2) return bwd_t<T, B / 2>(P, G, ch, dch, twb, modes, p3, sign, s, skip);
+  if (tc == B / 4) return bwd_t<T, B / 4>(P, G, ch, dch, twb, modes, p3, sign, s, skip);
   return cudaErrorInvalidValue;
 }
 
@@ -323,11 +324,13 @@ cudaError_t launch_forward_f32(snac_plan* P, const float* in3, void* modes, cuda
   return fwd_any<float, float>(P, plan_geom(P), P->chunks32, P->d_chunks32, P->d_tw32, in3, modes, 0.0, false, s);
 }
 
-cudaError_t launch_backward_update(snac_plan* P, const void* modes, double* p3, cudaStream_t s, bool subtract) {
+cudaError_t launch_backward_update(snac_plan* P, const void* modes, double* p3, cudaStream_t s, bool subtract,
+                                   const int* skip) {
   const double sign = subtract ? -1.0 : 1.0;
+  if (skip && !P->zsmooth) return cudaErrorInvalidValue;
   if (P->precision == SNAC_FP64)
-    return bwd_any<double>(P, plan_geom(P), P->chunks64, P->d_chunks64, P->d_tw64, modes, p3, sign, s);
-  return bwd_any<float>(P, plan_geom(P), P->chunks32, P->d_chunks32, P->d_tw32, modes, p3, sign, s);
+    return bwd_any<double>(P, plan_geom(P), P->chunks64, P->d_chunks64, P->d_tw64, modes, p3, sign, s, skip);
+  return bwd_any<float>(P, plan_geom(P), P->chunks32, P->d_chunks32, P->d_tw32, modes, p3, sign, s, skip);
 }
 
 // Pencil of a sharded solve: ncols columns stored [z][c], one pseudo-block (nx = ncols, ny = 1,

@@ -1229,11 +1229,11 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     // per-CTA partial sums: the 3-D residual grid (tiles x z split) or a plane reduction (MEAN_CTAS)
     P->npartial = std::max((int)P->lev[0].tiles.size() * zsplit, MEAN_CTAS);
     if ((st = dmalloc(P, &P->d_partial, (size_t)P->npartial * 4))) break;
-    if ((st = dmalloc(P, &P->d_sums, SUM_SLOTS)) || (st = dmalloc(P, &P->d_flag, 1))) break;
+    if ((st = dmalloc(P, &P->d_sums, SUM_SLOTS)) || (st = dmalloc(P, &P->d_flag, 2))) break;
     // per-mode, per-tile partial sums (basic tiles; the fused tiles are fewer)
     if ((st = dmalloc(P, &P->d_mode_part, (size_t)P->nz * std::max<size_t>(P->lev[0].tiles.size(), 64)))) break;
     if ((st = dmalloc(P, &P->d_mode_norm2, (size_t)P->nz))) break;
-    if (P->onchip && (st = dmalloc(P, &P->d_fused, 2))) break;
+    if (P->onchip && (st = dmalloc(P, &P->d_fused, 3))) break;
     if ((st = dmalloc(P, &P->d_active, (size_t)P->nz)) || (st = dmalloc(P, &P->d_check, (size_t)P->nz))) break;
     auto mapped = [](auto** h, auto** dh, size_t n) {
       return cudaHostAlloc((void**)h, n * sizeof(**h), cudaHostAllocMapped) == cudaSuccess &&
@@ -1246,11 +1246,12 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
       break;
     }
     {
-      // the pre-pass flag starts at zero (its reduction resets it after each use); on a private
-      // non-blocking stream, like every other device write of plan creation
+      // the pre-pass flag, the ticket of the sums and the counters of the fused launch start at zero (each
+      // use resets them); on a private non-blocking stream, like every other device write of plan creation
       cudaStream_t cs = nullptr;
       bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
-                cudaMemsetAsync(P->d_flag, 0, sizeof(int), cs) == cudaSuccess && cudaStreamSynchronize(cs) == cudaSuccess;
+                cudaMemsetAsync(P->d_flag, 0, 2 * sizeof(int), cs) == cudaSuccess &&
+                (!P->d_fused || cudaMemsetAsync(P->d_fused, 0, 3 * sizeof(int), cs) == cudaSuccess) && cudaStreamSynchronize(cs) == cudaSuccess;
       if (cs) cudaStreamDestroy(cs);
       if (!ok) {
         st = fail(SNAC_ERR_CUDA, "initialising the pre-pass flag failed");

@@ -237,7 +237,8 @@ struct snac_plan {
   double* d_pweight = nullptr;
   int* h_cycles = nullptr;    // per wavenumber: V-cycles of the last on-chip solve (mapped pinned)
   int* dh_cycles = nullptr;
-  int* d_fused = nullptr;     // the fused transform + on-chip launch's counters: next item, chunks done
+  int* d_fused = nullptr;     // the fused transform + on-chip launch's counters: next item, chunks done;
+                              // [2]: 1 if a wait of the last launch gave up
   int* h_wait = nullptr;      // set by that launch when a bounded wait gave up (mapped pinned)
   int* dh_wait = nullptr;
   int nblk = 0;
@@ -297,7 +298,7 @@ struct snac_plan {
   double* d_partial = nullptr;  // per-CTA partial sums
   int npartial = 0;
   double* d_sums = nullptr;     // reduced sums (SUM_SLOTS)
-  int* d_flag = nullptr;        // nonzero-initial-guess flag of the pre-pass
+  int* d_flag = nullptr;        // [0] nonzero-initial-guess flag of the pre-pass, [1] ticket of the sums
   double* d_mode_part = nullptr;  // per-mode, per-tile partial sums of squares
   double* d_mode_norm2 = nullptr; // per-mode ||r_q||^2
   int* d_active = nullptr;
@@ -392,7 +393,9 @@ cudaError_t launch_forward_f32(snac_plan* P, const float* in3, void* modes, cuda
 // Level-0 mode planes from plain to colour-split order.
 cudaError_t launch_to_split(snac_plan* P, const double* src, double* dst, cudaStream_t s);
 // p3 += F^-1(modes) / theta; subtract: p3 -= F^-1(modes) / theta (takes a correction back)
-cudaError_t launch_backward_update(snac_plan* P, const void* modes, double* p3, cudaStream_t s, bool subtract = false);
+// skip (smooth lengths): device flag; nonzero leaves p3 as it is
+cudaError_t launch_backward_update(snac_plan* P, const void* modes, double* p3, cudaStream_t s, bool subtract = false,
+                                   const int* skip = nullptr);
 // Pencils of a sharded solve ([z][c] fields of ncols columns): forward transform, backward update.
 cudaError_t launch_pencil_forward(snac_plan* P, long long ncols, const double* in, void* modes, cudaStream_t s);
 cudaError_t launch_pencil_backward(snac_plan* P, long long ncols, const void* modes, double* p, cudaStream_t s);
@@ -456,7 +459,7 @@ cudaError_t launch_direct(snac_plan* P, cudaStream_t s);
 // The reciprocal pivots of an FP64 plan's tridiagonal systems, once per plan (d_qof: a wavenumber of
 // every set).
 cudaError_t launch_tri_factor(snac_plan* P, const int* d_qof, int rows, cudaStream_t s);
-// *h_wait = 1 if any of the n values (inner type) is NaN or Inf, else 0.
+// h_check[0] = 1 if any of the n values (inner type) is NaN or Inf, else 0.
 cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStream_t s);
 // Where a solve leaves the mode-space solution: the level-0 iterate, or (direct solves of planes too
 // large for one CTA, whose last pass goes back to the planes' order) the level-0 right-hand side.

@@ -311,10 +311,7 @@ int mode_solves(snac_plan* P, double target, cudaStream_t s, int* cycles_out) {
   if (P->direct.on) {  // (the V-cycle paths see a non-finite right-hand side in its norms)
     CK(launch_nonfinite(P, P->lev[0].d_f, (long long)P->nz * P->lev[0].ncell, s));
     CK(cudaStreamSynchronize(s));
-    if (*P->h_wait) {
-      *P->h_wait = 0;
-      return SNAC_ERR_NONFINITE;
-    }
+    if (P->h_check[0]) return SNAC_ERR_NONFINITE;
     if (!P->onchip) {
       CK(launch_direct(P, s));
       direct_results(P, cycles_out);
@@ -338,11 +335,16 @@ int mode_solves(snac_plan* P, double target, cudaStream_t s, int* cycles_out) {
   return r.st;
 }
 
-int read_sums(snac_plan* P, cudaStream_t s, int n = 4) {
-  CK(launch_to_host(P->d_sums, P->dh_sums, n, s));
+// After a 3-D pass: its sums are in h_sums.
+int read_sums(snac_plan* P, cudaStream_t s) {
   CK(cudaStreamSynchronize(s));
-    profile_resolve(P);
+  profile_resolve(P);
   return SNAC_OK;
+}
+
+int wait_gave_up() {
+  set_error("a device-side wait gave up (transform chunks not counted within the limit)");
+  return SNAC_ERR_TIMEOUT;
 }
 
 // One problem's solve as a sequence of steps, so that several problems can run in lock-step: their
@@ -357,6 +359,7 @@ struct Job {
   int st = SNAC_OK;
   bool finished = false;
   bool p_zero = false, updated = false, aim_final = false, r32 = false, ff = false, redo = false;
+  bool late_wait = false;  // the status of the step's bounded waits is read with the next residual
   bool fused = false;  // this step's forward transform runs inside the on-chip launch
   FusedInput fin{};
   double fshift = 0.0, fn = 0.0, fn_pre = 0.0, prev_rel = INFINITY, rn = 0.0, target = 0.0;
@@ -385,9 +388,7 @@ cudaError_t job_begin(Job& J, cudaStream_t s) {
   P->info.n_modes = P->nz;
   std::fill(P->mode_cycles.begin(), P->mode_cycles.end(), 0);
   J.cyc.assign(P->nz, 0);
-  cudaError_t e = launch_prepass(P, J.f, J.p, s);
-  if (e == cudaSuccess) e = launch_to_host(P->d_sums, P->dh_sums, SUM_NONZERO + 1, s);
-  return e;
+  return launch_prepass(P, J.f, J.p, s);
 }
 
 void job_begin_read(Job& J) {
@@ -432,7 +433,6 @@ cudaError_t job_resid_launch(Job& J, cudaStream_t s) {
   } else {
     e = launch_field3d(P, 0, J.f, J.p, P->d_r3, J.fshift, J.k == 0, need_vp, s);
   }
-  if (e == cudaSuccess) e = launch_to_host(P->d_sums, P->dh_sums, 4, s);
   return e;
 }
 
@@ -442,6 +442,11 @@ cudaError_t job_resid_read(Job& J, cudaStream_t s) {
   snac_plan* P = J.P;
   profile_resolve(P);
   if (J.k == 0 && J.p_zero) return cudaSuccess;
+  if (J.late_wait && *P->h_wait) {  // the last step's update was skipped on the device
+    J.finish(wait_gave_up());
+    return cudaSuccess;
+  }
+  J.late_wait = false;
   if (J.ff && !J.redo) {
     J.rn = std::sqrt(P->h_sums[0]);
     // (NaN stays: reported by the decision). Direct plans take another step anyway above half the
@@ -450,9 +455,7 @@ cudaError_t job_resid_read(Job& J, cudaStream_t s) {
     if (J.r32) return cudaSuccess;
     J.redo = true;
     const bool need_vp = P->singular;
-    cudaError_t e = launch_field3d(P, 0, J.f, J.p, P->d_r3, J.fshift, false, need_vp, s);
-    if (e == cudaSuccess) e = launch_to_host(P->d_sums, P->dh_sums, 4, s);
-    return e;
+    return launch_field3d(P, 0, J.f, J.p, P->d_r3, J.fshift, false, need_vp, s);
   }
   if (J.k == 0) J.fn = std::sqrt(P->h_sums[1]);
   J.rn = std::sqrt(P->h_sums[0]);
@@ -543,7 +546,8 @@ cudaError_t job_update(Job& J, cudaStream_t s) {
   }
   cudaError_t e = cudaSuccess;
   if (P->singular) e = launch_fix_mean(P, mode_solution(P), s);
-  if (e == cudaSuccess) e = launch_backward_update(P, mode_solution(P), J.p, s);
+  if (e == cudaSuccess)
+    e = launch_backward_update(P, mode_solution(P), J.p, s, false, J.late_wait ? P->d_fused + 2 : nullptr);
   J.updated = true;
   ++J.k;
   return e;
@@ -629,9 +633,13 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
     bool any = false;
     for (Job& J : jobs) any = any || !J.finished;
     if (!any) break;
+    bool wait = false;  // (a step from a zero guess has no residual pass)
     for (Job& J : jobs)
-      if (!J.finished) job_cuda(J, job_resid_launch(J, js(J)), "residual");
-    if ((e = sync()) != cudaSuccess) { status = cuda_fail(e, "cudaStreamSynchronize"); break; }
+      if (!J.finished) {
+        job_cuda(J, job_resid_launch(J, js(J)), "residual");
+        wait = wait || !(J.k == 0 && J.p_zero);
+      }
+    if (wait && (e = sync()) != cudaSuccess) { status = cuda_fail(e, "cudaStreamSynchronize"); break; }
     bool redo = false;
     for (Job& J : jobs)
       if (!J.finished && job_cuda(J, job_resid_read(J, js(J)), "residual") == SNAC_OK) redo = redo || J.redo;
@@ -744,7 +752,21 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
           if (runs[k].st) owners[k]->finish(runs[k].st);
       }
     }
-    if (!chip[0].empty() || !chip[1].empty() || !fusedj[0].empty() || !fusedj[1].empty()) {
+    // direct on-chip solves run one step whatever their numbers: their update and the next residual follow
+    // on the device, and the host looks at the status of their waits with that residual (the update skips
+    // itself where a wait gave up)
+    bool look = !chip[0].empty() || !chip[1].empty();
+    for (int g = 0; g < 2; ++g)
+      for (Job* J : fusedj[g]) look = look || !(J->P->direct.on && J->P->zsmooth);
+    if (!look && (!fusedj[0].empty() || !fusedj[1].empty())) {
+      if ((e = ss.fork()) != cudaSuccess) { status = cuda_fail(e, "cudaStreamWaitEvent"); break; }
+      for (int g = 0; g < 2; ++g)
+        for (Job* J : fusedj[g])
+          if (!J->finished) {
+            direct_results(J->P, J->cyc.data());
+            J->late_wait = true;
+          }
+    } else if (look) {
       if ((e = sync()) != cudaSuccess) { status = cuda_fail(e, "cudaStreamSynchronize"); break; }
       for (int g = 0; g < 2; ++g) {
         for (Job* J : chip[g])
@@ -757,8 +779,7 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
           if (!J->finished) {
             profile_resolve(J->P);
             if (*J->P->h_wait) {
-              set_error("a device-side wait gave up (transform chunks not counted within the limit)");
-              J->finish(SNAC_ERR_TIMEOUT);
+              J->finish(wait_gave_up());
               continue;
             }
             const int st = onchip_results(J->P, J->cyc.data());
