@@ -8,6 +8,12 @@
 // V-cycles. "m" numbers cells along the transformed axis (M of them), "n" along the tridiagonal one
 // (N); spectral slot kappa stands for one eigenvector of the transformed axis.
 //
+// Layouts of several such rectangles (pieces) that meet along parts of their first or last rows are solved
+// piece by piece with Neumann faces there; the fluxes through the shared faces are the unknowns of a dense
+// system per wavenumber, whose right-hand side needs only the first and last rows of the pieces' solutions.
+// So a solve is: transforms, end values, interface systems (fluxes added to the end rows), tridiagonal
+// solves, inverse transforms.
+//
 // Transforms work on complex columns of a shared-memory buffer (fft_dev.cuh):
 //   pair kinds (PP, NN, DD): column c holds lines 2c and 2c+1 as real and imaginary part of one
 //       length-M FFT; with Z_k = A_k + i B_k the two spectra separate by additions. PP is kept at twice
@@ -24,6 +30,8 @@
 // where the system is nearly singular, and an exactly singular one (all tau = 0) ends in an exactly zero
 // pivot, whose unknown is set to zero (the caller fixes the mean).
 #pragma once
+
+#include <algorithm>
 
 #include "fft_dev.cuh"
 
@@ -51,8 +59,10 @@ struct DirectArgs {
   const T* lam;            // eigenvalue of slot kappa (<= 0), times cscale
   const TriRow<T>* tri;    // [N], times cscale
   const T* sigma;          // per wavenumber
-  const unsigned* cellmn;  // per plane cell: m | n << 16
+  const T* w;              // [N] cell widths along the tridiagonal axis
   long long ncell;
+  int soff;                // the piece's first spectral element within a plane
+  int e0, e1;              // where its first / last row's values start in the end vector, -1: not needed
   T cscale;                // power of two that brings the couplings of tri (and lam) to about 1
   T scale;                 // cscale / 2M
   // plane offset of (m, n): base[n nbm + mblk[m]] + m mstr[n]
@@ -63,9 +73,14 @@ struct DirectArgs {
 };
 
 template <typename T>
-inline DirectArgs<T> direct_args(const snac_plan* P) {
-  const DirectTab& D = P->direct;
+inline DirectArgs<T> direct_args(const snac_plan* P, const DirectTab& D) {
   DirectArgs<T> A{};
+  const IfaceTab& I = P->direct.it;
+  A.e0 = A.e1 = -1;
+  for (int u = 0; u < I.nends; ++u)
+    if (&P->direct.pc[I.ep[u]] == &D) (I.ee[u] == 0 ? A.e0 : A.e1) = I.eo[u];
+  A.soff = D.soff;
+  A.w = (const T*)D.d_w;
   A.F = D.fft;
   A.M = D.M;
   A.N = D.N;
@@ -81,7 +96,6 @@ inline DirectArgs<T> direct_args(const snac_plan* P) {
   A.tri = (const TriRow<T>*)D.d_tri;
   if constexpr (sizeof(T) == 8) A.sigma = P->d_sigma64;
   else A.sigma = P->d_sigma32;
-  A.cellmn = D.d_cellmn;
   A.ncell = P->lev[0].ncell;
   A.cscale = (T)D.cscale;
   A.scale = (T)(D.cscale / (2.0 * D.M));
@@ -92,6 +106,109 @@ inline DirectArgs<T> direct_args(const snac_plan* P) {
   A.xl = D.xl;
   A.vec = D.vec;
   return A;
+}
+
+template <typename T>
+struct IfaceArgs {
+  int k, kk, E, ns, qs, gs;         // gs: the whole problem is singular (the last constraint is implied)
+  int sp[IFACE_MAX_ENDS];
+  int nends, eo[IFACE_MAX_ENDS + 1];
+  int row[IFACE_MAX_ENDS];          // first spectral element of every end row within a plane
+  const double* Y;
+  const T* Z;
+  const double* KT;
+  T* ends;
+  T* alpha;
+  T* ssum;
+};
+
+template <typename T>
+inline IfaceArgs<T> iface_args(const snac_plan* P) {
+  const IfaceTab& I = P->direct.it;
+  IfaceArgs<T> A{};
+  A.k = I.k;
+  A.kk = I.kk;
+  A.E = I.E;
+  A.ns = I.ns;
+  A.qs = I.qs;
+  A.gs = P->singular ? 1 : 0;
+  A.nends = I.nends;
+  for (int u = 0; u < I.nends; ++u) {
+    const DirectTab& D = P->direct.pc[I.ep[u]];
+    A.eo[u] = I.eo[u];
+    A.row[u] = D.soff + (I.ee[u] ? (D.N - 1) * D.M : 0);
+  }
+  A.eo[I.nends] = I.E;
+  for (int a = 0; a < I.ns; ++a) A.sp[a] = I.sp[a];
+  A.Y = I.d_Y;
+  A.Z = (const T*)I.d_Z;
+  A.KT = I.d_KT;
+  A.ends = (T*)I.d_ends;
+  A.alpha = (T*)I.d_alpha;
+  A.ssum = (T*)I.d_ssum;
+  return A;
+}
+
+// out[j] = sum_e A[e ld + j] x[e] for j < n by a CTA of nt threads (part: nt values); x in shared memory.
+template <typename TA>
+__device__ void gemv_cols(const TA* __restrict__ A, int ld, int n, int E, const TA* __restrict__ x, TA* __restrict__ out,
+                          TA* __restrict__ part, int nt) {
+  const int np = (n + 31) & ~31, tid = threadIdx.x;
+  if (np <= nt) {  // the rows e split over nt / np groups of threads
+    const int G = nt / np, g = tid / np, j = tid - g * np;
+    TA acc = 0;
+    if (g < G && j < n) {
+#pragma unroll 16
+      for (int e = g; e < E; e += G) acc = fma(A[(long long)e * ld + j], x[e], acc);
+    }
+    part[tid] = acc;
+    __syncthreads();
+    if (tid < n) {
+      TA s = 0;
+      for (int q = 0; q < G; ++q) s += part[q * np + tid];
+      out[tid] = s;
+    }
+  } else {
+    for (int j = tid; j < n; j += nt) {
+      TA acc = 0;
+#pragma unroll 16
+      for (int e = 0; e < E; ++e) acc = fma(A[(long long)e * ld + j], x[e], acc);
+      out[j] = acc;
+    }
+  }
+  __syncthreads();
+}
+
+// The fluxes of wavenumber q from its end values: jumps of u across the interface cells, the dense system,
+// and what the fluxes add to the end rows' right-hand sides (add(e, v)); alpha: the singular pieces'
+// constants (by piece). The jumps are differences of nearly equal end values and K^-1 damps their smooth
+// part by the pieces' size in cells, so both products are formed in FP64 in every plan (in FP32 their
+// rounding left a second correction step at 1e-9 .. 2e-8 of ||f|| on the L-shaped 512 x 512 x 128 duct).
+// work (doubles, shared): ends (complete), y, phi, part: E + 2 kk + nt; ssum by piece.
+template <typename T, typename Add>
+__device__ void iface_solve(const IfaceArgs<T>& I, int q, double* work, const T* ssum, T* alpha, int nt, Add&& add) {
+  double* ends = work;
+  double* y = ends + I.E;
+  double* phi = y + I.kk;
+  double* part = phi + I.kk;
+  gemv_cols(I.Y, I.kk, I.k, I.E, ends, y, part, nt);
+  if ((int)threadIdx.x < I.ns) {
+    const int a = threadIdx.x;
+    y[I.k + a] = q == I.qs && !(I.gs && a == I.ns - 1) ? -(double)ssum[I.sp[a]] : 0.0;
+  }
+  __syncthreads();
+  gemv_cols(I.KT + (long long)q * I.kk * I.kk, I.kk, I.kk, I.kk, y, phi, part, nt);
+  if ((int)threadIdx.x < I.ns && q == I.qs) alpha[I.sp[threadIdx.x]] = (T)phi[I.k + threadIdx.x];
+  T* ph = reinterpret_cast<T*>(part);  // (kk <= 1040 values of T fit in nt doubles)
+  for (int j = threadIdx.x; j < I.k; j += nt) ph[j] = (T)phi[j];
+  __syncthreads();
+  for (int e = threadIdx.x; e < I.E; e += nt) {
+    T acc = 0;
+#pragma unroll 16
+    for (int j = 0; j < I.k; ++j) acc = fma(I.Z[(long long)j * I.E + e], ph[j], acc);
+    add(e, acc);
+  }
+  __syncthreads();
 }
 
 // Two spectra from one pair column: z1 = Z_k, z2 = Z_{M-k}; slots k -> y1 (line a, line b), M-k -> y2.
@@ -136,13 +253,13 @@ __device__ __forceinline__ double tri_recip(double x) { return recip(x); }
 // unknown), the segments' last unknowns form a tridiagonal system of P rows that the first segment's
 // thread solves, and each thread substitutes back. load(n) gives the right-hand side, store(n, u)
 // takes the solution; ex: 7 x P x kg values, this system's column kk. Every thread of the CTA calls it
-// (three barriers). tq = -lambda - sigma >= 0.
+// (three barriers). tq = -lambda - sigma >= 0; alpha: the last unknown of an exactly singular system.
 // `act` is false for threads past the last segment, which only take part in the barriers; `live`
 // for those with a system to solve.
 template <typename T, int R, typename Load, typename Store>
 __device__ __forceinline__ void tri_segment(const TriRow<T>* __restrict__ tri, int N, int P, int seg, int kk, int kg,
-                                            bool act, bool live, T tq, T scale, T* __restrict__ ex, Load&& load,
-                                            Store&& store) {
+                                            bool act, bool live, T tq, T scale, T alpha, T* __restrict__ ex,
+                                            Load&& load, Store&& store) {
   const int n0 = seg * R - (P * R - N);
   T D[R], c[R];
 #pragma unroll
@@ -196,7 +313,7 @@ __device__ __forceinline__ void tri_segment(const TriRow<T>* __restrict__ tri, i
       const T den = sum + hi;
       const T inv = den > (T)0 ? tri_recip(den) : (T)0;
       g = sum * inv;
-      y = fma(lo, y, d) * inv;
+      y = den > (T)0 ? fma(lo, y, d) * inv : alpha;
       z[o] = y;
       z[o + st] = hi * inv;
     }
@@ -229,45 +346,55 @@ constexpr int PLANE_R = 8;  // rows per thread of the tridiagonal phase
 
 struct PlaneShape {
   int cols, rp, s1;
-  size_t buf, bytes;  // elements of the buffer (real), bytes in all
+  size_t buf;  // elements of the buffer (real)
 };
-__host__ __device__ inline PlaneShape plane_shape(const FftTab& F, int M, int N, int cls, size_t w, int nt) {
+__host__ __device__ inline PlaneShape plane_shape(const FftTab& F, int M, int N, int cls) {
   PlaneShape s;
   s.cols = cls == LINES_PAIR ? (N + 1) / 2 : N;
   s.rp = s.cols | 1;
   s.s1 = F.l1 * s.rp;
   s.s1 += (1 - s.s1) & 15;  // consecutive slots of the first radix on different banks
   s.buf = 2 * (size_t)(F.n / F.l1) * s.s1;
-  s.bytes = (s.buf + 7 * (size_t)nt) * w;
   return s;
 }
+// Elements of shared memory of a whole-plane solve: the pieces' buffers, the exchange of the tridiagonal
+// segments, the singular pieces' constants and sums, and (doubles) the work space of an interface solve.
+inline size_t onchip_elements(size_t buffers, int nt) {
+  return ((buffers + 1) & ~(size_t)1) + 7 * (size_t)nt + 2 * IFACE_MAX_ENDS;
+}
+inline size_t iface_doubles(int E, int kk, int nt) {
+  return E ? E + 2 * (size_t)kk + std::max((size_t)nt, (size_t)kk) : 0;
+}
 
-// One wavenumber's solve by one CTA of nt threads, the whole plane in shared memory: f -> u (global
-// plane of this wavenumber, caller cell order).
 template <typename T>
-__device__ void plane_direct(const DirectArgs<T>& A, int q, const T* __restrict__ f, T* __restrict__ u,
-                             unsigned char* smem, int nt) {
-  const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls, sizeof(T), nt);
-  Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
-  T* bt = reinterpret_cast<T*>(smem);
-  T* ex = bt + S.buf;
+struct PlaneArgs {
+  int np;
+  const DirectArgs<T>* pc;   // device table
+  const unsigned* celloff;   // per plane cell: element of the shared buffers | sign flip << 31
+  long long ncell;
+  size_t buffers;            // elements of all pieces' buffers (even)
+  IfaceArgs<T> I;
+};
+
+template <typename T>
+inline PlaneArgs<T> plane_args(const snac_plan* P) {
+  PlaneArgs<T> A{};
+  A.np = (int)P->direct.pc.size();
+  A.pc = (const DirectArgs<T>*)P->direct.d_args;
+  A.celloff = P->direct.d_celloff;
+  A.ncell = P->lev[0].ncell;
+  for (const DirectTab& d : P->direct.pc) A.buffers += plane_shape(d.fft, d.M, d.N, d.cls).buf;
+  A.buffers = (A.buffers + 1) & ~(size_t)1;
+  A.I = iface_args<T>(P);
+  return A;
+}
+
+// Planes to spectra of one piece in its buffer (complete on entry, behind a barrier on return).
+template <typename T>
+__device__ void piece_forward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T>* buf, int nt) {
   const ColsAny cm{S.cols, S.rp};
-  const int M = A.M, N = A.N, kind = A.kind, l1 = A.F.l1;
-  const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
-  const int ncell = (int)A.ncell;
-  if (pair && (N & 1)) {  // the last column's missing line
-    for (int m = threadIdx.x; m < M; m += nt) bt[2 * (fft_row(m, l1, S.s1, S.rp) + S.cols - 1) + 1] = 0;
-  }
-  for (int c = threadIdx.x; c < ncell; c += nt) {
-    const unsigned mn = A.cellmn[c];
-    const int m = mn & 0xffffu, n = mn >> 16;
-    const T v = neg_if(flip && (m & 1), f[c]);
-    int o;
-    if (pair) o = 2 * (fft_row(pair_pos(kind, m, M), l1, S.s1, S.rp) + (n >> 1)) + (n & 1);
-    else o = 2 * (fft_row((m & 1) ? (M - 1 - m) >> 1 : m >> 1, l1, S.s1, S.rp) + n) + (m & 1);
-    bt[o] = v;
-  }
-  __syncthreads();
+  const int M = A.M, kind = A.kind, l1 = A.F.l1;
+  const bool pair = A.cls == LINES_PAIR;
   if (!pair) {
     for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
       int j, c;
@@ -299,30 +426,52 @@ __device__ void plane_direct(const DirectArgs<T>& A, int q, const T* __restrict_
     }
   }
   __syncthreads();
-  {
-    const int P = (N + PLANE_R - 1) / PLANE_R, kg = nt / P;
-    const int seg = quot16(threadIdx.x, kg), kk = threadIdx.x - seg * kg;
-    const bool mine = seg < P;
-    const T sg = A.sigma[q];
-    for (int k0 = 0; k0 < M; k0 += kg) {
-      const int kap = k0 + kk;
-      const bool live = mine && kap < M;
-      int o = 0, ns = 1;
-      T tq = 0;
-      if (live) {
-        tq = -fma(sg, A.cscale, A.lam[kap]);
-        if (pair) {
-          o = 2 * fft_row(A.perm[kap], l1, S.s1, S.rp);
-        } else {
-          ns = 2;
-          o = 2 * fft_row(A.perm[(kap & 1) ? (M - 1 - kap) >> 1 : kap >> 1], l1, S.s1, S.rp) + (kap & 1);
-        }
-      }
-      tri_segment<T, PLANE_R>(A.tri, N, P, mine ? seg : 0, kk, kg, mine, live, tq, A.scale, ex,
-                              [&](int n) { return bt[o + n * ns]; }, [&](int n, T v) { bt[o + n * ns] = v; });
+}
+
+// Where slot kappa of a piece stands in its buffer: element o + n ns for row n.
+template <typename T>
+__device__ __forceinline__ int slot_at(const DirectArgs<T>& A, const PlaneShape& S, int kap) {
+  if (A.cls == LINES_PAIR) return 2 * fft_row(A.perm[kap], A.F.l1, S.s1, S.rp);
+  return 2 * fft_row(A.perm[(kap & 1) ? (A.M - 1 - kap) >> 1 : kap >> 1], A.F.l1, S.s1, S.rp) + (kap & 1);
+}
+
+// The tridiagonal systems of one piece; ENDS: only the first and last rows' solutions, into the end vector.
+template <typename T, bool ENDS>
+__device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T sg, T alpha, T* ex, double* ends, int nt) {
+  const int N = A.N, M = A.M;
+  const int P = (N + PLANE_R - 1) / PLANE_R, kg = nt / P;
+  const int seg = quot16(threadIdx.x, kg), kk = threadIdx.x - seg * kg;
+  const bool mine = seg < P;
+  const int ns = A.cls == LINES_PAIR ? 1 : 2;
+  for (int k0 = 0; k0 < M; k0 += kg) {
+    const int kap = k0 + kk;
+    const bool live = mine && kap < M;
+    int o = 0;
+    T tq = 0;
+    if (live) {
+      tq = -fma(sg, A.cscale, A.lam[kap]);
+      o = slot_at(A, S, kap);
     }
+    tri_segment<T, PLANE_R>(A.tri, N, P, mine ? seg : 0, kk, kg, mine, live, tq, A.scale, alpha, ex,
+                            [&](int n) { return bt[o + n * ns]; },
+                            [&](int n, T v) {
+                              if (!ENDS) {
+                                bt[o + n * ns] = v;
+                              } else {
+                                if (n == 0 && A.e0 >= 0) ends[A.e0 + kap] = v;
+                                if (n == N - 1 && A.e1 >= 0) ends[A.e1 + kap] = v;
+                              }
+                            });
   }
   __syncthreads();
+}
+
+// Spectra back to planes of one piece.
+template <typename T>
+__device__ void piece_backward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T>* buf, int nt) {
+  const ColsAny cm{S.cols, S.rp};
+  const int M = A.M, kind = A.kind, l1 = A.F.l1;
+  const bool pair = A.cls == LINES_PAIR;
   if (pair) {
     for (int t = threadIdx.x; t < (M / 2 + 1) * S.cols; t += nt) {
       int k, c;
@@ -342,24 +491,91 @@ __device__ void plane_direct(const DirectArgs<T>& A, int q, const T* __restrict_
       cm.split(t, j, c);
       const int o = fft_row(A.perm[j], l1, S.s1, S.rp) + c;
       const Cpl<T> v = cx_mul(buf[o], A.t4a[j]);
-      buf[o] = Cpl<T>{v.re, -v.im};
+      buf[o] = Cpl<T>{v.re, -v.im};  // forward = conj(inverse(conj))
     }
   }
   __syncthreads();
   fft_all<true>(buf, A.F, S.s1, cm, A.tw, nt);
-  for (int c = threadIdx.x; c < ncell; c += nt) {
-    const unsigned mn = A.cellmn[c];
-    const int m = mn & 0xffffu, n = mn >> 16;
-    T v;
-    if (pair) {
-      v = bt[2 * (fft_row(pair_pos(kind, m, M), l1, S.s1, S.rp) + (n >> 1)) + (n & 1)];
-    } else {
-      const int k = (m & 1) ? (M - 1 - m) >> 1 : m >> 1;
-      const Cpl<T> z = buf[fft_row(k, l1, S.s1, S.rp) + n];
+  if (!pair) {
+    for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
+      int k, c;
+      cm.split(t, k, c);
+      const int o = fft_row(k, l1, S.s1, S.rp) + c;
+      const Cpl<T> z = buf[o];
       const Cpl<T> y = cx_mul(Cpl<T>{z.re, -z.im}, A.t4b[k]);
-      v = (m & 1) ? (T)-2 * y.im : (T)2 * y.re;
+      buf[o] = Cpl<T>{(T)2 * y.re, (T)-2 * y.im};
     }
-    u[c] = neg_if(flip && (m & 1), v);
+    __syncthreads();
+  }
+}
+
+// One wavenumber's solve by one CTA of nt threads, the whole plane in shared memory: f -> u (global
+// plane of this wavenumber, plane cell order).
+template <typename T>
+__device__ void plane_direct(const PlaneArgs<T>& O, T sg, int q, const T* __restrict__ f, T* __restrict__ u,
+                             unsigned char* smem, int nt) {
+  T* bt = reinterpret_cast<T*>(smem);
+  T* ex = bt + O.buffers;
+  T* alpha = ex + 7 * nt;
+  T* ssum = alpha + IFACE_MAX_ENDS;
+  double* work = reinterpret_cast<double*>(ssum + IFACE_MAX_ENDS);
+  const int ncell = (int)O.ncell;
+  if (threadIdx.x < 2 * IFACE_MAX_ENDS) alpha[threadIdx.x] = 0;
+  size_t b0 = 0;
+  for (int p = 0; p < O.np; ++p) {  // an odd number of lines: the last pair column's missing one
+    const DirectArgs<T>& A = O.pc[p];
+    const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
+    if (A.cls == LINES_PAIR && (A.N & 1))
+      for (int m = threadIdx.x; m < A.M; m += nt) bt[b0 + 2 * (fft_row(m, A.F.l1, S.s1, S.rp) + S.cols - 1) + 1] = 0;
+    b0 += S.buf;
+  }
+  for (int c = threadIdx.x; c < ncell; c += nt) {
+    const unsigned o = O.celloff[c];
+    bt[o & 0x7fffffffu] = neg_if(o >> 31, f[c]);
+  }
+  __syncthreads();
+  b0 = 0;
+  for (int p = 0; p < O.np; ++p) {
+    const DirectArgs<T> A = O.pc[p];
+    const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
+    piece_forward(A, S, reinterpret_cast<Cpl<T>*>(bt + b0), nt);
+    if (O.I.k) {
+      piece_tri<T, true>(A, S, bt + b0, sg, (T)0, ex, work, nt);
+      if (q == O.I.qs && threadIdx.x < 32) {
+        const int o = slot_at(A, S, 0), ns = A.cls == LINES_PAIR ? 1 : 2;
+        T s = 0;
+        for (int n = threadIdx.x; n < A.N; n += 32) s = fma(A.w[n], bt[b0 + o + n * ns], s);
+        s = warp_sum_t(s);
+        if (threadIdx.x == 0) ssum[p] = s;
+      }
+    }
+    b0 += S.buf;
+  }
+  if (O.I.k) {
+    __syncthreads();
+    iface_solve(O.I, q, work, ssum, alpha, nt, [&](int e, T v) {
+      size_t b = 0;
+      for (int p = 0; p < O.np; ++p) {
+        const DirectArgs<T>& A = O.pc[p];
+        const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
+        const int ns = A.cls == LINES_PAIR ? 1 : 2;
+        if (A.e0 >= 0 && e >= A.e0 && e < A.e0 + A.M) bt[b + slot_at(A, S, e - A.e0)] += v;
+        if (A.e1 >= 0 && e >= A.e1 && e < A.e1 + A.M) bt[b + slot_at(A, S, e - A.e1) + (A.N - 1) * ns] += v;
+        b += S.buf;
+      }
+    });
+  }
+  b0 = 0;
+  for (int p = 0; p < O.np; ++p) {
+    const DirectArgs<T> A = O.pc[p];
+    const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
+    piece_tri<T, false>(A, S, bt + b0, sg, O.I.k && q == O.I.qs ? alpha[p] : (T)0, ex, nullptr, nt);
+    piece_backward(A, S, reinterpret_cast<Cpl<T>*>(bt + b0), nt);
+    b0 += S.buf;
+  }
+  for (int c = threadIdx.x; c < ncell; c += nt) {
+    const unsigned o = O.celloff[c];
+    u[c] = neg_if(o >> 31, bt[o & 0x7fffffffu]);
   }
   __syncthreads();  // the shared memory is free for the next wavenumber
 }

@@ -1,0 +1,562 @@
+// Plan creation for direct solves of the reduced equations (direct_dev.cuh): which layouts allow them, the
+// pieces, and their tables.
+//
+// Blocks connected along the transformed axis form chains; chains stacked on one another along the other
+// axis with every face connected form a piece: a rectangle with one tensor grid. A layout of one piece (any
+// assembled rectangle) separates as it stands. Several pieces (L and T shapes, a channel with a side
+// branch) meet along parts of their first and last rows: each piece is solved with a Neumann condition
+// there, and the fluxes through the shared faces follow from a dense system per wavenumber (kern_iface.cu).
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <vector>
+
+#include "direct_dev.cuh"
+
+namespace snac {
+void set_error(const std::string& s);
+
+// Passes of an in-place FFT of n points: the factors 2 spread evenly over the fewest passes of at most
+// max_log2 each, then 7, 5, 3. False if another prime divides n.
+bool fft_tab(int n, int max_log2, FftTab& F) {
+  F = FftTab{};
+  F.n = n;
+  int twos = 0, rest = n;
+  while (rest % 2 == 0) rest /= 2, ++twos;
+  std::vector<int> rad;
+  for (int left = twos, np = (twos + max_log2 - 1) / max_log2; np > 0; --np) {
+    const int b = (left + np - 1) / np;
+    rad.push_back(1 << b);
+    left -= b;
+  }
+  for (int p : {7, 5, 3})
+    while (rest % p == 0) rest /= p, rad.push_back(p);
+  if (rest != 1 || rad.size() > FFT_MAX_PASS) return false;
+  if (rad.empty()) rad.push_back(1);
+  F.np = n == 1 ? 0 : (int)rad.size();
+  F.l1 = n / rad[0];
+  int span = n;
+  for (int k = 0; k < F.np; ++k) {
+    F.rad[k] = rad[k];
+    F.span[k] = span;
+    span /= rad[k];
+  }
+  return true;
+}
+
+// Row of every frequency after the forward passes (digit-reversed order).
+std::vector<int> fft_perm(const FftTab& F) {
+  std::vector<int> perm(F.n);
+  for (int k = 0; k < F.n; ++k) {
+    int q = k, p = 0;
+    for (int s = 0; s < F.np; ++s) {
+      p += (q % F.rad[s]) * (F.span[s] / F.rad[s]);
+      q /= F.rad[s];
+    }
+    perm[k] = p;
+  }
+  return perm;
+}
+
+namespace {
+
+// Boundary pair of an axis from its two outer face kinds.
+int pair_kind(int lo, int hi) {
+  if (lo == SNAC_BC_PERIODIC) return KIND_PP;
+  if (lo == SNAC_BC_NEUMANN) return hi == SNAC_BC_NEUMANN ? KIND_NN : KIND_ND;
+  return hi == SNAC_BC_NEUMANN ? KIND_DN : KIND_DD;
+}
+
+struct Chain {
+  std::vector<int> blk;
+  bool ring = false;
+};
+
+// A piece while it is being described: its chains from the first row of blocks to the last.
+struct Piece {
+  std::vector<Chain> rows;
+  int kind = 0;
+  int side[2] = {0, 0};        // face kind of the first / last row (SNAC_BC_NEUMANN where it has interface cells)
+  bool iface[2] = {false, false};
+};
+
+struct IfaceCell {
+  int pa, ma, pb, mb;  // last row of piece pa, first row of piece pb
+  double ca, cb;       // their couplings
+};
+
+struct Layout {
+  int axis = 0;  // transformed axis
+  std::vector<Piece> pc;
+  std::vector<IfaceCell> cells;
+};
+
+// The pieces of the layout for a transformed axis; false if it does not fit the scheme.
+bool pieces_along(const snac_plan* P, const std::vector<FaceKinds>& faces, int t, Layout& out) {
+  const HostLevel& l0 = P->lev[0];
+  const std::vector<BlockDev>& B = l0.blk;
+  const int nb = (int)B.size(), tl = 2 * t, th = 2 * t + 1, nl = 2 * (1 - t), nh = 2 * (1 - t) + 1;
+  out = Layout{};
+  out.axis = t;
+  std::vector<Chain> ch;
+  std::vector<int> of(nb, -1), at(nb, -1);
+  auto add = [&](int b0, bool ring) {
+    Chain c;
+    c.ring = ring;
+    for (int b = b0; b >= 0 && of[b] < 0; b = B[b].nbr[th]) {
+      of[b] = (int)ch.size();
+      at[b] = (int)c.blk.size();
+      c.blk.push_back(b);
+    }
+    ch.push_back(c);
+  };
+  for (int b = 0; b < nb; ++b)
+    if (B[b].nbr[tl] < 0) add(b, false);
+  for (int b = 0; b < nb; ++b)
+    if (of[b] < 0) add(b, true);
+  // the chain above, where every face matches
+  const int nc = (int)ch.size();
+  std::vector<int> up(nc, -1), down(nc, -1);
+  for (int c = 0; c < nc; ++c) {
+    const int b0 = B[ch[c].blk[0]].nbr[nh];
+    if (b0 < 0 || of[b0] == c) continue;
+    const int d = of[b0];
+    const int n = (int)ch[c].blk.size();
+    bool ok = (int)ch[d].blk.size() == n && ch[d].ring == ch[c].ring && (ch[c].ring || at[b0] == 0);
+    for (int i = 0; i < n && ok; ++i) ok = B[ch[c].blk[i]].nbr[nh] == ch[d].blk[(at[b0] + i) % n];
+    const FaceKinds &f0 = faces[ch[c].blk[0]], &f1 = faces[ch[c].blk.back()];
+    const FaceKinds &g0 = faces[ch[d].blk[0]], &g1 = faces[ch[d].blk.back()];
+    ok = ok && (ch[c].ring || (f0.k[tl] == g0.k[tl] && f1.k[th] == g1.k[th]));
+    if (ok) up[c] = d, down[d] = c;
+  }
+  std::vector<int> piece_of(nc, -1);
+  for (int c = 0; c < nc; ++c) {
+    if (down[c] >= 0) continue;
+    Piece p;
+    for (int d = c; d >= 0; d = up[d]) {
+      Chain row = ch[d];
+      if (row.ring && !p.rows.empty()) {  // a ring starts wherever it was met: start above the first block
+        const int b0 = B[p.rows.back().blk[0]].nbr[nh];
+        std::rotate(row.blk.begin(), std::find(row.blk.begin(), row.blk.end(), b0), row.blk.end());
+      }
+      piece_of[d] = (int)out.pc.size();
+      p.rows.push_back(row);
+    }
+    const Chain& r0 = p.rows[0];
+    p.kind = r0.ring ? KIND_PP : pair_kind(faces[r0.blk[0]].k[tl], faces[r0.blk.back()].k[th]);
+    out.pc.push_back(p);
+  }
+  for (int c = 0; c < nc; ++c)
+    if (piece_of[c] < 0) return false;  // stacked in a circle: periodic along the tridiagonal axis
+  // position of every block along its piece's transformed axis
+  std::vector<int> m0(nb, 0), pof(nb, 0);
+  auto ext = [&](int b, int a) { return a == 0 ? B[b].nx : B[b].ny; };
+  for (size_t p = 0; p < out.pc.size(); ++p)
+    for (const Chain& r : out.pc[p].rows) {
+      int m = 0;
+      for (int b : r.blk) {
+        m0[b] = m;
+        pof[b] = (int)p;
+        m += ext(b, t);
+      }
+    }
+  for (size_t p = 0; p < out.pc.size(); ++p)
+    for (int e = 0; e < 2; ++e) {
+      Piece& pc = out.pc[p];
+      const Chain& r = e == 0 ? pc.rows.front() : pc.rows.back();
+      const int f = e == 0 ? nl : nh;
+      int wall = -1, links = 0;
+      for (int b : r.blk) {
+        if (B[b].nbr[f] >= 0) {
+          ++links;
+          if (pof[B[b].nbr[f]] == (int)p) return false;  // the piece meets itself
+          continue;
+        }
+        if (wall >= 0 && wall != faces[b].k[f]) return false;
+        wall = faces[b].k[f];
+      }
+      if (links && wall >= 0 && wall != SNAC_BC_NEUMANN) return false;  // (a Dirichlet wall beside an interface)
+      pc.iface[e] = links > 0;
+      pc.side[e] = links ? (int)SNAC_BC_NEUMANN : wall;
+      if (e == 0 || !links) continue;
+      for (int b : r.blk) {
+        const int c = B[b].nbr[f];
+        if (c < 0) continue;
+        const Coef<double>*ka, *kb;
+        if (t == 0) {
+          ka = &l0.cy[B[b].yo + B[b].ny - 1];
+          kb = &l0.cy[B[c].yo];
+        } else {
+          ka = &l0.cx[B[b].xo + B[b].nx - 1];
+          kb = &l0.cx[B[c].xo];
+        }
+        for (int i = 0; i < ext(b, t); ++i)
+          out.cells.push_back({(int)p, m0[b] + i, pof[c], m0[c] + i, ka->hi, kb->lo});
+      }
+    }
+  return true;
+}
+
+// Widths of a piece along an axis: the blocks of its first row (transformed axis) or first column.
+std::vector<double> piece_widths(const snac_plan* P, const Piece& p, int axis, bool transformed) {
+  const HostLevel& l0 = P->lev[0];
+  std::vector<double> w;
+  auto put = [&](int b) {
+    const BlockDev& d = l0.blk[b];
+    if (axis == 0)
+      for (int i = 0; i < d.nx; ++i) w.push_back(l0.cx[d.xo + i].w);
+    else
+      for (int j = 0; j < d.ny; ++j) w.push_back(l0.cy[d.yo + j].w);
+  };
+  if (transformed)
+    for (int b : p.rows[0].blk) put(b);
+  else
+    for (const Chain& r : p.rows) put(r.blk[0]);
+  return w;
+}
+
+bool uniform(const std::vector<double>& w) {
+  for (double v : w)
+    if (std::fabs(v - w[0]) > 1e-12 * w[0]) return false;
+  return true;
+}
+
+// Whether every piece can be transformed along the layout's axis.
+bool transformable(const snac_plan* P, const Layout& L) {
+  for (const Piece& p : L.pc) {
+    const std::vector<double> w = piece_widths(P, p, L.axis, true);
+    const int m = (int)w.size(), n = (int)piece_widths(P, p, 1 - L.axis, false).size();
+    if (m % 2 || m < 4 || m > MAX_NZ || n < 2 || n > 65535 || !uniform(w)) return false;
+    FftTab F;
+    const bool four = p.kind == KIND_ND || p.kind == KIND_DN;
+    if (!fft_tab(four ? m / 2 : m, 4, F)) return false;
+  }
+  return true;
+}
+
+std::vector<float> to_float(const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); }
+
+// A table in the plan's inner type.
+int up_inner(snac_plan* P, void** d, const std::vector<double>& v) {
+  if (P->precision == SNAC_FP64) return plan_upload(P, d, v.data(), v.size() * sizeof(double));
+  const std::vector<float> f = to_float(v);
+  return plan_upload(P, d, f.data(), f.size() * sizeof(float));
+}
+template <typename V>
+int up_vec(snac_plan* P, V** d, const std::vector<V>& v) {
+  return plan_upload(P, reinterpret_cast<void**>(d), v.data(), v.size() * sizeof(V));
+}
+
+int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
+  const HostLevel& l0 = P->lev[0];
+  const bool f64 = P->precision == SNAC_FP64;
+  const std::vector<double> wm = piece_widths(P, p, ax, true);
+  D.w = piece_widths(P, p, 1 - ax, false);
+  D.M = (int)wm.size();
+  D.N = (int)D.w.size();
+  D.kind = p.kind;
+  D.cls = p.kind == KIND_ND || p.kind == KIND_DN ? LINES_DCT4 : LINES_PAIR;
+  D.xl = ax == 0 ? 1 : 0;
+  D.soff = soff;
+  fft_tab(D.cls == LINES_PAIR ? D.M : D.M / 2, f64 ? 3 : 4, D.fft);
+  const int nf = D.fft.n, M = D.M, N = D.N;
+  D.w2n = nf;
+  D.t4a = D.w2n + M + 1;
+  D.t4b = D.t4a + M / 2;
+  std::vector<double> tw(2 * (size_t)(D.t4b + M / 2));
+  auto put = [&](int k, double ang) {
+    tw[2 * k] = std::cos(ang);
+    tw[2 * k + 1] = std::sin(ang);
+  };
+  for (int k = 0; k < nf; ++k) put(k, -2.0 * M_PI * k / nf);
+  for (int k = 0; k <= M; ++k) put(D.w2n + k, -M_PI * k / (2.0 * M));
+  for (int k = 0; k < M / 2; ++k) put(D.t4a + k, -M_PI * (4.0 * k + 1.0) / (4.0 * M));
+  for (int k = 0; k < M / 2; ++k) put(D.t4b + k, -M_PI * k / (double)M);
+  const std::vector<int> perm = fft_perm(D.fft);
+  // eigenvalues of the slots and the tridiagonal rows, scaled by a power of two to couplings of about 1
+  double h = 0.0;
+  for (double v : wm) h += v;
+  h /= M;
+  std::vector<Coef<double>> ct;
+  for (const Chain& r : p.rows) {
+    const BlockDev& d = l0.blk[r.blk[0]];
+    if (ax == 0) ct.insert(ct.end(), l0.cy.begin() + d.yo, l0.cy.begin() + d.yo + d.ny);
+    else ct.insert(ct.end(), l0.cx.begin() + d.xo, l0.cx.begin() + d.xo + d.nx);
+  }
+  ct.front().lo = 0.0;  // (an interface is a Neumann face of the piece)
+  ct.back().hi = 0.0;
+  double big = 4.0 / (h * h);
+  for (const Coef<double>& c : ct) big = std::max(big, c.lo + c.hi);
+  int ex = 0;
+  std::frexp(big, &ex);
+  D.cscale = std::ldexp(1.0, -ex);
+  D.lam.resize(M);
+  for (int k = 0; k < M; ++k)
+    D.lam[k] = D.cscale * mode_lambda(p.kind, M, p.kind == KIND_DD || p.kind == KIND_DN ? M - 1 - k : k) / (h * h);
+  std::vector<double> tri(4 * (size_t)N);
+  for (int n = 0; n < N; ++n) {
+    const Coef<double>& c = ct[n];
+    double tau = 0.0;
+    if (n == 0 && p.side[0] == SNAC_BC_DIRICHLET) tau += 2.0 / (c.w * c.w);
+    if (n == N - 1 && p.side[1] == SNAC_BC_DIRICHLET) tau += 2.0 / (c.w * c.w);
+    tri[4 * n] = D.cscale * c.lo;
+    tri[4 * n + 1] = D.cscale * c.hi;
+    tri[4 * n + 2] = D.cscale * tau;
+    tri[4 * n + 3] = c.hi > 0.0 ? c.lo / c.hi : 0.0;
+  }
+  D.singular = (p.kind == KIND_PP || p.kind == KIND_NN) && p.side[0] != SNAC_BC_DIRICHLET && p.side[1] != SNAC_BC_DIRICHLET;
+  // where the lines live: plane offset of (m, n) = base[n nbm + mblk[m]] + m mstr[n]
+  const int gm = (int)p.rows[0].blk.size();
+  std::vector<int> mblk(M), base((size_t)N * gm), mstr(N);
+  bool vec = l0.ncell % 2 == 0 && (ax == 0 || N % 2 == 0);
+  int n0 = 0;
+  for (const Chain& r : p.rows) {
+    int m0 = 0;
+    for (int i = 0; i < gm; ++i) {
+      const BlockDev& d = l0.blk[r.blk[i]];
+      const int em = ax == 0 ? d.nx : d.ny, en = ax == 0 ? d.ny : d.nx;
+      // pairs are two cells of a line (x lines), or the same cell of two adjacent lines (the first even)
+      vec = vec && d.off % 2 == 0 && d.nx % 2 == 0 && (ax == 0 ? m0 : n0) % 2 == 0;
+      for (int m = m0; m < m0 + em; ++m) mblk[m] = i;
+      for (int n = n0; n < n0 + en; ++n) {
+        mstr[n] = ax == 0 ? 1 : d.nx;
+        const long long c = ax == 0 ? d.off + (long long)(n - n0) * d.nx : d.off + (n - n0);
+        base[(size_t)n * gm + i] = (int)(c - (long long)m0 * mstr[n]);
+      }
+      m0 += em;
+    }
+    n0 += ax == 0 ? l0.blk[r.blk[0]].ny : l0.blk[r.blk[0]].nx;
+  }
+  D.vec = vec;
+  D.nbm = gm;
+  int st;
+  if (!f64) {
+    // the systems with the smallest -(lambda + sigma): up to LOW_SPAN times the smallest nonzero one, 1/64 of
+    // all at most (kern_direct.cu, k_tri_low; rows of longer systems do not fit its CTA)
+    constexpr double LOW_SPAN = 256.0;
+    std::vector<std::pair<double, int>> by;
+    std::vector<unsigned char> low((size_t)P->nz * M, 0);
+    double least = INFINITY;
+    for (int l = 0; l < P->nz; ++l)
+      for (int k = 0; k < M; ++k) {
+        const double v = -(P->sigma[l] * D.cscale + D.lam[k]);
+        if (v > 0.0) least = std::min(least, v);
+      }
+    if (N <= 512 && !P->ranged)
+      for (int l = 0; l < P->nz; ++l)
+        for (int k = 0; k < M; ++k) {
+          const double v = -(P->sigma[l] * D.cscale + D.lam[k]);
+          if (v <= LOW_SPAN * least) by.push_back({v, l * M + k});
+        }
+    std::sort(by.begin(), by.end());
+    by.resize(std::min(by.size(), low.size() / 64));
+    std::vector<int> list;
+    for (const auto& v : by) {
+      list.push_back(v.second);
+      low[v.second] = 1;
+    }
+    D.nlow = (int)list.size();
+    if ((st = up_vec(P, &D.d_lam64, D.lam)) || (st = up_vec(P, &D.d_tri64, tri)) ||
+        (st = up_vec(P, &D.d_lowlist, list)) || (st = up_vec(P, &D.d_low, low)))
+      return st;
+  }
+  if ((st = up_inner(P, &D.d_tw, tw)) || (st = up_inner(P, &D.d_lam, D.lam)) || (st = up_inner(P, &D.d_tri, tri)) ||
+      (st = up_inner(P, &D.d_w, D.w)) || (st = up_vec(P, &D.d_perm, perm)) || (st = up_vec(P, &D.d_base, base)) ||
+      (st = up_vec(P, &D.d_mblk, mblk)) || (st = up_vec(P, &D.d_mstr, mstr)))
+    return st;
+  return SNAC_OK;
+}
+
+// Entries of the transforms as the line kernels scale them (direct_dev.cuh): forward F[kappa][m], inverse
+// B[m][kappa], B F = 2 M.
+double fwd_entry(int kind, int M, int kap, int m) {
+  const double pi = M_PI;
+  switch (kind) {
+    case KIND_PP: return kap <= M / 2 ? 2.0 * std::cos(2.0 * pi * ((long long)kap * m % M) / M)
+                                      : -2.0 * std::sin(2.0 * pi * ((long long)(M - kap) * m % M) / M);
+    case KIND_NN: return 2.0 * std::cos(pi * ((2LL * m + 1) * kap % (4LL * M)) / (2.0 * M));
+    case KIND_DD: return 2.0 * std::sin(pi * ((2LL * m + 1) * (M - kap) % (4LL * M)) / (2.0 * M));
+    case KIND_ND: return 2.0 * std::cos(pi * ((2LL * m + 1) * (2LL * kap + 1) % (8LL * M)) / (4.0 * M));
+    default: return 2.0 * std::sin(pi * ((2LL * m + 1) * (2LL * (M - 1 - kap) + 1) % (8LL * M)) / (4.0 * M));
+  }
+}
+double bwd_entry(int kind, int M, int m, int kap) {
+  const double f = fwd_entry(kind, M, kap, m);
+  const bool half = (kind == KIND_PP && (kap == 0 || kap == M / 2)) || ((kind == KIND_NN || kind == KIND_DD) && kap == 0);
+  return half ? 0.5 * f : f;
+}
+
+// The matrices between end values, jumps and fluxes.
+int build_iface(snac_plan* P, const Layout& L) {
+  DirectPlan& D = P->direct;
+  IfaceTab& I = D.it;
+  I.k = (int)L.cells.size();
+  if (I.k == 0) return SNAC_OK;
+  std::map<int, int> end_of;  // 2 piece + end -> number
+  for (size_t p = 0; p < L.pc.size(); ++p)
+    for (int e = 0; e < 2; ++e)
+      if (L.pc[p].iface[e]) {
+        const int u = I.nends++;
+        end_of[(int)(2 * p + e)] = u;
+        I.ep[u] = (int)p;
+        I.ee[u] = e;
+        I.eo[u + 1] = I.eo[u] + D.pc[p].M;
+      }
+  I.E = I.eo[I.nends];
+  for (int l = 0; l < P->nz; ++l)
+    if (P->sigma[l] == 0.0) I.qs = l;
+  if (I.qs >= 0)
+    for (size_t p = 0; p < L.pc.size(); ++p)
+      if (D.pc[p].singular) I.sp[I.ns++] = (int)p;
+  if (I.ns == 0) I.qs = -1;
+  I.kk = I.k + I.ns;
+  std::vector<double> Y((size_t)I.E * I.kk, 0.0), Z((size_t)I.kk * I.E, 0.0);
+  for (int j = 0; j < I.k; ++j) {
+    const IfaceCell& c = L.cells[j];
+    for (int side = 0; side < 2; ++side) {
+      const int p = side == 0 ? c.pa : c.pb, m = side == 0 ? c.ma : c.mb;
+      const int u = end_of[2 * p + (side == 0 ? 1 : 0)];
+      const DirectTab& T = D.pc[p];
+      for (int k = 0; k < T.M; ++k) {
+        Y[(size_t)(I.eo[u] + k) * I.kk + j] = (side == 0 ? -1.0 : 1.0) * bwd_entry(T.kind, T.M, m, k);
+        Z[(size_t)j * I.E + I.eo[u] + k] = (side == 0 ? -c.ca : c.cb) * fwd_entry(T.kind, T.M, k, m);
+      }
+    }
+  }
+  const size_t w = P->precision == SNAC_FP64 ? sizeof(double) : sizeof(float);
+  int st;
+  if ((st = up_vec(P, &I.d_Y, Y)) || (st = up_inner(P, &I.d_Z, Z)) ||
+      (st = plan_alloc(P, (void**)&I.d_KT, (size_t)P->nz * I.kk * I.kk * sizeof(double))) ||
+      (st = plan_alloc(P, &I.d_ends, (size_t)P->nz * I.E * w)) || (st = plan_alloc(P, &I.d_alpha, D.pc.size() * w)) ||
+      (st = plan_alloc(P, &I.d_ssum, D.pc.size() * w)))
+    return st;
+  I.Zh.swap(Z);
+  return SNAC_OK;
+}
+
+// The interface systems are dense: k^2 values per wavenumber kept, k^2 (E + k) operations to set them up.
+bool iface_affordable(const snac_plan* P, const Layout& L) {
+  const double k = (double)L.cells.size();
+  double E = 0.0;
+  int ends = 0;
+  for (const Piece& p : L.pc)
+    for (int e = 0; e < 2; ++e)
+      if (p.iface[e]) {
+        int m = 0;
+        for (int b : p.rows[0].blk) m += L.axis == 0 ? P->lev[0].blk[b].nx : P->lev[0].blk[b].ny;
+        E += m;
+        ++ends;
+      }
+  return ends <= IFACE_MAX_ENDS && (int)L.pc.size() <= IFACE_MAX_ENDS && k <= 1024 && E <= 8192 &&
+         P->nz * k * k <= 64e6 && P->nz * k * k * (E + k) <= 4e10;
+}
+
+}  // namespace
+
+// Only with the default schedule: a caller who sets a multigrid option gets the multigrid. Of the two plane
+// axes the one with fewer interface cells is transformed, x where they tie (its lines are contiguous).
+int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
+  if (P->nu1 != 2 || P->nu2 != 2 || P->max_cycles != 40 || P->max_coarse != 64 || P->fused != -1 ||
+      P->onchip_opt != 0 || P->bottom_cells != 0 || P->inner_reduction != 0.0 || P->lev[0].ncell >= (1LL << 31))
+    return SNAC_OK;
+  Layout best;
+  bool found = false;
+  for (int t = 0; t < 2; ++t) {
+    Layout L;
+    if (!pieces_along(P, faces, t, L) || !transformable(P, L) || !iface_affordable(P, L)) continue;
+    if (!found || L.cells.size() < best.cells.size()) best = L;
+    found = true;
+  }
+  if (!found) return SNAC_OK;
+  DirectPlan& D = P->direct;
+  int soff = 0, st;
+  for (const Piece& p : best.pc) {
+    D.pc.emplace_back();
+    if ((st = build_piece(P, p, best.axis, soff, D.pc.back()))) return st;
+    soff += D.pc.back().M * D.pc.back().N;
+  }
+  if ((st = build_iface(P, best))) return st;
+  D.on = true;
+  return SNAC_OK;
+}
+
+int finish_direct(snac_plan* P) {
+  DirectPlan& D = P->direct;
+  const bool f64 = P->precision == SNAC_FP64;
+  const size_t w = f64 ? sizeof(double) : sizeof(float);
+  int st;
+  std::vector<int> qrow(P->nz), qof;
+  int* d_qof = nullptr;
+  if (!P->onchip) {
+    std::map<int, int> seen;  // wavenumbers q and n - q of the real DFT have one eigenvalue
+    for (int l = 0; l < P->nz; ++l) {
+      const int q = P->q0 + l;
+      const auto it = seen.emplace(P->kind == KIND_PP ? std::min(q, P->nzt - q) : q, (int)qof.size());
+      if (it.second) qof.push_back(l);
+      qrow[l] = it.first->second;
+    }
+    if ((st = up_vec(P, &D.d_qrow, qrow)) || (st = up_vec(P, &d_qof, qof))) return st;
+    for (DirectTab& T : D.pc)
+      // (FP32 plans of few systems use the segments of k_tri_seg; the end values need the pivots)
+      if (f64 || D.pc.size() > 1 || (long long)P->nz * T.M >= 256LL * P->sms)
+        if ((st = plan_alloc(P, &T.d_fac, qof.size() * (size_t)T.M * T.N * w))) return st;
+  } else {
+    // the cells' places in the on-chip buffer, and the pieces' arguments
+    std::vector<unsigned> off(P->lev[0].ncell, 0u);
+    const auto place = [&](auto tag) {
+      using T = decltype(tag);
+      std::vector<DirectArgs<T>> args;
+      size_t base = 0;
+      for (const DirectTab& d : D.pc) {
+        const DirectArgs<T> A = direct_args<T>(P, d);
+        args.push_back(A);
+        const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
+        std::vector<int> hb((size_t)d.N * d.nbm), hm(d.M), hs(d.N);
+        cudaMemcpy(hb.data(), d.d_base, hb.size() * sizeof(int), cudaMemcpyDeviceToHost);
+        cudaMemcpy(hm.data(), d.d_mblk, hm.size() * sizeof(int), cudaMemcpyDeviceToHost);
+        cudaMemcpy(hs.data(), d.d_mstr, hs.size() * sizeof(int), cudaMemcpyDeviceToHost);
+        auto row = [&](int p) { return (size_t)(p / A.F.l1) * S.s1 + (size_t)(p % A.F.l1) * S.rp; };
+        const bool flip = d.kind == KIND_DD || d.kind == KIND_DN;
+        for (int n = 0; n < d.N; ++n)
+          for (int m = 0; m < d.M; ++m) {
+            const long long c = hb[(size_t)n * d.nbm + (d.nbm == 1 ? 0 : hm[m])] + (long long)m * hs[n];
+            size_t o;
+            if (d.cls == LINES_PAIR) {
+              const int t = d.kind == KIND_PP ? m : ((m & 1) ? d.M - 1 - (m >> 1) : m >> 1);
+              o = 2 * (row(t) + (n >> 1)) + (n & 1);
+            } else {
+              o = 2 * (row((m & 1) ? (d.M - 1 - m) >> 1 : m >> 1) + n) + (m & 1);
+            }
+            off[c] = (unsigned)(base + o) | (flip && (m & 1) ? 0x80000000u : 0u);
+          }
+        base += S.buf;
+      }
+      return plan_upload(P, &D.d_args, args.data(), args.size() * sizeof(DirectArgs<T>));
+    };
+    if ((st = f64 ? place(double{}) : place(float{})) || (st = up_vec(P, &D.d_celloff, off))) return st;
+  }
+  // on a private non-blocking stream, like every other device work of plan creation
+  cudaStream_t cs = nullptr;
+  bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
+  for (DirectTab& T : D.pc)
+    if (ok && T.d_fac) ok = launch_tri_factor(P, T, d_qof, (int)qof.size(), cs) == cudaSuccess;
+  if (ok && D.it.k) ok = setup_iface(P, cs) == cudaSuccess;
+  ok = ok && cudaStreamSynchronize(cs) == cudaSuccess;
+  if (cs) cudaStreamDestroy(cs);
+  if (!ok) {
+    const cudaError_t e = cudaGetLastError();
+    set_error(std::string("setting up the direct solves failed: ") + cudaGetErrorString(e));
+    return e == cudaErrorMemoryAllocation ? SNAC_ERR_OOM : SNAC_ERR_CUDA;
+  }
+  return SNAC_OK;
+}
+
+size_t direct_onchip_smem(const snac_plan* P) {
+  const DirectPlan& D = P->direct;
+  size_t el = 0;
+  for (const DirectTab& d : D.pc) el += plane_shape(d.fft, d.M, d.N, d.cls).buf;
+  return onchip_elements(el, BOTTOM_THREADS) * (P->precision == SNAC_FP64 ? sizeof(double) : sizeof(float)) +
+         iface_doubles(D.it.E, D.it.kk, BOTTOM_THREADS) * sizeof(double);
+}
+
+}  // namespace snac

@@ -417,7 +417,7 @@ struct OnchipArgs {
   int* cycles;              // per wavenumber: V-cycles run
   double* norm2;            // per wavenumber: ||r_q||^2 on return
   int direct;               // separable plans: the direct solve (direct_dev.cuh) in place of the V-cycles
-  DirectArgs<T> D;
+  PlaneArgs<T> D;
 };
 
 // One wavenumber's solve, from a zero iterate, by one CTA.
@@ -426,7 +426,7 @@ __device__ void onchip_mode(const OnchipArgs<T>& O, int q, unsigned char* smem_r
   const BottomArgs<T>& A = O.B;
   if (O.direct) {
     const long long o = (long long)q * O.D.ncell;
-    plane_direct<T>(O.D, q, A.f_top + o, A.u_top + o, smem_raw, BT);
+    plane_direct<T>(O.D, A.sigma[q], q, A.f_top + o, A.u_top + o, smem_raw, BT);
     if (threadIdx.x == 0) {
       O.cycles[q] = 1;
       O.norm2[q] = 0.0;
@@ -723,20 +723,20 @@ OnchipArgs<T> onchip_args(snac_plan* P, double target) {
   O.cycles = P->dh_cycles;
   O.norm2 = P->dh_mode_norm2;
   O.direct = P->direct.on ? 1 : 0;
-  if (P->direct.on) O.D = direct_args<T>(P);
+  if (P->direct.on) O.D = plane_args<T>(P);
   return O;
 }
 
 // Dynamic shared memory of one wavenumber's on-chip solve.
 template <typename T>
 size_t onchip_smem(const snac_plan* P) {
-  const DirectTab& D = P->direct;
-  return D.on ? plane_shape(D.fft, D.M, D.N, D.cls, sizeof(T), BT).bytes : bottom_layout(P, 0, sizeof(T)).bytes;
+  return P->direct.on ? direct_onchip_smem(P) : bottom_layout(P, 0, sizeof(T)).bytes;
 }
 
 // algorithmic bytes and flops of one on-chip V-cycle of one wavenumber, and of its load and store
 double onchip_cycle_flops(const snac_plan* P) {
-  if (P->direct.on) return (5.0 * std::log2((double)P->direct.M) + 28.0) * P->lev[0].ncell / 4.0;  // one direct solve
+  if (P->direct.on)  // one direct solve
+    return (5.0 * std::log2((double)P->direct.pc[0].M) + 28.0) * P->lev[0].ncell / 4.0;
   double fl = 0.0;
   const int L = (int)P->lev.size() - 1;
   for (int l = 0; l < L; ++l) fl += (double)P->lev[l].ncell * (12.0 * (P->nu1 + P->nu2) + 15.0 + 8.0);

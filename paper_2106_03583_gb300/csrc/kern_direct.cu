@@ -34,9 +34,10 @@ struct ColsLine : ColsShift {
   __device__ __forceinline__ int total8(int rows) const { return ((rows + 7) & ~7) << lc; }
 };
 
-// Lines of one CTA: global line number g = q N + n; per line the plane base of q and n.
+// Lines of one CTA: global line number g = q N + n; per line the plane base of q, its spectrum and n.
 struct LineSet {
   long long* plane;  // q ncell, or -1 past the last line
+  long long* spec;   // first element of the line's spectrum
   int* n;
 };
 
@@ -48,7 +49,7 @@ __device__ __forceinline__ long long line_off(const DirectArgs<T>& A, const Line
 }
 
 template <typename T>
-__device__ __forceinline__ int line_setup(const DirectArgs<T>& A, int lines, long long* plane, int* ln) {
+__device__ __forceinline__ int line_setup(const DirectArgs<T>& A, int lines, long long* plane, long long* spec, int* ln) {
   const int g0 = blockIdx.x * lines;
   const int total = A.nq * A.N;
   for (int l = threadIdx.x; l < lines; l += LNT) {
@@ -56,6 +57,7 @@ __device__ __forceinline__ int line_setup(const DirectArgs<T>& A, int lines, lon
     const int q = g / A.N;
     plane[l] = g < total ? (long long)q * A.ncell : -1;
     ln[l] = g < total ? g - q * A.N : 0;
+    spec[l] = (long long)q * A.ncell + A.soff + (long long)(g - q * A.N) * A.M;
   }
   __syncthreads();
   return g0;
@@ -69,6 +71,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const
                                                                          T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long plane[MAX_LINES];
+  __shared__ long long spec[MAX_LINES];
   __shared__ int ln[MAX_LINES];
   Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
   T* bt = reinterpret_cast<T*>(smem);
@@ -76,8 +79,8 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const
   const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
   const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
   const int lines = pair ? 2 * C : C;
-  const int g0 = line_setup(A, lines, plane, ln);
-  const LineSet S{plane, ln};
+  const int g0 = line_setup(A, lines, plane, spec, ln);
+  const LineSet S{plane, spec, ln};
   const int nlive = min(lines, A.nq * A.N - g0);
   if (pair) {
     if (A.xl) {  // items: two consecutive cells of both lines of a column
@@ -159,8 +162,6 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const
   }
   __syncthreads();
   fft_all<false>(buf, A.F, s1, cm, A.tw, LNT);
-  // spectra: line g of the CTA at out[g M + kappa]
-  T* o0 = out + (long long)g0 * M;
   if (pair) {
     const int total = cm.total8(M / 2 + 1);
     for (int t = threadIdx.x; t < total; t += LNT) {
@@ -171,15 +172,16 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const
       const Cpl<T> z2 = k == 0 ? z1 : buf[fft_row(A.perm[M - k], l1, s1, C) + c];
       Cpl<T> y1, y2;
       pair_post(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], z1, z2, y1, y2);
-      T* oa = o0 + (long long)(2 * c) * M;
       const bool mirror = k > 0 && 2 * k < M;
       if (2 * c < nlive) {
+        T* oa = out + spec[2 * c];
         oa[k] = y1.re;
         if (mirror) oa[M - k] = y2.re;
       }
       if (2 * c + 1 < nlive) {
-        oa[M + k] = y1.im;
-        if (mirror) oa[M + M - k] = y2.im;
+        T* ob = out + spec[2 * c + 1];
+        ob[k] = y1.im;
+        if (mirror) ob[M - k] = y2.im;
       }
     }
   } else {
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const
       const int kk = h - 1 - k;
       const Cpl<T> v = cx_mul(buf[fft_row(A.perm[k], l1, s1, C) + c], A.t4b[k]);
       const Cpl<T> w = cx_mul(buf[fft_row(A.perm[kk], l1, s1, C) + c], A.t4b[kk]);
-      T* o = o0 + (long long)c * M;
+      T* o = out + spec[c];
       o[2 * k] = (T)2 * v.re;
       o[2 * k + 1] = (T)-2 * w.im;
       o[2 * kk] = (T)2 * w.re;
@@ -205,16 +207,16 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
                                                                          T* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long plane[MAX_LINES];
+  __shared__ long long spec[MAX_LINES];
   __shared__ int ln[MAX_LINES];
   Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
   const ColsLine cm{{lc}};
   const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
   const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
   const int lines = pair ? 2 * C : C;
-  const int g0 = line_setup(A, lines, plane, ln);
-  const LineSet S{plane, ln};
+  const int g0 = line_setup(A, lines, plane, spec, ln);
+  const LineSet S{plane, spec, ln};
   const int nlive = min(lines, A.nq * A.N - g0);
-  const T* i0 = in + (long long)g0 * M;
   if (pair) {
     const int total = cm.total8(M / 2 + 1);
     for (int t0 = threadIdx.x; t0 < total; t0 += LB * LNT) {
@@ -225,15 +227,16 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
         cm.split8(t0 + u * LNT, k, c);
         x1[u] = x2[u] = Cpl<T>{0, 0};
         if (t0 + u * LNT < total && 2 * k <= M) {
-          const T* ia = i0 + (long long)(2 * c) * M;
           const bool two = k > 0 && !(kind == KIND_PP && 2 * k == M);
           if (2 * c < nlive) {
+            const T* ia = in + spec[2 * c];
             x1[u].re = ia[k];
             if (two) x2[u].re = ia[M - k];
           }
           if (2 * c + 1 < nlive) {
-            x1[u].im = ia[M + k];
-            if (two) x2[u].im = ia[M + M - k];
+            const T* ib = in + spec[2 * c + 1];
+            x1[u].im = ib[k];
+            if (two) x2[u].im = ib[M - k];
           }
         }
       }
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
       const int jj = h - 1 - j;
       Cpl<T> p{0, 0}, r{0, 0};
       if (c < nlive) {
-        const T* i = i0 + (long long)c * M;
+        const T* i = in + spec[c];
         p = Cpl<T>{i[2 * j], i[2 * j + 1]};
         r = Cpl<T>{i[2 * jj], i[2 * jj + 1]};
       }
@@ -333,15 +336,16 @@ constexpr int TRI_R = 16;
 
 template <typename T, int KG>
 __global__ void __launch_bounds__(1024, 1) k_tri_seg(const DirectArgs<T> A, int P, const unsigned char* __restrict__ low,
-                                                   T* __restrict__ x) {
+                                                   const T* __restrict__ alpha, T* __restrict__ x) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int kk = threadIdx.x % KG, seg = threadIdx.x / KG;
   const long long sys = (long long)blockIdx.x * KG + kk;
   const bool live = sys < (long long)A.nq * A.M && !low[sys];  // (k_tri_low solves the others)
   const int q = live ? (int)(sys / A.M) : 0, kap = live ? (int)(sys - (long long)q * A.M) : 0;
-  T* col = x + (long long)q * A.N * A.M + kap;
+  T* col = x + (long long)q * A.ncell + A.soff + kap;
   const T tq = live ? -fma(A.sigma[q], A.cscale, A.lam[kap]) : (T)1;
-  tri_segment<T, TRI_R>(A.tri, A.N, P, seg, kk, KG, true, live, tq, A.scale, reinterpret_cast<T*>(smem),
+  tri_segment<T, TRI_R>(A.tri, A.N, P, seg, kk, KG, true, live, tq, A.scale, alpha ? *alpha : (T)0,
+                        reinterpret_cast<T*>(smem),
                         [&](int n) { return col[(long long)n * A.M]; },
                         [&](int n, T v) { col[(long long)n * A.M] = v; });
 }
@@ -352,22 +356,30 @@ __global__ void __launch_bounds__(1024, 1) k_tri_seg(const DirectArgs<T> A, int 
 // largest where lambda + sigma is smallest. These few systems (list) therefore set the residual a
 // correction step can reach: with all of them in FP32 the second step on the 1024 x 512 x 512 channel ends
 // at 0.9-1.5e-10 relative residual, with the list in FP64 at 5e-11.
+// ENDS: only the first and last unknowns, into the end vector of the interface systems.
 constexpr int LOW_KG = 8, LOW_R = 8;
+template <bool ENDS>
 __global__ void __launch_bounds__(512, 1) k_tri_low(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
                                                   const double* __restrict__ sigma, double cscale, double scale,
                                                   const int* __restrict__ list, int nlist, int M, int N, int P,
-                                                  float* __restrict__ x) {
+                                                  long long ncell, int soff, const float* __restrict__ alpha,
+                                                  float* __restrict__ x, float* __restrict__ ends, int E, int e0, int e1) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int kk = threadIdx.x % LOW_KG, seg = threadIdx.x / LOW_KG;
   const int k = blockIdx.x * LOW_KG + kk;
   const bool live = k < nlist;
   const int sys = live ? list[k] : 0;
   const int q = sys / M, kap = sys - q * M;
-  float* col = x + (long long)q * N * M + kap;
+  float* col = x + (long long)q * ncell + soff + kap;
   const double tq = live ? -fma(sigma[q], cscale, lam[kap]) : 1.0;
-  tri_segment<double, LOW_R>(tri, N, P, seg, kk, LOW_KG, true, live, tq, scale, reinterpret_cast<double*>(smem),
+  tri_segment<double, LOW_R>(tri, N, P, seg, kk, LOW_KG, true, live, tq, scale, alpha ? (double)*alpha : 0.0,
+                             reinterpret_cast<double*>(smem),
                              [&](int n) { return (double)col[(long long)n * M]; },
-                             [&](int n, double v) { col[(long long)n * M] = (float)v; });
+                             [&](int n, double v) {
+                               if (!ENDS) col[(long long)n * M] = (float)v;
+                               else if (n == 0 && e0 >= 0) ends[(long long)q * E + e0 + kap] = (float)v;
+                               else if (n == N - 1 && e1 >= 0) ends[(long long)q * E + e1 + kap] = (float)v;
+                             });
 }
 
 // Rows in order, one thread per system, for systems too long for the segments of one CTA (FP32; the
@@ -377,7 +389,7 @@ __global__ void __launch_bounds__(128) k_tri_seq(const DirectArgs<T> A, T* __res
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= (long long)A.nq * A.M) return;
   const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
-  const long long o = (long long)q * A.N * A.M + kap;
+  const long long o = (long long)q * A.ncell + A.soff + kap;
   x += o;
   cw += o;
   const T tq = -fma(A.sigma[q], A.cscale, A.lam[kap]);
@@ -448,12 +460,12 @@ constexpr int TRI_U = 8;  // rows whose loads are in flight per thread
 template <typename T>
 __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const int* __restrict__ qrow,
                                                   const unsigned char* __restrict__ low, const T* __restrict__ fac,
-                                                  T* __restrict__ x) {
+                                                  const T* __restrict__ alpha, T* __restrict__ x) {
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= (long long)A.nq * A.M || (sizeof(T) == 4 && low[sys])) return;
   const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
   const int N = A.N, M = A.M;
-  x += (long long)q * N * M + kap;
+  x += (long long)q * A.ncell + A.soff + kap;
   fac += (long long)qrow[q] * N * M + kap;
   const T sc = -A.scale;
   T d = 0;
@@ -485,9 +497,54 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
     for (int u = TRI_U - 1; u >= 0; --u) {
       if (n0 + u >= N) continue;
       y = fma(A.tri[n0 + u].hi * f[u], y, v[u]);
+      // an exactly singular system ends in a zero pivot: its last unknown is the piece's constant
+      if (n0 + u == N - 1 && alpha != nullptr && f[u] == (T)0) y = *alpha;
       x[(long long)(n0 + u) * M] = y;
     }
   }
+}
+
+// First and last unknowns of every system of a piece (the end values of the interface systems), from the
+// kept pivots (the listed systems of an FP32 plan: k_tri_low). ssum (slot 0 of the singular wavenumber): the
+// weighted sum of its right-hand side.
+template <typename T>
+__global__ void __launch_bounds__(128, 8) k_tri_ends(const DirectArgs<T> A, const int* __restrict__ qrow,
+                                                   const unsigned char* __restrict__ low, const T* __restrict__ fac,
+                                                   const T* __restrict__ x, T* __restrict__ ends, int E, int qs,
+                                                   T* __restrict__ ssum) {
+  const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (sys >= (long long)A.nq * A.M) return;
+  const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
+  const int N = A.N, M = A.M;
+  x += (long long)q * A.ncell + A.soff + kap;
+  if (q == qs && kap == 0) {
+    T s = 0;
+    for (int n = 0; n < N; ++n) s = fma(A.w[n], x[(long long)n * M], s);
+    *ssum = s;
+  }
+  if (sizeof(T) == 4 && low[sys]) return;
+  fac += (long long)qrow[q] * N * M + kap;
+  const T sc = -A.scale;
+  T d = 0, pi = 1, F = 0;
+  for (int n0 = 0; n0 < N; n0 += TRI_U) {
+    T v[TRI_U], f[TRI_U];
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      const bool in = n0 + u < N;
+      v[u] = in ? x[(long long)(n0 + u) * M] : (T)0;
+      f[u] = in ? fac[(long long)(n0 + u) * M] : (T)0;
+    }
+#pragma unroll
+    for (int u = 0; u < TRI_U; ++u) {
+      if (n0 + u >= N) break;
+      const TriRow<T> w = A.tri[n0 + u];
+      d = fma(w.lo, d, sc * v[u]) * f[u];
+      F = fma(pi, d, F);
+      pi *= w.hi * f[u];
+    }
+  }
+  if (A.e0 >= 0) ends[(long long)q * E + A.e0 + kap] = F;
+  if (A.e1 >= 0) ends[(long long)q * E + A.e1 + kap] = d;
 }
 
 template <typename T>
@@ -498,59 +555,89 @@ __global__ void __launch_bounds__(256) k_nonfinite(const T* __restrict__ v, long
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
 }
 
+// Complex columns per line CTA: about 32 KB of shared memory, 2 to 16 columns.
 template <typename T>
-cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
-  const DirectArgs<T> A = direct_args<T>(P);
-  const double cells = (double)P->nz * P->lev[0].ncell, w = sizeof(T);
-  // complex columns per line CTA: about 32 KB of shared memory, 2 to 16 columns
+int line_columns(const DirectArgs<T>& A) {
   int lc = 1;
-  while (lc < 4 && ((size_t)A.F.n << (lc + 1)) * 2 * w <= 36 * 1024) ++lc;
-  const int lines = A.cls == LINES_PAIR ? 2 << lc : 1 << lc;
-  const long long total = (long long)A.nq * A.N;
-  const unsigned grid = (unsigned)((total + lines - 1) / lines);
-  const size_t smem = line_smem(A.F, lc, w);
-  T* f = (T*)P->lev[0].d_f;
-  T* u = (T*)P->lev[0].d_u;
-  const double fl = (2.5 * std::log2((double)A.M) + 4.0) * cells;
+  while (lc < 4 && ((size_t)A.F.n << (lc + 1)) * 2 * sizeof(T) <= 36 * 1024) ++lc;
+  return lc;
+}
+
+template <typename T>
+cudaError_t lines_t(snac_plan* P, const DirectArgs<T>& A, bool fwd, const T* in, T* out, cudaStream_t s) {
+  const int lc = line_columns(A), lines = A.cls == LINES_PAIR ? 2 << lc : 1 << lc;
+  const unsigned grid = (unsigned)(((long long)A.nq * A.N + lines - 1) / lines);
+  const size_t smem = line_smem(A.F, lc, sizeof(T));
+  const double cells = (double)A.nq * A.M * A.N;
   constexpr int kMax = 160 * 1024;  // the largest need (4096-point FP64 lines): function-wide, never lowered
-  {
-    LaunchScope ls(P, K_LINES_FWD, 2.0 * w * cells, fl, s);
-    cudaFuncSetAttribute(k_lines_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-    k_lines_fwd<T><<<grid, LNT, smem, s>>>(A, lc, f, u);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  {
-    LaunchScope ls(P, K_TRI, 2.0 * w * cells, 20.0 * cells, s);
-    const long long sys = (long long)A.nq * A.M;
-    const int segs = (A.N + TRI_R - 1) / TRI_R;
-    if constexpr (sizeof(T) == 4) {
-      const DirectTab& D = P->direct;
-      const int lsegs = (A.N + LOW_R - 1) / LOW_R;
-      if (D.nlow)
-        k_tri_low<<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
-            (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / (2.0 * A.M), D.d_lowlist,
-            D.nlow, A.M, A.N, lsegs, u);
-      if (D.d_fac) {
-        k_tri_pre<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A, D.d_qrow, D.d_low, (const T*)D.d_fac, u);
-      } else if (segs <= 32) {
-        k_tri_seg<T, 32><<<(unsigned)((sys + 31) / 32), 32 * segs, 7 * sizeof(T) * 32 * segs, s>>>(A, segs, D.d_low, u);
-      } else if (segs <= 64) {
-        k_tri_seg<T, 16><<<(unsigned)((sys + 15) / 16), 16 * segs, 7 * sizeof(T) * 16 * segs, s>>>(A, segs, D.d_low, u);
-      } else {
-        k_tri_seq<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A, u, f);
-      }
-    } else {
-      k_tri_pre<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A, P->direct.d_qrow, nullptr, (const T*)P->direct.d_fac, u);
-    }
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  {
-    LaunchScope ls(P, K_LINES_BWD, 2.0 * w * cells, fl, s);
-    cudaFuncSetAttribute(k_lines_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-    k_lines_bwd<T><<<grid, LNT, smem, s>>>(A, lc, u, f);
+  LaunchScope ls(P, fwd ? K_LINES_FWD : K_LINES_BWD, 2.0 * sizeof(T) * cells, (2.5 * std::log2((double)A.M) + 4.0) * cells, s);
+  auto kern = fwd ? k_lines_fwd<T> : k_lines_bwd<T>;
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+  kern<<<grid, LNT, smem, s>>>(A, lc, in, out);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t tri_t(snac_plan* P, const DirectTab& D, const DirectArgs<T>& A, const T* alpha, T* u, T* f, cudaStream_t s) {
+  const double cells = (double)A.nq * A.M * A.N;
+  LaunchScope ls(P, K_TRI, 2.0 * sizeof(T) * cells, 20.0 * cells, s);
+  const long long sys = (long long)A.nq * A.M;
+  const int segs = (A.N + TRI_R - 1) / TRI_R;
+  const unsigned g128 = (unsigned)((sys + 127) / 128);
+  if constexpr (sizeof(T) == 4) {
+    const int lsegs = (A.N + LOW_R - 1) / LOW_R;
+    if (D.nlow)
+      k_tri_low<false><<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
+          (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / (2.0 * A.M), D.d_lowlist,
+          D.nlow, A.M, A.N, lsegs, A.ncell, A.soff, alpha, u, nullptr, 0, -1, -1);
+    if (D.d_fac)
+      k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u);
+    else if (segs <= 32)
+      k_tri_seg<T, 32><<<(unsigned)((sys + 31) / 32), 32 * segs, 7 * sizeof(T) * 32 * segs, s>>>(A, segs, D.d_low, alpha, u);
+    else if (segs <= 64)
+      k_tri_seg<T, 16><<<(unsigned)((sys + 15) / 16), 16 * segs, 7 * sizeof(T) * 16 * segs, s>>>(A, segs, D.d_low, alpha, u);
+    else
+      k_tri_seq<T><<<g128, 128, 0, s>>>(A, u, f);
+  } else {
+    k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, nullptr, (const T*)D.d_fac, alpha, u);
   }
   return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
+  DirectPlan& D = P->direct;
+  T* f = (T*)P->lev[0].d_f;
+  T* u = (T*)P->lev[0].d_u;
+  const int np = (int)D.pc.size();
+  std::vector<DirectArgs<T>> A;
+  for (const DirectTab& d : D.pc) A.push_back(direct_args<T>(P, d));
+  cudaError_t e = cudaSuccess;
+  for (int p = 0; p < np && e == cudaSuccess; ++p) e = lines_t(P, A[p], true, f, u, s);
+  if (D.it.k) {
+    for (int p = 0; p < np && e == cudaSuccess; ++p) {
+      const DirectTab& d = D.pc[p];
+      const double cells = (double)A[p].nq * d.M * d.N;
+      LaunchScope ls(P, K_TRI, 2.0 * sizeof(T) * cells, 7.0 * cells, s);
+      const long long sys = (long long)A[p].nq * d.M;
+      if constexpr (sizeof(T) == 4) {
+        const int lsegs = (d.N + LOW_R - 1) / LOW_R;
+        if (d.nlow)
+          k_tri_low<true><<<(d.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
+              (const TriRow<double>*)d.d_tri64, d.d_lam64, P->d_sigma64, d.cscale, d.cscale / (2.0 * d.M), d.d_lowlist,
+              d.nlow, d.M, d.N, lsegs, A[p].ncell, A[p].soff, nullptr, u, (T*)D.it.d_ends, D.it.E, A[p].e0, A[p].e1);
+      }
+      k_tri_ends<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A[p], D.d_qrow, d.d_low, (const T*)d.d_fac, u,
+                                                                 (T*)D.it.d_ends, D.it.E, d.singular ? D.it.qs : -1,
+                                                                 (T*)D.it.d_ssum + p);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = launch_iface(P, s);
+  }
+  for (int p = 0; p < np && e == cudaSuccess; ++p)
+    e = tri_t<T>(P, D.pc[p], A[p], D.it.ns ? (const T*)D.it.d_alpha + p : nullptr, u, f, s);
+  for (int p = 0; p < np && e == cudaSuccess; ++p) e = lines_t(P, A[p], false, (const T*)u, f, s);
+  return e;
 }
 
 }  // namespace
@@ -562,8 +649,7 @@ cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStrea
   return cudaGetLastError();
 }
 
-cudaError_t launch_tri_factor(snac_plan* P, const int* d_qof, int rows, cudaStream_t s) {
-  const DirectTab& D = P->direct;
+cudaError_t launch_tri_factor(snac_plan* P, const DirectTab& D, const int* d_qof, int rows, cudaStream_t s) {
   const bool f64 = P->precision == SNAC_FP64;
   const TriRow<double>* tri = (const TriRow<double>*)(f64 ? D.d_tri : (void*)D.d_tri64);
   const double* lam = f64 ? (const double*)D.d_lam : D.d_lam64;

@@ -1,0 +1,249 @@
+// The interface systems of direct solves with several pieces (direct_dev.cuh). With the pieces solved under
+// Neumann faces where they meet, the jump of u across interface cell j is
+//   u_b - u_a = phi_j,   A_p u = f + sum_j (-c_a phi_j at a_j, +c_b phi_j at b_j),
+// so (I - Y^T R_q Z^T) phi = Y^T (end values of the solution for f): Z takes the fluxes to the spectral
+// right-hand sides of the pieces' end rows, R_q holds each system's response of its end rows to its end
+// rows, Y takes end values to jumps. A piece whose slot 0 is singular for the wavenumber of zero shift (no
+// Dirichlet face) is solved up to a constant alpha, an extra unknown, with the compatibility of its
+// right-hand side as the extra equation. The inverse of every system is kept with the plan.
+#include <cmath>
+#include <vector>
+
+#include "direct_dev.cuh"
+
+namespace snac {
+namespace {
+
+// R of one system: responses of the first / last unknown to a unit right-hand side in the first / last row
+// (as the solve scales them), {00, 0N, N0, NN}.
+__global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
+                                            const double* __restrict__ sigma, double cscale, double scale, int nq,
+                                            int M, int N, double4* __restrict__ resp) {
+  const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (sys >= (long long)nq * M) return;
+  const int q = (int)(sys / M), kap = (int)(sys - (long long)q * M);
+  const double tq = -fma(sigma[q], cscale, lam[kap]);
+  double g = 0, d = 0, pi = 1, F = 0, inv = 0, plast = 1;
+  for (int n = 0; n < N; ++n) {
+    const TriRow<double> w = tri[n];
+    const double s = fma(w.lo, g, w.tau + tq), den = s + w.hi;
+    inv = den > 0 ? 1.0 / den : 0.0;
+    g = s * inv;
+    d = (n == 0 ? 1.0 : w.lo * d) * inv;
+    F = fma(pi, d, F);
+    plast = pi;
+    pi *= w.hi * inv;
+  }
+  resp[sys] = make_double4(-scale * F, -scale * plast * inv, -scale * d, -scale * inv);
+}
+
+struct BuildArgs {
+  int k, kk, E, ns, qs, gs, nends;
+  int ep[IFACE_MAX_ENDS], ee[IFACE_MAX_ENDS], eo[IFACE_MAX_ENDS + 1], sp[IFACE_MAX_ENDS];
+  int em[IFACE_MAX_ENDS];                 // slots of the end's piece
+  double we[IFACE_MAX_ENDS];              // width of the end's row
+  const double4* resp[IFACE_MAX_ENDS];    // of the end's piece, [q][kappa]
+  const double* Y;
+  const double* Z;
+};
+
+// K = I - Y^T R_q Z^T, a 32 x 32 tile per CTA of 256 threads (2 x 2 entries each); the rows and columns of
+// the singular pieces' constants beyond.
+constexpr int KT = 32;
+__global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __restrict__ K) {
+  __shared__ double ys[KT][KT + 1], ws[KT][KT + 1];
+  const int q = blockIdx.z, j0 = blockIdx.y * KT, i0 = blockIdx.x * KT;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  double acc[2][2] = {{0, 0}, {0, 0}};
+  for (int u = 0; u < A.nends; ++u) {
+    const int M = A.em[u];
+    for (int k0 = 0; k0 < M; k0 += KT) {
+      for (int t = threadIdx.x; t < KT * KT; t += 256) {
+        const int r = t / KT, c = t % KT;
+        // ys[slot][j]
+        ys[r][c] = k0 + r < M && j0 + c < A.k ? A.Y[(size_t)(A.eo[u] + k0 + r) * A.kk + j0 + c] : 0.0;
+        // ws[slot][i] = sum over the ends of the same piece of R Z
+        double w = 0.0;
+        const int kap = k0 + c, i = i0 + r;
+        if (kap < M && i < A.k) {
+          const double4 R = A.resp[u][(size_t)q * M + kap];
+          for (int v = 0; v < A.nends; ++v)
+            if (A.ep[v] == A.ep[u]) {
+              const double rr = A.ee[u] ? (A.ee[v] ? R.w : R.z) : (A.ee[v] ? R.y : R.x);
+              w = fma(rr, A.Z[(size_t)i * A.E + A.eo[v] + kap], w);
+            }
+        }
+        ws[c][r] = w;
+      }
+      __syncthreads();
+#pragma unroll 8
+      for (int e = 0; e < KT; ++e) {
+        const double a0 = ys[e][ty], a1 = ys[e][ty + 16], b0 = ws[e][tx], b1 = ws[e][tx + 16];
+        acc[0][0] = fma(a0, b0, acc[0][0]);
+        acc[0][1] = fma(a0, b1, acc[0][1]);
+        acc[1][0] = fma(a1, b0, acc[1][0]);
+        acc[1][1] = fma(a1, b1, acc[1][1]);
+      }
+      __syncthreads();
+    }
+  }
+  for (int a = 0; a < 2; ++a)
+    for (int b = 0; b < 2; ++b) {
+      const int j = j0 + ty + 16 * a, i = i0 + tx + 16 * b;
+      if (j >= A.kk || i >= A.kk) continue;
+      double v = (j == i ? 1.0 : 0.0) - acc[a][b];
+      if (j >= A.k || i >= A.k) {
+        v = j == i ? 1.0 : 0.0;
+        if (q == A.qs) {
+          const bool implied = A.gs && j == A.kk - 1;  // the last constraint of a singular problem
+          v = implied && i == j ? 1.0 : 0.0;
+          if (!implied && (j < A.k || i < A.k)) {
+            const int p = A.sp[(j < A.k ? i : j) - A.k];
+            for (int u = 0; u < A.nends; ++u)
+              if (A.ep[u] == p)
+                v += j < A.k ? -A.Y[(size_t)A.eo[u] * A.kk + j] : A.we[u] * A.Z[(size_t)i * A.E + A.eo[u]];
+          }
+        }
+      }
+      K[((size_t)q * A.kk + j) * A.kk + i] = v;
+    }
+}
+
+// In-place Gauss-Jordan inverse of every K, one CTA each. No pivoting: K is the identity plus a product
+// of positive operators, and the constraints come last.
+__global__ void __launch_bounds__(1024) k_invert(double* __restrict__ Kq, int n) {
+  extern __shared__ double sh[];
+  double* rp = sh;        // pivot row / pivot
+  double* cp = sh + n;    // pivot column
+  double* K = Kq + (size_t)blockIdx.x * n * n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int p = 0; p < n; ++p) {
+    const double piv = 1.0 / K[(size_t)p * n + p];
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      rp[j] = j == p ? piv : K[(size_t)p * n + j] * piv;
+      cp[j] = K[(size_t)j * n + p];
+    }
+    __syncthreads();
+    for (int i = warp; i < n; i += nw) {
+      double* row = K + (size_t)i * n;
+      const double c = cp[i];
+      for (int j = lane; j < n; j += 32)
+        row[j] = i == p ? rp[j] : (j == p ? -c * piv : fma(-c, rp[j], row[j]));
+    }
+    __syncthreads();
+  }
+}
+
+// Kept transposed: the solve's threads read consecutive entries of a column of K^-1.
+__global__ void __launch_bounds__(256) k_keep(const double* __restrict__ K, int n, double* __restrict__ out) {
+  const size_t o = (size_t)blockIdx.y * n * n;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * n; t += (size_t)gridDim.x * blockDim.x)
+    out[o + (t % n) * n + t / n] = K[o + t];
+}
+
+constexpr int INT = 1024;
+
+// One wavenumber per CTA: fluxes from the end values, added to the spectral right-hand sides. Bound by
+// reading Y, Z (shared by all wavenumbers, L2) and the kept inverse.
+template <typename T>
+__global__ void __launch_bounds__(INT) k_iface(const IfaceArgs<T> I, long long ncell, T* __restrict__ x) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  double* work = reinterpret_cast<double*>(raw);
+  const int q = blockIdx.x;
+  for (int e = threadIdx.x; e < I.E; e += INT) work[e] = (double)I.ends[(size_t)q * I.E + e];
+  __syncthreads();
+  T* xq = x + (long long)q * ncell;
+  iface_solve(I, q, work, I.ssum, I.alpha, INT, [&](int e, T v) {
+    int u = 0;
+    while (u + 1 < I.nends && e >= I.eo[u + 1]) ++u;
+    xq[I.row[u] + e - I.eo[u]] += v;
+  });
+}
+
+template <typename T>
+cudaError_t iface_t(snac_plan* P, cudaStream_t s) {
+  const IfaceArgs<T> I = iface_args<T>(P);
+  const size_t smem = iface_doubles(I.E, I.kk, INT) * sizeof(double);
+  LaunchScope ls(P, K_IFACE, P->nz * (8.0 * I.kk * I.kk + 3.0 * sizeof(T) * I.E),
+                 2.0 * P->nz * ((double)I.kk * I.kk + 2.0 * I.k * I.E), s);
+  cudaFuncSetAttribute(k_iface<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
+  k_iface<T><<<P->nz, INT, smem, s>>>(I, P->lev[0].ncell, (T*)P->lev[0].d_u);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_iface(snac_plan* P, cudaStream_t s) {
+  return P->precision == SNAC_FP64 ? iface_t<double>(P, s) : iface_t<float>(P, s);
+}
+
+cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
+  DirectPlan& D = P->direct;
+  IfaceTab& I = D.it;
+  const bool f64 = P->precision == SNAC_FP64;
+  std::vector<void*> tmp;
+  cudaError_t e = cudaSuccess;
+  auto get = [&](size_t bytes) -> void* {
+    void* p = nullptr;
+    if (e == cudaSuccess) e = cudaMalloc(&p, bytes);
+    if (p) tmp.push_back(p);
+    return p;
+  };
+  BuildArgs A{};
+  A.k = I.k;
+  A.kk = I.kk;
+  A.E = I.E;
+  A.ns = I.ns;
+  A.qs = I.qs;
+  A.gs = P->singular ? 1 : 0;
+  A.nends = I.nends;
+  for (int a = 0; a < I.ns; ++a) A.sp[a] = I.sp[a];
+  double* dZ = (double*)get(I.Zh.size() * sizeof(double));
+  double* K = (double*)get((size_t)P->nz * I.kk * I.kk * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dZ, I.Zh.data(), I.Zh.size() * sizeof(double), cudaMemcpyHostToDevice, s);
+  A.Y = I.d_Y;
+  A.Z = dZ;
+  std::vector<double4*> resp(D.pc.size(), nullptr);
+  for (size_t p = 0; p < D.pc.size(); ++p) {
+    const DirectTab& d = D.pc[p];
+    resp[p] = (double4*)get((size_t)P->nz * d.M * sizeof(double4));
+    if (e != cudaSuccess) break;
+    const TriRow<double>* tri = (const TriRow<double>*)(f64 ? d.d_tri : (void*)d.d_tri64);
+    const double* lam = f64 ? (const double*)d.d_lam : d.d_lam64;
+    const long long sys = (long long)P->nz * d.M;
+    k_resp<<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(tri, lam, P->d_sigma64, d.cscale, d.cscale / (2.0 * d.M), P->nz,
+                                                        d.M, d.N, resp[p]);
+    e = cudaGetLastError();
+  }
+  for (int u = 0; u <= I.nends; ++u) A.eo[u] = I.eo[u];
+  for (int u = 0; u < I.nends; ++u) {
+    const DirectTab& d = D.pc[I.ep[u]];
+    A.ep[u] = I.ep[u];
+    A.ee[u] = I.ee[u];
+    A.em[u] = d.M;
+    A.we[u] = I.ee[u] ? d.w.back() : d.w.front();
+    A.resp[u] = resp[I.ep[u]];
+  }
+  if (e == cudaSuccess) {
+    const unsigned t = (unsigned)((I.kk + KT - 1) / KT);
+    k_build<<<dim3(t, t, (unsigned)P->nz), 256, 0, s>>>(A, K);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) {
+    const size_t smem = 2 * (size_t)I.kk * sizeof(double);
+    k_invert<<<P->nz, I.kk >= 256 ? 1024 : 256, smem, s>>>(K, I.kk);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) {
+    const dim3 g((unsigned)std::max<size_t>(1, std::min<size_t>(64, (size_t)I.kk * I.kk / 1024)), (unsigned)P->nz);
+    k_keep<<<g, 256, 0, s>>>(K, I.kk, I.d_KT);
+    e = cudaGetLastError();
+  }
+  const cudaError_t es = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = es;
+  for (void* p : tmp) cudaFree(p);
+  std::vector<double>().swap(I.Zh);
+  return e;
+}
+
+}  // namespace snac

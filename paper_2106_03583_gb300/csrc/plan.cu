@@ -13,7 +13,6 @@
 #include <cstring>
 #include <new>
 
-#include "direct_dev.cuh"
 #include "fused_tab.h"
 #include "kern_common.cuh"
 #include "snac_impl.h"
@@ -339,17 +338,6 @@ int build_levels(snac_plan* P, const std::vector<HBlock>& hb) {
   return SNAC_OK;
 }
 
-double mode_lambda(int kind, int n, int q) {
-  double m;
-  switch (kind) {
-    case KIND_PP: m = q; break;
-    case KIND_NN: m = 0.5 * q; break;
-    case KIND_DD: m = 0.5 * (q + 1); break;
-    default: m = 0.25 * (2 * q + 1); break;
-  }
-  return 2.0 * (std::cos(2.0 * M_PI * m / n) - 1.0);
-}
-
 // Weight w_q with sum_k x_k^2 = sum_q w_q Xhat_q^2 for the unnormalised transforms of Table 1.
 double parseval_weight(int kind, int n, int q) {
   switch (kind) {
@@ -358,260 +346,6 @@ double parseval_weight(int kind, int n, int q) {
     case KIND_DD: return q == n - 1 ? 0.25 / n : 0.5 / n;
     default: return 0.5 / n;
   }
-}
-
-// Boundary pair of an assembled plane axis from its two outer face kinds.
-int pair_kind(int lo, int hi) {
-  if (lo == SNAC_BC_PERIODIC) return KIND_PP;
-  if (lo == SNAC_BC_NEUMANN) return hi == SNAC_BC_NEUMANN ? KIND_NN : KIND_ND;
-  return hi == SNAC_BC_NEUMANN ? KIND_DN : KIND_DD;
-}
-
-// Passes of an in-place FFT of n points: the factors 2 spread evenly over the fewest passes of at most
-// max_log2 each, then 7, 5, 3. False if another prime divides n.
-bool fft_tab(int n, int max_log2, FftTab& F) {
-  F = FftTab{};
-  F.n = n;
-  int twos = 0, rest = n;
-  while (rest % 2 == 0) rest /= 2, ++twos;
-  std::vector<int> rad;
-  for (int left = twos, np = (twos + max_log2 - 1) / max_log2; np > 0; --np) {
-    const int b = (left + np - 1) / np;
-    rad.push_back(1 << b);
-    left -= b;
-  }
-  for (int p : {7, 5, 3})
-    while (rest % p == 0) rest /= p, rad.push_back(p);
-  if (rest != 1 || rad.size() > FFT_MAX_PASS) return false;
-  if (rad.empty()) rad.push_back(1);
-  F.np = n == 1 ? 0 : (int)rad.size();
-  F.l1 = n / rad[0];
-  int span = n;
-  for (int k = 0; k < F.np; ++k) {
-    F.rad[k] = rad[k];
-    F.span[k] = span;
-    span /= rad[k];
-  }
-  return true;
-}
-
-// Row of every frequency after the forward passes (digit-reversed order).
-std::vector<int> fft_perm(const FftTab& F) {
-  std::vector<int> perm(F.n);
-  for (int k = 0; k < F.n; ++k) {
-    int q = k, p = 0;
-    for (int s = 0; s < F.np; ++s) {
-      p += (q % F.rad[s]) * (F.span[s] / F.rad[s]);
-      q /= F.rad[s];
-    }
-    perm[k] = p;
-  }
-  return perm;
-}
-
-// The direct solve of the reduced equations (direct_dev.cuh), where the layout allows it: the blocks
-// tile a rectangle with one cell grid per axis, each outer side has one face kind, one plane axis is
-// uniform with an even length whose half or whole has no prime factor above 7, and the other is not
-// periodic. Only with the default schedule: a caller who sets a multigrid option gets the multigrid.
-// The x axis is taken where both qualify (its lines are contiguous).
-int build_direct(snac_plan* P, const std::vector<HBlock>& hb) {
-  if (P->nu1 != 2 || P->nu2 != 2 || P->max_cycles != 40 || P->max_coarse != 64 || P->fused != -1 ||
-      P->onchip_opt != 0 || P->bottom_cells != 0 || P->inner_reduction != 0.0)
-    return SNAC_OK;
-  const int nb = (int)hb.size();
-  // the block grid
-  std::vector<long long> at[2];
-  for (int a = 0; a < 2; ++a) {
-    for (const HBlock& h : hb) at[a].push_back(h.lo[a]);
-    std::sort(at[a].begin(), at[a].end());
-    at[a].erase(std::unique(at[a].begin(), at[a].end()), at[a].end());
-  }
-  const int gx = (int)at[0].size(), gy = (int)at[1].size();
-  if ((long long)gx * gy != nb) return SNAC_OK;
-  std::vector<int> grid(nb, -1);
-  for (int b = 0; b < nb; ++b) {
-    const int ix = (int)(std::lower_bound(at[0].begin(), at[0].end(), hb[b].lo[0]) - at[0].begin());
-    const int iy = (int)(std::lower_bound(at[1].begin(), at[1].end(), hb[b].lo[1]) - at[1].begin());
-    if (grid[iy * gx + ix] >= 0) return SNAC_OK;
-    grid[iy * gx + ix] = b;
-  }
-  auto blk = [&](int ix, int iy) { return grid[iy * gx + ix]; };
-  int outer[2][2] = {{-1, -1}, {-1, -1}};
-  for (int iy = 0; iy < gy; ++iy)
-    for (int ix = 0; ix < gx; ++ix) {
-      const HBlock& h = hb[blk(ix, iy)];
-      const int g[2] = {gx, gy}, i[2] = {ix, iy};
-      for (int a = 0; a < 2; ++a) {
-        // one extent and one set of widths per block column / row, with no gap to the next
-        const HBlock& first = hb[a == 0 ? blk(ix, 0) : blk(0, iy)];
-        if (h.lo[a] != first.lo[a] || h.hi[a] != first.hi[a] || h.w[a] != first.w[a]) return SNAC_OK;
-        if (i[a] + 1 < g[a] && h.hi[a] + 1 != at[a][i[a] + 1]) return SNAC_OK;
-        for (int sd = 0; sd < 2; ++sd) {
-          const int to = i[a] + (sd ? 1 : -1);
-          const bool inner = to >= 0 && to < g[a];
-          const int wrap = (to + g[a]) % g[a];
-          const int nbr = a == 0 ? blk(wrap, iy) : blk(ix, wrap);
-          const bool linked = h.bc[a][sd] == SNAC_BC_BLOCK && h.nbr[a][sd] == nbr;
-          if (inner) {
-            // (with two blocks along an axis that also wraps, both faces name the same neighbour)
-            if (!linked) return SNAC_OK;
-            continue;
-          }
-          int k = h.bc[a][sd];
-          if (k == SNAC_BC_BLOCK) {
-            if (!linked || g[a] < 2) return SNAC_OK;
-            k = SNAC_BC_PERIODIC;
-          }
-          if (outer[a][sd] >= 0 && outer[a][sd] != k) return SNAC_OK;
-          outer[a][sd] = k;
-        }
-      }
-    }
-  std::vector<double> w[2];
-  std::vector<Coef<double>> cf[2];
-  const HostLevel& l0 = P->lev[0];
-  for (int ix = 0; ix < gx; ++ix) {
-    const int b = blk(ix, 0);
-    w[0].insert(w[0].end(), hb[b].w[0].begin(), hb[b].w[0].end());
-    cf[0].insert(cf[0].end(), l0.cx.begin() + l0.blk[b].xo, l0.cx.begin() + l0.blk[b].xo + l0.blk[b].nx);
-  }
-  for (int iy = 0; iy < gy; ++iy) {
-    const int b = blk(0, iy);
-    w[1].insert(w[1].end(), hb[b].w[1].begin(), hb[b].w[1].end());
-    cf[1].insert(cf[1].end(), l0.cy.begin() + l0.blk[b].yo, l0.cy.begin() + l0.blk[b].yo + l0.blk[b].ny);
-  }
-  const bool f64 = P->precision == SNAC_FP64;
-  int ax = -1, kind = 0, cls = 0;
-  FftTab F{};
-  for (int a = 0; a < 2 && ax < 0; ++a) {
-    const int m = (int)w[a].size(), n = (int)w[1 - a].size();
-    if (m % 2 || m < 4 || m > MAX_NZ || n < 2 || n > 65535 || outer[1 - a][0] == SNAC_BC_PERIODIC) continue;
-    bool uniform = true;
-    for (double v : w[a]) uniform = uniform && std::fabs(v - w[a][0]) <= 1e-12 * w[a][0];
-    const int kd = pair_kind(outer[a][0], outer[a][1]);
-    const int cl = kd == KIND_ND || kd == KIND_DN ? LINES_DCT4 : LINES_PAIR;
-    if (!uniform || !fft_tab(cl == LINES_PAIR ? m : m / 2, f64 ? 3 : 4, F)) continue;
-    ax = a;
-    kind = kd;
-    cls = cl;
-  }
-  if (ax < 0 || P->lev[0].ncell >= (1LL << 31)) return SNAC_OK;
-  DirectTab& D = P->direct;
-  D.M = (int)w[ax].size();
-  D.N = (int)w[1 - ax].size();
-  D.cls = cls;
-  D.kind = kind;
-  D.xl = ax == 0 ? 1 : 0;
-  D.fft = F;
-  // twiddles
-  const int nf = F.n, M = D.M, N = D.N;
-  D.w2n = nf;
-  D.t4a = D.w2n + M + 1;
-  D.t4b = D.t4a + M / 2;
-  std::vector<double> tw(2 * (size_t)(D.t4b + M / 2));
-  auto put = [&](int k, double ang) {
-    tw[2 * k] = std::cos(ang);
-    tw[2 * k + 1] = std::sin(ang);
-  };
-  for (int k = 0; k < nf; ++k) put(k, -2.0 * M_PI * k / nf);
-  for (int k = 0; k <= M; ++k) put(D.w2n + k, -M_PI * k / (2.0 * M));
-  for (int k = 0; k < M / 2; ++k) put(D.t4a + k, -M_PI * (4.0 * k + 1.0) / (4.0 * M));
-  for (int k = 0; k < M / 2; ++k) put(D.t4b + k, -M_PI * k / (double)M);
-  const std::vector<int> perm = fft_perm(F);
-  // eigenvalues of the slots and the tridiagonal rows, scaled by a power of two to couplings of about 1
-  double h = 0.0;
-  for (double v : w[ax]) h += v;
-  h /= M;
-  const std::vector<Coef<double>>& ct = cf[1 - ax];
-  double big = 4.0 / (h * h);
-  for (const Coef<double>& c : ct) big = std::max(big, c.lo + c.hi);
-  int ex = 0;
-  std::frexp(big, &ex);
-  D.cscale = std::ldexp(1.0, -ex);
-  std::vector<double> lam(M), tri(4 * (size_t)N);
-  for (int k = 0; k < M; ++k)
-    lam[k] = D.cscale * mode_lambda(kind, M, kind == KIND_DD || kind == KIND_DN ? M - 1 - k : k) / (h * h);
-  for (int n = 0; n < N; ++n) {
-    const Coef<double>& c = ct[n];
-    double tau = 0.0;
-    if (n == 0 && outer[1 - ax][0] == SNAC_BC_DIRICHLET) tau += 2.0 / (c.w * c.w);
-    if (n == N - 1 && outer[1 - ax][1] == SNAC_BC_DIRICHLET) tau += 2.0 / (c.w * c.w);
-    tri[4 * n] = D.cscale * c.lo;
-    tri[4 * n + 1] = D.cscale * c.hi;
-    tri[4 * n + 2] = D.cscale * tau;
-    tri[4 * n + 3] = c.hi > 0.0 ? c.lo / c.hi : 0.0;
-  }
-  // where the lines live: plane offset of (m, n) = base[n nbm + mblk[m]] + m mstr[n]
-  const int gm = ax == 0 ? gx : gy;
-  std::vector<int> mblk(M), base((size_t)N * gm), mstr(N);
-  std::vector<unsigned> cellmn(l0.ncell);
-  bool vec = true;
-  for (int iy = 0, y0 = 0; iy < gy; y0 += l0.blk[blk(0, iy)].ny, ++iy)
-    for (int ix = 0, x0 = 0; ix < gx; x0 += l0.blk[blk(ix, 0)].nx, ++ix) {
-      const BlockDev& d = l0.blk[blk(ix, iy)];
-      vec = vec && d.off % 2 == 0 && d.nx % 2 == 0 && x0 % 2 == 0;
-      for (int j = 0; j < d.ny; ++j)
-        for (int i = 0; i < d.nx; ++i) {
-          const int m = ax == 0 ? x0 + i : y0 + j, n = ax == 0 ? y0 + j : x0 + i;
-          const long long c = d.off + (long long)j * d.nx + i;
-          cellmn[c] = (unsigned)m | (unsigned)n << 16;
-          mblk[m] = ax == 0 ? ix : iy;
-          mstr[n] = ax == 0 ? 1 : d.nx;
-          base[(size_t)n * gm + mblk[m]] = (int)(c - (long long)m * mstr[n]);
-        }
-    }
-  // pairs: two cells of a line (x lines), or the same cell of two adjacent lines (first one even)
-  D.vec = vec && (ax == 0 || N % 2 == 0) && l0.ncell % 2 == 0;
-  D.nbm = gm;
-  auto up = [&](void** d, const std::vector<double>& v) -> int {
-    if (f64) {
-      double* p = nullptr;
-      const int st = upload(P, &p, v);
-      *d = p;
-      return st;
-    }
-    float* p = nullptr;
-    const int st = upload(P, &p, to32(v));
-    *d = p;
-    return st;
-  };
-  int st;
-  if (!f64) {
-    // the systems with the smallest -(lambda + sigma): up to LOW_SPAN times the smallest nonzero one, 1/64 of
-    // all at most (kern_direct.cu, k_tri_low; rows of longer systems do not fit its CTA)
-    constexpr double LOW_SPAN = 256.0;
-    std::vector<std::pair<double, int>> by;
-    std::vector<unsigned char> low((size_t)P->nz * M, 0);
-    double least = INFINITY;
-    for (int l = 0; l < P->nz; ++l)
-      for (int k = 0; k < M; ++k) {
-        const double t = -(P->sigma[l] * D.cscale + lam[k]);
-        if (t > 0.0) least = std::min(least, t);
-      }
-    if (N <= 512 && !P->ranged)
-      for (int l = 0; l < P->nz; ++l)
-        for (int k = 0; k < M; ++k) {
-          const double t = -(P->sigma[l] * D.cscale + lam[k]);
-          if (t <= LOW_SPAN * least) by.push_back({t, l * M + k});
-        }
-    std::sort(by.begin(), by.end());
-    by.resize(std::min(by.size(), low.size() / 64));
-    std::vector<int> list;
-    for (const auto& v : by) {
-      list.push_back(v.second);
-      low[v.second] = 1;
-    }
-    D.nlow = (int)list.size();
-    if ((st = upload(P, &D.d_lam64, lam)) || (st = upload(P, &D.d_tri64, tri)) || (st = upload(P, &D.d_lowlist, list)) ||
-        (st = upload(P, &D.d_low, low)))
-      return st;
-  }
-  if ((st = up(&D.d_tw, tw)) || (st = up(&D.d_lam, lam)) || (st = up(&D.d_tri, tri)) ||
-      (st = upload(P, &D.d_perm, perm)) || (st = upload(P, &D.d_cellmn, cellmn)) || (st = upload(P, &D.d_base, base)) ||
-      (st = upload(P, &D.d_mblk, mblk)) || (st = upload(P, &D.d_mstr, mstr)))
-    return st;
-  D.on = true;
-  return SNAC_OK;
 }
 
 int build_coarse(snac_plan* P) {
@@ -1073,7 +807,13 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     for (int l = 0; l < P->nz; ++l) sm[l] = (P->singular && mode_lambda(P->kind, P->nzt, P->q0 + l) == 0.0) ? 1 : 0;
     if ((st = upload(P, &P->d_singular_mode, sm))) break;
     if ((st = build_coarse(P))) break;
-    if ((st = build_direct(P, hb))) break;
+    {
+      std::vector<FaceKinds> faces(hb.size());
+      for (size_t b = 0; b < hb.size(); ++b)
+        for (int a = 0; a < 2; ++a)
+          for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
+      if ((st = build_direct(P, faces))) break;
+    }
     // the bottom of the cycle in one launch: from the first level below 0 whose planes, with all
     // coarser ones, fit in one CTA's shared memory (at least one smoothed level above the coarsest)
     // and whose plane has at most bottom_cells cells
@@ -1094,32 +834,11 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
       const int L = (int)P->lev.size() - 1;
       P->onchip = P->onchip_opt == 0 && P->nu1 >= 1 && P->nu2 >= 1 && L >= 1 && L < BOTTOM_MAX_LEVELS &&
                   P->lev[0].ncell <= BOTTOM_MAX_CELLS && bottom_layout(P, 0, inner).bytes <= (size_t)BOTTOM_MAX_SMEM;
+      if (P->onchip && P->direct.on && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) P->direct.on = false;
     }
     // the automatic inner reduction: an on-chip plan's V-cycles are cheap next to an outer step,
     // so it asks more of each step (measured on c64: 3 outer steps at 1e-4, 2 at 3e-5, 18 % faster)
     if (P->inner_reduction == 0.0) P->inner_reduction = P->onchip ? 3e-5 : 1e-4;
-    if (P->direct.on && !P->onchip && (P->precision == SNAC_FP64 || (long long)P->nz * P->direct.M >= 256LL * P->sms)) {
-      std::vector<int> qrow(P->nz), qof;
-      std::map<int, int> seen;  // wavenumbers q and n - q of the real DFT have one eigenvalue
-      for (int l = 0; l < P->nz; ++l) {
-        const int q = P->q0 + l;
-        const auto it = seen.emplace(P->kind == KIND_PP ? std::min(q, P->nzt - q) : q, (int)qof.size());
-        if (it.second) qof.push_back(l);
-        qrow[l] = it.first->second;
-      }
-      int* d_qof = nullptr;
-      if ((st = upload(P, &P->direct.d_qrow, qrow)) || (st = upload(P, &d_qof, qof)) ||
-          (st = dmalloc(P, (char**)&P->direct.d_fac, qof.size() * (size_t)P->direct.M * P->direct.N * inner)))
-        break;
-      cudaStream_t cs = nullptr;
-      bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
-      ok = ok && launch_tri_factor(P, d_qof, (int)qof.size(), cs) == cudaSuccess && cudaStreamSynchronize(cs) == cudaSuccess;
-      if (cs) cudaStreamDestroy(cs);
-      if (!ok) {
-        st = fail(SNAC_ERR_CUDA, "factoring the tridiagonal systems failed");
-        break;
-      }
-    }
     // fused FP32 tile kernels on the levels whose blocks all keep the halo inside their neighbours
     // (above the bottom sub-cycle; not needed when the whole solve runs on chip)
     const bool want_fused = !P->onchip && (P->fused == 1 || (P->fused < 0 && P->precision == SNAC_MIXED));
@@ -1258,6 +977,7 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
         break;
       }
     }
+    if (P->direct.on && (st = finish_direct(P))) break;
   } while (0);
   if (st) {
     free_plan(P);
@@ -1273,6 +993,32 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
 }  // namespace
 
 namespace snac {
+int plan_alloc(snac_plan* P, void** p, size_t bytes) {
+  char* c = nullptr;
+  const int st = dmalloc(P, &c, bytes);
+  *p = c;
+  return st;
+}
+
+int plan_upload(snac_plan* P, void** p, const void* src, size_t bytes) {
+  const int st = plan_alloc(P, p, bytes);
+  if (st) return st;
+  if (bytes && cudaMemcpy(*p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess)
+    return fail(SNAC_ERR_CUDA, "cudaMemcpy upload failed");
+  return SNAC_OK;
+}
+
+double mode_lambda(int kind, int n, int q) {
+  double m;
+  switch (kind) {
+    case KIND_PP: m = q; break;
+    case KIND_NN: m = 0.5 * q; break;
+    case KIND_DD: m = 0.5 * (q + 1); break;
+    default: m = 0.25 * (2 * q + 1); break;
+  }
+  return 2.0 * (std::cos(2.0 * M_PI * m / n) - 1.0);
+}
+
 int plan_inner_size(const snac_plan* P) { return P->precision == SNAC_FP64 ? 8 : 4; }
 
 int check_layout(int nblocks, const snac_block* blocks, int homog_axis) {

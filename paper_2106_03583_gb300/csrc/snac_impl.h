@@ -167,19 +167,19 @@ struct FftTab {
   int rad[FFT_MAX_PASS], span[FFT_MAX_PASS];
 };
 
-// Separable plans (the blocks assemble into a rectangle with a uniform plane axis): the reduced
-// equations are solved by a transform along that axis and tridiagonal systems along the other
-// (direct_dev.cuh). Tables in the plan's inner type.
+// One piece of a plan solved directly (direct_dev.cuh): a rectangle of blocks with one tensor grid, its
+// reduced equations solved by a transform along one plane axis and tridiagonal systems along the other.
+// Tables in the plan's inner type.
 struct DirectTab {
-  bool on = false;
   int M = 0, N = 0;        // cells along the transformed / the tridiagonal axis
   int cls = 0, kind = 0;   // LINES_PAIR / LINES_DCT4; boundary pair of the transformed axis
   int xl = 0, vec = 0, nbm = 1;
+  int soff = 0;            // first spectral element within a plane (the pieces' spectra follow each other)
   FftTab fft{};
   int w2n = 0, t4a = 0, t4b = 0;  // offsets in the twiddle table
   double cscale = 1.0;
+  bool singular = false;   // all-Neumann / periodic: a zero shift makes slot 0's system singular
   void* d_fac = nullptr;             // plans not on chip: reciprocal pivots (k_tri_pre), inner type
-  int* d_qrow = nullptr;             // per wavenumber: its set of them
   int nlow = 0;                      // mixed plans: systems solved in FP64 arithmetic (k_tri_low)
   int* d_lowlist = nullptr;          // their numbers q M + kappa
   unsigned char* d_low = nullptr;    // per system: 1 if listed
@@ -189,17 +189,46 @@ struct DirectTab {
   void* d_tri = nullptr;
   double* d_lam64 = nullptr;  // the same in FP64 (mixed plans; FP64 plans: the tables above)
   double* d_tri64 = nullptr;
-  unsigned* d_cellmn = nullptr;
+  void* d_w = nullptr;        // cell widths along the tridiagonal axis
   int* d_base = nullptr;
   int* d_mblk = nullptr;
   int* d_mstr = nullptr;
+  // host copies the interface setup needs
+  std::vector<double> w, lam;
+};
+
+// The interfaces between the pieces of a plan (kern_iface.cu).
+constexpr int IFACE_MAX_ENDS = 16;
+struct IfaceTab {
+  int k = 0, kk = 0, E = 0;  // interface cells; with one unknown per singular piece; spectral end values
+  int nends = 0;             // ends (piece, first or last row) that carry interface cells
+  int ep[IFACE_MAX_ENDS] = {}, ee[IFACE_MAX_ENDS] = {}, eo[IFACE_MAX_ENDS + 1] = {};
+  int qs = -1;               // wavenumber (local) with a zero shift, where pieces are singular; -1: none
+  int ns = 0;                // singular pieces
+  int sp[IFACE_MAX_ENDS] = {};
+  double* d_Y = nullptr;     // [E][kk]: end values -> jump of u across every interface cell
+  void* d_Z = nullptr;       // [kk][E]: fluxes -> right-hand sides of the end rows
+  double* d_KT = nullptr;    // [q][kk][kk]: transposed inverse of the interface system
+  void* d_ends = nullptr;    // [q][E]: end values of a solve
+  void* d_alpha = nullptr;   // [piece]: constant of every singular piece
+  void* d_ssum = nullptr;    // [piece]: weighted sum of its slot-0 right-hand side
+  std::vector<double> Zh;    // host copy, until the systems are set up
+};
+
+struct DirectPlan {
+  bool on = false;
+  std::vector<DirectTab> pc;
+  IfaceTab it;
+  int* d_qrow = nullptr;        // per wavenumber: its set of pivots in d_fac
+  unsigned* d_celloff = nullptr;  // on chip: per plane cell, element of the shared buffer | sign flip << 31
+  void* d_args = nullptr;       // on chip: the pieces' DirectArgs
 };
 
 // Kernel kinds counted by the tracing facility.
 enum KernelKind {
   K_FIELD3D = 0, K_REDUCE, K_FIX_MEAN, K_SHIFT, K_FORWARD, K_BACKWARD, K_SMOOTH, K_RESTRICT, K_PROLONG,
   K_COARSE, K_MODE_RESID, K_MODE_REDUCE, K_MODE_APPLY, K_FDOWN, K_FUP, K_BOTTOM, K_FIELD3D_FF, K_ONCHIP, K_FWD_ONCHIP,
-  K_LINES_FWD, K_TRI, K_LINES_BWD, K_COUNT
+  K_LINES_FWD, K_TRI, K_LINES_BWD, K_IFACE, K_COUNT
 };
 
 struct KernelStat {
@@ -233,7 +262,7 @@ struct snac_plan {
   int onchip_opt = 0;         // snac_options.onchip
   int bottom_cells = 0;       // snac_options.bottom_cells
   void* d_onchip = nullptr;   // BottomLevel<inner type> table from level 0
-  snac::DirectTab direct;     // separable plans: direct solves of the reduced equations
+  snac::DirectPlan direct;    // direct solves of the reduced equations, where the layout allows them
   double* d_pweight = nullptr;
   int* h_cycles = nullptr;    // per wavenumber: V-cycles of the last on-chip solve (mapped pinned)
   int* dh_cycles = nullptr;
@@ -456,9 +485,27 @@ BottomLayout bottom_layout(const snac_plan* P, int lb, size_t w);
 // Separable plans: every wavenumber's solution of the reduced equations for the right-hand sides in
 // lev[0].d_f (plain order), into mode_solution(P).
 cudaError_t launch_direct(snac_plan* P, cudaStream_t s);
-// The reciprocal pivots of an FP64 plan's tridiagonal systems, once per plan (d_qof: a wavenumber of
-// every set).
-cudaError_t launch_tri_factor(snac_plan* P, const int* d_qof, int rows, cudaStream_t s);
+// Plan creation: the pieces and their tables, where the layout allows direct solves (direct_plan.cu;
+// faces: the face kinds W, E, S, N of every block), and, once the launch shape is known, the pivots, the
+// interface systems and the on-chip tables.
+struct FaceKinds {
+  int k[4];
+};
+int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces);
+int finish_direct(snac_plan* P);
+cudaError_t launch_tri_factor(snac_plan* P, const DirectTab& D, const int* d_qof, int rows, cudaStream_t s);
+// Interface systems of plans of several pieces: setup (once per plan) and the solve of every wavenumber's
+// fluxes from the end values, added to the spectral right-hand sides.
+cudaError_t setup_iface(snac_plan* P, cudaStream_t s);
+cudaError_t launch_iface(snac_plan* P, cudaStream_t s);
+// Plan-owned device memory (freed with the plan).
+int plan_alloc(snac_plan* P, void** p, size_t bytes);
+int plan_upload(snac_plan* P, void** p, const void* src, size_t bytes);
+double mode_lambda(int kind, int n, int q);
+bool fft_tab(int n, int max_log2, FftTab& F);
+std::vector<int> fft_perm(const FftTab& F);
+// Dynamic shared memory of a direct on-chip solve (0: does not fit).
+size_t direct_onchip_smem(const snac_plan* P);
 // h_check[0] = 1 if any of the n values (inner type) is NaN or Inf, else 0.
 cudaError_t launch_nonfinite(snac_plan* P, const void* v, long long n, cudaStream_t s);
 // Where a solve leaves the mode-space solution: the level-0 iterate, or (direct solves of planes too
