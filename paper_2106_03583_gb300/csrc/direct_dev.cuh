@@ -22,6 +22,8 @@
 //   DCT-IV kinds (ND; DN = ND of (-1)^m x_m, slots reversed likewise): column c holds line c as a
 //       half-length sequence t_j = (x_2j + i x_M-1-2j) e^{-i pi (4j+1)/4M}.
 // Forward then inverse multiplies by 2 M for every kind; the tridiagonal solve divides by it.
+//   dense (an axis that is not uniform, or a length with another prime factor; planes of several passes):
+//       the eigenvectors of the one-dimensional operator, one M x M matrix product per line and way.
 //
 // Tridiagonal systems: (lo + hi + tau) u_n - lo u_{n-1} - hi u_{n+1} = -f_n / 2M with couplings lo, hi
 // >= 0 and tau = -lambda_kappa - sigma_q + (Dirichlet face terms) >= 0. Elimination carries the row
@@ -38,7 +40,7 @@
 namespace snac {
 namespace {
 
-enum { LINES_PAIR = 0, LINES_DCT4 = 1 };
+enum { LINES_PAIR = 0, LINES_DCT4 = 1, LINES_DENSE = 2 };
 
 // One row of the tridiagonal axis: couplings, face term, and lo / hi (0 where hi = 0).
 template <typename T>
@@ -64,7 +66,9 @@ struct DirectArgs {
   int soff;                // the piece's first spectral element within a plane
   int e0, e1;              // where its first / last row's values start in the end vector, -1: not needed
   T cscale;                // power of two that brings the couplings of tri (and lam) to about 1
-  T scale;                 // cscale / 2M
+  T scale;                 // cscale / theta (2M, dense: 1)
+  const T* F1;             // LINES_DENSE: matrices [m][kappa], [kappa][m]
+  const T* B1;
   // plane offset of (m, n): base[n nbm + mblk[m]] + m mstr[n]
   const int* base;
   const int* mblk;
@@ -98,7 +102,9 @@ inline DirectArgs<T> direct_args(const snac_plan* P, const DirectTab& D) {
   else A.sigma = P->d_sigma32;
   A.ncell = P->lev[0].ncell;
   A.cscale = (T)D.cscale;
-  A.scale = (T)(D.cscale / (2.0 * D.M));
+  A.scale = (T)(D.cscale / D.theta);
+  A.F1 = (const T*)D.d_F;
+  A.B1 = (const T*)D.d_B;
   A.base = D.d_base;
   A.mblk = D.d_mblk;
   A.mstr = D.d_mstr;

@@ -215,23 +215,94 @@ std::vector<double> piece_widths(const snac_plan* P, const Piece& p, int axis, b
   return w;
 }
 
+// Eigenvalues (into d) and orthonormal eigenvectors (rows of Z) of a symmetric tridiagonal matrix with
+// diagonal d and off-diagonal e (e[i] couples i and i + 1): shifted QR steps by Givens rotations chased down
+// the unreduced block (Wilkinson's shift). False if the block of one eigenvalue takes more than 60 steps.
+bool tridiag_eigen(std::vector<double>& d, std::vector<double> e, std::vector<double>& Z) {
+  const int n = (int)d.size();
+  Z.assign((size_t)n * n, 0.0);
+  for (int i = 0; i < n; ++i) Z[(size_t)i * n + i] = 1.0;
+  auto small = [&](int i) { return std::fabs(e[i]) <= 1.1e-16 * (std::fabs(d[i]) + std::fabs(d[i + 1])); };
+  int steps = 0;
+  for (int hi = n - 1; hi > 0;) {
+    if (small(hi - 1)) {
+      e[--hi] = 0.0;
+      steps = 0;
+      continue;
+    }
+    if (++steps > 60) return false;
+    int lo = hi - 1;
+    while (lo > 0 && !small(lo - 1)) --lo;
+    // the eigenvalue of the trailing 2 x 2 block closer to its last entry
+    const double h = 0.5 * (d[hi - 1] - d[hi]), b = e[hi - 1];
+    const double mu = d[hi] - b * b / (h + std::copysign(std::hypot(h, b), h));
+    double x = d[lo] - mu, z = e[lo];
+    for (int k = lo; k < hi; ++k) {
+      // rotate rows and columns k, k + 1 so that (x, z) becomes (r, 0)
+      const double r = std::hypot(x, z), c = r > 0.0 ? x / r : 1.0, s = r > 0.0 ? z / r : 0.0;
+      if (k > lo) e[k - 1] = r;
+      const double d0 = d[k], d1 = d[k + 1], ek = e[k];
+      d[k] = c * c * d0 + 2.0 * c * s * ek + s * s * d1;
+      d[k + 1] = s * s * d0 - 2.0 * c * s * ek + c * c * d1;
+      e[k] = c * s * (d1 - d0) + (c * c - s * s) * ek;
+      if (k + 1 < hi) {
+        x = e[k];
+        z = s * e[k + 1];
+        e[k + 1] *= c;
+      }
+      double* z0 = &Z[(size_t)k * n];
+      double* z1 = z0 + n;
+      for (int i = 0; i < n; ++i) {
+        const double u = z0[i], v = z1[i];
+        z0[i] = c * u + s * v;
+        z1[i] = c * v - s * u;
+      }
+    }
+  }
+  return true;
+}
+
 bool uniform(const std::vector<double>& w) {
   for (double v : w)
     if (std::fabs(v - w[0]) > 1e-12 * w[0]) return false;
   return true;
 }
 
-// Whether every piece can be transformed along the layout's axis.
-bool transformable(const snac_plan* P, const Layout& L) {
+// Whether a piece's lines take the FFT: a uniform axis of even length whose half (DCT-IV kinds) or whole
+// has no prime factor above 7.
+bool fft_piece(const Piece& p, const std::vector<double>& w) {
+  const int m = (int)w.size();
+  FftTab F;
+  const bool four = p.kind == KIND_ND || p.kind == KIND_DN;
+  return m % 2 == 0 && m >= 4 && m <= MAX_NZ && uniform(w) && fft_tab(four ? m / 2 : m, 4, F);
+}
+
+// Operations per plane cell of a layout's transforms and interfaces; negative if some piece can't be
+// transformed. Dense transforms (2 M FMA per cell and solve) only for planes of several passes, and where they
+// beat the V-cycles they replace, which take the longer the more the plane is stretched: measured on M x M x 160
+// cells, stretched mildly both ways, FP64 3.2 -> 1.9 ms at M = 128, 5.9 -> 5.2 at 192, but 9.9 -> 11.3 at 256:
+// up to 200 cells on average over the plane; mixed 2.1 -> 0.7, 2.9 -> 1.2, 4.4 -> 3.2 and 8.3 -> 7.7 at 384: up
+// to there (the eigenvectors, O(M^3) on the host, take 0.02 s of plan creation). 336 x 192 x 150 mixed 6.1 -> 1.6
+// to 2.1 ms; three rectangles of 64 to 128 cells by 192, FP64, 3.6 -> 2.0 ms.
+double layout_cost(const snac_plan* P, const Layout& L) {
+  const bool f64 = P->precision == SNAC_FP64;
+  double ops = 0.0, cells = 0.0, dense = 0.0, ends = 0.0;
   for (const Piece& p : L.pc) {
     const std::vector<double> w = piece_widths(P, p, L.axis, true);
-    const int m = (int)w.size(), n = (int)piece_widths(P, p, 1 - L.axis, false).size();
-    if (m % 2 || m < 4 || m > MAX_NZ || n < 2 || n > 65535 || !uniform(w)) return false;
-    FftTab F;
-    const bool four = p.kind == KIND_ND || p.kind == KIND_DN;
-    if (!fft_tab(four ? m / 2 : m, 4, F)) return false;
+    const double m = (double)w.size(), n = (double)piece_widths(P, p, 1 - L.axis, false).size();
+    if (n < 2 || n > 65535) return -1.0;
+    cells += m * n;
+    for (int e = 0; e < 2; ++e) ends += p.iface[e] ? m : 0.0;
+    if (fft_piece(p, w)) {
+      ops += 30.0 * m * n;
+      continue;
+    }
+    if (P->onchip || p.kind == KIND_PP || m < 4 || m > 384) return -1.0;
+    dense += m * m * n;
   }
-  return true;
+  if (f64 && dense > 200.0 * cells) return -1.0;
+  const double k = (double)L.cells.size();
+  return (ops + 2.0 * dense + k * (k + 2.0 * ends)) / cells;
 }
 
 std::vector<float> to_float(const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); }
@@ -255,11 +326,13 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   D.M = (int)wm.size();
   D.N = (int)D.w.size();
   D.kind = p.kind;
-  D.cls = p.kind == KIND_ND || p.kind == KIND_DN ? LINES_DCT4 : LINES_PAIR;
+  D.cls = !fft_piece(p, wm) ? LINES_DENSE : p.kind == KIND_ND || p.kind == KIND_DN ? LINES_DCT4 : LINES_PAIR;
   D.xl = ax == 0 ? 1 : 0;
   D.soff = soff;
-  fft_tab(D.cls == LINES_PAIR ? D.M : D.M / 2, f64 ? 3 : 4, D.fft);
+  if (D.cls == LINES_DENSE) fft_tab(2, 1, D.fft);  // (not used)
+  else fft_tab(D.cls == LINES_PAIR ? D.M : D.M / 2, f64 ? 3 : 4, D.fft);
   const int nf = D.fft.n, M = D.M, N = D.N;
+  D.theta = D.cls == LINES_DENSE ? 1.0 : 2.0 * M;
   D.w2n = nf;
   D.t4a = D.w2n + M + 1;
   D.t4b = D.t4a + M / 2;
@@ -285,14 +358,51 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   }
   ct.front().lo = 0.0;  // (an interface is a Neumann face of the piece)
   ct.back().hi = 0.0;
-  double big = 4.0 / (h * h);
+  // dense: A = W^-1/2 Q Lam Q^T W^1/2 along the axis, F = Q^T W^1/2, B = W^-1/2 Q, smallest |lambda| first
+  std::vector<double> ev;
+  if (D.cls == LINES_DENSE) {
+    std::vector<Coef<double>> cm;
+    for (int b : p.rows[0].blk) {
+      const BlockDev& d = l0.blk[b];
+      if (ax == 0) cm.insert(cm.end(), l0.cx.begin() + d.xo, l0.cx.begin() + d.xo + d.nx);
+      else cm.insert(cm.end(), l0.cy.begin() + d.yo, l0.cy.begin() + d.yo + d.ny);
+    }
+    std::vector<double> dd(M), ee(M, 0.0), Z;
+    for (int m = 0; m < M; ++m) {
+      dd[m] = cm[m].d;
+      if (m + 1 < M) ee[m] = std::sqrt(cm[m].hi * cm[m + 1].lo);
+    }
+    if (!tridiag_eigen(dd, ee, Z)) {
+      set_error("the eigenvectors along a plane axis did not converge");
+      return SNAC_ERR_LAYOUT;
+    }
+    std::vector<int> order(M);
+    for (int k = 0; k < M; ++k) order[k] = k;
+    std::sort(order.begin(), order.end(), [&](int a, int b) { return dd[a] > dd[b]; });
+    D.F.resize((size_t)M * M);
+    D.B.resize((size_t)M * M);
+    std::vector<double> ft((size_t)M * M), bt((size_t)M * M);
+    ev.resize(M);
+    for (int k = 0; k < M; ++k) {
+      ev[k] = std::min(0.0, dd[order[k]]);
+      if (k == 0 && p.kind == KIND_NN) ev[k] = 0.0;
+      for (int m = 0; m < M; ++m) {
+        const double q = Z[(size_t)order[k] * M + m], r = std::sqrt(wm[m]);
+        D.F[(size_t)k * M + m] = ft[(size_t)m * M + k] = q * r;
+        D.B[(size_t)m * M + k] = bt[(size_t)k * M + m] = q / r;
+      }
+    }
+    int se;
+    if ((se = up_inner(P, &D.d_F, ft)) || (se = up_inner(P, &D.d_B, bt))) return se;
+  }
+  double big = ev.empty() ? 4.0 / (h * h) : -ev.back();
   for (const Coef<double>& c : ct) big = std::max(big, c.lo + c.hi);
   int ex = 0;
   std::frexp(big, &ex);
   D.cscale = std::ldexp(1.0, -ex);
   D.lam.resize(M);
   for (int k = 0; k < M; ++k)
-    D.lam[k] = D.cscale * mode_lambda(p.kind, M, p.kind == KIND_DD || p.kind == KIND_DN ? M - 1 - k : k) / (h * h);
+    D.lam[k] = !ev.empty() ? D.cscale * ev[k] : D.cscale * mode_lambda(p.kind, M, p.kind == KIND_DD || p.kind == KIND_DN ? M - 1 - k : k) / (h * h);
   std::vector<double> tri(4 * (size_t)N);
   for (int n = 0; n < N; ++n) {
     const Coef<double>& c = ct[n];
@@ -418,8 +528,8 @@ int build_iface(snac_plan* P, const Layout& L) {
       const int u = end_of[2 * p + (side == 0 ? 1 : 0)];
       const DirectTab& T = D.pc[p];
       for (int k = 0; k < T.M; ++k) {
-        Y[(size_t)(I.eo[u] + k) * I.kk + j] = (side == 0 ? -1.0 : 1.0) * bwd_entry(T.kind, T.M, m, k);
-        Z[(size_t)j * I.E + I.eo[u] + k] = (side == 0 ? -c.ca : c.cb) * fwd_entry(T.kind, T.M, k, m);
+        Y[(size_t)(I.eo[u] + k) * I.kk + j] = (side == 0 ? -1.0 : 1.0) * (T.cls == LINES_DENSE ? T.B[(size_t)m * T.M + k] : bwd_entry(T.kind, T.M, m, k));
+        Z[(size_t)j * I.E + I.eo[u] + k] = (side == 0 ? -c.ca : c.cb) * (T.cls == LINES_DENSE ? T.F[(size_t)k * T.M + m] : fwd_entry(T.kind, T.M, k, m));
       }
     }
   }
@@ -454,20 +564,22 @@ bool iface_affordable(const snac_plan* P, const Layout& L) {
 }  // namespace
 
 // Only with the default schedule: a caller who sets a multigrid option gets the multigrid. Of the two plane
-// axes the one with fewer interface cells is transformed, x where they tie (its lines are contiguous).
+// axes the cheaper one is transformed, x where they tie (its lines are contiguous).
 int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
   if (P->nu1 != 2 || P->nu2 != 2 || P->max_cycles != 40 || P->max_coarse != 64 || P->fused != -1 ||
       P->onchip_opt != 0 || P->bottom_cells != 0 || P->inner_reduction != 0.0 || P->lev[0].ncell >= (1LL << 31))
     return SNAC_OK;
   Layout best;
-  bool found = false;
+  double least = INFINITY;
   for (int t = 0; t < 2; ++t) {
     Layout L;
-    if (!pieces_along(P, faces, t, L) || !transformable(P, L) || !iface_affordable(P, L)) continue;
-    if (!found || L.cells.size() < best.cells.size()) best = L;
-    found = true;
+    if (!pieces_along(P, faces, t, L) || !iface_affordable(P, L)) continue;
+    const double cost = layout_cost(P, L);
+    if (cost < 0.0 || cost >= least) continue;
+    best = L;
+    least = cost;
   }
-  if (!found) return SNAC_OK;
+  if (!std::isfinite(least)) return SNAC_OK;
   DirectPlan& D = P->direct;
   int soff = 0, st;
   for (const Piece& p : best.pc) {
@@ -476,6 +588,10 @@ int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
     soff += D.pc.back().M * D.pc.back().N;
   }
   if ((st = build_iface(P, best))) return st;
+  for (DirectTab& d : D.pc) {
+    std::vector<double>().swap(d.F);
+    std::vector<double>().swap(d.B);
+  }
   D.on = true;
   return SNAC_OK;
 }

@@ -330,6 +330,102 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
   }
 }
 
+// Dense transform of DL lines x DK outputs per CTA of 256 threads (16 x 16, each RL lines x RO outputs):
+// out[line][o] = sum_i in[line][i] mat[i][o]. Thread columns run over lines, so both orders of the plane's
+// lines load and store whole sectors (16 lines of one cell, or 8 cells of one line). FWD: planes -> spectra;
+// else spectra -> planes. 2 M FMA per cell and way: FP32 issue-bound, FP64 bound by the FP64 pipe.
+template <typename T>
+struct DenseTile {
+  // FP64: 16 outputs wide, so that no FP64 operation is spent on padding of common lengths
+  static constexpr int RL = 8, RO = sizeof(T) == 4 ? 4 : 1, DL = 16 * RL, DK = 16 * RO, DM = 16;
+};
+
+template <typename T, bool FWD>
+__global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T* __restrict__ in, T* __restrict__ out) {
+  constexpr int RL = DenseTile<T>::RL, RO = DenseTile<T>::RO, DL = DenseTile<T>::DL, DK = DenseTile<T>::DK,
+                DM = DenseTile<T>::DM;
+  __shared__ long long plane[DL];
+  __shared__ long long spec[DL];
+  __shared__ int ln[DL];
+  __shared__ T as[DM][DL];
+  __shared__ __align__(16) T bs[DM][DK];
+  const int M = A.M;
+  const long long total = (long long)A.nq * A.N, g0 = (long long)blockIdx.x * DL;
+  for (int l = threadIdx.x; l < DL; l += 256) {
+    const long long g = g0 + l;
+    const int q = g < total ? (int)(g / A.N) : 0, n = g < total ? (int)(g - (long long)q * A.N) : 0;
+    plane[l] = (long long)q * A.ncell;
+    spec[l] = (long long)q * A.ncell + A.soff + (long long)n * M;
+    ln[l] = n;
+  }
+  __syncthreads();
+  const LineSet S{plane, spec, ln};
+  const int nlive = (int)min((long long)DL, total - g0);
+  const T* __restrict__ mat = FWD ? A.F1 : A.B1;
+  const int o0 = blockIdx.y * DK;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const bool along = !FWD || A.xl;  // the inputs of a line are contiguous
+  T acc[RL][RO];
+#pragma unroll
+  for (int i = 0; i < RL; ++i)
+#pragma unroll
+    for (int j = 0; j < RO; ++j) acc[i][j] = 0;
+  constexpr int NA = DM * DL / 256, NB = DM * DK / 256;
+  T ra[NA], rb[NB];
+  auto fetch = [&](int m0) {
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int t = threadIdx.x + u * 256;
+      const int l = along ? t / DM : t % DL, m = m0 + (along ? t % DM : t / DL);
+      ra[u] = l < nlive && m < M ? in[FWD ? line_off(A, S, l, m) : spec[l] + m] : (T)0;
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int t = threadIdx.x + u * 256, m = m0 + t / DK, o = o0 + t % DK;
+      rb[u] = m < M && o < M ? mat[(long long)m * M + o] : (T)0;
+    }
+  };
+  fetch(0);
+  for (int m0 = 0; m0 < M; m0 += DM) {
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int t = threadIdx.x + u * 256;
+      if (along) as[t % DM][t / DM] = ra[u];
+      else as[t / DL][t % DL] = ra[u];
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int t = threadIdx.x + u * 256;
+      bs[t / DK][t % DK] = rb[u];
+    }
+    __syncthreads();
+    if (m0 + DM < M) fetch(m0 + DM);
+#pragma unroll
+    for (int k = 0; k < DM; ++k) {
+      T a[RL], b[RO];
+#pragma unroll
+      for (int i = 0; i < RL; ++i) a[i] = as[k][tx + 16 * i];
+#pragma unroll
+      for (int j = 0; j < RO; ++j) b[j] = bs[k][RO * ty + j];
+#pragma unroll
+      for (int i = 0; i < RL; ++i)
+#pragma unroll
+        for (int j = 0; j < RO; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < RL; ++i) {
+    const int l = tx + 16 * i;
+    if (l >= nlive) continue;
+#pragma unroll
+    for (int j = 0; j < RO; ++j) {
+      const int o = o0 + RO * ty + j;
+      if (o < M) out[FWD ? spec[l] + o : line_off(A, S, l, o)] = acc[i][j];
+    }
+  }
+}
+
 // FP32: KG systems x P segments of TRI_R rows per CTA, the rows in registers: the field is read and
 // written once (a sequential sweep per system would write and re-read both factors).
 constexpr int TRI_R = 16;
@@ -565,6 +661,15 @@ int line_columns(const DirectArgs<T>& A) {
 
 template <typename T>
 cudaError_t lines_t(snac_plan* P, const DirectArgs<T>& A, bool fwd, const T* in, T* out, cudaStream_t s) {
+  if (A.cls == LINES_DENSE) {
+    const double cells = (double)A.nq * A.M * A.N;
+    LaunchScope ls(P, fwd ? K_LINES_FWD : K_LINES_BWD, 2.0 * sizeof(T) * cells, 2.0 * A.M * cells, s);
+    const dim3 g((unsigned)(((long long)A.nq * A.N + DenseTile<T>::DL - 1) / DenseTile<T>::DL),
+                 (unsigned)((A.M + DenseTile<T>::DK - 1) / DenseTile<T>::DK));
+    if (fwd) k_dense<T, true><<<g, 256, 0, s>>>(A, in, out);
+    else k_dense<T, false><<<g, 256, 0, s>>>(A, in, out);
+    return cudaGetLastError();
+  }
   const int lc = line_columns(A), lines = A.cls == LINES_PAIR ? 2 << lc : 1 << lc;
   const unsigned grid = (unsigned)(((long long)A.nq * A.N + lines - 1) / lines);
   const size_t smem = line_smem(A.F, lc, sizeof(T));
@@ -588,7 +693,7 @@ cudaError_t tri_t(snac_plan* P, const DirectTab& D, const DirectArgs<T>& A, cons
     const int lsegs = (A.N + LOW_R - 1) / LOW_R;
     if (D.nlow)
       k_tri_low<false><<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
-          (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / (2.0 * A.M), D.d_lowlist,
+          (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / D.theta, D.d_lowlist,
           D.nlow, A.M, A.N, lsegs, A.ncell, A.soff, alpha, u, nullptr, 0, -1, -1);
     if (D.d_fac)
       k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u);
@@ -624,7 +729,7 @@ cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
         const int lsegs = (d.N + LOW_R - 1) / LOW_R;
         if (d.nlow)
           k_tri_low<true><<<(d.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
-              (const TriRow<double>*)d.d_tri64, d.d_lam64, P->d_sigma64, d.cscale, d.cscale / (2.0 * d.M), d.d_lowlist,
+              (const TriRow<double>*)d.d_tri64, d.d_lam64, P->d_sigma64, d.cscale, d.cscale / d.theta, d.d_lowlist,
               d.nlow, d.M, d.N, lsegs, A[p].ncell, A[p].soff, nullptr, u, (T*)D.it.d_ends, D.it.E, A[p].e0, A[p].e1);
       }
       k_tri_ends<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A[p], D.d_qrow, d.d_low, (const T*)d.d_fac, u,

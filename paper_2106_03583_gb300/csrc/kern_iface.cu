@@ -211,7 +211,7 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
     const TriRow<double>* tri = (const TriRow<double>*)(f64 ? d.d_tri : (void*)d.d_tri64);
     const double* lam = f64 ? (const double*)d.d_lam : d.d_lam64;
     const long long sys = (long long)P->nz * d.M;
-    k_resp<<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(tri, lam, P->d_sigma64, d.cscale, d.cscale / (2.0 * d.M), P->nz,
+    k_resp<<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(tri, lam, P->d_sigma64, d.cscale, d.cscale / d.theta, P->nz,
                                                         d.M, d.N, resp[p]);
     e = cudaGetLastError();
   }

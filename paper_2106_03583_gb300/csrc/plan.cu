@@ -807,13 +807,6 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     for (int l = 0; l < P->nz; ++l) sm[l] = (P->singular && mode_lambda(P->kind, P->nzt, P->q0 + l) == 0.0) ? 1 : 0;
     if ((st = upload(P, &P->d_singular_mode, sm))) break;
     if ((st = build_coarse(P))) break;
-    {
-      std::vector<FaceKinds> faces(hb.size());
-      for (size_t b = 0; b < hb.size(); ++b)
-        for (int a = 0; a < 2; ++a)
-          for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
-      if ((st = build_direct(P, faces))) break;
-    }
     // the bottom of the cycle in one launch: from the first level below 0 whose planes, with all
     // coarser ones, fit in one CTA's shared memory (at least one smoothed level above the coarsest)
     // and whose plane has at most bottom_cells cells
@@ -834,8 +827,15 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
       const int L = (int)P->lev.size() - 1;
       P->onchip = P->onchip_opt == 0 && P->nu1 >= 1 && P->nu2 >= 1 && L >= 1 && L < BOTTOM_MAX_LEVELS &&
                   P->lev[0].ncell <= BOTTOM_MAX_CELLS && bottom_layout(P, 0, inner).bytes <= (size_t)BOTTOM_MAX_SMEM;
-      if (P->onchip && P->direct.on && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) P->direct.on = false;
     }
+    {
+      std::vector<FaceKinds> faces(hb.size());
+      for (size_t b = 0; b < hb.size(); ++b)
+        for (int a = 0; a < 2; ++a)
+          for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
+      if ((st = build_direct(P, faces))) break;
+    }
+    if (P->onchip && P->direct.on && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) P->direct.on = false;
     // the automatic inner reduction: an on-chip plan's V-cycles are cheap next to an outer step,
     // so it asks more of each step (measured on c64: 3 outer steps at 1e-4, 2 at 3e-5, 18 % faster)
     if (P->inner_reduction == 0.0) P->inner_reduction = P->onchip ? 3e-5 : 1e-4;

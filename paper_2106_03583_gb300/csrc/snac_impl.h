@@ -172,12 +172,15 @@ struct FftTab {
 // Tables in the plan's inner type.
 struct DirectTab {
   int M = 0, N = 0;        // cells along the transformed / the tridiagonal axis
-  int cls = 0, kind = 0;   // LINES_PAIR / LINES_DCT4; boundary pair of the transformed axis
+  int cls = 0, kind = 0;   // LINES_PAIR / LINES_DCT4 / LINES_DENSE; boundary pair of the transformed axis
   int xl = 0, vec = 0, nbm = 1;
   int soff = 0;            // first spectral element within a plane (the pieces' spectra follow each other)
   FftTab fft{};
   int w2n = 0, t4a = 0, t4b = 0;  // offsets in the twiddle table
   double cscale = 1.0;
+  double theta = 1.0;      // inverse times forward transform
+  void* d_F = nullptr;     // LINES_DENSE: [m][kappa] and [kappa][m] matrices of the transform and its inverse
+  void* d_B = nullptr;
   bool singular = false;   // all-Neumann / periodic: a zero shift makes slot 0's system singular
   void* d_fac = nullptr;             // plans not on chip: reciprocal pivots (k_tri_pre), inner type
   int nlow = 0;                      // mixed plans: systems solved in FP64 arithmetic (k_tri_low)
@@ -194,7 +197,7 @@ struct DirectTab {
   int* d_mblk = nullptr;
   int* d_mstr = nullptr;
   // host copies the interface setup needs
-  std::vector<double> w, lam;
+  std::vector<double> w, lam, F, B;  // F[kappa M + m], B[m M + kappa] (LINES_DENSE)
 };
 
 // The interfaces between the pieces of a plan (kern_iface.cu).

@@ -75,6 +75,12 @@ DIRECT = [
     ("L", 160, 256, 0.0, 0.0, "NNNN", "PP", (False, False)),
     ("O", 192, 192, 0.0, 0.0, "DNNN", "ND", (False, False)),
     ("T", 192, 320, 1.0, 0.0, "NNNN", "NN", (False, False)),    # y lines, singular
+    # dense transforms: axes clustered both ways, or a length with a prime factor 11
+    ("1", 160, 96, 1.3, 1.5, "DNNN", "DN", (False, False)),
+    ("2x2", 96, 160, 1.0, 1.0, "NNNN", "NN", (False, False)),   # singular, x lines
+    ("1", 88, 96, 0.0, 1.2, "NNDN", "DD", (False, False)),
+    ("L", 160, 128, 1.0, 1.0, "DDNN", "NN", (False, False)),
+    ("T", 240, 128, 1.0, 1.0, "NNNN", "PP", (False, False)),    # singular
 ]
 
 
@@ -83,7 +89,7 @@ def _passes(pl):
     return st["lines_forward"]["launches"] + st["onchip"]["launches"], st
 
 
-def _check_modes(blocks, precision, shift=0.0, modes=None):
+def _check_modes(blocks, precision, shift=0.0, modes=None, dense=False):
     import torch
     g = ogrid.Grid(blocks, shift=shift)
     pl = plan(blocks, precision=precision, shift=shift, modes=modes)
@@ -106,6 +112,7 @@ def _check_modes(blocks, precision, shift=0.0, modes=None):
     # (several pieces: the dense interface systems add sums of up to nmax terms, 1/2 u sqrt(nmax) each way, and the
     # solution is formed twice)
     pieces = len(np.unique(g.plane.gx)) * len(np.unique(g.plane.gy)) != g.plane.n
+    pieces = pieces or dense   # (the same for dense transforms: sums of nmax terms twice)
     c = 16 * eps * (np.log2(nmax) + 4) * (1 + (2 + 0.25 * np.sqrt(nmax)) * pieces)
     for k in range(q1 - q0):
         r = F[k] - (g.plane.A @ U[k] + lam[k] * U[k])
@@ -120,7 +127,7 @@ def _check_modes(blocks, precision, shift=0.0, modes=None):
 @pytest.mark.parametrize("case", DIRECT, ids=lambda c: "-".join(map(str, c[:6])))
 def test_direct_mode_solve(case, precision):
     layout, nx, ny, xf, yf, walls, zp, per = case
-    _check_modes(build(layout, nx, ny, xf, yf, walls, zp, per=per), precision)
+    _check_modes(build(layout, nx, ny, xf, yf, walls, zp, per=per), precision, dense=(xf > 0 and yf > 0) or nx % 11 == 0)
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
