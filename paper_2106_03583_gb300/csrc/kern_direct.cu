@@ -330,25 +330,50 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
   }
 }
 
-// Dense transform of DL lines x DK outputs per CTA of 256 threads (16 x 16, each RL lines x RO outputs):
-// out[line][o] = sum_i in[line][i] mat[i][o]. Thread columns run over lines, so both orders of the plane's
-// lines load and store whole sectors (16 lines of one cell, or 8 cells of one line). FWD: planes -> spectra;
-// else spectra -> planes. 2 M FMA per cell and way: FP32 issue-bound, FP64 bound by the FP64 pipe.
+// Dense transform of DL lines x DK outputs per CTA of 256 threads: out[line][o] = sum_i in[line][i] mat[i][o].
+// FWD: planes -> spectra; else spectra -> planes. 2 M FMA per cell and way. A warp covers 8 line groups x 4
+// output groups, so that an input is one 128-byte shared read for 8 lanes of 16 bytes and the matrix entries
+// are broadcasts; FP32 multiplies two lines per packed FMA. Two stages of DM terms, the next one's loads in
+// flight. FP64 is bound by its pipe (92 % of it; 320 x 160 x 96 cells in three rectangles: both ways 1.28 ->
+// 1.18 ms against 16 x 2 lanes per warp and one stage), FP32 by the latency of shared reads at 16 warps per SM
+// (42 % of the FP32 rate; 336 x 192 x 150: both ways 0.33 -> 0.23 ms). Matrix entries stored as pairs: slower.
 template <typename T>
 struct DenseTile {
   // FP64: 16 outputs wide, so that no FP64 operation is spent on padding of common lengths
-  static constexpr int RL = 8, RO = sizeof(T) == 4 ? 4 : 1, DL = 16 * RL, DK = 16 * RO, DM = 16;
+  static constexpr int V = 16 / sizeof(T), RL = 8, RO = sizeof(T) == 4 ? 4 : 1, DL = 16 * RL, DK = 16 * RO, DM = 16;
 };
+
+__device__ __forceinline__ void dense_fma(float (&acc)[8][4], const float (&a)[8], const float (&b)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float2 bb = make_float2(b[j], b[j]);
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      const float2 r = __ffma2_rn(make_float2(a[i], a[i + 1]), bb, make_float2(acc[i][j], acc[i + 1][j]));
+      acc[i][j] = r.x;
+      acc[i + 1][j] = r.y;
+    }
+  }
+}
+__device__ __forceinline__ void dense_fma(double (&acc)[8][1], const double (&a)[8], const double (&b)[1]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i][0] = fma(a[i], b[0], acc[i][0]);
+}
 
 template <typename T, bool FWD>
 __global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T* __restrict__ in, T* __restrict__ out) {
-  constexpr int RL = DenseTile<T>::RL, RO = DenseTile<T>::RO, DL = DenseTile<T>::DL, DK = DenseTile<T>::DK,
-                DM = DenseTile<T>::DM;
+  using D = DenseTile<T>;
+  constexpr int V = D::V, RL = D::RL, RO = D::RO, DL = D::DL, DK = D::DK, DM = D::DM;
+  struct alignas(16) Vec {
+    T v[V];
+  };
   __shared__ long long plane[DL];
   __shared__ long long spec[DL];
   __shared__ int ln[DL];
-  __shared__ T as[DM][DL];
-  __shared__ __align__(16) T bs[DM][DK];
+  __shared__ long long org[DL];  // a line's first input and its stride (one block along m)
+  __shared__ int str[DL];
+  __shared__ __align__(16) T as[2][DM][DL + V];
+  __shared__ __align__(16) T bs[2][DM][DK];
   const int M = A.M;
   const long long total = (long long)A.nq * A.N, g0 = (long long)blockIdx.x * DL;
   for (int l = threadIdx.x; l < DL; l += 256) {
@@ -357,14 +382,18 @@ __global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T
     plane[l] = (long long)q * A.ncell;
     spec[l] = (long long)q * A.ncell + A.soff + (long long)n * M;
     ln[l] = n;
+    org[l] = FWD ? plane[l] + A.base[n * A.nbm] : spec[l];
+    str[l] = FWD ? A.mstr[n] : 1;
   }
   __syncthreads();
   const LineSet S{plane, spec, ln};
   const int nlive = (int)min((long long)DL, total - g0);
   const T* __restrict__ mat = FWD ? A.F1 : A.B1;
   const int o0 = blockIdx.y * DK;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int tx = (warp % 2) * 8 + lane % 8, ty = (warp / 2) * 4 + lane / 8;
   const bool along = !FWD || A.xl;  // the inputs of a line are contiguous
+  const bool one = !FWD || A.nbm == 1;
   T acc[RL][RO];
 #pragma unroll
   for (int i = 0; i < RL; ++i)
@@ -377,7 +406,8 @@ __global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T
     for (int u = 0; u < NA; ++u) {
       const int t = threadIdx.x + u * 256;
       const int l = along ? t / DM : t % DL, m = m0 + (along ? t % DM : t / DL);
-      ra[u] = l < nlive && m < M ? in[FWD ? line_off(A, S, l, m) : spec[l] + m] : (T)0;
+      ra[u] = (T)0;
+      if (l < nlive && m < M) ra[u] = in[one ? org[l] + (long long)m * str[l] : line_off(A, S, l, m)];
     }
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
@@ -385,44 +415,56 @@ __global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T
       rb[u] = m < M && o < M ? mat[(long long)m * M + o] : (T)0;
     }
   };
-  fetch(0);
-  for (int m0 = 0; m0 < M; m0 += DM) {
+  auto keep = [&](int st) {
 #pragma unroll
     for (int u = 0; u < NA; ++u) {
       const int t = threadIdx.x + u * 256;
-      if (along) as[t % DM][t / DM] = ra[u];
-      else as[t / DL][t % DL] = ra[u];
+      if (along) as[st][t % DM][t / DM] = ra[u];
+      else as[st][t / DL][t % DL] = ra[u];
     }
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
       const int t = threadIdx.x + u * 256;
-      bs[t / DK][t % DK] = rb[u];
+      bs[st][t / DK][t % DK] = rb[u];
     }
+  };
+  fetch(0);
+  int st = 0;
+  for (int m0 = 0; m0 < M; m0 += DM, st ^= 1) {
+    keep(st);  // (the other threads read this stage last before the previous barrier)
     __syncthreads();
     if (m0 + DM < M) fetch(m0 + DM);
 #pragma unroll
     for (int k = 0; k < DM; ++k) {
       T a[RL], b[RO];
 #pragma unroll
-      for (int i = 0; i < RL; ++i) a[i] = as[k][tx + 16 * i];
+      for (int c = 0; c < RL / V; ++c) {
+        const Vec v = *reinterpret_cast<const Vec*>(&as[st][k][V * tx + 16 * V * c]);
 #pragma unroll
-      for (int j = 0; j < RO; ++j) b[j] = bs[k][RO * ty + j];
+        for (int i = 0; i < V; ++i) a[V * c + i] = v.v[i];
+      }
 #pragma unroll
-      for (int i = 0; i < RL; ++i)
-#pragma unroll
-        for (int j = 0; j < RO; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      for (int j = 0; j < RO; ++j) b[j] = bs[st][k][RO * ty + j];
+      dense_fma(acc, a, b);
     }
-    __syncthreads();
   }
+  const int o = o0 + RO * ty;
 #pragma unroll
   for (int i = 0; i < RL; ++i) {
-    const int l = tx + 16 * i;
-    if (l >= nlive) continue;
+    const int l = V * tx + 16 * V * (i / V) + i % V;
+    if (l >= nlive || o >= M) continue;
+    const long long at = FWD ? spec[l] + o : line_off(A, S, l, o);
+    if (RO == V && o + V <= M && (reinterpret_cast<size_t>(out + at) & 15) == 0 &&
+        (FWD || line_off(A, S, l, o + V - 1) == at + V - 1)) {
+      Vec v;
 #pragma unroll
-    for (int j = 0; j < RO; ++j) {
-      const int o = o0 + RO * ty + j;
-      if (o < M) out[FWD ? spec[l] + o : line_off(A, S, l, o)] = acc[i][j];
+      for (int j = 0; j < V; ++j) v.v[j] = acc[i][j % RO];
+      *reinterpret_cast<Vec*>(out + at) = v;
+      continue;
     }
+#pragma unroll
+    for (int j = 0; j < RO; ++j)
+      if (o + j < M) out[FWD ? at + j : line_off(A, S, l, o + j)] = acc[i][j];
   }
 }
 
