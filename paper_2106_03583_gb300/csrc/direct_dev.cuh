@@ -73,7 +73,7 @@ struct DirectArgs {
   const int* base;
   const int* mblk;
   const int* mstr;
-  int nbm, xl, vec;        // xl: the transformed axis is the contiguous one; vec: pairs may be loaded as vectors
+  int nbm, m1, xl, vec;    // m1: first m of the second block; xl: the transformed axis is the contiguous one; vec: pairs may be loaded as vectors
 };
 
 template <typename T>
@@ -109,6 +109,7 @@ inline DirectArgs<T> direct_args(const snac_plan* P, const DirectTab& D) {
   A.mblk = D.d_mblk;
   A.mstr = D.d_mstr;
   A.nbm = D.nbm;
+  A.m1 = D.m1;
   A.xl = D.xl;
   A.vec = D.vec;
   return A;
@@ -398,14 +399,14 @@ inline PlaneArgs<T> plane_args(const snac_plan* P) {
 // Planes to spectra of one piece in its buffer (complete on entry, behind a barrier on return).
 template <typename T>
 __device__ void piece_forward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T>* buf, int nt) {
-  const ColsAny cm{S.cols, S.rp};
-  const int M = A.M, kind = A.kind, l1 = A.F.l1;
+  const ColsAny cm{S.cols, S.rp, recip16(S.cols)};
+  const int M = A.M, kind = A.kind;
   const bool pair = A.cls == LINES_PAIR;
   if (!pair) {
     for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
       int j, c;
       cm.split(t, j, c);
-      const int o = fft_row(j, l1, S.s1, S.rp) + c;
+      const int o = fft_row(j, A.F, S.s1, S.rp) + c;
       buf[o] = cx_mul(buf[o], A.t4a[j]);
     }
     __syncthreads();
@@ -415,8 +416,8 @@ __device__ void piece_forward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T
     for (int t = threadIdx.x; t < (M / 2 + 1) * S.cols; t += nt) {
       int k, c;
       cm.split(t, k, c);
-      const int o1 = fft_row(A.perm[k], l1, S.s1, S.rp) + c;
-      const int o2 = k == 0 ? o1 : fft_row(A.perm[M - k], l1, S.s1, S.rp) + c;
+      const int o1 = fft_row(A.perm[k], A.F, S.s1, S.rp) + c;
+      const int o2 = k == 0 ? o1 : fft_row(A.perm[M - k], A.F, S.s1, S.rp) + c;
       Cpl<T> y1, y2;
       pair_post(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], buf[o1], buf[o2], y1, y2);
       if (o2 != o1) buf[o2] = y2;
@@ -426,7 +427,7 @@ __device__ void piece_forward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T
     for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
       int k, c;
       cm.split(t, k, c);
-      const int o = fft_row(A.perm[k], l1, S.s1, S.rp) + c;
+      const int o = fft_row(A.perm[k], A.F, S.s1, S.rp) + c;
       const Cpl<T> v = cx_mul(buf[o], A.t4b[k]);
       buf[o] = Cpl<T>{(T)2 * v.re, (T)-2 * v.im};
     }
@@ -437,8 +438,8 @@ __device__ void piece_forward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T
 // Where slot kappa of a piece stands in its buffer: element o + n ns for row n.
 template <typename T>
 __device__ __forceinline__ int slot_at(const DirectArgs<T>& A, const PlaneShape& S, int kap) {
-  if (A.cls == LINES_PAIR) return 2 * fft_row(A.perm[kap], A.F.l1, S.s1, S.rp);
-  return 2 * fft_row(A.perm[(kap & 1) ? (A.M - 1 - kap) >> 1 : kap >> 1], A.F.l1, S.s1, S.rp) + (kap & 1);
+  if (A.cls == LINES_PAIR) return 2 * fft_row(A.perm[kap], A.F, S.s1, S.rp);
+  return 2 * fft_row(A.perm[(kap & 1) ? (A.M - 1 - kap) >> 1 : kap >> 1], A.F, S.s1, S.rp) + (kap & 1);
 }
 
 // The tridiagonal systems of one piece; ENDS: only the first and last rows' solutions, into the end vector.
@@ -446,7 +447,7 @@ template <typename T, bool ENDS>
 __device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T sg, T alpha, T* ex, double* ends, int nt) {
   const int N = A.N, M = A.M;
   const int P = (N + PLANE_R - 1) / PLANE_R, kg = nt / P;
-  const int seg = quot16(threadIdx.x, kg), kk = threadIdx.x - seg * kg;
+  const int seg = (int)threadIdx.x / kg, kk = threadIdx.x - seg * kg;
   const bool mine = seg < P;
   const int ns = A.cls == LINES_PAIR ? 1 : 2;
   for (int k0 = 0; k0 < M; k0 += kg) {
@@ -475,15 +476,15 @@ __device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T 
 // Spectra back to planes of one piece.
 template <typename T>
 __device__ void piece_backward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<T>* buf, int nt) {
-  const ColsAny cm{S.cols, S.rp};
-  const int M = A.M, kind = A.kind, l1 = A.F.l1;
+  const ColsAny cm{S.cols, S.rp, recip16(S.cols)};
+  const int M = A.M, kind = A.kind;
   const bool pair = A.cls == LINES_PAIR;
   if (pair) {
     for (int t = threadIdx.x; t < (M / 2 + 1) * S.cols; t += nt) {
       int k, c;
       cm.split(t, k, c);
-      const int o1 = fft_row(A.perm[k], l1, S.s1, S.rp) + c;
-      const int o2 = k == 0 ? o1 : fft_row(A.perm[M - k], l1, S.s1, S.rp) + c;
+      const int o1 = fft_row(A.perm[k], A.F, S.s1, S.rp) + c;
+      const int o2 = k == 0 ? o1 : fft_row(A.perm[M - k], A.F, S.s1, S.rp) + c;
       const Cpl<T> x1 = buf[o1];
       const Cpl<T> x2 = k == 0 || (kind == KIND_PP && 2 * k == M) ? Cpl<T>{0, 0} : buf[o2];
       Cpl<T> z1, z2;
@@ -495,7 +496,7 @@ __device__ void piece_backward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<
     for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
       int j, c;
       cm.split(t, j, c);
-      const int o = fft_row(A.perm[j], l1, S.s1, S.rp) + c;
+      const int o = fft_row(A.perm[j], A.F, S.s1, S.rp) + c;
       const Cpl<T> v = cx_mul(buf[o], A.t4a[j]);
       buf[o] = Cpl<T>{v.re, -v.im};  // forward = conj(inverse(conj))
     }
@@ -506,7 +507,7 @@ __device__ void piece_backward(const DirectArgs<T>& A, const PlaneShape& S, Cpl<
     for (int t = threadIdx.x; t < A.F.n * S.cols; t += nt) {
       int k, c;
       cm.split(t, k, c);
-      const int o = fft_row(k, l1, S.s1, S.rp) + c;
+      const int o = fft_row(k, A.F, S.s1, S.rp) + c;
       const Cpl<T> z = buf[o];
       const Cpl<T> y = cx_mul(Cpl<T>{z.re, -z.im}, A.t4b[k]);
       buf[o] = Cpl<T>{(T)2 * y.re, (T)-2 * y.im};
@@ -532,7 +533,7 @@ __device__ void plane_direct(const PlaneArgs<T>& O, T sg, int q, const T* __rest
     const DirectArgs<T>& A = O.pc[p];
     const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
     if (A.cls == LINES_PAIR && (A.N & 1))
-      for (int m = threadIdx.x; m < A.M; m += nt) bt[b0 + 2 * (fft_row(m, A.F.l1, S.s1, S.rp) + S.cols - 1) + 1] = 0;
+      for (int m = threadIdx.x; m < A.M; m += nt) bt[b0 + 2 * (fft_row(m, A.F, S.s1, S.rp) + S.cols - 1) + 1] = 0;
     b0 += S.buf;
   }
   for (int c = threadIdx.x; c < ncell; c += nt) {

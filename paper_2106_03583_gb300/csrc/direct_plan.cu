@@ -35,10 +35,13 @@ bool fft_tab(int n, int max_log2, FftTab& F) {
   if (rad.empty()) rad.push_back(1);
   F.np = n == 1 ? 0 : (int)rad.size();
   F.l1 = n / rad[0];
+  F.l1r = recip16(F.l1);
   int span = n;
   for (int k = 0; k < F.np; ++k) {
     F.rad[k] = rad[k];
     F.span[k] = span;
+    F.lr[k] = recip16(span / rad[k]);
+    F.pr[k] = recip16(std::max(F.l1 / span, 1));
     span /= rad[k];
   }
   return true;
@@ -439,6 +442,7 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   }
   D.vec = vec;
   D.nbm = gm;
+  D.m1 = (int)(std::find(mblk.begin(), mblk.end(), 1) - mblk.begin());
   int st;
   if (!f64) {
     // the systems with the smallest -(lambda + sigma): up to LOW_SPAN times the smallest nonzero one, 1/64 of

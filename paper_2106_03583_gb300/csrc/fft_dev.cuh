@@ -156,15 +156,9 @@ __device__ __forceinline__ void dft_reg(Cpl<T> (&x)[R]) {
   }
 }
 
-// n / d for 0 <= n < 2^16 and 1 <= d < 2^16: an approximate quotient (error below 2^-5), corrected by
-// one step either way.
-__device__ __forceinline__ int quot16(int n, int d) {
-  int q = __float2int_rz(__fdividef((float)n, (float)d));
-  const int r = n - q * d;
-  q += r >= d ? 1 : 0;
-  q -= r < 0 ? 1 : 0;
-  return q;
-}
+// n / d for 0 <= n < 2^16 - 1 and 1 <= d < 2^16 with r = recip16(d) = floor((2^32 - 1) / d): (n + 1) r / 2^32 is
+// less than (n + 1) / d, and by less than 1 / d.
+__device__ __forceinline__ int quot16(int n, unsigned r) { return (int)__umulhi((unsigned)n + 1u, r); }
 
 // The columns of a buffer: item t of a pass is (index t / columns, column t % columns).
 struct ColsShift {  // 2^lc columns
@@ -178,24 +172,24 @@ struct ColsShift {  // 2^lc columns
 };
 struct ColsAny {
   int C, RP;
+  unsigned r;  // recip16(C)
   __device__ __forceinline__ int cols() const { return C; }
   __device__ __forceinline__ int pitch() const { return RP; }
   __device__ __forceinline__ void split(int t, int& idx, int& c) const {
-    idx = quot16(t, C);
+    idx = quot16(t, r);
     c = t - idx * C;
   }
 };
 
 // Row p of the buffer (p a natural index, or perm[k]).
-__device__ __forceinline__ int fft_row(int p, int l1, int s1, int rp) {
-  const int b = quot16(p, l1);
-  return b * s1 + (p - b * l1) * rp;
+__device__ __forceinline__ int fft_row(int p, const FftTab& F, int s1, int rp) {
+  return quot16(p, F.l1r) * (s1 - F.l1 * rp) + p * rp;
 }
 
 template <int R, bool INV, typename T, typename Cols>
-__device__ __forceinline__ void fft_pass(Cpl<T>* __restrict__ buf, const FftTab& F, int span, int s1, const Cols cm,
+__device__ __forceinline__ void fft_pass(Cpl<T>* __restrict__ buf, const FftTab& F, int s, int s1, const Cols cm,
                                          const Cpl<T>* __restrict__ tw, int nt) {
-  const int L = span / R, tws = F.n / span, rp = cm.pitch();
+  const int span = F.span[s], L = span / R, tws = F.n / span, rp = cm.pitch();
   const bool first = span == F.n;
   const int stride = first ? s1 : L * rp;
   const int per = first ? 1 : F.l1 / span;
@@ -205,9 +199,9 @@ __device__ __forceinline__ void fft_pass(Cpl<T>* __restrict__ buf, const FftTab&
     cm.split(t, idx, c);
     int i = idx, o = idx * rp + c;
     if (!first) {
-      const int bb = quot16(idx, L);
+      const int bb = quot16(idx, F.lr[s]);
       i = idx - bb * L;
-      const int sub = quot16(bb, per);
+      const int sub = quot16(bb, F.pr[s]);
       o = sub * s1 + ((bb - sub * per) * span + i) * rp + c;
     }
     Cpl<T> x[R];
@@ -239,17 +233,16 @@ __device__ void fft_all(Cpl<T>* __restrict__ buf, const FftTab& F, int s1, const
                         int nt) {
   for (int k = 0; k < F.np; ++k) {
     const int s = INV ? F.np - 1 - k : k;
-    const int span = F.span[s];
     switch (F.rad[s]) {
       case 16:
-        if constexpr (sizeof(T) == 4) fft_pass<16, INV>(buf, F, span, s1, cm, tw, nt);
+        if constexpr (sizeof(T) == 4) fft_pass<16, INV>(buf, F, s, s1, cm, tw, nt);
         break;
-      case 8: fft_pass<8, INV>(buf, F, span, s1, cm, tw, nt); break;
-      case 4: fft_pass<4, INV>(buf, F, span, s1, cm, tw, nt); break;
-      case 2: fft_pass<2, INV>(buf, F, span, s1, cm, tw, nt); break;
-      case 3: fft_pass<3, INV>(buf, F, span, s1, cm, tw, nt); break;
-      case 5: fft_pass<5, INV>(buf, F, span, s1, cm, tw, nt); break;
-      default: fft_pass<7, INV>(buf, F, span, s1, cm, tw, nt); break;
+      case 8: fft_pass<8, INV>(buf, F, s, s1, cm, tw, nt); break;
+      case 4: fft_pass<4, INV>(buf, F, s, s1, cm, tw, nt); break;
+      case 2: fft_pass<2, INV>(buf, F, s, s1, cm, tw, nt); break;
+      case 3: fft_pass<3, INV>(buf, F, s, s1, cm, tw, nt); break;
+      case 5: fft_pass<5, INV>(buf, F, s, s1, cm, tw, nt); break;
+      default: fft_pass<7, INV>(buf, F, s, s1, cm, tw, nt); break;
     }
   }
 }

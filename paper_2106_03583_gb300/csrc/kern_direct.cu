@@ -31,7 +31,6 @@ struct ColsLine : ColsShift {
     c = ((hi & ((1 << ch) - 1)) << cl) | lo;
     idx = ((hi >> ch) << 3) | kk;
   }
-  __device__ __forceinline__ int total8(int rows) const { return ((rows + 7) & ~7) << lc; }
 };
 
 // Lines of one CTA: global line number g = q N + n; per line the plane base of q, its spectrum and n.
@@ -47,6 +46,23 @@ __device__ __forceinline__ long long line_off(const DirectArgs<T>& A, const Line
   const int b = A.nbm == 1 ? 0 : A.mblk[m];
   return S.plane[l] + A.base[n * A.nbm + b] + (long long)m * A.mstr[n];
 }
+
+// A line's place in the plane, kept by the thread that walks it: at(m) is the offset of cell m. Up to two
+// blocks along m cost a selection; more take line_off.
+template <typename T>
+struct LineAt {
+  long long o0, o1;
+  int l;
+  bool live;
+  __device__ __forceinline__ LineAt(const DirectArgs<T>& A, const LineSet& S, int l_, int nlive) : l(l_), live(l_ < nlive) {
+    const int n = live ? S.n[l] : 0;
+    o0 = live ? S.plane[l] + A.base[n * A.nbm] : 0;
+    o1 = live && A.nbm == 2 ? S.plane[l] + A.base[n * 2 + 1] : o0;
+  }
+  __device__ __forceinline__ long long at(const DirectArgs<T>& A, const LineSet& S, int str, int m) const {
+    return A.nbm > 2 ? line_off(A, S, l, m) : (m < A.m1 ? o0 : o1) + (long long)m * str;
+  }
+};
 
 template <typename T>
 __device__ __forceinline__ int line_setup(const DirectArgs<T>& A, int lines, long long* plane, long long* spec, int* ln) {
@@ -66,6 +82,10 @@ __device__ __forceinline__ int line_setup(const DirectArgs<T>& A, int lines, lon
 constexpr int MAX_LINES = 64;
 constexpr int LB = 4;  // loads of a batch in flight per thread
 
+// Every thread keeps its column through all loops (LNT is a multiple of the threads of one index), so the line
+// pointers are made once and an item costs no division. Bound by: FP64, its pipe (85 %, 512 x 512 x 256 cells 2.05 ms
+// a launch); FP32, instruction issue and the latency of the passes (81 instructions per cell, down from 104: 0.25
+// -> 0.21 ms, 2.6 TB/s).
 template <typename T>
 __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const DirectArgs<T> A, int lc, const T* __restrict__ in,
                                                                          T* __restrict__ out) {
@@ -76,124 +96,123 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_fwd(const
   Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
   T* bt = reinterpret_cast<T*>(smem);
   const ColsLine cm{{lc}};
-  const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
+  const int C = 1 << lc, M = A.M, kind = A.kind, s1 = line_s1(A.F, lc);
   const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
   const int lines = pair ? 2 * C : C;
   const int g0 = line_setup(A, lines, plane, spec, ln);
   const LineSet S{plane, spec, ln};
   const int nlive = min(lines, A.nq * A.N - g0);
+  // LNT is a multiple of a column group's threads: a thread keeps its column(s) and walks the indices
+  const int is = LNT >> lc;
   if (pair) {
+    int i0, c;
+    if (A.xl) cm.split8(threadIdx.x, i0, c);
+    else cm.split(threadIdx.x, i0, c);
+    const LineAt<T> pa(A, S, 2 * c, nlive), pb(A, S, 2 * c + 1, nlive);
     if (A.xl) {  // items: two consecutive cells of both lines of a column
-      const int total = cm.total8(M / 2);
-      for (int t0 = threadIdx.x; t0 < total; t0 += LB * LNT) {
+      for (int h0 = i0; 2 * h0 < M; h0 += LB * is) {
         Cpl<T> a[LB], b[LB];
 #pragma unroll
         for (int u = 0; u < LB; ++u) {
-          int h, c;
-          cm.split8(t0 + u * LNT, h, c);
+          const int m = 2 * (h0 + u * is);
           a[u] = b[u] = Cpl<T>{0, 0};
-          if (t0 + u * LNT < total && 2 * h < M) {
-            const int m = 2 * h;
+          if (m < M) {
             if (A.vec) {
-              if (2 * c < nlive) a[u] = *reinterpret_cast<const Cpl<T>*>(in + line_off(A, S, 2 * c, m));
-              if (2 * c + 1 < nlive) b[u] = *reinterpret_cast<const Cpl<T>*>(in + line_off(A, S, 2 * c + 1, m));
+              if (pa.live) a[u] = *reinterpret_cast<const Cpl<T>*>(in + pa.at(A, S, 1, m));
+              if (pb.live) b[u] = *reinterpret_cast<const Cpl<T>*>(in + pb.at(A, S, 1, m));
             } else {
-              if (2 * c < nlive) a[u] = Cpl<T>{in[line_off(A, S, 2 * c, m)], in[line_off(A, S, 2 * c, m + 1)]};
-              if (2 * c + 1 < nlive) b[u] = Cpl<T>{in[line_off(A, S, 2 * c + 1, m)], in[line_off(A, S, 2 * c + 1, m + 1)]};
+              if (pa.live) a[u] = Cpl<T>{in[pa.at(A, S, 1, m)], in[pa.at(A, S, 1, m + 1)]};
+              if (pb.live) b[u] = Cpl<T>{in[pb.at(A, S, 1, m)], in[pb.at(A, S, 1, m + 1)]};
             }
           }
         }
 #pragma unroll
         for (int u = 0; u < LB; ++u) {
-          int h, c;
-          cm.split8(t0 + u * LNT, h, c);
-          if (t0 + u * LNT >= total || 2 * h >= M) continue;
+          const int m = 2 * (h0 + u * is);
+          if (m >= M) continue;
           a[u].im = neg_if(flip, a[u].im), b[u].im = neg_if(flip, b[u].im);
-          buf[fft_row(pair_pos(kind, 2 * h, M), l1, s1, C) + c] = Cpl<T>{a[u].re, b[u].re};
-          buf[fft_row(pair_pos(kind, 2 * h + 1, M), l1, s1, C) + c] = Cpl<T>{a[u].im, b[u].im};
+          buf[fft_row(pair_pos(kind, m, M), A.F, s1, C) + c] = Cpl<T>{a[u].re, b[u].re};
+          buf[fft_row(pair_pos(kind, m + 1, M), A.F, s1, C) + c] = Cpl<T>{a[u].im, b[u].im};
         }
       }
     } else {  // the lines are adjacent in memory: one element of both lines of a column
-      const int total = M << lc;
-      for (int t0 = threadIdx.x; t0 < total; t0 += 2 * LB * LNT) {
+      const int str = A.mstr[S.n[2 * c]], strb = A.mstr[S.n[2 * c + 1]];
+      for (int m0 = i0; m0 < M; m0 += 2 * LB * is) {
         Cpl<T> v[2 * LB];
 #pragma unroll
         for (int u = 0; u < 2 * LB; ++u) {
-          int m, c;
-          cm.split(t0 + u * LNT, m, c);
+          const int m = m0 + u * is;
           v[u] = Cpl<T>{0, 0};
-          if (t0 + u * LNT < total) {
+          if (m < M) {
             if (A.vec) {
-              if (2 * c < nlive) v[u] = *reinterpret_cast<const Cpl<T>*>(in + line_off(A, S, 2 * c, m));
+              if (pa.live) v[u] = *reinterpret_cast<const Cpl<T>*>(in + pa.at(A, S, str, m));
             } else {
-              if (2 * c < nlive) v[u].re = in[line_off(A, S, 2 * c, m)];
-              if (2 * c + 1 < nlive) v[u].im = in[line_off(A, S, 2 * c + 1, m)];
+              if (pa.live) v[u].re = in[pa.at(A, S, str, m)];
+              if (pb.live) v[u].im = in[pb.at(A, S, strb, m)];
             }
           }
         }
 #pragma unroll
         for (int u = 0; u < 2 * LB; ++u) {
-          int m, c;
-          cm.split(t0 + u * LNT, m, c);
-          if (t0 + u * LNT >= total) continue;
+          const int m = m0 + u * is;
+          if (m >= M) continue;
           v[u] = Cpl<T>{neg_if(flip && (m & 1), v[u].re), neg_if(flip && (m & 1), v[u].im)};
-          buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c] = v[u];
+          buf[fft_row(pair_pos(kind, m, M), A.F, s1, C) + c] = v[u];
         }
       }
     }
   } else {
     // t_j and t_j' (j' = M/2 - 1 - j) from cells 2j, 2j+1, 2j', 2j'+1 of the column's line
-    const int h = M / 2, items = (h + 1) / 2, total = A.xl ? cm.total8(items) : items << lc;
-    for (int t = threadIdx.x; t < total; t += LNT) {
-      int j, c;
-      if (A.xl) cm.split8(t, j, c);
-      else cm.split(t, j, c);
-      if (j >= items) continue;
+    const int h = M / 2, items = (h + 1) / 2;
+    int j0, c;
+    if (A.xl) cm.split8(threadIdx.x, j0, c);
+    else cm.split(threadIdx.x, j0, c);
+    const LineAt<T> pa(A, S, c, nlive);
+    const int str = A.mstr[S.n[c]];
+    for (int j = j0; j < items; j += is) {
       const int jj = h - 1 - j;
       Cpl<T> p{0, 0}, r{0, 0};
       if (c < nlive) {
-        p = Cpl<T>{in[line_off(A, S, c, 2 * j)], in[line_off(A, S, c, 2 * j + 1)]};
-        r = Cpl<T>{in[line_off(A, S, c, 2 * jj)], in[line_off(A, S, c, 2 * jj + 1)]};
+        p = Cpl<T>{in[pa.at(A, S, str, 2 * j)], in[pa.at(A, S, str, 2 * j + 1)]};
+        r = Cpl<T>{in[pa.at(A, S, str, 2 * jj)], in[pa.at(A, S, str, 2 * jj + 1)]};
       }
       p.im = neg_if(flip, p.im), r.im = neg_if(flip, r.im);
-      buf[fft_row(j, l1, s1, C) + c] = cx_mul(Cpl<T>{p.re, r.im}, A.t4a[j]);
-      buf[fft_row(jj, l1, s1, C) + c] = cx_mul(Cpl<T>{r.re, p.im}, A.t4a[jj]);
+      buf[fft_row(j, A.F, s1, C) + c] = cx_mul(Cpl<T>{p.re, r.im}, A.t4a[j]);
+      buf[fft_row(jj, A.F, s1, C) + c] = cx_mul(Cpl<T>{r.re, p.im}, A.t4a[jj]);
     }
   }
   __syncthreads();
   fft_all<false>(buf, A.F, s1, cm, A.tw, LNT);
   if (pair) {
-    const int total = cm.total8(M / 2 + 1);
-    for (int t = threadIdx.x; t < total; t += LNT) {
-      int k, c;
-      cm.split8(t, k, c);
-      if (2 * k > M) continue;
-      const Cpl<T> z1 = buf[fft_row(A.perm[k], l1, s1, C) + c];
-      const Cpl<T> z2 = k == 0 ? z1 : buf[fft_row(A.perm[M - k], l1, s1, C) + c];
+    int k0, c;
+    cm.split8(threadIdx.x, k0, c);
+    const bool la = 2 * c < nlive, lb = 2 * c + 1 < nlive;
+    T* oa = out + (la ? spec[2 * c] : 0);
+    T* ob = out + (lb ? spec[2 * c + 1] : 0);
+    for (int k = k0; 2 * k <= M; k += is) {
+      const Cpl<T> z1 = buf[fft_row(A.perm[k], A.F, s1, C) + c];
+      const Cpl<T> z2 = k == 0 ? z1 : buf[fft_row(A.perm[M - k], A.F, s1, C) + c];
       Cpl<T> y1, y2;
       pair_post(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], z1, z2, y1, y2);
       const bool mirror = k > 0 && 2 * k < M;
-      if (2 * c < nlive) {
-        T* oa = out + spec[2 * c];
+      if (la) {
         oa[k] = y1.re;
         if (mirror) oa[M - k] = y2.re;
       }
-      if (2 * c + 1 < nlive) {
-        T* ob = out + spec[2 * c + 1];
+      if (lb) {
         ob[k] = y1.im;
         if (mirror) ob[M - k] = y2.im;
       }
     }
   } else {
-    const int h = M / 2, items = (h + 1) / 2, total = cm.total8(items);
-    for (int t = threadIdx.x; t < total; t += LNT) {
-      int k, c;
-      cm.split8(t, k, c);
-      if (k >= items || c >= nlive) continue;
+    const int h = M / 2, items = (h + 1) / 2;
+    int k0, c;
+    cm.split8(threadIdx.x, k0, c);
+    T* o = out + (c < nlive ? spec[c] : 0);
+    for (int k = c < nlive ? k0 : items; k < items; k += is) {
       const int kk = h - 1 - k;
-      const Cpl<T> v = cx_mul(buf[fft_row(A.perm[k], l1, s1, C) + c], A.t4b[k]);
-      const Cpl<T> w = cx_mul(buf[fft_row(A.perm[kk], l1, s1, C) + c], A.t4b[kk]);
-      T* o = out + spec[c];
+      const Cpl<T> v = cx_mul(buf[fft_row(A.perm[k], A.F, s1, C) + c], A.t4b[k]);
+      const Cpl<T> w = cx_mul(buf[fft_row(A.perm[kk], A.F, s1, C) + c], A.t4b[kk]);
       o[2 * k] = (T)2 * v.re;
       o[2 * k + 1] = (T)-2 * w.im;
       o[2 * kk] = (T)2 * w.re;
@@ -211,30 +230,32 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
   __shared__ int ln[MAX_LINES];
   Cpl<T>* buf = reinterpret_cast<Cpl<T>*>(smem);
   const ColsLine cm{{lc}};
-  const int C = 1 << lc, M = A.M, kind = A.kind, l1 = A.F.l1, s1 = line_s1(A.F, lc);
+  const int C = 1 << lc, M = A.M, kind = A.kind, s1 = line_s1(A.F, lc);
   const bool flip = flip_kind(kind), pair = A.cls == LINES_PAIR;
   const int lines = pair ? 2 * C : C;
   const int g0 = line_setup(A, lines, plane, spec, ln);
   const LineSet S{plane, spec, ln};
   const int nlive = min(lines, A.nq * A.N - g0);
+  const int is = LNT >> lc;
   if (pair) {
-    const int total = cm.total8(M / 2 + 1);
-    for (int t0 = threadIdx.x; t0 < total; t0 += LB * LNT) {
+    int k0, c;
+    cm.split8(threadIdx.x, k0, c);
+    const bool la = 2 * c < nlive, lb = 2 * c + 1 < nlive;
+    const T* ia = in + (la ? spec[2 * c] : 0);
+    const T* ib = in + (lb ? spec[2 * c + 1] : 0);
+    for (; 2 * k0 <= M; k0 += LB * is) {
       Cpl<T> x1[LB], x2[LB];
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        int k, c;
-        cm.split8(t0 + u * LNT, k, c);
+        const int k = k0 + u * is;
         x1[u] = x2[u] = Cpl<T>{0, 0};
-        if (t0 + u * LNT < total && 2 * k <= M) {
+        if (2 * k <= M) {
           const bool two = k > 0 && !(kind == KIND_PP && 2 * k == M);
-          if (2 * c < nlive) {
-            const T* ia = in + spec[2 * c];
+          if (la) {
             x1[u].re = ia[k];
             if (two) x2[u].re = ia[M - k];
           }
-          if (2 * c + 1 < nlive) {
-            const T* ib = in + spec[2 * c + 1];
+          if (lb) {
             x1[u].im = ib[k];
             if (two) x2[u].im = ib[M - k];
           }
@@ -242,21 +263,19 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
       }
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        int k, c;
-        cm.split8(t0 + u * LNT, k, c);
-        if (t0 + u * LNT >= total || 2 * k > M) continue;
+        const int k = k0 + u * is;
+        if (2 * k > M) continue;
         Cpl<T> z1, z2;
         pair_pre(kind, kind == KIND_PP ? Cpl<T>{1, 0} : A.w2n[k], x1[u], x2[u], z1, z2);
-        buf[fft_row(A.perm[k], l1, s1, C) + c] = z1;
-        if (k > 0 && 2 * k < M) buf[fft_row(A.perm[M - k], l1, s1, C) + c] = z2;
+        buf[fft_row(A.perm[k], A.F, s1, C) + c] = z1;
+        if (k > 0 && 2 * k < M) buf[fft_row(A.perm[M - k], A.F, s1, C) + c] = z2;
       }
     }
   } else {
-    const int h = M / 2, items = (h + 1) / 2, total = cm.total8(items);
-    for (int t = threadIdx.x; t < total; t += LNT) {
-      int j, c;
-      cm.split8(t, j, c);
-      if (j >= items) continue;
+    const int h = M / 2, items = (h + 1) / 2;
+    int j0, c;
+    cm.split8(threadIdx.x, j0, c);
+    for (int j = j0; j < items; j += is) {
       const int jj = h - 1 - j;
       Cpl<T> p{0, 0}, r{0, 0};
       if (c < nlive) {
@@ -265,67 +284,65 @@ __global__ void __launch_bounds__(LNT, sizeof(T) == 4 ? 4 : 3) k_lines_bwd(const
         r = Cpl<T>{i[2 * jj], i[2 * jj + 1]};
       }
       const Cpl<T> v = cx_mul(Cpl<T>{p.re, r.im}, A.t4a[j]), w = cx_mul(Cpl<T>{r.re, p.im}, A.t4a[jj]);
-      buf[fft_row(A.perm[j], l1, s1, C) + c] = Cpl<T>{v.re, -v.im};  // forward = conj(inverse(conj))
-      buf[fft_row(A.perm[jj], l1, s1, C) + c] = Cpl<T>{w.re, -w.im};
+      buf[fft_row(A.perm[j], A.F, s1, C) + c] = Cpl<T>{v.re, -v.im};  // forward = conj(inverse(conj))
+      buf[fft_row(A.perm[jj], A.F, s1, C) + c] = Cpl<T>{w.re, -w.im};
     }
   }
   __syncthreads();
   fft_all<true>(buf, A.F, s1, cm, A.tw, LNT);
   if (pair) {
+    int i0, c;
+    if (A.xl) cm.split8(threadIdx.x, i0, c);
+    else cm.split(threadIdx.x, i0, c);
+    const LineAt<T> pa(A, S, 2 * c, nlive), pb(A, S, 2 * c + 1, nlive);
     if (A.xl) {
-      const int total = cm.total8(M / 2);
-      for (int t = threadIdx.x; t < total; t += LNT) {
-        int h, c;
-        cm.split8(t, h, c);
-        const int m = 2 * h;
-        if (m >= M) continue;
-        const Cpl<T> e = buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c];
-        Cpl<T> o = buf[fft_row(pair_pos(kind, m + 1, M), l1, s1, C) + c];
+      for (int m = 2 * i0; m < M; m += 2 * is) {
+        const Cpl<T> e = buf[fft_row(pair_pos(kind, m, M), A.F, s1, C) + c];
+        Cpl<T> o = buf[fft_row(pair_pos(kind, m + 1, M), A.F, s1, C) + c];
         o = Cpl<T>{neg_if(flip, o.re), neg_if(flip, o.im)};
         if (A.vec) {
-          if (2 * c < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c, m)) = Cpl<T>{e.re, o.re};
-          if (2 * c + 1 < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c + 1, m)) = Cpl<T>{e.im, o.im};
+          if (pa.live) *reinterpret_cast<Cpl<T>*>(out + pa.at(A, S, 1, m)) = Cpl<T>{e.re, o.re};
+          if (pb.live) *reinterpret_cast<Cpl<T>*>(out + pb.at(A, S, 1, m)) = Cpl<T>{e.im, o.im};
         } else {
-          if (2 * c < nlive) {
-            out[line_off(A, S, 2 * c, m)] = e.re;
-            out[line_off(A, S, 2 * c, m + 1)] = o.re;
+          if (pa.live) {
+            out[pa.at(A, S, 1, m)] = e.re;
+            out[pa.at(A, S, 1, m + 1)] = o.re;
           }
-          if (2 * c + 1 < nlive) {
-            out[line_off(A, S, 2 * c + 1, m)] = e.im;
-            out[line_off(A, S, 2 * c + 1, m + 1)] = o.im;
+          if (pb.live) {
+            out[pb.at(A, S, 1, m)] = e.im;
+            out[pb.at(A, S, 1, m + 1)] = o.im;
           }
         }
       }
     } else {
-      const int total = M << lc;
-      for (int t = threadIdx.x; t < total; t += LNT) {
-        int m, c;
-        cm.split(t, m, c);
-        Cpl<T> v = buf[fft_row(pair_pos(kind, m, M), l1, s1, C) + c];
+      const int str = A.mstr[S.n[2 * c]], strb = A.mstr[S.n[2 * c + 1]];
+      for (int m = i0; m < M; m += is) {
+        Cpl<T> v = buf[fft_row(pair_pos(kind, m, M), A.F, s1, C) + c];
         v = Cpl<T>{neg_if(flip && (m & 1), v.re), neg_if(flip && (m & 1), v.im)};
         if (A.vec) {
-          if (2 * c < nlive) *reinterpret_cast<Cpl<T>*>(out + line_off(A, S, 2 * c, m)) = v;
+          if (pa.live) *reinterpret_cast<Cpl<T>*>(out + pa.at(A, S, str, m)) = v;
         } else {
-          if (2 * c < nlive) out[line_off(A, S, 2 * c, m)] = v.re;
-          if (2 * c + 1 < nlive) out[line_off(A, S, 2 * c + 1, m)] = v.im;
+          if (pa.live) out[pa.at(A, S, str, m)] = v.re;
+          if (pb.live) out[pb.at(A, S, strb, m)] = v.im;
         }
       }
     }
   } else {
-    const int h = M / 2, items = (h + 1) / 2, total = A.xl ? cm.total8(items) : items << lc;
-    for (int t = threadIdx.x; t < total; t += LNT) {
-      int k, c;
-      if (A.xl) cm.split8(t, k, c);
-      else cm.split(t, k, c);
-      if (k >= items || c >= nlive) continue;
+    const int h = M / 2, items = (h + 1) / 2;
+    int k0, c;
+    if (A.xl) cm.split8(threadIdx.x, k0, c);
+    else cm.split(threadIdx.x, k0, c);
+    const LineAt<T> pa(A, S, c, nlive);
+    const int str = A.mstr[S.n[c]];
+    for (int k = pa.live ? k0 : items; k < items; k += is) {
       const int kk = h - 1 - k;
-      const Cpl<T> z = buf[fft_row(k, l1, s1, C) + c], y = buf[fft_row(kk, l1, s1, C) + c];
+      const Cpl<T> z = buf[fft_row(k, A.F, s1, C) + c], y = buf[fft_row(kk, A.F, s1, C) + c];
       const Cpl<T> v = cx_mul(Cpl<T>{z.re, -z.im}, A.t4b[k]), w = cx_mul(Cpl<T>{y.re, -y.im}, A.t4b[kk]);
       const T sg = flip ? (T)2 : (T)-2;  // cells 2k + 1 carry -2 Im, sign-flipped for DN
-      out[line_off(A, S, c, 2 * k)] = (T)2 * v.re;
-      out[line_off(A, S, c, 2 * k + 1)] = sg * w.im;
-      out[line_off(A, S, c, 2 * kk)] = (T)2 * w.re;
-      out[line_off(A, S, c, 2 * kk + 1)] = sg * v.im;
+      out[pa.at(A, S, str, 2 * k)] = (T)2 * v.re;
+      out[pa.at(A, S, str, 2 * k + 1)] = sg * w.im;
+      out[pa.at(A, S, str, 2 * kk)] = (T)2 * w.re;
+      out[pa.at(A, S, str, 2 * kk + 1)] = sg * v.im;
     }
   }
 }

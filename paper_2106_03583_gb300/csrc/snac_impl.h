@@ -165,7 +165,10 @@ constexpr int FFT_MAX_PASS = 12;
 struct FftTab {
   int n, np, l1;
   int rad[FFT_MAX_PASS], span[FFT_MAX_PASS];
+  // reciprocals for quot16 (fft_dev.cuh) of l1, and per pass of the sub-length and of l1 / span
+  unsigned l1r, lr[FFT_MAX_PASS], pr[FFT_MAX_PASS];
 };
+__host__ __device__ constexpr unsigned recip16(int d) { return 0xffffffffu / (unsigned)d; }
 
 // One piece of a plan solved directly (direct_dev.cuh): a rectangle of blocks with one tensor grid, its
 // reduced equations solved by a transform along one plane axis and tridiagonal systems along the other.
@@ -174,6 +177,7 @@ struct DirectTab {
   int M = 0, N = 0;        // cells along the transformed / the tridiagonal axis
   int cls = 0, kind = 0;   // LINES_PAIR / LINES_DCT4 / LINES_DENSE; boundary pair of the transformed axis
   int xl = 0, vec = 0, nbm = 1;
+  int m1 = 0;              // first cell along the transformed axis of its second block (M: one block)
   int soff = 0;            // first spectral element within a plane (the pieces' spectra follow each other)
   FftTab fft{};
   int w2n = 0, t4a = 0, t4b = 0;  // offsets in the twiddle table
