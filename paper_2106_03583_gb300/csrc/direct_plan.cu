@@ -617,9 +617,7 @@ int finish_direct(snac_plan* P) {
     }
     if ((st = up_vec(P, &D.d_qrow, qrow)) || (st = up_vec(P, &d_qof, qof))) return st;
     for (DirectTab& T : D.pc)
-      // (FP32 plans of few systems use the segments of k_tri_seg; the end values need the pivots)
-      if (f64 || D.pc.size() > 1 || (long long)P->nz * T.M >= 256LL * P->sms)
-        if ((st = plan_alloc(P, &T.d_fac, qof.size() * (size_t)T.M * T.N * w))) return st;
+      if ((st = plan_alloc(P, &T.d_fac, qof.size() * (size_t)T.M * T.N * w))) return st;
   } else {
     // the cells' places in the on-chip buffer, and the pieces' arguments
     std::vector<unsigned> off(P->lev[0].ncell, 0u);

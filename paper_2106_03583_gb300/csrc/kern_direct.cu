@@ -1,7 +1,7 @@
 // Separable solve of the reduced equations (Eq. 9) for planes too large for one CTA's shared memory:
 // three passes over the mode-space field, each reading and writing it once --
 //   k_lines_fwd  transform along the uniform plane axis, planes -> spectral [q][n][kappa]
-//   k_tri        one tridiagonal system per (q, kappa) along the other axis, in place
+//   k_tri_*      one tridiagonal system per (q, kappa) along the other axis, in place
 //   k_lines_bwd  inverse transform, spectral -> planes
 // and the plan-side tables of the method (see direct_dev.cuh for the transforms and the systems).
 #include <algorithm>
@@ -485,26 +485,6 @@ __global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T
   }
 }
 
-// FP32: KG systems x P segments of TRI_R rows per CTA, the rows in registers: the field is read and
-// written once (a sequential sweep per system would write and re-read both factors).
-constexpr int TRI_R = 16;
-
-template <typename T, int KG>
-__global__ void __launch_bounds__(1024, 1) k_tri_seg(const DirectArgs<T> A, int P, const unsigned char* __restrict__ low,
-                                                   const T* __restrict__ alpha, T* __restrict__ x) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int kk = threadIdx.x % KG, seg = threadIdx.x / KG;
-  const long long sys = (long long)blockIdx.x * KG + kk;
-  const bool live = sys < (long long)A.nq * A.M && !low[sys];  // (k_tri_low solves the others)
-  const int q = live ? (int)(sys / A.M) : 0, kap = live ? (int)(sys - (long long)q * A.M) : 0;
-  T* col = x + (long long)q * A.ncell + A.soff + kap;
-  const T tq = live ? -fma(A.sigma[q], A.cscale, A.lam[kap]) : (T)1;
-  tri_segment<T, TRI_R>(A.tri, A.N, P, seg, kk, KG, true, live, tq, A.scale, alpha ? *alpha : (T)0,
-                        reinterpret_cast<T*>(smem),
-                        [&](int n) { return col[(long long)n * A.M]; },
-                        [&](int n, T v) { col[(long long)n * A.M] = v; });
-}
-
 // The smoothest systems of an FP32 plan in FP64 arithmetic (FP32 right-hand side and solution). A
 // rounded elimination leaves errors that differ from row to row, relative to the solution; the outer
 // residual sees them times the row coupling (1e6 and more on a stretched axis), and the solution is
@@ -537,60 +517,11 @@ __global__ void __launch_bounds__(512, 1) k_tri_low(const TriRow<double>* __rest
                              });
 }
 
-// Rows in order, one thread per system, for systems too long for the segments of one CTA (FP32; the
-// factors c go to the plan's other mode buffer).
-template <typename T>
-__global__ void __launch_bounds__(128) k_tri_seq(const DirectArgs<T> A, T* __restrict__ x, T* __restrict__ cw) {
-  const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (sys >= (long long)A.nq * A.M) return;
-  const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
-  const long long o = (long long)q * A.ncell + A.soff + kap;
-  x += o;
-  cw += o;
-  const T tq = -fma(A.sigma[q], A.cscale, A.lam[kap]);
-  constexpr int U = 8;
-  T g = 0, d = 0;
-  for (int n0 = 0; n0 < A.N; n0 += U) {
-    T v[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = n0 + u < A.N ? x[(long long)(n0 + u) * A.M] : (T)0;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (n0 + u >= A.N) break;
-      const TriRow<T> w = A.tri[n0 + u];
-      const T s = fma(w.lo, g, w.tau + tq);
-      const T den = s + w.hi;
-      const T inv = den > (T)0 ? tri_recip(den) : (T)0;
-      g = s * inv;
-      d = fma(w.lo, d, -A.scale * v[u]) * inv;
-      x[(long long)(n0 + u) * A.M] = d;
-      cw[(long long)(n0 + u) * A.M] = w.hi * inv;
-    }
-  }
-  T y = 0;
-  for (int n0 = (A.N - 1) / U * U; n0 >= 0; n0 -= U) {
-    T v[U], c[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const bool in = n0 + u < A.N;
-      v[u] = in ? x[(long long)(n0 + u) * A.M] : (T)0;
-      c[u] = in ? cw[(long long)(n0 + u) * A.M] : (T)0;
-    }
-#pragma unroll
-    for (int u = U - 1; u >= 0; --u) {
-      if (n0 + u >= A.N) continue;
-      y = fma(c[u], y, v[u]);
-      x[(long long)(n0 + u) * A.M] = y;
-    }
-  }
-}
-
-// FP64 plans: the elimination is bound by the FP64 pipe (14 operations per row, half of them for the
-// pivot's reciprocal, which depends on the plan only), so the reciprocals are kept: [row of
-// DirectTab::qrow][n][kappa], wavenumbers of equal sigma (q and n - q of the real DFT) sharing one set. The
-// solve is then 5 operations per row at 48 bytes per cell. Measured on 512 x 512 x 256: 1.89 -> 0.71 ms (FP32 plans,
-// kept in FP32: 24 bytes per cell, 0.44 -> 0.36 ms, from 256 systems per multiprocessor on; below that the
-// segments of k_tri_seg have the shorter chain).
+// The elimination would be bound by arithmetic (14 operations per row, half of them for the pivot's reciprocal,
+// which depends on the plan only), so the reciprocals are kept: [row of DirectTab::qrow][n][kappa], wavenumbers of
+// equal sigma (q and n - q of the real DFT) sharing one set. The solve is then 5 operations per row. FP64 plans walk
+// the rows twice (k_tri_pre, 48 bytes per cell; 512 x 512 x 256: 1.89 -> 0.69 ms, the FP64 pipe alone takes 0.53);
+// FP32 plans take k_tri_scan, and k_tri_pre only for systems of more than 1024 rows.
 template <typename T>
 __global__ void __launch_bounds__(128) k_tri_factor(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
                                                   const double* __restrict__ sigma, double cscale, int M, int N,
@@ -657,6 +588,131 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
       x[(long long)(n0 + u) * M] = y;
     }
   }
+}
+
+// FP32 plans: the field is read and written once (12 bytes per cell instead of k_tri_pre's 24; FP64 would pay the
+// 12 operations per row). Measured with the listed systems' k_tri_low: 512 x 512 x 256 cells 0.345 -> 0.262 ms,
+// 1024 x 512 x 512 1.14 -> 0.81 ms (5.3 TB/s); 256 x 256 x 32 50 -> 47 us, 336 x 192 x 150 0.11 -> 0.085 ms against
+// the segments eliminated without kept pivots.
+// One thread per system and segment of TRI_R rows, which stay in its registers; with the pivots known, both
+// sweeps are first-order recurrences, so a segment is an affine map of the value that enters it: the segments'
+// maps are composed in order by the first segment's thread, then each thread runs its rows again from the right
+// value, rounding as the sequential sweep does. All coefficients are >= 0. 2^lg systems per CTA.
+// ENDS: only the first and last unknowns (and ssum, see k_tri_ends), nothing is written to the field.
+constexpr int SCAN_NT = 512, TRI_R = 16;
+template <bool ENDS>
+__global__ void __launch_bounds__(SCAN_NT, 2) k_tri_scan(const DirectArgs<float> A, int lg, int P, const int* __restrict__ qrow,
+                                                        const unsigned char* __restrict__ low, const float* __restrict__ fac,
+                                                        const float* __restrict__ alpha, float* __restrict__ x,
+                                                        float* __restrict__ ends, int E, int qs, float* __restrict__ ssum) {
+  constexpr int R = TRI_R;
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* lohi = reinterpret_cast<float2*>(smem);             // [P R] couplings
+  float2* ex = lohi + P * R;                                  // [P][2^lg] segment maps, then entering values
+  float* w = reinterpret_cast<float*>(ex + (P << lg));        // ENDS: [P][2^lg] partial sums
+  const int N = A.N, M = A.M, KG = 1 << lg;
+  const int kk = threadIdx.x & (KG - 1), seg = threadIdx.x >> lg;
+  const long long sys = ((long long)blockIdx.x << lg) + kk;
+  const bool in = sys < (long long)A.nq * M;
+  const bool live = in && !low[sys];  // (k_tri_low solves the others)
+  const int q = in ? (int)(sys / M) : 0, kap = in ? (int)(sys - (long long)q * M) : 0;
+  const bool sum = ENDS && in && q == qs && kap == 0;
+  const int n0 = seg * R;
+  float* col = x + (long long)q * A.ncell + A.soff + kap + (long long)n0 * M;
+  const float* fc = fac + (long long)qrow[q] * N * M + kap + (long long)n0 * M;
+  float v[R], f[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const bool ok = n0 + r < N;
+    v[r] = ok && (live || sum) ? col[(long long)r * M] : 0.0f;
+    f[r] = ok && live ? fc[(long long)r * M] : 0.0f;
+  }
+  for (int n = threadIdx.x; n < P * R; n += blockDim.x) {
+    const bool ok = n < N;
+    lohi[n] = make_float2(ok ? A.tri[n].lo : 0.0f, ok ? A.tri[n].hi : 0.0f);
+  }
+  if (sum) {
+    float t = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (n0 + r < N) t = fma(A.w[n0 + r], v[r], t);
+    w[threadIdx.x] = t;
+  }
+  __syncthreads();
+  float2* e = ex + threadIdx.x;
+  float d = 0, a = 1;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float lo = lohi[n0 + r].x;
+    v[r] *= -A.scale;
+    d = fma(lo, d, v[r]) * f[r];
+    a *= lo * f[r];
+  }
+  *e = make_float2(d, a);
+  __syncthreads();
+  if (seg == 0) {
+    float g = 0, t = 0;
+    for (int k = kk; k < P << lg; k += KG) {
+      const float2 m = ex[k];
+      ex[k].x = g;
+      g = fma(m.y, g, m.x);
+      if (sum) t += w[k];
+    }
+    if (sum) *ssum = t;
+  }
+  __syncthreads();
+  d = e->x;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    d = fma(lohi[n0 + r].x, d, v[r]) * f[r];
+    v[r] = d;
+    // an exactly singular system ends in a zero pivot: its last unknown is the piece's constant
+    if (n0 + r == N - 1 && alpha != nullptr && f[r] == 0.0f) v[r] = *alpha;
+    if (ENDS && n0 + r == N - 1 && live && A.e1 >= 0) ends[(long long)q * E + A.e1 + kap] = v[r];
+  }
+  float y = 0, c = 1;
+#pragma unroll
+  for (int r = R - 1; r >= 0; --r) {
+    const float h = lohi[n0 + r].y * f[r];
+    y = fma(h, y, v[r]);
+    c *= h;
+  }
+  *e = make_float2(y, c);
+  __syncthreads();
+  if (seg == 0) {
+    float g = 0;
+    for (int k = ((P - 1) << lg) + kk; k >= 0; k -= KG) {
+      const float2 m = ex[k];
+      ex[k].x = g;
+      g = fma(m.y, g, m.x);
+    }
+    if (ENDS && live && A.e0 >= 0) ends[(long long)q * E + A.e0 + kap] = g;
+  }
+  if (ENDS) return;
+  __syncthreads();
+  y = e->x;
+#pragma unroll
+  for (int r = R - 1; r >= 0; --r) {
+    y = fma(lohi[n0 + r].y * f[r], y, v[r]);
+    if (live && n0 + r < N) col[(long long)r * M] = y;
+  }
+}
+
+// Systems per CTA (log2) of k_tri_scan: 8 to 32, so that its rows are whole sectors; -1: too many segments.
+inline int scan_lg(int P) {
+  for (int lg = 5; lg >= 3; --lg)
+    if (P << lg <= SCAN_NT) return lg;
+  return -1;
+}
+
+template <bool ENDS>
+void launch_scan(const DirectArgs<float>& A, int lg, const int* qrow, const unsigned char* low, const float* fac,
+                 const float* alpha, float* x, float* ends, int E, int qs, float* ssum, cudaStream_t s) {
+  const int P = (A.N + TRI_R - 1) / TRI_R;
+  const long long sys = (long long)A.nq * A.M;
+  const size_t smem = sizeof(float2) * ((size_t)P * TRI_R + ((size_t)P << lg)) + (ENDS ? sizeof(float) * ((size_t)P << lg) : 0);
+  k_tri_scan<ENDS><<<(unsigned)((sys + (1 << lg) - 1) >> lg), P << lg, smem, s>>>(A, lg, P, qrow, low, fac, alpha, x, ends, E,
+                                                                                  qs, ssum);
 }
 
 // First and last unknowns of every system of a piece (the end values of the interface systems), from the
@@ -742,11 +798,10 @@ cudaError_t lines_t(snac_plan* P, const DirectArgs<T>& A, bool fwd, const T* in,
 }
 
 template <typename T>
-cudaError_t tri_t(snac_plan* P, const DirectTab& D, const DirectArgs<T>& A, const T* alpha, T* u, T* f, cudaStream_t s) {
+cudaError_t tri_t(snac_plan* P, const DirectTab& D, const DirectArgs<T>& A, const T* alpha, T* u, cudaStream_t s) {
   const double cells = (double)A.nq * A.M * A.N;
   LaunchScope ls(P, K_TRI, 2.0 * sizeof(T) * cells, 20.0 * cells, s);
   const long long sys = (long long)A.nq * A.M;
-  const int segs = (A.N + TRI_R - 1) / TRI_R;
   const unsigned g128 = (unsigned)((sys + 127) / 128);
   if constexpr (sizeof(T) == 4) {
     const int lsegs = (A.N + LOW_R - 1) / LOW_R;
@@ -754,14 +809,11 @@ cudaError_t tri_t(snac_plan* P, const DirectTab& D, const DirectArgs<T>& A, cons
       k_tri_low<false><<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
           (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / D.theta, D.d_lowlist,
           D.nlow, A.M, A.N, lsegs, A.ncell, A.soff, alpha, u, nullptr, 0, -1, -1);
-    if (D.d_fac)
-      k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u);
-    else if (segs <= 32)
-      k_tri_seg<T, 32><<<(unsigned)((sys + 31) / 32), 32 * segs, 7 * sizeof(T) * 32 * segs, s>>>(A, segs, D.d_low, alpha, u);
-    else if (segs <= 64)
-      k_tri_seg<T, 16><<<(unsigned)((sys + 15) / 16), 16 * segs, 7 * sizeof(T) * 16 * segs, s>>>(A, segs, D.d_low, alpha, u);
+    const int lg = scan_lg((A.N + TRI_R - 1) / TRI_R);
+    if (lg >= 0)
+      launch_scan<false>(A, lg, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u, nullptr, 0, -1, nullptr, s);
     else
-      k_tri_seq<T><<<g128, 128, 0, s>>>(A, u, f);
+      k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u);
   } else {
     k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, nullptr, (const T*)D.d_fac, alpha, u);
   }
@@ -791,15 +843,24 @@ cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
               (const TriRow<double>*)d.d_tri64, d.d_lam64, P->d_sigma64, d.cscale, d.cscale / d.theta, d.d_lowlist,
               d.nlow, d.M, d.N, lsegs, A[p].ncell, A[p].soff, nullptr, u, (T*)D.it.d_ends, D.it.E, A[p].e0, A[p].e1);
       }
-      k_tri_ends<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A[p], D.d_qrow, d.d_low, (const T*)d.d_fac, u,
-                                                                 (T*)D.it.d_ends, D.it.E, d.singular ? D.it.qs : -1,
-                                                                 (T*)D.it.d_ssum + p);
+      const int qs = d.singular ? D.it.qs : -1;
+      bool done = false;
+      if constexpr (sizeof(T) == 4) {
+        const int lg = scan_lg((d.N + TRI_R - 1) / TRI_R);
+        done = lg >= 0;
+        if (done)
+          launch_scan<true>(A[p], lg, D.d_qrow, d.d_low, (const T*)d.d_fac, nullptr, u, (T*)D.it.d_ends, D.it.E, qs,
+                            (T*)D.it.d_ssum + p, s);
+      }
+      if (!done)
+        k_tri_ends<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A[p], D.d_qrow, d.d_low, (const T*)d.d_fac, u,
+                                                                   (T*)D.it.d_ends, D.it.E, qs, (T*)D.it.d_ssum + p);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = launch_iface(P, s);
   }
   for (int p = 0; p < np && e == cudaSuccess; ++p)
-    e = tri_t<T>(P, D.pc[p], A[p], D.it.ns ? (const T*)D.it.d_alpha + p : nullptr, u, f, s);
+    e = tri_t<T>(P, D.pc[p], A[p], D.it.ns ? (const T*)D.it.d_alpha + p : nullptr, u, s);
   for (int p = 0; p < np && e == cudaSuccess; ++p) e = lines_t(P, A[p], false, (const T*)u, f, s);
   return e;
 }

@@ -81,6 +81,13 @@ DIRECT = [
     ("1", 88, 96, 0.0, 1.2, "NNDN", "DD", (False, False)),
     ("L", 160, 128, 1.0, 1.0, "DDNN", "NN", (False, False)),
     ("T", 240, 128, 1.0, 1.0, "NNNN", "PP", (False, False)),    # singular
+    # segments of 16 rows, 32 / 16 / 8 systems per CTA: a last CTA not full, a last segment not full, 17 segments,
+    # the most segments, and the end values of 17 segments (singular)
+    ("1", 72, 128, 0.0, 1.0, "NNNN", "NN", (False, False)),
+    ("1", 128, 72, 0.0, 1.0, "DDNN", "PP", (False, False)),
+    ("1", 40, 264, 0.0, 1.0, "NNDN", "DD", (False, False)),
+    ("1", 16, 1024, 0.0, 1.0, "DNNN", "NN", (False, False)),
+    ("L", 64, 544, 0.0, 1.0, "NNNN", "NN", (False, False)),
 ]
 
 
