@@ -50,7 +50,7 @@ FP64_ALU_PEAK = 152 * 2 * 2 * 2.07e9   # SMs x FP64 FMA/clk/SM x 2 flop x max SM
 # roof is the FP64 pipe, not HBM
 FP64_ALWAYS = {"field3d"}
 FP64_IN_FP64_PLAN = {"smooth", "restrict", "prolong", "mode_resid", "mode_apply", "forward_transform",
-                     "backward_update", "coarse_solve"}
+                     "backward_update", "coarse_solve", "lines_forward", "lines_backward"}
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum from one ncu capture of the
 # kernel on the workload at 1/2 scale per axis), divided by that launch's algorithmic bytes, with the
 # sha256 of the kernel's source file when it was captured. The bench scales the ratio to its own
@@ -59,13 +59,27 @@ FP64_IN_FP64_PLAN = {"smooth", "restrict", "prolong", "mode_resid", "mode_apply"
 # launches of the first cycles (fused kernels), the first launch of the others.
 _FUSED = {"src": "paper_2106_03583_gb300/csrc/kern_fused.cu",
           "sha256": "2b68f2b1fd20f060bc103825a18f00981660e81a8b8743649cd5d4ea215d0b23"}
+_LINES = {"src": "paper_2106_03583_gb300/csrc/kern_direct.cu",
+          "sha256": "c0763ff0c6fcd5f30b169ee3af517f2db2eb63673f4b5fb9ddd0cec79e4c4850"}
+_Z = {"src": "paper_2106_03583_gb300/csrc/ztrans_dev.cuh",
+      "sha256": "679b1e33500a8b243667ab6f2b42e3757d317f4c597ba14d788b8b0b14d5ce08"}
+_FF = {"src": "paper_2106_03583_gb300/csrc/kern_ffresid.cu",
+       "sha256": "5fc9d13b4f578ffb67c8becdd7bbe4938c8cf9a95398023890909415df383606"}
+_F64 = {"src": "paper_2106_03583_gb300/csrc/kern_field.cu",
+        "sha256": "578895333e01efacaf9ddf5dd66b9c5265fe393489eecd8d074588eceb81523c"}
 TRAFFIC = {
     ("chan", "fused_up", "mixed"): dict(_FUSED, ratio=413.18 / 436.21),       # 3.25 w x 131072 cells x 256 modes
     ("chan", "fused_down", "mixed"): dict(_FUSED, ratio=404.67 / 335.54),     # zero iterate: 2.5 w x 131072 x 256
-    ("chan", "field3d_ff", "mixed"): {"src": "paper_2106_03583_gb300/csrc/kern_ffresid.cu", "ratio": 663.60 / 671.09,
-                                      "sha256": "ff6d20a1b921f85afe1735f14a91eeaa722ae4089ac4238709efb70ea0c6242f"},
-    ("chan", "smooth", "fp64"): {"src": "paper_2106_03583_gb300/csrc/kern_mg.cu", "ratio": 755.85 / 402.65,
-                                 "sha256": "7ff5bf650cac1bff272ed46562c8e0a873024af37927a04949010cce6a4b6037"},
+    ("chan", "backward_update", "mixed"): dict(_Z, ratio=641.9 / 671.1),      # 4 + 8 + 8 B per cell
+    ("chan", "field3d_ff", "mixed"): dict(_FF, ratio=662.7 / 671.1),
+    ("chan", "field3d", "mixed"): dict(_F64, ratio=1270.2 / 805.3),           # 24 B; edges of the tiles re-read
+    ("chan", "lines_forward", "mixed"): dict(_LINES, ratio=218.0 / 268.4),
+    ("chan", "lines_backward", "mixed"): dict(_LINES, ratio=221.4 / 268.4),
+    ("chan", "tridiagonal", "mixed"): dict(_LINES, ratio=332.1 / 268.4),      # the kept pivots beside the field
+    ("chan", "lines_forward", "fp64"): dict(_LINES, ratio=486.9 / 536.9),
+    ("chan", "lines_backward", "fp64"): dict(_LINES, ratio=487.8 / 536.9),
+    ("chan", "forward_transform", "fp64"): dict(_Z, ratio=490.0 / 536.9),
+    ("chan", "backward_update", "fp64"): dict(_Z, ratio=760.1 / 805.3),
 }
 
 
@@ -181,7 +195,7 @@ def whole_job_rate(world, steps, max_ms):
 
 
 def _dtype(precision):
-    return "f64" if precision == "fp64" else "f32 transforms and multigrid, f64 residual and update (mixed)"
+    return "f64" if precision == "fp64" else "f32 transforms and reduced solves, f64 residual and update (mixed)"
 
 
 def workload_config(name, blocks, tol, precision, world, scale=1):

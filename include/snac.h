@@ -86,10 +86,13 @@ typedef enum { SNAC_FP64 = 0, SNAC_MIXED = 1 } snac_precision;
 
 /* Solver options; pass NULL to snac_plan_create for the defaults shown.
  * With the default schedule (nu1, nu2, max_cycles, max_coarse, fused, inner_reduction, onchip and
- * bottom_cells as shown) a layout whose blocks assemble into a rectangle with one uniform plane axis (an
- * even number of cells, half or all of it a product of 2, 3, 5 and 7; the other axis not periodic) solves the
- * reduced equations directly -- a transform along that axis (Table 1) and tridiagonal systems along the
- * other -- in place of V-cycles; setting any of these options asks for the multigrid. */
+ * bottom_cells as shown) the reduced equations are solved directly in place of V-cycles where the layout
+ * allows it: its blocks assemble into one rectangle, or into several that meet along parts of their sides (L, T, U
+ * shapes, rings); each rectangle is transformed along one plane axis (the same one for all; Table 1 kinds on a
+ * uniform axis of an even number of cells, half or all of it a product of 2, 3, 5 and 7; the eigenvectors of the
+ * axis otherwise, for planes that do not solve on chip, up to 384 (SNAC_MIXED) or about 200 (SNAC_FP64) cells along
+ * it), tridiagonal systems run along the other axis (not periodic), and a dense system per wavenumber gives the
+ * fluxes between rectangles. Setting any of these options asks for the multigrid. */
 typedef struct {
   int32_t precision;   /* SNAC_FP64 (default): every stage in FP64. SNAC_MIXED: transforms and
                           multigrid in FP32 inside the FP64 defect-correction loop; the outer
