@@ -60,7 +60,7 @@ FP64_IN_FP64_PLAN = {"smooth", "restrict", "prolong", "mode_resid", "mode_apply"
 _FUSED = {"src": "paper_2106_03583_gb300/csrc/kern_fused.cu",
           "sha256": "2b68f2b1fd20f060bc103825a18f00981660e81a8b8743649cd5d4ea215d0b23"}
 _LINES = {"src": "paper_2106_03583_gb300/csrc/kern_direct.cu",
-          "sha256": "c0763ff0c6fcd5f30b169ee3af517f2db2eb63673f4b5fb9ddd0cec79e4c4850"}
+          "sha256": "1832384e88e19c3a8140116062612f72d8836fcf770a7029d709bfa33dfb88f9"}
 _Z = {"src": "paper_2106_03583_gb300/csrc/ztrans_dev.cuh",
       "sha256": "679b1e33500a8b243667ab6f2b42e3757d317f4c597ba14d788b8b0b14d5ce08"}
 _FF = {"src": "paper_2106_03583_gb300/csrc/kern_ffresid.cu",

@@ -592,9 +592,9 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
 
 // FP32 plans: the field is read and written once (12 bytes per cell instead of k_tri_pre's 24; FP64 would pay the
 // 12 operations per row). Measured with the listed systems' k_tri_low: 512 x 512 x 256 cells 0.345 -> 0.262 ms,
-// 1024 x 512 x 512 1.14 -> 0.81 ms (4.0 TB/s; what is
-// left is the barriers between its phases); 256 x 256 x 32 50 -> 47 us, 336 x 192 x 150 0.11 -> 0.085 ms against
-// the segments eliminated without kept pivots.
+// 1024 x 512 x 512 1.14 -> 0.81 ms (4.0 TB/s; what is left is the barriers between its phases); 256 x 256 x 32 50 ->
+// 47 us, 336 x 192 x 150 0.11 -> 0.085 ms against the segments eliminated without kept pivots. Two CTAs of 512
+// threads per multiprocessor: four of 256 (shorter rows of systems) take 0.31 ms, one of 1024 0.29 ms.
 // One thread per system and segment of TRI_R rows, which stay in its registers; with the pivots known, both
 // sweeps are first-order recurrences, so a segment is an affine map of the value that enters it: the segments'
 // maps are composed in order by the first segment's thread, then each thread runs its rows again from the right
