@@ -73,7 +73,8 @@ struct DirectArgs {
   const int* base;
   const int* mblk;
   const int* mstr;
-  int nbm, m1, xl, vec;    // m1: first m of the second block; xl: the transformed axis is the contiguous one; vec: pairs may be loaded as vectors
+  int nbm, m1, xl, vec;    // m1: first m of the second block (M: one block); xl: the transformed axis is the
+                           // contiguous one; vec: pairs may be loaded as vectors
 };
 
 template <typename T>
