@@ -653,14 +653,13 @@ int finish_direct(snac_plan* P) {
     };
     if ((st = f64 ? place(double{}) : place(float{})) || (st = up_vec(P, &D.d_celloff, off))) return st;
   }
-  // on a private non-blocking stream, like every other device work of plan creation
-  cudaStream_t cs = nullptr;
-  bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
+  // on the private stream, like every other device work of plan creation
+  const cudaStream_t cs = P->setup_stream;
+  bool ok = true;
   for (DirectTab& T : D.pc)
     if (ok && T.d_fac) ok = launch_tri_factor(P, T, d_qof, (int)qof.size(), cs) == cudaSuccess;
   if (ok && D.it.k) ok = setup_iface(P, cs) == cudaSuccess;
   ok = ok && cudaStreamSynchronize(cs) == cudaSuccess;
-  if (cs) cudaStreamDestroy(cs);
   if (!ok) {
     const cudaError_t e = cudaGetLastError();
     set_error(std::string("setting up the direct solves failed: ") + cudaGetErrorString(e));

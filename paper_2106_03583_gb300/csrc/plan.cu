@@ -174,8 +174,7 @@ template <typename T>
 int upload(snac_plan* P, T** ptr, const std::vector<T>& v) {
   int st = dmalloc(P, ptr, v.size());
   if (st) return st;
-  if (!v.empty() && cudaMemcpy(*ptr, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess)
-    return fail(SNAC_ERR_CUDA, "cudaMemcpy upload failed");
+  if (copy_in(P, *ptr, v.data(), v.size() * sizeof(T)) != cudaSuccess) return fail(SNAC_ERR_CUDA, "upload failed");
   return SNAC_OK;
 }
 
@@ -503,6 +502,7 @@ void free_plan(snac_plan* P) {
   profile_release(P);
   for (auto& kv : P->round_graphs)
     if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
+  if (P->setup_stream) cudaStreamDestroy(P->setup_stream);
   if (P->capture_stream) cudaStreamDestroy(P->capture_stream);
   for (void* p : P->allocs) cudaFree(p);
   for (void* p : P->pen_tallocs) cudaFree(p);
@@ -869,12 +869,8 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
       for (size_t l = 0; l + 1 < P->lev.size(); ++l)
         if ((st = dmalloc(P, &P->lev[l].d_invd, (size_t)P->nz * P->lev[l].ncell))) break;
       if (st) break;
-      // on a private non-blocking stream: plan creation does not wait for other streams' work
-      cudaStream_t cs = nullptr;
-      bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
-      ok = ok && launch_inverse_diagonals(P, cs) == cudaSuccess && cudaStreamSynchronize(cs) == cudaSuccess;
-      if (cs) cudaStreamDestroy(cs);
-      if (!ok) {
+      // on the private stream: plan creation does not wait for other streams' work
+      if (launch_inverse_diagonals(P, P->setup_stream) != cudaSuccess || cudaStreamSynchronize(P->setup_stream) != cudaSuccess) {
         st = fail(SNAC_ERR_CUDA, "computing the inverse diagonals failed");
         break;
       }
@@ -966,12 +962,11 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     }
     {
       // the pre-pass flag, the ticket of the sums and the counters of the fused launch start at zero (each
-      // use resets them); on a private non-blocking stream, like every other device write of plan creation
-      cudaStream_t cs = nullptr;
-      bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
-                cudaMemsetAsync(P->d_flag, 0, 2 * sizeof(int), cs) == cudaSuccess &&
-                (!P->d_fused || cudaMemsetAsync(P->d_fused, 0, 3 * sizeof(int), cs) == cudaSuccess) && cudaStreamSynchronize(cs) == cudaSuccess;
-      if (cs) cudaStreamDestroy(cs);
+      // use resets them); on the private stream, like every other device write of plan creation
+      const cudaStream_t cs = P->setup_stream;
+      const bool ok = cudaMemsetAsync(P->d_flag, 0, 2 * sizeof(int), cs) == cudaSuccess &&
+                      (!P->d_fused || cudaMemsetAsync(P->d_fused, 0, 3 * sizeof(int), cs) == cudaSuccess) &&
+                      cudaStreamSynchronize(cs) == cudaSuccess;
       if (!ok) {
         st = fail(SNAC_ERR_CUDA, "initialising the pre-pass flag failed");
         break;
@@ -993,6 +988,13 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
 }  // namespace
 
 namespace snac {
+cudaError_t copy_in(snac_plan* P, void* dst, const void* src, size_t bytes) {
+  cudaError_t e = cudaSuccess;
+  if (!P->setup_stream) e = cudaStreamCreateWithFlags(&P->setup_stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, P->setup_stream);
+  return e != cudaSuccess || !bytes ? e : cudaStreamSynchronize(P->setup_stream);
+}
+
 int plan_alloc(snac_plan* P, void** p, size_t bytes) {
   char* c = nullptr;
   const int st = dmalloc(P, &c, bytes);
@@ -1003,8 +1005,7 @@ int plan_alloc(snac_plan* P, void** p, size_t bytes) {
 int plan_upload(snac_plan* P, void** p, const void* src, size_t bytes) {
   const int st = plan_alloc(P, p, bytes);
   if (st) return st;
-  if (bytes && cudaMemcpy(*p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess)
-    return fail(SNAC_ERR_CUDA, "cudaMemcpy upload failed");
+  if (copy_in(P, *p, src, bytes) != cudaSuccess) return fail(SNAC_ERR_CUDA, "upload failed");
   return SNAC_OK;
 }
 

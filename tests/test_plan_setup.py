@@ -1,0 +1,53 @@
+"""Plan creation on the host (no GPU: tests/fake_cudart.cpp stands in for the CUDA runtime)."""
+import pytest
+
+import fake_cuda
+
+# an L of three blocks, a rectangle clustered both ways (dense transforms), small planes of one piece and of
+# three, and a plan that keeps its V-cycles (a prime axis)
+LAYOUTS = """
+def face(n, f):
+    return inputs.tanh_faces(n, 0, f, 0.0, 1.0)
+def problem(rects, nx, ny, nz=8, xf=0.0, yf=0.0, z=("N", "N"), walls="DNNN"):
+    return inputs.make_blocks(face(nx, xf), face(ny, yf), np.linspace(0.0, 1.0, nz + 1), rects,
+                              dict(zip(("x-", "x+", "y-", "y+"), walls)), z)
+L = lambda n: [(0, n, 0, n), (n, 2 * n, 0, n), (0, n, n, 2 * n)]
+PROBLEMS = {
+    "L": lambda: problem(L(80), 160, 160, z=("P", "P")), "L on chip": lambda: problem(L(16), 32, 32),
+    "dense": lambda: problem([(0, 160, 0, 128)], 160, 128, xf=1.0, yf=1.0),
+    "on chip": lambda: problem([(0, 32, 0, 32)], 32, 32, yf=1.0),
+    "planes": lambda: problem([(0, 160, 0, 128)], 160, 128, yf=1.0),
+    "V-cycles": lambda: problem([(0, 416, 0, 416)], 416, 416, xf=1.0, yf=1.0),
+}
+"""
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_setup_kernels_run_after_the_tables_have_arrived(precision):
+    out = fake_cuda.run(LAYOUTS + f"""
+out = dict()
+for name, make in PROBLEMS.items():
+    fake.fake_reset()
+    st, h = create(make(), {precision!r})
+    out[name] = [st, len(launches()), fake.fake_unordered().decode().split()]
+    lib.snac_plan_destroy(h)
+""")
+    assert sum(n for _, n, _ in out.values()) > 0
+    for name, (st, _, unordered) in out.items():
+        assert st == 0 and unordered == [], name
+    assert len(out) == 6
+
+
+def test_pencil_kernels_run_after_their_tables_have_arrived():
+    out = fake_cuda.run(LAYOUTS + """
+st, h = create(PROBLEMS["on chip"]())
+buf = (ctypes.c_double * (8 * 1024))()
+s = ctypes.c_void_p(8)
+halo, n = (ctypes.c_int64 * 4096)(), ctypes.c_int64()
+sums = (ctypes.c_double * 5)()
+fake.fake_reset()
+r = [lib.snac_pencil_setup(h, 0, 1024, halo, 4096, ctypes.byref(n)),
+     lib.snac_pencil_residual(h, buf, buf, buf, 0.0, sums, s), lib.snac_pencil_forward(h, 1024, buf, buf, s)]
+out = [st, r, len(launches()), fake.fake_unordered().decode().split()]
+""")
+    assert out[:2] == [0, [0, 0, 0]] and out[2] >= 3 and out[3] == []
