@@ -30,7 +30,8 @@
 // sums (tau) instead of the diagonal, so that every operation adds or multiplies non-negative numbers:
 // no cancellation, the factors are accurate to a few units in the last place of the working type even
 // where the system is nearly singular, and an exactly singular one (all tau = 0) ends in an exactly zero
-// pivot, whose unknown is set to zero (the caller fixes the mean).
+// pivot, whose unknown is set to zero (the caller fixes the mean). A piece of several without a Dirichlet face
+// has the last unknown of its slot 0 given (pinned): its value alpha comes from the interface system.
 #pragma once
 
 #include <algorithm>
@@ -61,7 +62,7 @@ struct DirectArgs {
   const T* lam;            // eigenvalue of slot kappa (<= 0), times cscale
   const TriRow<T>* tri;    // [N], times cscale
   const T* sigma;          // per wavenumber
-  const T* w;              // [N] cell widths along the tridiagonal axis
+  int pin;                 // slot 0 is pinned
   long long ncell;
   int soff;                // the piece's first spectral element within a plane
   int e0, e1;              // where its first / last row's values start in the end vector, -1: not needed
@@ -85,7 +86,7 @@ inline DirectArgs<T> direct_args(const snac_plan* P, const DirectTab& D) {
   for (int u = 0; u < I.nends; ++u)
     if (&P->direct.pc[I.ep[u]] == &D) (I.ee[u] == 0 ? A.e0 : A.e1) = I.eo[u];
   A.soff = D.soff;
-  A.w = (const T*)D.d_w;
+  A.pin = D.pin;
   A.F = D.fft;
   A.M = D.M;
   A.N = D.N;
@@ -118,7 +119,7 @@ inline DirectArgs<T> direct_args(const snac_plan* P, const DirectTab& D) {
 
 template <typename T>
 struct IfaceArgs {
-  int k, kk, E, ns, qs, gs;         // gs: the whole problem is singular (the last constraint is implied)
+  int k, kk, E, ns, qs;             // qs: wavenumber whose whole system is singular (the last equation is implied)
   int sp[IFACE_MAX_ENDS];
   int nends, eo[IFACE_MAX_ENDS + 1];
   int row[IFACE_MAX_ENDS];          // first spectral element of every end row within a plane
@@ -127,7 +128,7 @@ struct IfaceArgs {
   const double* KT;
   T* ends;
   T* alpha;
-  T* ssum;
+  T* num;
 };
 
 template <typename T>
@@ -139,7 +140,6 @@ inline IfaceArgs<T> iface_args(const snac_plan* P) {
   A.E = I.E;
   A.ns = I.ns;
   A.qs = I.qs;
-  A.gs = P->singular ? 1 : 0;
   A.nends = I.nends;
   for (int u = 0; u < I.nends; ++u) {
     const DirectTab& D = P->direct.pc[I.ep[u]];
@@ -153,7 +153,7 @@ inline IfaceArgs<T> iface_args(const snac_plan* P) {
   A.KT = I.d_KT;
   A.ends = (T*)I.d_ends;
   A.alpha = (T*)I.d_alpha;
-  A.ssum = (T*)I.d_ssum;
+  A.num = (T*)I.d_num;
   return A;
 }
 
@@ -188,13 +188,13 @@ __device__ void gemv_cols(const TA* __restrict__ A, int ld, int n, int E, const 
 }
 
 // The fluxes of wavenumber q from its end values: jumps of u across the interface cells, the dense system,
-// and what the fluxes add to the end rows' right-hand sides (add(e, v)); alpha: the singular pieces'
-// constants (by piece). The jumps are differences of nearly equal end values and K^-1 damps their smooth
+// and what the fluxes add to the end rows' right-hand sides (add(e, v)); num, alpha: the pinned pieces'
+// eliminated last right-hand sides and unknowns (by piece). The jumps are differences of nearly equal end values and K^-1 damps their smooth
 // part by the pieces' size in cells, so both products are formed in FP64 in every plan (in FP32 their
 // rounding left a second correction step at 1e-9 .. 2e-8 of ||f|| on the L-shaped 512 x 512 x 128 duct).
-// work (doubles, shared): ends (complete), y, phi, part: E + 2 kk + nt; ssum by piece.
+// work (doubles, shared): ends (complete), y, phi, part: E + 2 kk + nt.
 template <typename T, typename Add>
-__device__ void iface_solve(const IfaceArgs<T>& I, int q, double* work, const T* ssum, T* alpha, int nt, Add&& add) {
+__device__ void iface_solve(const IfaceArgs<T>& I, int q, double* work, const T* num, T* alpha, int nt, Add&& add) {
   double* ends = work;
   double* y = ends + I.E;
   double* phi = y + I.kk;
@@ -202,11 +202,11 @@ __device__ void iface_solve(const IfaceArgs<T>& I, int q, double* work, const T*
   gemv_cols(I.Y, I.kk, I.k, I.E, ends, y, part, nt);
   if ((int)threadIdx.x < I.ns) {
     const int a = threadIdx.x;
-    y[I.k + a] = q == I.qs && !(I.gs && a == I.ns - 1) ? -(double)ssum[I.sp[a]] : 0.0;
+    y[I.k + a] = q == I.qs && a == I.ns - 1 ? 0.0 : (double)num[I.sp[a]];
   }
   __syncthreads();
   gemv_cols(I.KT + (long long)q * I.kk * I.kk, I.kk, I.kk, I.kk, y, phi, part, nt);
-  if ((int)threadIdx.x < I.ns && q == I.qs) alpha[I.sp[threadIdx.x]] = (T)phi[I.k + threadIdx.x];
+  if ((int)threadIdx.x < I.ns) alpha[I.sp[threadIdx.x]] = (T)phi[I.k + threadIdx.x];
   T* ph = reinterpret_cast<T*>(part);  // (kk <= 1040 values of T fit in nt doubles)
   for (int j = threadIdx.x; j < I.k; j += nt) ph[j] = (T)phi[j];
   __syncthreads();
@@ -261,13 +261,14 @@ __device__ __forceinline__ double tri_recip(double x) { return recip(x); }
 // unknown), the segments' last unknowns form a tridiagonal system of P rows that the first segment's
 // thread solves, and each thread substitutes back. load(n) gives the right-hand side, store(n, u)
 // takes the solution; ex: 7 x P x kg values, this system's column kk. Every thread of the CTA calls it
-// (three barriers). tq = -lambda - sigma >= 0; alpha: the last unknown of an exactly singular system.
+// (three barriers). tq = -lambda - sigma >= 0; pin: the last unknown is alpha, and num takes what its row is
+// left with by the elimination; an exactly singular system that is not pinned ends in zero.
 // `act` is false for threads past the last segment, which only take part in the barriers; `live`
 // for those with a system to solve.
-template <typename T, int R, typename Load, typename Store>
+template <typename T, int R, typename Load, typename Store, typename Num>
 __device__ __forceinline__ void tri_segment(const TriRow<T>* __restrict__ tri, int N, int P, int seg, int kk, int kg,
-                                            bool act, bool live, T tq, T scale, T alpha, T* __restrict__ ex,
-                                            Load&& load, Store&& store) {
+                                            bool act, bool live, T tq, T scale, bool pin, T alpha, T* __restrict__ ex,
+                                            Load&& load, Store&& store, Num&& num) {
   const int n0 = seg * R - (P * R - N);
   T D[R], c[R];
 #pragma unroll
@@ -282,7 +283,8 @@ __device__ __forceinline__ void tri_segment(const TriRow<T>* __restrict__ tri, i
     }
     const T la = w.lo * a, ls = fma(w.lo, sl, w.tau);
     const T den = la + ls + w.hi;
-    const T inv = den > (T)0 ? tri_recip(den) : (T)0;
+    // (a pinned last row stays as it is: num and the segments' system need it unscaled)
+    const T inv = pin && r == R - 1 && seg == P - 1 ? (T)1 : den > (T)0 ? tri_recip(den) : (T)0;
     c[r] = w.hi * inv;
     a = la * inv;
     sl = ls * inv;
@@ -321,7 +323,13 @@ __device__ __forceinline__ void tri_segment(const TriRow<T>* __restrict__ tri, i
       const T den = sum + hi;
       const T inv = den > (T)0 ? tri_recip(den) : (T)0;
       g = sum * inv;
-      y = den > (T)0 ? fma(lo, y, d) * inv : alpha;
+      y = fma(lo, y, d);
+      if (pin && !more) {
+        num(y);
+        y = alpha;
+      } else {
+        y *= inv;
+      }
       z[o] = y;
       z[o + st] = hi * inv;
     }
@@ -366,7 +374,7 @@ __host__ __device__ inline PlaneShape plane_shape(const FftTab& F, int M, int N,
   return s;
 }
 // Elements of shared memory of a whole-plane solve: the pieces' buffers, the exchange of the tridiagonal
-// segments, the singular pieces' constants and sums, and (doubles) the work space of an interface solve.
+// segments, the pinned pieces' unknowns and right-hand sides, and (doubles) the work space of an interface solve.
 inline size_t onchip_elements(size_t buffers, int nt) {
   return ((buffers + 1) & ~(size_t)1) + 7 * (size_t)nt + 2 * IFACE_MAX_ENDS;
 }
@@ -443,9 +451,10 @@ __device__ __forceinline__ int slot_at(const DirectArgs<T>& A, const PlaneShape&
   return 2 * fft_row(A.perm[(kap & 1) ? (A.M - 1 - kap) >> 1 : kap >> 1], A.F, S.s1, S.rp) + (kap & 1);
 }
 
-// The tridiagonal systems of one piece; ENDS: only the first and last rows' solutions, into the end vector.
+// The tridiagonal systems of one piece; ENDS: only the first and last rows' solutions, into the end vector, and
+// the pinned system's eliminated last right-hand side (*num).
 template <typename T, bool ENDS>
-__device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T sg, T alpha, T* ex, double* ends, int nt) {
+__device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T sg, T alpha, T* ex, double* ends, T* num, int nt) {
   const int N = A.N, M = A.M;
   const int P = (N + PLANE_R - 1) / PLANE_R, kg = nt / P;
   const int seg = (int)threadIdx.x / kg, kk = threadIdx.x - seg * kg;
@@ -460,7 +469,7 @@ __device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T 
       tq = -fma(sg, A.cscale, A.lam[kap]);
       o = slot_at(A, S, kap);
     }
-    tri_segment<T, PLANE_R>(A.tri, N, P, mine ? seg : 0, kk, kg, mine, live, tq, A.scale, alpha, ex,
+    tri_segment<T, PLANE_R>(A.tri, N, P, mine ? seg : 0, kk, kg, mine, live, tq, A.scale, A.pin && live && kap == 0, alpha, ex,
                             [&](int n) { return bt[o + n * ns]; },
                             [&](int n, T v) {
                               if (!ENDS) {
@@ -469,6 +478,9 @@ __device__ void piece_tri(const DirectArgs<T>& A, const PlaneShape& S, T* bt, T 
                                 if (n == 0 && A.e0 >= 0) ends[A.e0 + kap] = v;
                                 if (n == N - 1 && A.e1 >= 0) ends[A.e1 + kap] = v;
                               }
+                            },
+                            [&](T v) {
+                              if (ENDS) *num = v;
                             });
   }
   __syncthreads();
@@ -525,8 +537,8 @@ __device__ void plane_direct(const PlaneArgs<T>& O, T sg, int q, const T* __rest
   T* bt = reinterpret_cast<T*>(smem);
   T* ex = bt + O.buffers;
   T* alpha = ex + 7 * nt;
-  T* ssum = alpha + IFACE_MAX_ENDS;
-  double* work = reinterpret_cast<double*>(ssum + IFACE_MAX_ENDS);
+  T* num = alpha + IFACE_MAX_ENDS;
+  double* work = reinterpret_cast<double*>(num + IFACE_MAX_ENDS);
   const int ncell = (int)O.ncell;
   if (threadIdx.x < 2 * IFACE_MAX_ENDS) alpha[threadIdx.x] = 0;
   size_t b0 = 0;
@@ -547,21 +559,12 @@ __device__ void plane_direct(const PlaneArgs<T>& O, T sg, int q, const T* __rest
     const DirectArgs<T> A = O.pc[p];
     const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
     piece_forward(A, S, reinterpret_cast<Cpl<T>*>(bt + b0), nt);
-    if (O.I.k) {
-      piece_tri<T, true>(A, S, bt + b0, sg, (T)0, ex, work, nt);
-      if (q == O.I.qs && threadIdx.x < 32) {
-        const int o = slot_at(A, S, 0), ns = A.cls == LINES_PAIR ? 1 : 2;
-        T s = 0;
-        for (int n = threadIdx.x; n < A.N; n += 32) s = fma(A.w[n], bt[b0 + o + n * ns], s);
-        s = warp_sum_t(s);
-        if (threadIdx.x == 0) ssum[p] = s;
-      }
-    }
+    if (O.I.k) piece_tri<T, true>(A, S, bt + b0, sg, (T)0, ex, work, num + p, nt);
     b0 += S.buf;
   }
   if (O.I.k) {
     __syncthreads();
-    iface_solve(O.I, q, work, ssum, alpha, nt, [&](int e, T v) {
+    iface_solve(O.I, q, work, num, alpha, nt, [&](int e, T v) {
       size_t b = 0;
       for (int p = 0; p < O.np; ++p) {
         const DirectArgs<T>& A = O.pc[p];
@@ -577,7 +580,7 @@ __device__ void plane_direct(const PlaneArgs<T>& O, T sg, int q, const T* __rest
   for (int p = 0; p < O.np; ++p) {
     const DirectArgs<T> A = O.pc[p];
     const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
-    piece_tri<T, false>(A, S, bt + b0, sg, O.I.k && q == O.I.qs ? alpha[p] : (T)0, ex, nullptr, nt);
+    piece_tri<T, false>(A, S, bt + b0, sg, alpha[p], ex, nullptr, nullptr, nt);
     piece_backward(A, S, reinterpret_cast<Cpl<T>*>(bt + b0), nt);
     b0 += S.buf;
   }

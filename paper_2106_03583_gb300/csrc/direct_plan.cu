@@ -325,9 +325,8 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   const HostLevel& l0 = P->lev[0];
   const bool f64 = P->precision == SNAC_FP64;
   const std::vector<double> wm = piece_widths(P, p, ax, true);
-  D.w = piece_widths(P, p, 1 - ax, false);
   D.M = (int)wm.size();
-  D.N = (int)D.w.size();
+  D.N = (int)piece_widths(P, p, 1 - ax, false).size();
   D.kind = p.kind;
   D.cls = !fft_piece(p, wm) ? LINES_DENSE : p.kind == KIND_ND || p.kind == KIND_DN ? LINES_DCT4 : LINES_PAIR;
   D.xl = ax == 0 ? 1 : 0;
@@ -417,7 +416,8 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
     tri[4 * n + 2] = D.cscale * tau;
     tri[4 * n + 3] = c.hi > 0.0 ? c.lo / c.hi : 0.0;
   }
-  D.singular = (p.kind == KIND_PP || p.kind == KIND_NN) && p.side[0] != SNAC_BC_DIRICHLET && p.side[1] != SNAC_BC_DIRICHLET;
+  D.pin = (p.iface[0] || p.iface[1]) && (p.kind == KIND_PP || p.kind == KIND_NN) && p.side[0] != SNAC_BC_DIRICHLET &&
+          p.side[1] != SNAC_BC_DIRICHLET;
   // where the lines live: plane offset of (m, n) = base[n nbm + mblk[m]] + m mstr[n]
   const int gm = (int)p.rows[0].blk.size();
   std::vector<int> mblk(M), base((size_t)N * gm), mstr(N);
@@ -475,8 +475,8 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
       return st;
   }
   if ((st = up_inner(P, &D.d_tw, tw)) || (st = up_inner(P, &D.d_lam, D.lam)) || (st = up_inner(P, &D.d_tri, tri)) ||
-      (st = up_inner(P, &D.d_w, D.w)) || (st = up_vec(P, &D.d_perm, perm)) || (st = up_vec(P, &D.d_base, base)) ||
-      (st = up_vec(P, &D.d_mblk, mblk)) || (st = up_vec(P, &D.d_mstr, mstr)))
+      (st = up_vec(P, &D.d_perm, perm)) || (st = up_vec(P, &D.d_base, base)) || (st = up_vec(P, &D.d_mblk, mblk)) ||
+      (st = up_vec(P, &D.d_mstr, mstr)))
     return st;
   return SNAC_OK;
 }
@@ -518,11 +518,9 @@ int build_iface(snac_plan* P, const Layout& L) {
       }
   I.E = I.eo[I.nends];
   for (int l = 0; l < P->nz; ++l)
-    if (P->sigma[l] == 0.0) I.qs = l;
-  if (I.qs >= 0)
-    for (size_t p = 0; p < L.pc.size(); ++p)
-      if (D.pc[p].singular) I.sp[I.ns++] = (int)p;
-  if (I.ns == 0) I.qs = -1;
+    if (P->singular && P->sigma[l] == 0.0) I.qs = l;
+  for (size_t p = 0; p < L.pc.size(); ++p)
+    if (D.pc[p].pin) I.sp[I.ns++] = (int)p;
   I.kk = I.k + I.ns;
   std::vector<double> Y((size_t)I.E * I.kk, 0.0), Z((size_t)I.kk * I.E, 0.0);
   for (int j = 0; j < I.k; ++j) {
@@ -541,8 +539,8 @@ int build_iface(snac_plan* P, const Layout& L) {
   int st;
   if ((st = up_vec(P, &I.d_Y, Y)) || (st = up_inner(P, &I.d_Z, Z)) ||
       (st = plan_alloc(P, (void**)&I.d_KT, (size_t)P->nz * I.kk * I.kk * sizeof(double))) ||
-      (st = plan_alloc(P, &I.d_ends, (size_t)P->nz * I.E * w)) || (st = plan_alloc(P, &I.d_alpha, D.pc.size() * w)) ||
-      (st = plan_alloc(P, &I.d_ssum, D.pc.size() * w)))
+      (st = plan_alloc(P, &I.d_ends, (size_t)P->nz * I.E * w)) || (st = plan_alloc(P, &I.d_alpha, (size_t)P->nz * IFACE_MAX_ENDS * w)) ||
+      (st = plan_alloc(P, &I.d_num, (size_t)P->nz * IFACE_MAX_ENDS * w)))
     return st;
   I.Zh.swap(Z);
   return SNAC_OK;

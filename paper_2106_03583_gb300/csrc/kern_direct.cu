@@ -491,14 +491,16 @@ __global__ void __launch_bounds__(256, 2) k_dense(const DirectArgs<T> A, const T
 // largest where lambda + sigma is smallest. These few systems (list) therefore set the residual a
 // correction step can reach: with all of them in FP32 the second step on the 1024 x 512 x 512 channel ends
 // at 0.9-1.5e-10 relative residual, with the list in FP64 at 5e-11.
-// ENDS: only the first and last unknowns, into the end vector of the interface systems.
+// ENDS: only the first and last unknowns, into the end vector of the interface systems, and num (tri_segment) of
+// the pinned ones; pin, alpha, num: of the piece, IFACE_MAX_ENDS apart per wavenumber.
 constexpr int LOW_KG = 8, LOW_R = 8;
 template <bool ENDS>
 __global__ void __launch_bounds__(512, 1) k_tri_low(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
                                                   const double* __restrict__ sigma, double cscale, double scale,
                                                   const int* __restrict__ list, int nlist, int M, int N, int P,
-                                                  long long ncell, int soff, const float* __restrict__ alpha,
-                                                  float* __restrict__ x, float* __restrict__ ends, int E, int e0, int e1) {
+                                                  long long ncell, int soff, int pin, const float* __restrict__ alpha,
+                                                  float* __restrict__ num, float* __restrict__ x,
+                                                  float* __restrict__ ends, int E, int e0, int e1) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int kk = threadIdx.x % LOW_KG, seg = threadIdx.x / LOW_KG;
   const int k = blockIdx.x * LOW_KG + kk;
@@ -507,24 +509,29 @@ __global__ void __launch_bounds__(512, 1) k_tri_low(const TriRow<double>* __rest
   const int q = sys / M, kap = sys - q * M;
   float* col = x + (long long)q * ncell + soff + kap;
   const double tq = live ? -fma(sigma[q], cscale, lam[kap]) : 1.0;
-  tri_segment<double, LOW_R>(tri, N, P, seg, kk, LOW_KG, true, live, tq, scale, alpha ? (double)*alpha : 0.0,
-                             reinterpret_cast<double*>(smem),
+  const bool pinned = pin && live && kap == 0;
+  tri_segment<double, LOW_R>(tri, N, P, seg, kk, LOW_KG, true, live, tq, scale, pinned,
+                             pinned && !ENDS ? (double)alpha[q * IFACE_MAX_ENDS] : 0.0, reinterpret_cast<double*>(smem),
                              [&](int n) { return (double)col[(long long)n * M]; },
                              [&](int n, double v) {
                                if (!ENDS) col[(long long)n * M] = (float)v;
                                else if (n == 0 && e0 >= 0) ends[(long long)q * E + e0 + kap] = (float)v;
                                else if (n == N - 1 && e1 >= 0) ends[(long long)q * E + e1 + kap] = (float)v;
+                             },
+                             [&](double v) {
+                               if (ENDS) num[q * IFACE_MAX_ENDS] = (float)v;
                              });
 }
 
 // The elimination would be bound by arithmetic (14 operations per row, half of them for the pivot's reciprocal,
 // which depends on the plan only), so the reciprocals are kept: [row of DirectTab::qrow][n][kappa], wavenumbers of
-// equal sigma (q and n - q of the real DFT) sharing one set. The solve is then 5 operations per row. FP64 plans walk
+// equal sigma (q and n - q of the real DFT) sharing one set; that of a pinned unknown is kept as zero. The solve is
+// then 5 operations per row. FP64 plans walk
 // the rows twice (k_tri_pre, 48 bytes per cell; 512 x 512 x 256: 1.89 -> 0.69 ms, the FP64 pipe alone takes 0.53);
 // FP32 plans take k_tri_scan, and k_tri_pre only for systems of more than 1024 rows.
 template <typename T>
 __global__ void __launch_bounds__(128) k_tri_factor(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
-                                                  const double* __restrict__ sigma, double cscale, int M, int N,
+                                                  const double* __restrict__ sigma, double cscale, int M, int N, int pin,
                                                   const int* __restrict__ qof, int rows, T* __restrict__ fac) {
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= (long long)rows * M) return;
@@ -538,7 +545,7 @@ __global__ void __launch_bounds__(128) k_tri_factor(const TriRow<double>* __rest
     const double den = s + w.hi;
     const double inv = den > 0 ? 1.0 / den : 0.0;
     g = s * inv;
-    f[(long long)n * M] = (T)inv;
+    f[(long long)n * M] = pin && kap == 0 && n == N - 1 ? (T)0 : (T)inv;
   }
 }
 
@@ -583,8 +590,7 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
     for (int u = TRI_U - 1; u >= 0; --u) {
       if (n0 + u >= N) continue;
       y = fma(A.tri[n0 + u].hi * f[u], y, v[u]);
-      // an exactly singular system ends in a zero pivot: its last unknown is the piece's constant
-      if (n0 + u == N - 1 && alpha != nullptr && f[u] == (T)0) y = *alpha;
+      if (n0 + u == N - 1 && A.pin && kap == 0) y = alpha[q * IFACE_MAX_ENDS];
       x[(long long)(n0 + u) * M] = y;
     }
   }
@@ -599,25 +605,24 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
 // sweeps are first-order recurrences, so a segment is an affine map of the value that enters it: the segments'
 // maps are composed in order by the first segment's thread, then each thread runs its rows again from the right
 // value, rounding as the sequential sweep does. All coefficients are >= 0. 2^lg systems per CTA.
-// ENDS: only the first and last unknowns (and ssum, see k_tri_ends), nothing is written to the field.
+// ENDS: only the first and last unknowns and num (see k_tri_ends), nothing is written to the field.
 constexpr int SCAN_NT = 512, TRI_R = 16;
 template <bool ENDS>
 __global__ void __launch_bounds__(SCAN_NT, 2) k_tri_scan(const DirectArgs<float> A, int lg, int P, const int* __restrict__ qrow,
                                                         const unsigned char* __restrict__ low, const float* __restrict__ fac,
                                                         const float* __restrict__ alpha, float* __restrict__ x,
-                                                        float* __restrict__ ends, int E, int qs, float* __restrict__ ssum) {
+                                                        float* __restrict__ ends, int E, float* __restrict__ num) {
   constexpr int R = TRI_R;
   extern __shared__ __align__(16) unsigned char smem[];
   float2* lohi = reinterpret_cast<float2*>(smem);             // [P R] couplings
   float2* ex = lohi + P * R;                                  // [P][2^lg] segment maps, then entering values
-  float* w = reinterpret_cast<float*>(ex + (P << lg));        // ENDS: [P][2^lg] partial sums
   const int N = A.N, M = A.M, KG = 1 << lg;
   const int kk = threadIdx.x & (KG - 1), seg = threadIdx.x >> lg;
   const long long sys = ((long long)blockIdx.x << lg) + kk;
   const bool in = sys < (long long)A.nq * M;
   const bool live = in && !low[sys];  // (k_tri_low solves the others)
   const int q = in ? (int)(sys / M) : 0, kap = in ? (int)(sys - (long long)q * M) : 0;
-  const bool sum = ENDS && in && q == qs && kap == 0;
+  const bool pinned = live && A.pin && kap == 0;
   const int n0 = seg * R;
   float* col = x + (long long)q * A.ncell + A.soff + kap + (long long)n0 * M;
   const float* fc = fac + (long long)qrow[q] * N * M + kap + (long long)n0 * M;
@@ -625,19 +630,12 @@ __global__ void __launch_bounds__(SCAN_NT, 2) k_tri_scan(const DirectArgs<float>
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const bool ok = n0 + r < N;
-    v[r] = ok && (live || sum) ? col[(long long)r * M] : 0.0f;
+    v[r] = ok && live ? col[(long long)r * M] : 0.0f;
     f[r] = ok && live ? fc[(long long)r * M] : 0.0f;
   }
   for (int n = threadIdx.x; n < P * R; n += blockDim.x) {
     const bool ok = n < N;
     lohi[n] = make_float2(ok ? A.tri[n].lo : 0.0f, ok ? A.tri[n].hi : 0.0f);
-  }
-  if (sum) {
-    float t = 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-      if (n0 + r < N) t = fma(A.w[n0 + r], v[r], t);
-    w[threadIdx.x] = t;
   }
   __syncthreads();
   float2* e = ex + threadIdx.x;
@@ -652,23 +650,25 @@ __global__ void __launch_bounds__(SCAN_NT, 2) k_tri_scan(const DirectArgs<float>
   *e = make_float2(d, a);
   __syncthreads();
   if (seg == 0) {
-    float g = 0, t = 0;
+    float g = 0;
     for (int k = kk; k < P << lg; k += KG) {
       const float2 m = ex[k];
       ex[k].x = g;
       g = fma(m.y, g, m.x);
-      if (sum) t += w[k];
     }
-    if (sum) *ssum = t;
   }
   __syncthreads();
   d = e->x;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    d = fma(lohi[n0 + r].x, d, v[r]) * f[r];
-    v[r] = d;
-    // an exactly singular system ends in a zero pivot: its last unknown is the piece's constant
-    if (n0 + r == N - 1 && alpha != nullptr && f[r] == 0.0f) v[r] = *alpha;
+    d = fma(lohi[n0 + r].x, d, v[r]);
+    if (n0 + r == N - 1 && pinned) {
+      if (ENDS) num[q * IFACE_MAX_ENDS] = d;
+      v[r] = ENDS ? 0.0f : alpha[q * IFACE_MAX_ENDS];
+    } else {
+      d *= f[r];
+      v[r] = d;
+    }
     if (ENDS && n0 + r == N - 1 && live && A.e1 >= 0) ends[(long long)q * E + A.e1 + kap] = v[r];
   }
   float y = 0, c = 1;
@@ -708,32 +708,27 @@ inline int scan_lg(int P) {
 
 template <bool ENDS>
 void launch_scan(const DirectArgs<float>& A, int lg, const int* qrow, const unsigned char* low, const float* fac,
-                 const float* alpha, float* x, float* ends, int E, int qs, float* ssum, cudaStream_t s) {
+                 const float* alpha, float* x, float* ends, int E, float* num, cudaStream_t s) {
   const int P = (A.N + TRI_R - 1) / TRI_R;
   const long long sys = (long long)A.nq * A.M;
-  const size_t smem = sizeof(float2) * ((size_t)P * TRI_R + ((size_t)P << lg)) + (ENDS ? sizeof(float) * ((size_t)P << lg) : 0);
+  const size_t smem = sizeof(float2) * ((size_t)P * TRI_R + ((size_t)P << lg));
   k_tri_scan<ENDS><<<(unsigned)((sys + (1 << lg) - 1) >> lg), P << lg, smem, s>>>(A, lg, P, qrow, low, fac, alpha, x, ends, E,
-                                                                                  qs, ssum);
+                                                                                  num);
 }
 
 // First and last unknowns of every system of a piece (the end values of the interface systems), from the
-// kept pivots (the listed systems of an FP32 plan: k_tri_low). ssum (slot 0 of the singular wavenumber): the
-// weighted sum of its right-hand side.
+// kept pivots (the listed systems of an FP32 plan: k_tri_low). num: what the elimination leaves in the last row
+// of the pinned systems (their last unknown is taken as zero).
 template <typename T>
 __global__ void __launch_bounds__(128, 8) k_tri_ends(const DirectArgs<T> A, const int* __restrict__ qrow,
                                                    const unsigned char* __restrict__ low, const T* __restrict__ fac,
-                                                   const T* __restrict__ x, T* __restrict__ ends, int E, int qs,
-                                                   T* __restrict__ ssum) {
+                                                   const T* __restrict__ x, T* __restrict__ ends, int E,
+                                                   T* __restrict__ num) {
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= (long long)A.nq * A.M) return;
   const int q = (int)(sys / A.M), kap = (int)(sys - (long long)q * A.M);
   const int N = A.N, M = A.M;
   x += (long long)q * A.ncell + A.soff + kap;
-  if (q == qs && kap == 0) {
-    T s = 0;
-    for (int n = 0; n < N; ++n) s = fma(A.w[n], x[(long long)n * M], s);
-    *ssum = s;
-  }
   if (sizeof(T) == 4 && low[sys]) return;
   fac += (long long)qrow[q] * N * M + kap;
   const T sc = -A.scale;
@@ -750,7 +745,9 @@ __global__ void __launch_bounds__(128, 8) k_tri_ends(const DirectArgs<T> A, cons
     for (int u = 0; u < TRI_U; ++u) {
       if (n0 + u >= N) break;
       const TriRow<T> w = A.tri[n0 + u];
-      d = fma(w.lo, d, sc * v[u]) * f[u];
+      d = fma(w.lo, d, sc * v[u]);
+      if (n0 + u == N - 1 && A.pin && kap == 0) num[q * IFACE_MAX_ENDS] = d;
+      d *= f[u];
       F = fma(pi, d, F);
       pi *= w.hi * f[u];
     }
@@ -809,10 +806,10 @@ cudaError_t tri_t(snac_plan* P, const DirectTab& D, const DirectArgs<T>& A, cons
     if (D.nlow)
       k_tri_low<false><<<(D.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
           (const TriRow<double>*)D.d_tri64, D.d_lam64, P->d_sigma64, D.cscale, D.cscale / D.theta, D.d_lowlist,
-          D.nlow, A.M, A.N, lsegs, A.ncell, A.soff, alpha, u, nullptr, 0, -1, -1);
+          D.nlow, A.M, A.N, lsegs, A.ncell, A.soff, A.pin, alpha, nullptr, u, nullptr, 0, -1, -1);
     const int lg = scan_lg((A.N + TRI_R - 1) / TRI_R);
     if (lg >= 0)
-      launch_scan<false>(A, lg, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u, nullptr, 0, -1, nullptr, s);
+      launch_scan<false>(A, lg, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u, nullptr, 0, nullptr, s);
     else
       k_tri_pre<T><<<g128, 128, 0, s>>>(A, P->direct.d_qrow, D.d_low, (const T*)D.d_fac, alpha, u);
   } else {
@@ -842,20 +839,20 @@ cudaError_t direct_t(snac_plan* P, cudaStream_t s) {
         if (d.nlow)
           k_tri_low<true><<<(d.nlow + LOW_KG - 1) / LOW_KG, LOW_KG * lsegs, 7 * sizeof(double) * LOW_KG * lsegs, s>>>(
               (const TriRow<double>*)d.d_tri64, d.d_lam64, P->d_sigma64, d.cscale, d.cscale / d.theta, d.d_lowlist,
-              d.nlow, d.M, d.N, lsegs, A[p].ncell, A[p].soff, nullptr, u, (T*)D.it.d_ends, D.it.E, A[p].e0, A[p].e1);
+              d.nlow, d.M, d.N, lsegs, A[p].ncell, A[p].soff, A[p].pin, nullptr, (T*)D.it.d_num + p, u, (T*)D.it.d_ends, D.it.E,
+              A[p].e0, A[p].e1);
       }
-      const int qs = d.singular ? D.it.qs : -1;
       bool done = false;
       if constexpr (sizeof(T) == 4) {
         const int lg = scan_lg((d.N + TRI_R - 1) / TRI_R);
         done = lg >= 0;
         if (done)
-          launch_scan<true>(A[p], lg, D.d_qrow, d.d_low, (const T*)d.d_fac, nullptr, u, (T*)D.it.d_ends, D.it.E, qs,
-                            (T*)D.it.d_ssum + p, s);
+          launch_scan<true>(A[p], lg, D.d_qrow, d.d_low, (const T*)d.d_fac, nullptr, u, (T*)D.it.d_ends, D.it.E,
+                            (T*)D.it.d_num + p, s);
       }
       if (!done)
         k_tri_ends<T><<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(A[p], D.d_qrow, d.d_low, (const T*)d.d_fac, u,
-                                                                   (T*)D.it.d_ends, D.it.E, qs, (T*)D.it.d_ssum + p);
+                                                                   (T*)D.it.d_ends, D.it.E, (T*)D.it.d_num + p);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = launch_iface(P, s);
@@ -880,8 +877,8 @@ cudaError_t launch_tri_factor(snac_plan* P, const DirectTab& D, const int* d_qof
   const TriRow<double>* tri = (const TriRow<double>*)(f64 ? D.d_tri : (void*)D.d_tri64);
   const double* lam = f64 ? (const double*)D.d_lam : D.d_lam64;
   const unsigned grid = (unsigned)(((long long)rows * D.M + 127) / 128);
-  if (f64) k_tri_factor<double><<<grid, 128, 0, s>>>(tri, lam, P->d_sigma64, D.cscale, D.M, D.N, d_qof, rows, (double*)D.d_fac);
-  else k_tri_factor<float><<<grid, 128, 0, s>>>(tri, lam, P->d_sigma64, D.cscale, D.M, D.N, d_qof, rows, (float*)D.d_fac);
+  if (f64) k_tri_factor<double><<<grid, 128, 0, s>>>(tri, lam, P->d_sigma64, D.cscale, D.M, D.N, D.pin, d_qof, rows, (double*)D.d_fac);
+  else k_tri_factor<float><<<grid, 128, 0, s>>>(tri, lam, P->d_sigma64, D.cscale, D.M, D.N, D.pin, d_qof, rows, (float*)D.d_fac);
   return cudaGetLastError();
 }
 

@@ -3,9 +3,12 @@
 //   u_b - u_a = phi_j,   A_p u = f + sum_j (-c_a phi_j at a_j, +c_b phi_j at b_j),
 // so (I - Y^T R_q Z^T) phi = Y^T (end values of the solution for f): Z takes the fluxes to the spectral
 // right-hand sides of the pieces' end rows, R_q holds each system's response of its end rows to its end
-// rows, Y takes end values to jumps. A piece whose slot 0 is singular for the wavenumber of zero shift (no
-// Dirichlet face) is solved up to a constant alpha, an extra unknown, with the compatibility of its
-// right-hand side as the extra equation. The inverse of every system is kept with the plan.
+// rows, Y takes end values to jumps. A piece without a Dirichlet face is singular for a zero shift, and nearly
+// so for a small one: R of its slot 0 then grows like 1 / shift and swamps the system (with shift -1e-8 of a
+// unit box no step reduced the residual in FP64, with -1e-4 none in FP32). So that slot's system is pinned for
+// every wavenumber: its last unknown alpha is an unknown of the interface system, all others follow from it by
+// h (1 at a zero shift) and its last row, eliminated, is the extra equation den alpha = num. The inverse of
+// every system is kept with the plan.
 #include <cmath>
 #include <vector>
 
@@ -15,10 +18,12 @@ namespace snac {
 namespace {
 
 // R of one system: responses of the first / last unknown to a unit right-hand side in the first / last row
-// (as the solve scales them), {00, 0N, N0, NN}.
+// (as the solve scales them), {00, 0N, N0, NN}. Of a pinned system also {h of the first row, what a unit in the
+// first row leaves in the eliminated last one, den}.
 __global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
                                             const double* __restrict__ sigma, double cscale, double scale, int nq,
-                                            int M, int N, double4* __restrict__ resp) {
+                                            int M, int N, int pin, double4* __restrict__ resp,
+                                            double4* __restrict__ pinned) {
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= (long long)nq * M) return;
   const int q = (int)(sys / M), kap = (int)(sys - (long long)q * M);
@@ -28,8 +33,13 @@ __global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__
     const TriRow<double> w = tri[n];
     const double s = fma(w.lo, g, w.tau + tq), den = s + w.hi;
     inv = den > 0 ? 1.0 / den : 0.0;
+    d = n == 0 ? 1.0 : w.lo * d;
+    if (n == N - 1 && pin && kap == 0) {
+      pinned[q] = make_double4(pi, d, den, 0.0);
+      inv = 0.0;
+    }
     g = s * inv;
-    d = (n == 0 ? 1.0 : w.lo * d) * inv;
+    d *= inv;
     F = fma(pi, d, F);
     plast = pi;
     pi *= w.hi * inv;
@@ -38,17 +48,18 @@ __global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__
 }
 
 struct BuildArgs {
-  int k, kk, E, ns, qs, gs, nends;
+  int k, kk, E, ns, qs, nends;
   int ep[IFACE_MAX_ENDS], ee[IFACE_MAX_ENDS], eo[IFACE_MAX_ENDS + 1], sp[IFACE_MAX_ENDS];
   int em[IFACE_MAX_ENDS];                 // slots of the end's piece
-  double we[IFACE_MAX_ENDS];              // width of the end's row
+  double sc[IFACE_MAX_ENDS];              // scale of the right-hand sides of a pinned piece
+  const double4* pinned[IFACE_MAX_ENDS];  // of a pinned piece, [q]
   const double4* resp[IFACE_MAX_ENDS];    // of the end's piece, [q][kappa]
   const double* Y;
   const double* Z;
 };
 
 // K = I - Y^T R_q Z^T, a 32 x 32 tile per CTA of 256 threads (2 x 2 entries each); the rows and columns of
-// the singular pieces' constants beyond.
+// the pinned pieces' unknowns beyond.
 constexpr int KT = 32;
 __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __restrict__ K) {
   __shared__ double ys[KT][KT + 1], ws[KT][KT + 1];
@@ -94,15 +105,15 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
       double v = (j == i ? 1.0 : 0.0) - acc[a][b];
       if (j >= A.k || i >= A.k) {
         v = j == i ? 1.0 : 0.0;
-        if (q == A.qs) {
-          const bool implied = A.gs && j == A.kk - 1;  // the last constraint of a singular problem
-          v = implied && i == j ? 1.0 : 0.0;
-          if (!implied && (j < A.k || i < A.k)) {
-            const int p = A.sp[(j < A.k ? i : j) - A.k];
+        if (!(q == A.qs && j == A.kk - 1)) {  // (the last equation of a singular problem is implied: alpha = 0)
+          const int a = (j < A.k ? i : j) - A.k, p = A.sp[a];
+          const double4 R = A.pinned[a][q];
+          v = j == i ? R.z : 0.0;
+          if (j < A.k || i < A.k)
             for (int u = 0; u < A.nends; ++u)
               if (A.ep[u] == p)
-                v += j < A.k ? -A.Y[(size_t)A.eo[u] * A.kk + j] : A.we[u] * A.Z[(size_t)i * A.E + A.eo[u]];
-          }
+                v += j < A.k ? -A.Y[(size_t)A.eo[u] * A.kk + j] * (A.ee[u] ? 1.0 : R.x)
+                             : A.sc[a] * A.Z[(size_t)i * A.E + A.eo[u]] * (A.ee[u] ? 1.0 : R.y);
         }
       }
       K[((size_t)q * A.kk + j) * A.kk + i] = v;
@@ -110,7 +121,7 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
 }
 
 // In-place Gauss-Jordan inverse of every K, one CTA each. No pivoting: K is the identity plus a product
-// of positive operators, and the constraints come last.
+// of positive operators, and the pinned unknowns come last.
 __global__ void __launch_bounds__(1024) k_invert(double* __restrict__ Kq, int n) {
   extern __shared__ double sh[];
   double* rp = sh;        // pivot row / pivot
@@ -153,7 +164,7 @@ __global__ void __launch_bounds__(INT) k_iface(const IfaceArgs<T> I, long long n
   for (int e = threadIdx.x; e < I.E; e += INT) work[e] = (double)I.ends[(size_t)q * I.E + e];
   __syncthreads();
   T* xq = x + (long long)q * ncell;
-  iface_solve(I, q, work, I.ssum, I.alpha, INT, [&](int e, T v) {
+  iface_solve(I, q, work, I.num + q * IFACE_MAX_ENDS, I.alpha + q * IFACE_MAX_ENDS, INT, [&](int e, T v) {
     int u = 0;
     while (u + 1 < I.nends && e >= I.eo[u + 1]) ++u;
     xq[I.row[u] + e - I.eo[u]] += v;
@@ -195,7 +206,6 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   A.E = I.E;
   A.ns = I.ns;
   A.qs = I.qs;
-  A.gs = P->singular ? 1 : 0;
   A.nends = I.nends;
   for (int a = 0; a < I.ns; ++a) A.sp[a] = I.sp[a];
   double* dZ = (double*)get(I.Zh.size() * sizeof(double));
@@ -203,16 +213,17 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(dZ, I.Zh.data(), I.Zh.size() * sizeof(double), cudaMemcpyHostToDevice, s);
   A.Y = I.d_Y;
   A.Z = dZ;
-  std::vector<double4*> resp(D.pc.size(), nullptr);
+  std::vector<double4*> resp(D.pc.size(), nullptr), pinned(D.pc.size(), nullptr);
   for (size_t p = 0; p < D.pc.size(); ++p) {
     const DirectTab& d = D.pc[p];
     resp[p] = (double4*)get((size_t)P->nz * d.M * sizeof(double4));
+    if (d.pin) pinned[p] = (double4*)get((size_t)P->nz * sizeof(double4));
     if (e != cudaSuccess) break;
     const TriRow<double>* tri = (const TriRow<double>*)(f64 ? d.d_tri : (void*)d.d_tri64);
     const double* lam = f64 ? (const double*)d.d_lam : d.d_lam64;
     const long long sys = (long long)P->nz * d.M;
     k_resp<<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(tri, lam, P->d_sigma64, d.cscale, d.cscale / d.theta, P->nz,
-                                                        d.M, d.N, resp[p]);
+                                                        d.M, d.N, d.pin, resp[p], pinned[p]);
     e = cudaGetLastError();
   }
   for (int u = 0; u <= I.nends; ++u) A.eo[u] = I.eo[u];
@@ -221,8 +232,11 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
     A.ep[u] = I.ep[u];
     A.ee[u] = I.ee[u];
     A.em[u] = d.M;
-    A.we[u] = I.ee[u] ? d.w.back() : d.w.front();
     A.resp[u] = resp[I.ep[u]];
+  }
+  for (int a = 0; a < I.ns; ++a) {
+    A.sc[a] = D.pc[I.sp[a]].cscale / D.pc[I.sp[a]].theta;
+    A.pinned[a] = pinned[I.sp[a]];
   }
   if (e == cudaSuccess) {
     const unsigned t = (unsigned)((I.kk + KT - 1) / KT);

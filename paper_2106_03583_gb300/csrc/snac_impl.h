@@ -185,7 +185,7 @@ struct DirectTab {
   double theta = 1.0;      // inverse times forward transform
   void* d_F = nullptr;     // LINES_DENSE: [m][kappa] and [kappa][m] matrices of the transform and its inverse
   void* d_B = nullptr;
-  bool singular = false;   // all-Neumann / periodic: a zero shift makes slot 0's system singular
+  bool pin = false;        // all-Neumann / periodic piece of several: its constant is an unknown of the interface system
   void* d_fac = nullptr;             // plans not on chip: reciprocal pivots (k_tri_pre), inner type
   int nlow = 0;                      // mixed plans: systems solved in FP64 arithmetic (k_tri_low)
   int* d_lowlist = nullptr;          // their numbers q M + kappa
@@ -196,29 +196,28 @@ struct DirectTab {
   void* d_tri = nullptr;
   double* d_lam64 = nullptr;  // the same in FP64 (mixed plans; FP64 plans: the tables above)
   double* d_tri64 = nullptr;
-  void* d_w = nullptr;        // cell widths along the tridiagonal axis
   int* d_base = nullptr;
   int* d_mblk = nullptr;
   int* d_mstr = nullptr;
   // host copies the interface setup needs
-  std::vector<double> w, lam, F, B;  // F[kappa M + m], B[m M + kappa] (LINES_DENSE)
+  std::vector<double> lam, F, B;  // F[kappa M + m], B[m M + kappa] (LINES_DENSE)
 };
 
 // The interfaces between the pieces of a plan (kern_iface.cu).
 constexpr int IFACE_MAX_ENDS = 16;
 struct IfaceTab {
-  int k = 0, kk = 0, E = 0;  // interface cells; with one unknown per singular piece; spectral end values
+  int k = 0, kk = 0, E = 0;  // interface cells; with one unknown per pinned piece; spectral end values
   int nends = 0;             // ends (piece, first or last row) that carry interface cells
   int ep[IFACE_MAX_ENDS] = {}, ee[IFACE_MAX_ENDS] = {}, eo[IFACE_MAX_ENDS + 1] = {};
-  int qs = -1;               // wavenumber (local) with a zero shift, where pieces are singular; -1: none
-  int ns = 0;                // singular pieces
+  int qs = -1;               // wavenumber (local) whose whole system is singular; -1: none
+  int ns = 0;                // pinned pieces
   int sp[IFACE_MAX_ENDS] = {};
   double* d_Y = nullptr;     // [E][kk]: end values -> jump of u across every interface cell
   void* d_Z = nullptr;       // [kk][E]: fluxes -> right-hand sides of the end rows
   double* d_KT = nullptr;    // [q][kk][kk]: transposed inverse of the interface system
   void* d_ends = nullptr;    // [q][E]: end values of a solve
-  void* d_alpha = nullptr;   // [piece]: constant of every singular piece
-  void* d_ssum = nullptr;    // [piece]: weighted sum of its slot-0 right-hand side
+  void* d_alpha = nullptr;   // [q][IFACE_MAX_ENDS]: by piece, the last unknown of its pinned system
+  void* d_num = nullptr;     // [q][IFACE_MAX_ENDS]: by piece, that unknown's eliminated right-hand side
   std::vector<double> Zh;    // host copy, until the systems are set up
 };
 
