@@ -321,6 +321,9 @@ int up_vec(snac_plan* P, V** d, const std::vector<V>& v) {
   return plan_upload(P, reinterpret_cast<void**>(d), v.data(), v.size() * sizeof(V));
 }
 
+// The layout has no direct solve after all: the plan keeps its V-cycles.
+constexpr int NOT_DIRECT = 1;
+
 int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   const HostLevel& l0 = P->lev[0];
   const bool f64 = P->precision == SNAC_FP64;
@@ -348,7 +351,8 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   for (int k = 0; k < M / 2; ++k) put(D.t4a + k, -M_PI * (4.0 * k + 1.0) / (4.0 * M));
   for (int k = 0; k < M / 2; ++k) put(D.t4b + k, -M_PI * k / (double)M);
   const std::vector<int> perm = fft_perm(D.fft);
-  // eigenvalues of the slots and the tridiagonal rows, scaled by a power of two to couplings of about 1
+  // eigenvalues of the slots and the tridiagonal rows, scaled by a power of two to couplings of about 1 (cell
+  // widths in any unit: their squares may lie near the ends of the range)
   double h = 0.0;
   for (double v : wm) h += v;
   h /= M;
@@ -360,24 +364,33 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   }
   ct.front().lo = 0.0;  // (an interface is a Neumann face of the piece)
   ct.back().hi = 0.0;
-  // dense: A = W^-1/2 Q Lam Q^T W^1/2 along the axis, F = Q^T W^1/2, B = W^-1/2 Q, smallest |lambda| first
-  std::vector<double> ev;
-  if (D.cls == LINES_DENSE) {
-    std::vector<Coef<double>> cm;
+  std::vector<Coef<double>> cm;
+  if (D.cls == LINES_DENSE)
     for (int b : p.rows[0].blk) {
       const BlockDev& d = l0.blk[b];
       if (ax == 0) cm.insert(cm.end(), l0.cx.begin() + d.xo, l0.cx.begin() + d.xo + d.nx);
       else cm.insert(cm.end(), l0.cy.begin() + d.yo, l0.cy.begin() + d.yo + d.ny);
     }
+  double big = D.cls == LINES_DENSE ? 0.0 : 4.0 / (h * h);
+  for (const Coef<double>& c : cm) big = std::max(big, -2.0 * c.d);
+  bool finite = true;
+  for (const Coef<double>& c : ct) {
+    big = std::max(big, c.lo + c.hi);
+    finite = finite && std::isfinite(c.d);
+  }
+  if (!finite || !std::isfinite(big)) return NOT_DIRECT;
+  int ex = 0;
+  std::frexp(big, &ex);
+  D.cscale = std::ldexp(1.0, -ex);
+  // dense: A = W^-1/2 Q Lam Q^T W^1/2 along the axis, F = Q^T W^1/2, B = W^-1/2 Q, smallest |lambda| first
+  std::vector<double> ev;
+  if (D.cls == LINES_DENSE) {
     std::vector<double> dd(M), ee(M, 0.0), Z;
     for (int m = 0; m < M; ++m) {
-      dd[m] = cm[m].d;
-      if (m + 1 < M) ee[m] = std::sqrt(cm[m].hi * cm[m + 1].lo);
+      dd[m] = D.cscale * cm[m].d;
+      if (m + 1 < M) ee[m] = std::sqrt((D.cscale * cm[m].hi) * (D.cscale * cm[m + 1].lo));
     }
-    if (!tridiag_eigen(dd, ee, Z)) {
-      set_error("the eigenvectors along a plane axis did not converge");
-      return SNAC_ERR_LAYOUT;
-    }
+    if (!tridiag_eigen(dd, ee, Z)) return NOT_DIRECT;
     std::vector<int> order(M);
     for (int k = 0; k < M; ++k) order[k] = k;
     std::sort(order.begin(), order.end(), [&](int a, int b) { return dd[a] > dd[b]; });
@@ -397,14 +410,9 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
     int se;
     if ((se = up_inner(P, &D.d_F, ft)) || (se = up_inner(P, &D.d_B, bt))) return se;
   }
-  double big = ev.empty() ? 4.0 / (h * h) : -ev.back();
-  for (const Coef<double>& c : ct) big = std::max(big, c.lo + c.hi);
-  int ex = 0;
-  std::frexp(big, &ex);
-  D.cscale = std::ldexp(1.0, -ex);
   D.lam.resize(M);
   for (int k = 0; k < M; ++k)
-    D.lam[k] = !ev.empty() ? D.cscale * ev[k] : D.cscale * mode_lambda(p.kind, M, p.kind == KIND_DD || p.kind == KIND_DN ? M - 1 - k : k) / (h * h);
+    D.lam[k] = !ev.empty() ? ev[k] : D.cscale * mode_lambda(p.kind, M, p.kind == KIND_DD || p.kind == KIND_DN ? M - 1 - k : k) / (h * h);
   std::vector<double> tri(4 * (size_t)N);
   for (int n = 0; n < N; ++n) {
     const Coef<double>& c = ct[n];
@@ -565,12 +573,8 @@ bool iface_affordable(const snac_plan* P, const Layout& L) {
 
 }  // namespace
 
-// Only with the default schedule: a caller who sets a multigrid option gets the multigrid. Of the two plane
-// axes the cheaper one is transformed, x where they tie (its lines are contiguous).
-int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
-  if (P->nu1 != 2 || P->nu2 != 2 || P->max_cycles != 40 || P->max_coarse != 64 || P->fused != -1 ||
-      P->onchip_opt != 0 || P->bottom_cells != 0 || P->inner_reduction != 0.0 || P->lev[0].ncell >= (1LL << 31))
-    return SNAC_OK;
+// Of the two plane axes the cheaper one is transformed, x where they tie (its lines are contiguous).
+static int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
   Layout best;
   double least = INFINITY;
   for (int t = 0; t < 2; ++t) {
@@ -598,7 +602,7 @@ int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
   return SNAC_OK;
 }
 
-int finish_direct(snac_plan* P) {
+static int finish_direct(snac_plan* P) {
   DirectPlan& D = P->direct;
   const bool f64 = P->precision == SNAC_FP64;
   const size_t w = f64 ? sizeof(double) : sizeof(float);
@@ -663,6 +667,20 @@ int finish_direct(snac_plan* P) {
     set_error(std::string("setting up the direct solves failed: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? SNAC_ERR_OOM : SNAC_ERR_CUDA;
   }
+  return SNAC_OK;
+}
+
+int setup_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
+  if (P->lev[0].ncell >= (1LL << 31)) return SNAC_OK;
+  const size_t mark = P->allocs.size(), bytes = P->bytes;
+  int st = build_direct(P, faces);
+  if (st == SNAC_OK && P->direct.on && P->onchip && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) P->direct.on = false;
+  if (st == SNAC_OK && P->direct.on) st = finish_direct(P);
+  if (st != NOT_DIRECT) return st;
+  for (size_t k = mark; k < P->allocs.size(); ++k) cudaFree(P->allocs[k]);
+  P->allocs.resize(mark);
+  P->bytes = bytes;
+  P->direct = DirectPlan{};
   return SNAC_OK;
 }
 

@@ -828,14 +828,9 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
       P->onchip = P->onchip_opt == 0 && P->nu1 >= 1 && P->nu2 >= 1 && L >= 1 && L < BOTTOM_MAX_LEVELS &&
                   P->lev[0].ncell <= BOTTOM_MAX_CELLS && bottom_layout(P, 0, inner).bytes <= (size_t)BOTTOM_MAX_SMEM;
     }
-    {
-      std::vector<FaceKinds> faces(hb.size());
-      for (size_t b = 0; b < hb.size(); ++b)
-        for (int a = 0; a < 2; ++a)
-          for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
-      if ((st = build_direct(P, faces))) break;
-    }
-    if (P->onchip && P->direct.on && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) P->direct.on = false;
+    // direct solves only with the default schedule: a caller who sets a multigrid option gets the multigrid
+    const bool direct = P->nu1 == 2 && P->nu2 == 2 && P->max_cycles == 40 && P->max_coarse == 64 && P->fused == -1 &&
+                        P->onchip_opt == 0 && P->bottom_cells == 0 && P->inner_reduction == 0.0;
     // the automatic inner reduction: an on-chip plan's V-cycles are cheap next to an outer step,
     // so it asks more of each step (measured on c64: 3 outer steps at 1e-4, 2 at 3e-5, 18 % faster)
     if (P->inner_reduction == 0.0) P->inner_reduction = P->onchip ? 3e-5 : 1e-4;
@@ -972,7 +967,13 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
         break;
       }
     }
-    if (P->direct.on && (st = finish_direct(P))) break;
+    if (direct) {
+      std::vector<FaceKinds> faces(hb.size());
+      for (size_t b = 0; b < hb.size(); ++b)
+        for (int a = 0; a < 2; ++a)
+          for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
+      if ((st = setup_direct(P, faces))) break;
+    }
   } while (0);
   if (st) {
     free_plan(P);

@@ -492,14 +492,13 @@ BottomLayout bottom_layout(const snac_plan* P, int lb, size_t w);
 // Separable plans: every wavenumber's solution of the reduced equations for the right-hand sides in
 // lev[0].d_f (plain order), into mode_solution(P).
 cudaError_t launch_direct(snac_plan* P, cudaStream_t s);
-// Plan creation: the pieces and their tables, where the layout allows direct solves (direct_plan.cu;
-// faces: the face kinds W, E, S, N of every block), and, once the launch shape is known, the pivots, the
-// interface systems and the on-chip tables.
+// End of plan creation: the pieces, their tables, the pivots, the interface systems and the on-chip tables, where
+// the layout allows direct solves (direct_plan.cu; faces: the face kinds W, E, S, N of every block). Direct solves
+// replace V-cycles that the plan has anyway: where their setup is not possible it keeps those.
 struct FaceKinds {
   int k[4];
 };
-int build_direct(snac_plan* P, const std::vector<FaceKinds>& faces);
-int finish_direct(snac_plan* P);
+int setup_direct(snac_plan* P, const std::vector<FaceKinds>& faces);
 cudaError_t launch_tri_factor(snac_plan* P, const DirectTab& D, const int* d_qof, int rows, cudaStream_t s);
 // Interface systems of plans of several pieces: setup (once per plan) and the solve of every wavenumber's
 // fluxes from the end values, added to the spectral right-hand sides.

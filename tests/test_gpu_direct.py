@@ -236,3 +236,21 @@ def test_direct_solve_with_a_nearly_singular_piece(case, precision):
             P = [spsolve((g.plane.A + s * identity(g.plane.n)).tocsc(), x) for s, x in zip(sigma, F)]
             assert rel(host(p), g.from_planes(T.backward(g.kind, np.array(P)))) <= 1e-9
     assert max(steps) <= steps[0] + 1
+
+
+@pytest.mark.parametrize("unit", [2.0 ** -250, 2.0 ** 266])
+def test_dense_transforms_in_any_unit_of_length(unit):
+    """Cell widths times a power of two: the same solution times its square, to rounding."""
+    import torch
+    out = []
+    for scale in (1.0, unit):
+        blocks = build("1", 160, 96, 1.3, 1.5, "DNNN", "DN")
+        f = inputs.divergence_rhs(blocks, 8)
+        for b in blocks:
+            b["dx"] = tuple(np.asarray(w) * scale for w in b["dx"])
+        pl = plan(blocks)
+        p = torch.zeros(len(f), dtype=torch.float64, device="cuda")
+        assert pl.solve(dev(f), p, tol=1e-10)["outer_iters"] == 1 and pl.kernel_stats()["lines_forward"]["launches"] == 1
+        pl.close()
+        out.append(host(p))
+    assert rel(out[1] / unit ** 2, out[0]) <= 1e-13

@@ -51,3 +51,24 @@ r = [lib.snac_pencil_setup(h, 0, 1024, halo, 4096, ctypes.byref(n)),
 out = [st, r, len(launches()), fake.fake_unordered().decode().split()]
 """)
     assert out[:2] == [0, [0, 0, 0]] and out[2] >= 3 and out[3] == []
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_cell_widths_of_any_size(precision):
+    """Widths whose squares or products leave the range of a double: no plan is refused for its eigenvectors, and
+    only couplings that are not numbers lose the direct solve."""
+    out = fake_cuda.run(LAYOUTS + f"""
+out = []
+for scale, first, walls in ((1.0, 1.0, "DNDN"), (1e-75, 1.0, "DNDN"), (1e-100, 1.0, "DNDN"), (1e80, 1.0, "DNDN"),
+                            (1.0, 1e-160, "DNNN"), (1.0, 1e-160, "NNDN")):
+    b = problem([(0, 160, 0, 128)], 160, 128, xf=1.0, yf=1.0, walls=walls)
+    for q in b:
+        q["dx"] = tuple(np.asarray(w) * scale for w in q["dx"])
+        for w in q["dx"][:2]:
+            w[0] *= first
+    fake.fake_reset()
+    st, h = create(b, {precision!r})
+    out.append([st, any("k_tri_factor" in n for n in launches())])
+    lib.snac_plan_destroy(h)
+""")
+    assert out == [[0, True]] * 4 + [[0, False]] * 2
