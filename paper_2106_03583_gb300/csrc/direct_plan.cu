@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <map>
+#include <new>
 #include <vector>
 
 #include "direct_dev.cuh"
@@ -673,10 +674,16 @@ static int finish_direct(snac_plan* P) {
 int setup_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
   if (P->lev[0].ncell >= (1LL << 31)) return SNAC_OK;
   const size_t mark = P->allocs.size(), bytes = P->bytes;
-  int st = build_direct(P, faces);
-  if (st == SNAC_OK && P->direct.on && P->onchip && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) P->direct.on = false;
-  if (st == SNAC_OK && P->direct.on) st = finish_direct(P);
-  if (st != NOT_DIRECT) return st;
+  int st;
+  try {
+    st = build_direct(P, faces);
+    if (st == SNAC_OK && P->direct.on && P->onchip && direct_onchip_smem(P) > (size_t)BOTTOM_MAX_SMEM) st = NOT_DIRECT;
+    if (st == SNAC_OK && P->direct.on) st = finish_direct(P);
+  } catch (const std::bad_alloc&) {
+    st = SNAC_ERR_OOM;
+  }
+  if (st != NOT_DIRECT && st != SNAC_ERR_OOM) return st;
+  set_error("");
   for (size_t k = mark; k < P->allocs.size(); ++k) cudaFree(P->allocs[k]);
   P->allocs.resize(mark);
   P->bytes = bytes;

@@ -72,3 +72,36 @@ for scale, first, walls in ((1.0, 1.0, "DNDN"), (1e-75, 1.0, "DNDN"), (1e-100, 1
     lib.snac_plan_destroy(h)
 """)
     assert out == [[0, True]] * 4 + [[0, False]] * 2
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("name", ["L", "L on chip", "dense", "planes"])
+def test_direct_setup_out_of_memory(name, precision):
+    """A plan whose multigrid fits is created whether the direct solve's tables fit or not, and keeps none of them
+    where they do not; every allocation fails once."""
+    out = fake_cuda.run(LAYOUTS + f"""
+out = []
+b = PROBLEMS[{name!r}]()
+st, h = create(b, {precision!r})
+want = workspace(h)
+lib.snac_plan_destroy(h)
+n = 0
+while True:
+    fake.fake_reset()
+    before = fake.fake_used()
+    fake.fake_fail_after(n)
+    st, h = create(b, {precision!r})
+    fake.fake_fail_after(-1)
+    out.append([st, workspace(h) == fake.fake_used() - before if st == 0 else True, workspace(h) if st == 0 else 0])
+    lib.snac_plan_destroy(h)
+    out[-1].append(fake.fake_used() == before)
+    if out[-1][2] == want:
+        break
+    n += 1
+""")
+    status = [o[0] for o in out]
+    first = status.index(0)
+    assert all(s == -3 for s in status[:first]) and all(s == 0 for s in status[first:])
+    assert all(o[1] and o[3] for o in out)
+    fallback = out[first:-1]   # plans that kept their V-cycles: the same memory, less than with the tables
+    assert len(fallback) >= 8 and len({o[2] for o in fallback}) == 1 and fallback[0][2] < out[-1][2]
