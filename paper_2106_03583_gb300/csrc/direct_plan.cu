@@ -429,7 +429,8 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
           p.side[1] != SNAC_BC_DIRICHLET;
   // where the lines live: plane offset of (m, n) = base[n nbm + mblk[m]] + m mstr[n]
   const int gm = (int)p.rows[0].blk.size();
-  std::vector<int> mblk(M), base((size_t)N * gm), mstr(N);
+  std::vector<int>&mblk = D.mblk, &base = D.base, &mstr = D.mstr;
+  mblk.resize(M), base.resize((size_t)N * gm), mstr.resize(N);
   bool vec = l0.ncell % 2 == 0 && (ax == 0 || N % 2 == 0);
   int n0 = 0;
   for (const Chain& r : p.rows) {
@@ -632,15 +633,11 @@ static int finish_direct(snac_plan* P) {
         const DirectArgs<T> A = direct_args<T>(P, d);
         args.push_back(A);
         const PlaneShape S = plane_shape(A.F, A.M, A.N, A.cls);
-        std::vector<int> hb((size_t)d.N * d.nbm), hm(d.M), hs(d.N);
-        cudaMemcpy(hb.data(), d.d_base, hb.size() * sizeof(int), cudaMemcpyDeviceToHost);
-        cudaMemcpy(hm.data(), d.d_mblk, hm.size() * sizeof(int), cudaMemcpyDeviceToHost);
-        cudaMemcpy(hs.data(), d.d_mstr, hs.size() * sizeof(int), cudaMemcpyDeviceToHost);
         auto row = [&](int p) { return (size_t)(p / A.F.l1) * S.s1 + (size_t)(p % A.F.l1) * S.rp; };
         const bool flip = d.kind == KIND_DD || d.kind == KIND_DN;
         for (int n = 0; n < d.N; ++n)
           for (int m = 0; m < d.M; ++m) {
-            const long long c = hb[(size_t)n * d.nbm + (d.nbm == 1 ? 0 : hm[m])] + (long long)m * hs[n];
+            const long long c = d.base[(size_t)n * d.nbm + d.mblk[m]] + (long long)m * d.mstr[n];
             size_t o;
             if (d.cls == LINES_PAIR) {
               const int t = d.kind == KIND_PP ? m : ((m & 1) ? d.M - 1 - (m >> 1) : m >> 1);
@@ -658,13 +655,15 @@ static int finish_direct(snac_plan* P) {
   }
   // on the private stream, like every other device work of plan creation
   const cudaStream_t cs = P->setup_stream;
-  bool ok = true;
-  for (DirectTab& T : D.pc)
-    if (ok && T.d_fac) ok = launch_tri_factor(P, T, d_qof, (int)qof.size(), cs) == cudaSuccess;
-  if (ok && D.it.k) ok = setup_iface(P, cs) == cudaSuccess;
-  ok = ok && cudaStreamSynchronize(cs) == cudaSuccess;
-  if (!ok) {
-    const cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  for (DirectTab& T : D.pc) {
+    if (e == cudaSuccess && T.d_fac) e = launch_tri_factor(P, T, d_qof, (int)qof.size(), cs);
+    for (std::vector<int>* v : {&T.base, &T.mblk, &T.mstr}) std::vector<int>().swap(*v);
+  }
+  if (e == cudaSuccess && D.it.k) e = setup_iface(P, cs);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
     set_error(std::string("setting up the direct solves failed: ") + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? SNAC_ERR_OOM : SNAC_ERR_CUDA;
   }

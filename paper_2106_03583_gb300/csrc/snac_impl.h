@@ -199,8 +199,9 @@ struct DirectTab {
   int* d_base = nullptr;
   int* d_mblk = nullptr;
   int* d_mstr = nullptr;
-  // host copies the interface setup needs
+  // host copies the rest of the set-up needs
   std::vector<double> lam, F, B;  // F[kappa M + m], B[m M + kappa] (LINES_DENSE)
+  std::vector<int> base, mblk, mstr;
 };
 
 // The interfaces between the pieces of a plan (kern_iface.cu).

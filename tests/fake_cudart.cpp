@@ -57,6 +57,7 @@ cudaError_t copy(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_
   std::memcpy(d, s, n);
   if (k == cudaMemcpyHostToDevice) ++pending[(uintptr_t)st];
   else if (wait) pending.erase((uintptr_t)st);
+  if (k == cudaMemcpyDeviceToHost) log_ += "read back\n";
   return cudaSuccess;
 }
 }  // namespace

@@ -105,3 +105,14 @@ while True:
     assert all(o[1] and o[3] for o in out)
     fallback = out[first:-1]   # plans that kept their V-cycles: the same memory, less than with the tables
     assert len(fallback) >= 8 and len({o[2] for o in fallback}) == 1 and fallback[0][2] < out[-1][2]
+
+
+def test_setup_reads_nothing_back():
+    """The cells' places come from the tables that were uploaded, not from unchecked copies of them."""
+    out = fake_cuda.run(LAYOUTS + """
+for make in PROBLEMS.values():
+    st, h = create(make())
+    lib.snac_plan_destroy(h)
+out = fake.fake_log().decode().count("read back")
+""")
+    assert out == 0
