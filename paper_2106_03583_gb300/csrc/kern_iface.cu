@@ -58,8 +58,9 @@ struct BuildArgs {
   const double* Z;
 };
 
-// K = I - Y^T R_q Z^T, a 32 x 32 tile per CTA of 256 threads (2 x 2 entries each); the rows and columns of
-// the pinned pieces' unknowns beyond.
+// The transpose of K = I - Y^T R_q Z^T (KT[q][i][j] = K[j][i]), a 32 x 32 tile per CTA of 256 threads (2 x 2
+// entries each); the rows and columns of the pinned pieces' unknowns beyond. Transposed, so that its inverse
+// stands as the solve reads it (consecutive entries of a column of K^-1) without another copy.
 constexpr int KT = 32;
 __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __restrict__ K) {
   __shared__ double ys[KT][KT + 1], ws[KT][KT + 1];
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
       __syncthreads();
 #pragma unroll 8
       for (int e = 0; e < KT; ++e) {
-        const double a0 = ys[e][ty], a1 = ys[e][ty + 16], b0 = ws[e][tx], b1 = ws[e][tx + 16];
+        const double a0 = ys[e][tx], a1 = ys[e][tx + 16], b0 = ws[e][ty], b1 = ws[e][ty + 16];
         acc[0][0] = fma(a0, b0, acc[0][0]);
         acc[0][1] = fma(a0, b1, acc[0][1]);
         acc[1][0] = fma(a1, b0, acc[1][0]);
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
   }
   for (int a = 0; a < 2; ++a)
     for (int b = 0; b < 2; ++b) {
-      const int j = j0 + ty + 16 * a, i = i0 + tx + 16 * b;
+      const int j = j0 + tx + 16 * a, i = i0 + ty + 16 * b;
       if (j >= A.kk || i >= A.kk) continue;
       double v = (j == i ? 1.0 : 0.0) - acc[a][b];
       if (j >= A.k || i >= A.k) {
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
                              : A.sc[a] * A.Z[(size_t)i * A.E + A.eo[u]] * (A.ee[u] ? 1.0 : R.y);
         }
       }
-      K[((size_t)q * A.kk + j) * A.kk + i] = v;
+      K[((size_t)q * A.kk + i) * A.kk + j] = v;
     }
 }
 
@@ -143,13 +144,6 @@ __global__ void __launch_bounds__(1024) k_invert(double* __restrict__ Kq, int n)
     }
     __syncthreads();
   }
-}
-
-// Kept transposed: the solve's threads read consecutive entries of a column of K^-1.
-__global__ void __launch_bounds__(256) k_keep(const double* __restrict__ K, int n, double* __restrict__ out) {
-  const size_t o = (size_t)blockIdx.y * n * n;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)n * n; t += (size_t)gridDim.x * blockDim.x)
-    out[o + (t % n) * n + t / n] = K[o + t];
 }
 
 constexpr int INT = 1024;
@@ -192,11 +186,12 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   DirectPlan& D = P->direct;
   IfaceTab& I = D.it;
   const bool f64 = P->precision == SNAC_FP64;
+  // temporaries in stream order: cudaFree would wait for every other stream of the device
   std::vector<void*> tmp;
   cudaError_t e = cudaSuccess;
   auto get = [&](size_t bytes) -> void* {
     void* p = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&p, bytes);
+    if (e == cudaSuccess) e = cudaMallocAsync(&p, bytes, s);
     if (p) tmp.push_back(p);
     return p;
   };
@@ -209,7 +204,6 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   A.nends = I.nends;
   for (int a = 0; a < I.ns; ++a) A.sp[a] = I.sp[a];
   double* dZ = (double*)get(I.Zh.size() * sizeof(double));
-  double* K = (double*)get((size_t)P->nz * I.kk * I.kk * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpyAsync(dZ, I.Zh.data(), I.Zh.size() * sizeof(double), cudaMemcpyHostToDevice, s);
   A.Y = I.d_Y;
   A.Z = dZ;
@@ -240,22 +234,20 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   }
   if (e == cudaSuccess) {
     const unsigned t = (unsigned)((I.kk + KT - 1) / KT);
-    k_build<<<dim3(t, t, (unsigned)P->nz), 256, 0, s>>>(A, K);
+    k_build<<<dim3(t, t, (unsigned)P->nz), 256, 0, s>>>(A, I.d_KT);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
     const size_t smem = 2 * (size_t)I.kk * sizeof(double);
-    k_invert<<<P->nz, I.kk >= 256 ? 1024 : 256, smem, s>>>(K, I.kk);
+    k_invert<<<P->nz, I.kk >= 256 ? 1024 : 256, smem, s>>>(I.d_KT, I.kk);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) {
-    const dim3 g((unsigned)std::max<size_t>(1, std::min<size_t>(64, (size_t)I.kk * I.kk / 1024)), (unsigned)P->nz);
-    k_keep<<<g, 256, 0, s>>>(K, I.kk, I.d_KT);
-    e = cudaGetLastError();
+  for (void* p : tmp) {
+    const cudaError_t ef = cudaFreeAsync(p, s);
+    if (e == cudaSuccess) e = ef;
   }
   const cudaError_t es = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = es;
-  for (void* p : tmp) cudaFree(p);
   std::vector<double>().swap(I.Zh);
   return e;
 }

@@ -116,3 +116,13 @@ for make in PROBLEMS.values():
 out = fake.fake_log().decode().count("read back")
 """)
     assert out == 0
+
+
+@pytest.mark.parametrize("name", ["L", "L on chip", "dense"])
+def test_setup_waits_for_no_other_stream(name):
+    """cudaFree waits for the whole device: plan creation does without, in stream order."""
+    out = fake_cuda.run(LAYOUTS + f"""
+st, h = create(PROBLEMS[{name!r}]())
+out = [st, fake.fake_log().decode().split().count("cudaFree"), fake.fake_used() == workspace(h)]
+""")
+    assert out == [0, 0, True]
