@@ -670,6 +670,26 @@ static int finish_direct(snac_plan* P) {
   return SNAC_OK;
 }
 
+size_t direct_interface_bytes(const snac_plan* P, const std::vector<FaceKinds>& faces) {
+  const size_t w = P->precision == SNAC_FP64 ? sizeof(double) : sizeof(float);
+  size_t most = 0;
+  for (int t = 0; t < 2; ++t) {
+    Layout L;
+    if (!pieces_along(P, faces, t, L) || L.cells.empty() || !iface_affordable(P, L)) continue;
+    size_t E = 0, M = 0;
+    for (const Piece& p : L.pc) {
+      const size_t m = piece_widths(P, p, t, true).size();
+      M += m;
+      for (int e = 0; e < 2; ++e) E += p.iface[e] ? m : 0;
+    }
+    const size_t kk = L.cells.size() + L.pc.size(), nz = (size_t)P->nz;
+    // kept: inverses, Y, Z, end values, pinned unknowns; while they are set up: responses, a second Z
+    most = std::max(most, nz * kk * kk * sizeof(double) + E * kk * (sizeof(double) + w) + nz * E * w +
+                              2 * nz * IFACE_MAX_ENDS * w + nz * (M + L.pc.size()) * sizeof(double4) + E * kk * sizeof(double));
+  }
+  return most;
+}
+
 int setup_direct(snac_plan* P, const std::vector<FaceKinds>& faces) {
   if (P->lev[0].ncell >= (1LL << 31)) return SNAC_OK;
   const size_t mark = P->allocs.size(), bytes = P->bytes;

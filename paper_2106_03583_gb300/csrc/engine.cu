@@ -60,6 +60,7 @@ struct Request {
   State state = State::Queued;
   PlanSlot* slot = nullptr;
   bool build_plan = false;
+  bool direct = true;  // false: the interface systems of a direct plan exceed the whole budget
   int status = SNAC_OK;
   snac_solve_info info{};
   snac_request_times times{};
@@ -104,9 +105,10 @@ std::string problem_key(const Request& r) {
   return k;
 }
 
-// Device bytes of a plan before it exists: the level hierarchy (u, f and, FP64, the inverse
-// diagonals, x 4/3 over levels; FP32 fused levels add a second iterate), the residual field and the
-// small tables, rounded up. Replaced by the plan's own count once it is built.
+// Device bytes of a plan before it exists, but for its interface systems (interface_bytes): the level hierarchy
+// (u, f and, FP64, the inverse diagonals, x 4/3 over levels; FP32 fused levels add a second iterate), the residual
+// field, the pivots of a direct plan and the small tables, rounded up. Replaced by the plan's own count once it
+// is built.
 uint64_t plan_estimate(long long n3, bool fp64) {
   const double per_cell = fp64 ? 64.0 : 40.0;
   return (uint64_t)(per_cell * (double)n3) + (64ull << 20);
@@ -259,8 +261,8 @@ int snac_engine::run(Request* r, cudaStream_t s) {
     bool have_opt = r->has_opt;
     if (r->tune && ok) {  // choose the schedule on this request's right-hand side
       snac_options chosen{};
-      if (snac_autotune((int32_t)r->blocks.size(), r->blocks.data(), r->homog_axis, r->has_opt ? &r->opt : nullptr,
-                        d_f, r->tol, &chosen, nullptr, s) == SNAC_OK) {
+      if (snac::autotune((int32_t)r->blocks.size(), r->blocks.data(), r->homog_axis, r->has_opt ? &r->opt : nullptr,
+                         d_f, r->tol, &chosen, nullptr, r->direct, s) == SNAC_OK) {
         use = chosen;
         have_opt = true;
         std::lock_guard<std::mutex> lk(mu);
@@ -276,7 +278,8 @@ int snac_engine::run(Request* r, cudaStream_t s) {
       }
     }
     snac_plan* pl = nullptr;
-    st = snac_plan_create(&pl, (int32_t)r->blocks.size(), r->blocks.data(), r->homog_axis, have_opt ? &use : nullptr);
+    st = snac::create_plan(&pl, (int32_t)r->blocks.size(), r->blocks.data(), r->homog_axis, have_opt ? &use : nullptr,
+                           r->direct);
     size_t bytes = 0;
     if (st == SNAC_OK) snac_plan_workspace_bytes(pl, &bytes);
     std::lock_guard<std::mutex> lk(mu);
@@ -522,6 +525,9 @@ int snac_engine_submit(snac_engine* e, int32_t nblocks, const snac_block* blocks
   r->buf_bytes = 16ull * (uint64_t)n3;
   r->plan_estimate = plan_estimate(n3, !(opt && opt->precision == SNAC_MIXED));
   r->tune_bytes = e->opt.autotune ? 8ull * (uint64_t)n3 : 0;
+  const uint64_t iface = snac::interface_bytes(nblocks, r->blocks.data(), homog_axis, opt);
+  r->direct = r->buf_bytes + r->plan_estimate + iface + r->tune_bytes <= e->opt.hbm_budget;
+  if (r->direct) r->plan_estimate += iface;
   if (r->buf_bytes + r->plan_estimate + r->tune_bytes > e->opt.hbm_budget) {
     delete r;
     return SNAC_ERR_OOM;

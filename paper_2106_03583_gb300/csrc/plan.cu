@@ -650,7 +650,36 @@ std::vector<snac_block> internal_blocks(int nblocks, const snac_block* blocks, i
   return out;
 }
 
-int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_t homog_axis, const snac_options* opt) {
+// Direct solves only with the default schedule: a caller who sets a multigrid option gets the multigrid.
+bool default_schedule(const snac_plan* P) {
+  return P->nu1 == 2 && P->nu2 == 2 && P->max_cycles == 40 && P->max_coarse == 64 && P->fused == -1 &&
+         P->onchip_opt == 0 && P->bottom_cells == 0 && P->inner_reduction == 0.0;
+}
+
+void take_options(snac_plan* P, const snac_options* opt) {
+  P->precision = opt->precision;
+  P->nu1 = opt->nu1;
+  P->nu2 = opt->nu2;
+  P->max_outer = opt->max_outer;
+  P->max_cycles = opt->max_cycles;
+  P->max_coarse = opt->max_coarse;
+  P->inner_reduction = opt->inner_reduction;
+  P->fused = opt->fused;
+  P->shift = opt->shift;
+  P->onchip_opt = opt->onchip;
+  P->bottom_cells = opt->bottom_cells;
+}
+
+std::vector<FaceKinds> face_kinds(const std::vector<HBlock>& hb) {
+  std::vector<FaceKinds> faces(hb.size());
+  for (size_t b = 0; b < hb.size(); ++b)
+    for (int a = 0; a < 2; ++a)
+      for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
+  return faces;
+}
+
+int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_t homog_axis, const snac_options* opt,
+           bool allow_direct) {
   if (!out || !blocks_in || nblocks < 1) return fail(SNAC_ERR_INVALID_ARG, "out/blocks NULL or nblocks < 1");
   *out = nullptr;
   if (homog_axis < 0 || homog_axis > 2) return fail(SNAC_ERR_INVALID_ARG, "homog_axis must be 0, 1 or 2");
@@ -662,21 +691,11 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
   snac_plan* P = new (std::nothrow) snac_plan();
   if (!P) return fail(SNAC_ERR_OOM, "host allocation");
   if (opt) {
-    P->precision = opt->precision;
-    P->nu1 = opt->nu1;
-    P->nu2 = opt->nu2;
-    P->max_outer = opt->max_outer;
-    P->max_cycles = opt->max_cycles;
-    P->max_coarse = opt->max_coarse;
-    P->inner_reduction = opt->inner_reduction;
-    P->fused = opt->fused;
-    P->shift = opt->shift;
-    P->onchip_opt = opt->onchip;
+    take_options(P, opt);
     if (opt->onchip != 0 && opt->onchip != -1) {
       delete P;
       return fail(SNAC_ERR_INVALID_ARG, "bad snac_options: onchip must be 0 or -1");
     }
-    P->bottom_cells = opt->bottom_cells;
     if (opt->bottom_cells != 0 && opt->bottom_cells != -1 &&
         (opt->bottom_cells < 16 || opt->bottom_cells > BOTTOM_MAX_CELLS)) {
       delete P;
@@ -828,9 +847,7 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
       P->onchip = P->onchip_opt == 0 && P->nu1 >= 1 && P->nu2 >= 1 && L >= 1 && L < BOTTOM_MAX_LEVELS &&
                   P->lev[0].ncell <= BOTTOM_MAX_CELLS && bottom_layout(P, 0, inner).bytes <= (size_t)BOTTOM_MAX_SMEM;
     }
-    // direct solves only with the default schedule: a caller who sets a multigrid option gets the multigrid
-    const bool direct = P->nu1 == 2 && P->nu2 == 2 && P->max_cycles == 40 && P->max_coarse == 64 && P->fused == -1 &&
-                        P->onchip_opt == 0 && P->bottom_cells == 0 && P->inner_reduction == 0.0;
+    const bool direct = allow_direct && default_schedule(P);
     // the automatic inner reduction: an on-chip plan's V-cycles are cheap next to an outer step,
     // so it asks more of each step (measured on c64: 3 outer steps at 1e-4, 2 at 3e-5, 18 % faster)
     if (P->inner_reduction == 0.0) P->inner_reduction = P->onchip ? 3e-5 : 1e-4;
@@ -967,13 +984,7 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
         break;
       }
     }
-    if (direct) {
-      std::vector<FaceKinds> faces(hb.size());
-      for (size_t b = 0; b < hb.size(); ++b)
-        for (int a = 0; a < 2; ++a)
-          for (int sd = 0; sd < 2; ++sd) faces[b].k[face(a, sd)] = hb[b].bc[a][sd];
-      if ((st = setup_direct(P, faces))) break;
-    }
+    if (direct && (st = setup_direct(P, face_kinds(hb)))) break;
   } while (0);
   if (st) {
     free_plan(P);
@@ -1030,17 +1041,34 @@ int check_layout(int nblocks, const snac_block* blocks, int homog_axis) {
   std::vector<HBlock> hb;
   return validate(nblocks, ib.data(), hb);
 }
+
+size_t interface_bytes(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt) {
+  const std::vector<snac_block> ib = internal_blocks(nblocks, blocks, homog_axis);
+  std::vector<HBlock> hb;
+  if (validate(nblocks, ib.data(), hb)) return 0;
+  snac_plan P;
+  if (opt) take_options(&P, opt);
+  if (!default_schedule(&P)) return 0;
+  P.nz = P.nzt = hb[0].n[2];
+  P.max_coarse = INT32_MAX;  // level 0 only
+  return build_levels(&P, hb) ? 0 : direct_interface_bytes(&P, face_kinds(hb));
+}
+
+int create_plan(snac_plan** out, int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt,
+                bool direct) {
+  try {
+    return create(out, nblocks, blocks, homog_axis, opt, direct);
+  } catch (...) {
+    return fail(SNAC_ERR_OOM, "exception during plan creation");
+  }
+}
 }  // namespace snac
 
 extern "C" {
 
 int snac_plan_create(snac_plan** out, int32_t nblocks, const snac_block* blocks, int32_t homog_axis,
                      const snac_options* opt) {
-  try {
-    return create(out, nblocks, blocks, homog_axis, opt);
-  } catch (...) {
-    return fail(SNAC_ERR_OOM, "exception during plan creation");
-  }
+  return create_plan(out, nblocks, blocks, homog_axis, opt, true);
 }
 
 int snac_plan_workspace_bytes(const snac_plan* plan, size_t* bytes) {

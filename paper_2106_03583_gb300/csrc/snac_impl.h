@@ -500,6 +500,15 @@ struct FaceKinds {
   int k[4];
 };
 int setup_direct(snac_plan* P, const std::vector<FaceKinds>& faces);
+// Device bytes that interface systems add to such a plan at most, their set-up included (0: none).
+size_t direct_interface_bytes(const snac_plan* P, const std::vector<FaceKinds>& faces);
+// snac_plan_create, and with direct = false a plan that keeps its V-cycles; the bytes above for a problem that
+// has no plan yet (a valid layout).
+int create_plan(snac_plan** out, int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt,
+                bool direct);
+size_t interface_bytes(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt);
+int autotune(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* base, const double* d_rhs,
+             double tol, snac_options* best, snac_tune_report* report, bool direct, void* stream);
 cudaError_t launch_tri_factor(snac_plan* P, const DirectTab& D, const int* d_qof, int rows, cudaStream_t s);
 // Interface systems of plans of several pieces: setup (once per plan) and the solve of every wavenumber's
 // fluxes from the end values, added to the spectral right-hand sides.

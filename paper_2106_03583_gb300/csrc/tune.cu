@@ -41,13 +41,14 @@ struct Trial {
   double tol;
   cudaStream_t s;
   cudaEvent_t e0, e1;
+  bool direct;
 };
 
 // Mean time of `reps` solves from p = 0 with options o, after one untimed solve; +inf if the plan
 // cannot be built or a solve does not reach tol.
 double time_options(const Trial& t, const snac_options& o, int reps) {
   snac_plan* pl = nullptr;
-  if (snac_plan_create(&pl, t.nblocks, t.blocks, t.homog, &o) != SNAC_OK) return INFINITY;
+  if (snac::create_plan(&pl, t.nblocks, t.blocks, t.homog, &o, t.direct) != SNAC_OK) return INFINITY;
   double ms = INFINITY;
   bool ok = cudaMemsetAsync(t.d_p, 0, t.bytes, t.s) == cudaSuccess &&
             snac_poisson_solve(pl, t.d_rhs, t.d_p, t.tol, t.s) == SNAC_OK;
@@ -72,6 +73,12 @@ double time_options(const Trial& t, const snac_options& o, int reps) {
 extern "C" int snac_autotune(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* base,
                              const double* d_rhs, double tol, snac_options* best, snac_tune_report* report,
                              void* stream) {
+  return snac::autotune(nblocks, blocks, homog_axis, base, d_rhs, tol, best, report, true, stream);
+}
+
+int snac::autotune(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* base,
+                   const double* d_rhs, double tol, snac_options* best, snac_tune_report* report, bool direct,
+                   void* stream) {
   if (!blocks || nblocks < 1 || !d_rhs || !best || !(tol > 0.0) || !std::isfinite(tol)) return SNAC_ERR_INVALID_ARG;
   if (base && (base->mode_begin != 0 || base->mode_end != 0)) return SNAC_ERR_INVALID_ARG;  // whole solves only
   int st = snac::check_layout(nblocks, blocks, homog_axis);
@@ -84,7 +91,7 @@ extern "C" int snac_autotune(int32_t nblocks, const snac_block* blocks, int32_t 
     n3 += c;
   }
   Trial t{nblocks, blocks, homog_axis, d_rhs, nullptr, (size_t)n3 * sizeof(double), tol, (cudaStream_t)stream,
-          nullptr, nullptr};
+          nullptr, nullptr, direct};
   if (cudaMalloc((void**)&t.d_p, t.bytes) != cudaSuccess) {
     cudaGetLastError();
     return SNAC_ERR_OOM;

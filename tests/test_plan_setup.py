@@ -126,3 +126,46 @@ st, h = create(PROBLEMS[{name!r}]())
 out = [st, fake.fake_log().decode().split().count("cudaFree"), fake.fake_used() == workspace(h)]
 """)
     assert out == [0, 0, True]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("name", ["thin", "L", "T", "dense", "on chip"])
+def test_engine_reserves_what_a_plan_takes(name, precision):
+    """What an engine has reserved covers the device's memory at its highest, the set-up of the interface systems
+    of two long thin rectangles included; where the budget has no room for those, the plan keeps its V-cycles."""
+    out = fake_cuda.run(LAYOUTS + f"""
+def thin():   # (the Dirichlet face beside an interface rules out rectangles that meet along their short sides)
+    b = problem([(0, 84, 0, 4), (0, 84, 4, 8), (84, 168, 4, 8)], 168, 8, nz=4096)
+    b[0]["bc"] = (("D", "D"),) + tuple(b[0]["bc"][1:])
+    return b
+PROBLEMS["thin"] = thin
+PROBLEMS["T"] = lambda: problem([(0, 80, 0, 80), (80, 160, 0, 80), (160, 240, 0, 80), (80, 160, 80, 160)], 240, 160, nz=32,
+                                xf=1.0, yf=1.0)
+b = PROBLEMS[{name!r}]()
+st, h = create(b, {precision!r})
+want = workspace(h)
+lib.snac_plan_destroy(h)
+arr, keep = snac._marshal_blocks(b)
+n3 = sum(int(np.prod([q["hi"][a] - q["lo"][a] + 1 for a in range(3)])) for q in b)
+f, p = np.zeros(n3), np.empty(n3)
+o = snac._Options(snac._PREC[{precision!r}], 2, 2, 20, 40, 64, -1, 0.0, 0.0, 0, 0, 0, 0)
+out = [st, want]
+vcycles = n3 * (16 + (64 if {precision!r} == "fp64" else 40)) + (64 << 20)
+for budget in (1 << 40, vcycles):
+    eo = snac._EngineOptions(1, 8, budget, 0, 16)
+    e, t = ctypes.c_void_p(), ctypes.c_int64()
+    fake.fake_reset()
+    before = fake.fake_used()
+    r = [lib.snac_engine_create(ctypes.byref(e), ctypes.byref(eo)),
+         lib.snac_engine_submit(e, len(b), arr, 2, ctypes.byref(o), f.ctypes.data, p.ctypes.data, 1e-10, ctypes.byref(t)),
+         lib.snac_engine_wait(e, t, None, None)]
+    s = snac._EngineStats()
+    lib.snac_engine_get_stats(e, ctypes.byref(s))
+    out.append([r, fake.fake_peak() - before, s.bytes_peak, any("k_resp" in l for l in launches())])
+    lib.snac_engine_destroy(e)
+""")
+    st, want, wide, tight = out
+    assert st == 0 and wide[0] == tight[0] == [0, 0, 0]
+    assert wide[1] <= wide[2] and tight[1] <= tight[2] and want <= wide[2]
+    pieces = name in ("thin", "L", "T")
+    assert wide[3] == pieces and not tight[3]
