@@ -519,11 +519,11 @@ int job_decide(Job& J, cudaStream_t s) {
   if (P->precision == SNAC_MIXED && P->inner_reduction * rn > J.tol * fn) J.target = P->inner_reduction * rn;
   J.aim_final = J.target <= 0.5 * J.tol * fn;
   if (P->direct.on && P->precision == SNAC_MIXED) {
-    // a direct step reduces the residual to the FP32 floor whatever the target: by 1e-4 or so from f, by
-    // about 3e-7 from the rough residual that such a step leaves (6e-7 with
-    // interfaces between pieces). The FP64 pass comes directly where
-    // that reaches the tolerance (with the margin above)
-    J.aim_final = J.k > 0 && (P->direct.it.k ? 6e-7 : 3e-7) * rel <= 0.5 * J.tol;
+    // a direct step reduces the residual to the FP32 floor whatever the target: from f to 1e-4 or so of it (6e-6
+    // to 1.1e-4 measured on planes of 64^2 to 512^2 cells), by about 3e-7 from the rough residual that such a step
+    // leaves (6e-7 with interfaces between pieces). The FP64 pass comes directly where that reaches the
+    // tolerance (with the margin above): at 1e-3 one step and no float-float pass, as with V-cycles
+    J.aim_final = (J.k == 0 ? 2e-4 : P->direct.it.k ? 6e-7 : 3e-7) * rel <= 0.5 * J.tol;
   }
   J.fused = fused_ready(P);
   if (J.fused) {  // the forward transform goes into the same launch as the wavenumber solves

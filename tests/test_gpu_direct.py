@@ -254,3 +254,21 @@ def test_dense_transforms_in_any_unit_of_length(unit):
         pl.close()
         out.append(host(p))
     assert rel(out[1] / unit ** 2, out[0]) <= 1e-13
+
+
+@pytest.mark.parametrize("case", [DIRECT[0], DIRECT[8], DIRECT[26]], ids=lambda c: "-".join(map(str, c[:6])))
+def test_loose_tolerance_takes_one_residual_pass(case):
+    """A mixed solve that one direct step finishes: the residual before it is f, the one after it FP64, and no
+    float-float pass between."""
+    import torch
+    layout, nx, ny, xf, yf, walls, zp, per = case
+    blocks = build(layout, nx, ny, xf, yf, walls, zp, per=per)
+    f = inputs.divergence_rhs(blocks, 8)
+    pl = plan(blocks, precision="mixed")
+    p = torch.zeros(len(f), dtype=torch.float64, device="cuda")
+    info = pl.solve(dev(f), p, tol=1e-3)
+    st = pl.kernel_stats()
+    assert info["status"] == 0 and info["outer_iters"] == 1
+    assert st["field3d_ff"]["launches"] == 0 and st["field3d"]["launches"] == 2   # the statistics of f, the residual
+    assert osv.rel_residual(blocks, f, host(p)) <= 1.01e-3
+    pl.close()
