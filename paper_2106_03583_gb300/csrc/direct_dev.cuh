@@ -126,6 +126,7 @@ struct IfaceArgs {
   const double* Y;
   const T* Z;
   const double* KT;
+  const int* qrow;
   T* ends;
   T* alpha;
   T* num;
@@ -151,6 +152,7 @@ inline IfaceArgs<T> iface_args(const snac_plan* P) {
   A.Y = I.d_Y;
   A.Z = (const T*)I.d_Z;
   A.KT = I.d_KT;
+  A.qrow = P->direct.d_qrow;
   A.ends = (T*)I.d_ends;
   A.alpha = (T*)I.d_alpha;
   A.num = (T*)I.d_num;
@@ -205,7 +207,7 @@ __device__ void iface_solve(const IfaceArgs<T>& I, int q, double* work, const T*
     y[I.k + a] = q == I.qs && a == I.ns - 1 ? 0.0 : (double)num[I.sp[a]];
   }
   __syncthreads();
-  gemv_cols(I.KT + (long long)q * I.kk * I.kk, I.kk, I.kk, I.kk, y, phi, part, nt);
+  gemv_cols(I.KT + (long long)I.qrow[q] * I.kk * I.kk, I.kk, I.kk, I.kk, y, phi, part, nt);
   if ((int)threadIdx.x < I.ns) alpha[I.sp[threadIdx.x]] = (T)phi[I.k + threadIdx.x];
   T* ph = reinterpret_cast<T*>(part);  // (kk <= 1040 values of T fit in nt doubles)
   for (int j = threadIdx.x; j < I.k; j += nt) ph[j] = (T)phi[j];

@@ -548,7 +548,6 @@ int build_iface(snac_plan* P, const Layout& L) {
   const size_t w = P->precision == SNAC_FP64 ? sizeof(double) : sizeof(float);
   int st;
   if ((st = up_vec(P, &I.d_Y, Y)) || (st = up_inner(P, &I.d_Z, Z)) ||
-      (st = plan_alloc(P, (void**)&I.d_KT, (size_t)P->nz * I.kk * I.kk * sizeof(double))) ||
       (st = plan_alloc(P, &I.d_ends, (size_t)P->nz * I.E * w)) || (st = plan_alloc(P, &I.d_alpha, (size_t)P->nz * IFACE_MAX_ENDS * w)) ||
       (st = plan_alloc(P, &I.d_num, (size_t)P->nz * IFACE_MAX_ENDS * w)))
     return st;
@@ -611,15 +610,16 @@ static int finish_direct(snac_plan* P) {
   int st;
   std::vector<int> qrow(P->nz), qof;
   int* d_qof = nullptr;
+  std::map<int, int> seen;  // wavenumbers q and n - q of the real DFT have one eigenvalue
+  for (int l = 0; l < P->nz; ++l) {
+    const int q = P->q0 + l;
+    const auto it = seen.emplace(P->kind == KIND_PP ? std::min(q, P->nzt - q) : q, (int)qof.size());
+    if (it.second) qof.push_back(l);
+    qrow[l] = it.first->second;
+  }
+  if ((st = up_vec(P, &D.d_qrow, qrow)) || (st = up_vec(P, &d_qof, qof))) return st;
+  if (D.it.k && (st = plan_alloc(P, (void**)&D.it.d_KT, qof.size() * D.it.kk * (size_t)D.it.kk * sizeof(double)))) return st;
   if (!P->onchip) {
-    std::map<int, int> seen;  // wavenumbers q and n - q of the real DFT have one eigenvalue
-    for (int l = 0; l < P->nz; ++l) {
-      const int q = P->q0 + l;
-      const auto it = seen.emplace(P->kind == KIND_PP ? std::min(q, P->nzt - q) : q, (int)qof.size());
-      if (it.second) qof.push_back(l);
-      qrow[l] = it.first->second;
-    }
-    if ((st = up_vec(P, &D.d_qrow, qrow)) || (st = up_vec(P, &d_qof, qof))) return st;
     for (DirectTab& T : D.pc)
       if ((st = plan_alloc(P, &T.d_fac, qof.size() * (size_t)T.M * T.N * w))) return st;
   } else {
@@ -660,7 +660,7 @@ static int finish_direct(snac_plan* P) {
     if (e == cudaSuccess && T.d_fac) e = launch_tri_factor(P, T, d_qof, (int)qof.size(), cs);
     for (std::vector<int>* v : {&T.base, &T.mblk, &T.mstr}) std::vector<int>().swap(*v);
   }
-  if (e == cudaSuccess && D.it.k) e = setup_iface(P, cs);
+  if (e == cudaSuccess && D.it.k) e = setup_iface(P, d_qof, (int)qof.size(), D.it.qs < 0 ? -1 : qrow[D.it.qs], cs);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -682,10 +682,10 @@ size_t direct_interface_bytes(const snac_plan* P, const std::vector<FaceKinds>& 
       M += m;
       for (int e = 0; e < 2; ++e) E += p.iface[e] ? m : 0;
     }
-    const size_t kk = L.cells.size() + L.pc.size(), nz = (size_t)P->nz;
+    const size_t kk = L.cells.size() + L.pc.size(), nz = (size_t)P->nz, rows = P->kind == KIND_PP ? nz / 2 + 1 : nz;
     // kept: inverses, Y, Z, end values, pinned unknowns; while they are set up: responses, a second Z
-    most = std::max(most, nz * kk * kk * sizeof(double) + E * kk * (sizeof(double) + w) + nz * E * w +
-                              2 * nz * IFACE_MAX_ENDS * w + nz * (M + L.pc.size()) * sizeof(double4) + E * kk * sizeof(double));
+    most = std::max(most, rows * kk * kk * sizeof(double) + E * kk * (sizeof(double) + w) + nz * E * w +
+                              2 * nz * IFACE_MAX_ENDS * w + rows * (M + L.pc.size()) * sizeof(double4) + E * kk * sizeof(double));
   }
   return most;
 }

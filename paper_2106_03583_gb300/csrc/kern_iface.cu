@@ -8,7 +8,7 @@
 // unit box no step reduced the residual in FP64, with -1e-4 none in FP32). So that slot's system is pinned for
 // every wavenumber: its last unknown alpha is an unknown of the interface system, all others follow from it by
 // h (1 at a zero shift) and its last row, eliminated, is the extra equation den alpha = num. The inverse of
-// every system is kept with the plan.
+// every system is kept with the plan, one for all wavenumbers of equal shift (a row of DirectPlan::d_qrow).
 #include <cmath>
 #include <vector>
 
@@ -21,13 +21,14 @@ namespace {
 // (as the solve scales them), {00, 0N, N0, NN}. Of a pinned system also {h of the first row, what a unit in the
 // first row leaves in the eliminated last one, den}.
 __global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__ tri, const double* __restrict__ lam,
-                                            const double* __restrict__ sigma, double cscale, double scale, int nq,
+                                            const double* __restrict__ sigma, const int* __restrict__ qof,
+                                            double cscale, double scale, int nq,
                                             int M, int N, int pin, double4* __restrict__ resp,
                                             double4* __restrict__ pinned) {
   const long long sys = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (sys >= (long long)nq * M) return;
   const int q = (int)(sys / M), kap = (int)(sys - (long long)q * M);
-  const double tq = -fma(sigma[q], cscale, lam[kap]);
+  const double tq = -fma(sigma[qof[q]], cscale, lam[kap]);
   double g = 0, d = 0, pi = 1, F = 0, inv = 0, plast = 1;
   for (int n = 0; n < N; ++n) {
     const TriRow<double> w = tri[n];
@@ -182,7 +183,7 @@ cudaError_t launch_iface(snac_plan* P, cudaStream_t s) {
   return P->precision == SNAC_FP64 ? iface_t<double>(P, s) : iface_t<float>(P, s);
 }
 
-cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
+cudaError_t setup_iface(snac_plan* P, const int* d_qof, int rows, int qs_row, cudaStream_t s) {
   DirectPlan& D = P->direct;
   IfaceTab& I = D.it;
   const bool f64 = P->precision == SNAC_FP64;
@@ -200,7 +201,7 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   A.kk = I.kk;
   A.E = I.E;
   A.ns = I.ns;
-  A.qs = I.qs;
+  A.qs = qs_row;
   A.nends = I.nends;
   for (int a = 0; a < I.ns; ++a) A.sp[a] = I.sp[a];
   double* dZ = (double*)get(I.Zh.size() * sizeof(double));
@@ -210,13 +211,13 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   std::vector<double4*> resp(D.pc.size(), nullptr), pinned(D.pc.size(), nullptr);
   for (size_t p = 0; p < D.pc.size(); ++p) {
     const DirectTab& d = D.pc[p];
-    resp[p] = (double4*)get((size_t)P->nz * d.M * sizeof(double4));
-    if (d.pin) pinned[p] = (double4*)get((size_t)P->nz * sizeof(double4));
+    resp[p] = (double4*)get((size_t)rows * d.M * sizeof(double4));
+    if (d.pin) pinned[p] = (double4*)get((size_t)rows * sizeof(double4));
     if (e != cudaSuccess) break;
     const TriRow<double>* tri = (const TriRow<double>*)(f64 ? d.d_tri : (void*)d.d_tri64);
     const double* lam = f64 ? (const double*)d.d_lam : d.d_lam64;
-    const long long sys = (long long)P->nz * d.M;
-    k_resp<<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(tri, lam, P->d_sigma64, d.cscale, d.cscale / d.theta, P->nz,
+    const long long sys = (long long)rows * d.M;
+    k_resp<<<(unsigned)((sys + 127) / 128), 128, 0, s>>>(tri, lam, P->d_sigma64, d_qof, d.cscale, d.cscale / d.theta, rows,
                                                         d.M, d.N, d.pin, resp[p], pinned[p]);
     e = cudaGetLastError();
   }
@@ -234,12 +235,12 @@ cudaError_t setup_iface(snac_plan* P, cudaStream_t s) {
   }
   if (e == cudaSuccess) {
     const unsigned t = (unsigned)((I.kk + KT - 1) / KT);
-    k_build<<<dim3(t, t, (unsigned)P->nz), 256, 0, s>>>(A, I.d_KT);
+    k_build<<<dim3(t, t, (unsigned)rows), 256, 0, s>>>(A, I.d_KT);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
     const size_t smem = 2 * (size_t)I.kk * sizeof(double);
-    k_invert<<<P->nz, I.kk >= 256 ? 1024 : 256, smem, s>>>(I.d_KT, I.kk);
+    k_invert<<<rows, I.kk >= 64 ? 1024 : 256, smem, s>>>(I.d_KT, I.kk);
     e = cudaGetLastError();
   }
   for (void* p : tmp) {

@@ -1050,6 +1050,7 @@ size_t interface_bytes(int32_t nblocks, const snac_block* blocks, int32_t homog_
   if (opt) take_options(&P, opt);
   if (!default_schedule(&P)) return 0;
   P.nz = P.nzt = hb[0].n[2];
+  P.kind = hb[0].bc[2][0] == SNAC_BC_PERIODIC ? KIND_PP : KIND_NN;
   P.max_coarse = INT32_MAX;  // level 0 only
   return build_levels(&P, hb) ? 0 : direct_interface_bytes(&P, face_kinds(hb));
 }

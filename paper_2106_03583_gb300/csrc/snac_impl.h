@@ -215,7 +215,7 @@ struct IfaceTab {
   int sp[IFACE_MAX_ENDS] = {};
   double* d_Y = nullptr;     // [E][kk]: end values -> jump of u across every interface cell
   void* d_Z = nullptr;       // [kk][E]: fluxes -> right-hand sides of the end rows
-  double* d_KT = nullptr;    // [q][kk][kk]: transposed inverse of the interface system
+  double* d_KT = nullptr;    // [row of DirectPlan::d_qrow][kk][kk]: transposed inverse of the interface system
   void* d_ends = nullptr;    // [q][E]: end values of a solve
   void* d_alpha = nullptr;   // [q][IFACE_MAX_ENDS]: by piece, the last unknown of its pinned system
   void* d_num = nullptr;     // [q][IFACE_MAX_ENDS]: by piece, that unknown's eliminated right-hand side
@@ -226,7 +226,7 @@ struct DirectPlan {
   bool on = false;
   std::vector<DirectTab> pc;
   IfaceTab it;
-  int* d_qrow = nullptr;        // per wavenumber: its set of pivots in d_fac
+  int* d_qrow = nullptr;        // per wavenumber: its set of pivots in d_fac and its interface system (shared by equal shifts)
   unsigned* d_celloff = nullptr;  // on chip: per plane cell, element of the shared buffer | sign flip << 31
   void* d_args = nullptr;       // on chip: the pieces' DirectArgs
 };
@@ -512,7 +512,8 @@ int autotune(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, cons
 cudaError_t launch_tri_factor(snac_plan* P, const DirectTab& D, const int* d_qof, int rows, cudaStream_t s);
 // Interface systems of plans of several pieces: setup (once per plan) and the solve of every wavenumber's
 // fluxes from the end values, added to the spectral right-hand sides.
-cudaError_t setup_iface(snac_plan* P, cudaStream_t s);
+// qof: the wavenumber of every row of d_qrow; qs_row: the row of it.qs, -1: none.
+cudaError_t setup_iface(snac_plan* P, const int* d_qof, int rows, int qs_row, cudaStream_t s);
 cudaError_t launch_iface(snac_plan* P, cudaStream_t s);
 // Plan-owned device memory (freed with the plan).
 int plan_alloc(snac_plan* P, void** p, size_t bytes);

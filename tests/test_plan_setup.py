@@ -169,3 +169,22 @@ for budget in (1 << 40, vcycles):
     assert wide[1] <= wide[2] and tight[1] <= tight[2] and want <= wide[2]
     pieces = name in ("thin", "L", "T")
     assert wide[3] == pieces and not tight[3]
+
+
+@pytest.mark.parametrize("name", ["L", "L on chip"])
+def test_equal_shifts_share_an_interface_system(name):
+    """Wavenumbers q and n - q of a periodic z have one eigenvalue: n / 2 + 1 inverses are kept, not n."""
+    out = fake_cuda.run(LAYOUTS + f"""
+out = []
+n, k = (160, 80) if {name!r} == "L" else (32, 16)
+pivots = 3 * k * k if {name!r} == "L" else 0   # (kept with the plan off chip, shared likewise)
+for nz in (32, 64):
+    ws = []
+    for walls in ("DNNN", "NNNN"):
+        for z in (("P", "P"), ("N", "N")):
+            st, h = create(problem(L(n // 2), n, n, nz=nz, z=z, walls=walls))
+            ws.append(workspace(h))
+    out.append([ws[1] - ws[0], ws[3] - ws[2]])
+out = [out[1][i] - out[0][i] - (31 - 15) * 8 * (k * k + pivots) for i in range(2)]
+""")
+    assert all(x >= 0 for x in out)
