@@ -535,6 +535,7 @@ int build_iface(snac_plan* P, const Layout& L) {
   std::vector<double> Y((size_t)I.E * I.kk, 0.0), Z((size_t)I.kk * I.E, 0.0);
   for (int j = 0; j < I.k; ++j) {
     const IfaceCell& c = L.cells[j];
+    I.cells.push_back({{end_of[2 * c.pa + 1], end_of[2 * c.pb]}, {c.ma, c.mb}, {-c.ca, c.cb}});
     for (int side = 0; side < 2; ++side) {
       const int p = side == 0 ? c.pa : c.pb, m = side == 0 ? c.ma : c.mb;
       const int u = end_of[2 * p + (side == 0 ? 1 : 0)];
@@ -683,9 +684,11 @@ size_t direct_interface_bytes(const snac_plan* P, const std::vector<FaceKinds>& 
       for (int e = 0; e < 2; ++e) E += p.iface[e] ? m : 0;
     }
     const size_t kk = L.cells.size() + L.pc.size(), nz = (size_t)P->nz, rows = P->kind == KIND_PP ? nz / 2 + 1 : nz;
-    // kept: inverses, Y, Z, end values, pinned unknowns; while they are set up: responses, a second Z
+    // kept: inverses, Y, Z, end values, pinned unknowns; while they are set up: responses and their cosine sums, a
+    // second Z, the cells
     most = std::max(most, rows * kk * kk * sizeof(double) + E * kk * (sizeof(double) + w) + nz * E * w +
-                              2 * nz * IFACE_MAX_ENDS * w + rows * (M + L.pc.size()) * sizeof(double4) + E * kk * sizeof(double));
+                              2 * nz * IFACE_MAX_ENDS * w + rows * (M + L.pc.size()) * sizeof(double4) +
+                              E * kk * sizeof(double) + rows * 4 * E * sizeof(double) + kk * sizeof(IfaceCellDev));
   }
   return most;
 }

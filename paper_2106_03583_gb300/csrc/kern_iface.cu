@@ -48,12 +48,57 @@ __global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__
   resp[sys] = make_double4(-scale * F, -scale * plast * inv, -scale * d, -scale * inv);
 }
 
+// R restricted to the cells of an end needs no product of matrices where the transform is a cosine or sine one:
+// the entries of B R F depend on the difference and the sum of the two cells only, through
+//   C(d) = sum_kappa h_kappa R_kappa cos(pi a_kappa d / 2M),   d < 2M
+// (products of cosines or sines as sums; h: 1/2 for the first and, periodic, the last slot). One CTA per row of
+// wavenumbers and piece, for every pair of its ends: 2 M^2 terms in place of k^2 M multiply-adds (with k_build, L of
+// 512 x 512 x 128 cells).
+struct CsumArgs {
+  int M, kind, slots, a0, da;    // a_kappa = a0 + kappa da, kappa < slots
+  int ne, u[2], ee[2];           // ends of the piece
+  long long off[2][2];           // of the pair's sums within a row
+  const double4* resp;           // [row][kappa]
+};
+__global__ void __launch_bounds__(512) k_csum(const CsumArgs A, long long stride, double* __restrict__ out) {
+  extern __shared__ double cs[];  // cos(pi t / 2M), t = 0..2M
+  const int M = A.M, T4 = 4 * M;
+  for (int t = threadIdx.x; t <= 2 * M; t += blockDim.x) cs[t] = cospi((double)t / (2 * M));
+  __syncthreads();
+  const double4* R = A.resp + (size_t)blockIdx.x * M;
+  double* o = out + (size_t)blockIdx.x * stride;
+  for (int d = threadIdx.x; d < 2 * M; d += blockDim.x) {
+    double acc[4] = {0, 0, 0, 0};
+    int t = (int)((long long)A.a0 * d % T4);
+    const int dt = (int)((long long)A.da * d % T4);  // (negative for the kinds with reversed slots)
+    for (int k = 0; k < A.slots; ++k) {
+      const bool half = A.kind != KIND_ND && A.kind != KIND_DN && (k == 0 || (A.kind == KIND_PP && 2 * k == M));
+      const double c = (half ? 0.5 : 1.0) * cs[t <= 2 * M ? t : T4 - t];
+      const double4 r = R[k];
+      acc[0] = fma(r.x, c, acc[0]);
+      acc[1] = fma(r.y, c, acc[1]);
+      acc[2] = fma(r.z, c, acc[2]);
+      acc[3] = fma(r.w, c, acc[3]);
+      t += dt;
+      t += t < 0 ? T4 : 0;
+      t -= t >= T4 ? T4 : 0;
+    }
+    for (int a = 0; a < A.ne; ++a)
+      for (int b = 0; b < A.ne; ++b) o[A.off[a][b] + d] = acc[2 * A.ee[a] + A.ee[b]];
+  }
+}
+
 struct BuildArgs {
   int k, kk, E, ns, qs, nends;
   int ep[IFACE_MAX_ENDS], ee[IFACE_MAX_ENDS], eo[IFACE_MAX_ENDS + 1], sp[IFACE_MAX_ENDS];
   int em[IFACE_MAX_ENDS];                 // slots of the end's piece
   double sc[IFACE_MAX_ENDS];              // scale of the right-hand sides of a pinned piece
   const double4* pinned[IFACE_MAX_ENDS];  // of a pinned piece, [q]
+  int kind[IFACE_MAX_ENDS];               // of the end's piece; -1: dense
+  int co[IFACE_MAX_ENDS][IFACE_MAX_ENDS];  // cosine sums of a pair of ends within a row, -1: other piece or dense
+  long long cstride;
+  const double* csum;
+  const IfaceCellDev* cells;
   const double4* resp[IFACE_MAX_ENDS];    // of the end's piece, [q][kappa]
   const double* Y;
   const double* Z;
@@ -68,7 +113,8 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
   const int q = blockIdx.z, j0 = blockIdx.y * KT, i0 = blockIdx.x * KT;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   double acc[2][2] = {{0, 0}, {0, 0}};
-  for (int u = 0; u < A.nends; ++u) {
+  for (int u = 0; u < A.nends; ++u) {  // dense transforms: products of matrices
+    if (A.kind[u] >= 0) continue;
     const int M = A.em[u];
     for (int k0 = 0; k0 < M; k0 += KT) {
       for (int t = threadIdx.x; t < KT * KT; t += 256) {
@@ -105,7 +151,20 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
       const int j = j0 + tx + 16 * a, i = i0 + ty + 16 * b;
       if (j >= A.kk || i >= A.kk) continue;
       double v = (j == i ? 1.0 : 0.0) - acc[a][b];
-      if (j >= A.k || i >= A.k) {
+      if (j < A.k && i < A.k) {
+        const IfaceCellDev cj = A.cells[j], ci = A.cells[i];
+        for (int x = 0; x < 2; ++x)
+          for (int y = 0; y < 2; ++y) {
+            const int o = A.co[cj.u[x]][ci.u[y]];
+            if (o < 0) continue;
+            const double* C = A.csum + (size_t)q * A.cstride + o;
+            const int kind = A.kind[cj.u[x]], mj = cj.m[x], mi = ci.m[y];
+            const double c0 = C[mj > mi ? mj - mi : mi - mj];
+            const double g = kind == KIND_PP ? 4.0 * c0
+                             : kind == KIND_NN || kind == KIND_ND ? 2.0 * (c0 + C[mj + mi + 1]) : 2.0 * (c0 - C[mj + mi + 1]);
+            v = fma(x == 0 ? g : -g, ci.z[y], v);  // - Y (R Z): Y is -1 below, +1 above
+          }
+      } else {
         v = j == i ? 1.0 : 0.0;
         if (!(q == A.qs && j == A.kk - 1)) {  // (the last equation of a singular problem is implied: alpha = 0)
           const int a = (j < A.k ? i : j) - A.k, p = A.sp[a];
@@ -229,6 +288,46 @@ cudaError_t setup_iface(snac_plan* P, const int* d_qof, int rows, int qs_row, cu
     A.em[u] = d.M;
     A.resp[u] = resp[I.ep[u]];
   }
+  // cosine sums of the pieces with a cosine or sine transform
+  for (auto& row : A.co)
+    for (int& o : row) o = -1;
+  std::vector<CsumArgs> cs;
+  for (size_t p = 0; p < D.pc.size(); ++p) {
+    const DirectTab& d = D.pc[p];
+    CsumArgs c{};
+    for (int u = 0; u < I.nends; ++u) {
+      if (I.ep[u] != (int)p) continue;
+      A.kind[u] = d.cls == LINES_DENSE ? -1 : d.kind;
+      c.u[c.ne] = u;
+      c.ee[c.ne++] = I.ee[u];
+    }
+    if (d.cls == LINES_DENSE || c.ne == 0) continue;
+    c.M = d.M;
+    c.kind = d.kind;
+    c.slots = d.kind == KIND_PP ? d.M / 2 + 1 : d.M;
+    c.a0 = d.kind == KIND_DD ? 2 * d.M : d.kind == KIND_DN ? 2 * d.M - 1 : d.kind == KIND_ND ? 1 : 0;
+    c.da = d.kind == KIND_PP ? 4 : d.kind == KIND_DD || d.kind == KIND_DN ? -2 : 2;
+    c.resp = resp[p];
+    for (int a = 0; a < c.ne; ++a)
+      for (int b = 0; b < c.ne; ++b) {
+        A.co[c.u[a]][c.u[b]] = (int)A.cstride;
+        c.off[a][b] = A.cstride;
+        A.cstride += 2 * d.M;
+      }
+    cs.push_back(c);
+  }
+  double* csum = (double*)get((size_t)rows * A.cstride * sizeof(double));
+  IfaceCellDev* cells = (IfaceCellDev*)get(I.cells.size() * sizeof(IfaceCellDev));
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(cells, I.cells.data(), I.cells.size() * sizeof(IfaceCellDev), cudaMemcpyHostToDevice, s);
+  A.csum = csum;
+  A.cells = cells;
+  for (const CsumArgs& c : cs) {
+    if (e != cudaSuccess) break;
+    cudaFuncSetAttribute(k_csum, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);  // (M <= MAX_NZ)
+    k_csum<<<rows, 512, (2 * (size_t)c.M + 1) * sizeof(double), s>>>(c, A.cstride, csum);
+    e = cudaGetLastError();
+  }
   for (int a = 0; a < I.ns; ++a) {
     A.sc[a] = D.pc[I.sp[a]].cscale / D.pc[I.sp[a]].theta;
     A.pinned[a] = pinned[I.sp[a]];
@@ -250,6 +349,7 @@ cudaError_t setup_iface(snac_plan* P, const int* d_qof, int rows, int qs_row, cu
   const cudaError_t es = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = es;
   std::vector<double>().swap(I.Zh);
+  std::vector<IfaceCellDev>().swap(I.cells);
   return e;
 }
 

@@ -206,6 +206,12 @@ struct DirectTab {
 
 // The interfaces between the pieces of a plan (kern_iface.cu).
 constexpr int IFACE_MAX_ENDS = 16;
+// An interface cell from below and above: the end it belongs to, its place along the transformed axis, and what a
+// unit flux adds to that end's row.
+struct IfaceCellDev {
+  int u[2], m[2];
+  double z[2];
+};
 struct IfaceTab {
   int k = 0, kk = 0, E = 0;  // interface cells; with one unknown per pinned piece; spectral end values
   int nends = 0;             // ends (piece, first or last row) that carry interface cells
@@ -219,7 +225,8 @@ struct IfaceTab {
   void* d_ends = nullptr;    // [q][E]: end values of a solve
   void* d_alpha = nullptr;   // [q][IFACE_MAX_ENDS]: by piece, the last unknown of its pinned system
   void* d_num = nullptr;     // [q][IFACE_MAX_ENDS]: by piece, that unknown's eliminated right-hand side
-  std::vector<double> Zh;    // host copy, until the systems are set up
+  std::vector<double> Zh;    // host copies, until the systems are set up
+  std::vector<IfaceCellDev> cells;
 };
 
 struct DirectPlan {
