@@ -7,9 +7,11 @@
 // branch) meet along parts of their first and last rows: each piece is solved with a Neumann condition
 // there, and the fluxes through the shared faces follow from a dense system per wavenumber (kern_iface.cu).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <map>
 #include <new>
+#include <thread>
 #include <vector>
 
 #include "direct_dev.cuh"
@@ -219,13 +221,45 @@ std::vector<double> piece_widths(const snac_plan* P, const Piece& p, int axis, b
   return w;
 }
 
+// Rotations of rows k, k + 1 for k = lo .. lo + length - 1: (u, v) -> (c u + s v, c v - s u).
+struct Sweep {
+  int lo, length;
+  size_t first;  // of their cosines and sines
+};
+
+// The sweeps in order on the identity's columns i0 .. i0 + W - 1, into Z (n x n). A row between two rotations stays
+// in registers, and W columns of 384 rows in the first-level cache.
+constexpr int EIG_W = 16;
+void rotate_columns(const std::vector<Sweep>& sw, const std::vector<double>& cs, int n, int i0, double* Z) {
+  constexpr int W = EIG_W;
+  std::vector<double> z((size_t)n * W, 0.0);
+  const int w = std::min(W, n - i0);
+  for (int i = 0; i < w; ++i) z[(size_t)(i0 + i) * W + i] = 1.0;
+  for (const Sweep& s : sw) {
+    double u[W];
+    double* row = &z[(size_t)s.lo * W];
+    const double* r = &cs[s.first];
+    for (int i = 0; i < W; ++i) u[i] = row[i];
+    for (int k = 0; k < s.length; ++k, row += W, r += 2)
+      for (int i = 0; i < W; ++i) {
+        const double v = row[W + i];
+        row[i] = r[0] * u[i] + r[1] * v;
+        u[i] = r[0] * v - r[1] * u[i];
+      }
+    for (int i = 0; i < W; ++i) row[i] = u[i];
+  }
+  for (int k = 0; k < n; ++k)
+    for (int i = 0; i < w; ++i) Z[(size_t)k * n + i0 + i] = z[(size_t)k * W + i];
+}
+
 // Eigenvalues (into d) and orthonormal eigenvectors (rows of Z) of a symmetric tridiagonal matrix with
 // diagonal d and off-diagonal e (e[i] couples i and i + 1): shifted QR steps by Givens rotations chased down
-// the unreduced block (Wilkinson's shift). False if the block of one eigenvalue takes more than 60 steps.
+// the unreduced block (Wilkinson's shift). False if the block of one eigenvalue takes more than 60 steps. The
+// rotations, about 1.2 n^2, are applied to blocks of columns afterwards, by a few threads.
 bool tridiag_eigen(std::vector<double>& d, std::vector<double> e, std::vector<double>& Z) {
   const int n = (int)d.size();
-  Z.assign((size_t)n * n, 0.0);
-  for (int i = 0; i < n; ++i) Z[(size_t)i * n + i] = 1.0;
+  std::vector<Sweep> sw;
+  std::vector<double> cs;
   auto small = [&](int i) { return std::fabs(e[i]) <= 1.1e-16 * (std::fabs(d[i]) + std::fabs(d[i + 1])); };
   int steps = 0;
   for (int hi = n - 1; hi > 0;) {
@@ -241,6 +275,7 @@ bool tridiag_eigen(std::vector<double>& d, std::vector<double> e, std::vector<do
     const double h = 0.5 * (d[hi - 1] - d[hi]), b = e[hi - 1];
     const double mu = d[hi] - b * b / (h + std::copysign(std::hypot(h, b), h));
     double x = d[lo] - mu, z = e[lo];
+    sw.push_back({lo, hi - lo, cs.size()});
     for (int k = lo; k < hi; ++k) {
       // rotate rows and columns k, k + 1 so that (x, z) becomes (r, 0)
       const double r = std::hypot(x, z), c = r > 0.0 ? x / r : 1.0, s = r > 0.0 ? z / r : 0.0;
@@ -254,15 +289,30 @@ bool tridiag_eigen(std::vector<double>& d, std::vector<double> e, std::vector<do
         z = s * e[k + 1];
         e[k + 1] *= c;
       }
-      double* z0 = &Z[(size_t)k * n];
-      double* z1 = z0 + n;
-      for (int i = 0; i < n; ++i) {
-        const double u = z0[i], v = z1[i];
-        z0[i] = c * u + s * v;
-        z1[i] = c * v - s * u;
-      }
+      cs.push_back(c);
+      cs.push_back(s);
     }
   }
+  Z.resize((size_t)n * n);
+  const int blocks = (n + EIG_W - 1) / EIG_W;
+  std::atomic<int> next{0};
+  std::atomic<bool> failed{false};
+  auto work = [&] {
+    try {
+      for (int b; (b = next.fetch_add(1)) < blocks;) rotate_columns(sw, cs, n, b * EIG_W, Z.data());
+    } catch (...) {
+      failed = true;
+    }
+  };
+  std::vector<std::thread> th;
+  const int want = std::min({7, blocks / 2, (int)std::thread::hardware_concurrency() - 1});
+  try {
+    for (int t = 0; t < want; ++t) th.emplace_back(work);
+  } catch (...) {  // no more threads: the ones there are do
+  }
+  work();
+  for (std::thread& t : th) t.join();
+  if (failed) throw std::bad_alloc();
   return true;
 }
 
@@ -460,17 +510,22 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
     constexpr double LOW_SPAN = 256.0;
     std::vector<std::pair<double, int>> by;
     std::vector<unsigned char> low((size_t)P->nz * M, 0);
+    std::vector<int> smooth(M);  // slots from the smallest -lambda up
+    for (int k = 0; k < M; ++k) smooth[k] = k;
+    std::stable_sort(smooth.begin(), smooth.end(), [&](int a, int b) { return D.lam[a] > D.lam[b]; });
+    const auto value = [&](int l, int k) { return -(P->sigma[l] * D.cscale + D.lam[k]); };
     double least = INFINITY;
     for (int l = 0; l < P->nz; ++l)
-      for (int k = 0; k < M; ++k) {
-        const double v = -(P->sigma[l] * D.cscale + D.lam[k]);
-        if (v > 0.0) least = std::min(least, v);
-      }
+      for (int k : smooth)
+        if (value(l, k) > 0.0) {
+          least = std::min(least, value(l, k));
+          break;
+        }
     if (N <= 512 && !P->ranged)
       for (int l = 0; l < P->nz; ++l)
-        for (int k = 0; k < M; ++k) {
-          const double v = -(P->sigma[l] * D.cscale + D.lam[k]);
-          if (v <= LOW_SPAN * least) by.push_back({v, l * M + k});
+        for (int k : smooth) {
+          if (value(l, k) > LOW_SPAN * least) break;
+          by.push_back({value(l, k), l * M + k});
         }
     std::sort(by.begin(), by.end());
     by.resize(std::min(by.size(), low.size() / 64));
@@ -492,23 +547,34 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
 }
 
 // Entries of the transforms as the line kernels scale them (direct_dev.cuh): forward F[kappa][m], inverse
-// B[m][kappa], B F = 2 M.
-double fwd_entry(int kind, int M, int kap, int m) {
-  const double pi = M_PI;
-  switch (kind) {
-    case KIND_PP: return kap <= M / 2 ? 2.0 * std::cos(2.0 * pi * ((long long)kap * m % M) / M)
-                                      : -2.0 * std::sin(2.0 * pi * ((long long)(M - kap) * m % M) / M);
-    case KIND_NN: return 2.0 * std::cos(pi * ((2LL * m + 1) * kap % (4LL * M)) / (2.0 * M));
-    case KIND_DD: return 2.0 * std::sin(pi * ((2LL * m + 1) * (M - kap) % (4LL * M)) / (2.0 * M));
-    case KIND_ND: return 2.0 * std::cos(pi * ((2LL * m + 1) * (2LL * kap + 1) % (8LL * M)) / (4.0 * M));
-    default: return 2.0 * std::sin(pi * ((2LL * m + 1) * (2LL * (M - 1 - kap) + 1) % (8LL * M)) / (4.0 * M));
+// B[m][kappa], B F = 2 M. From one table of 2 cos(pi t / 4M) or 2 sin(pi t / 4M), t < 8M: the interfaces of the L
+// of 512 x 512 cells need 4e5 entries.
+struct Entries {
+  int kind, M;
+  std::vector<double> c, s;
+  Entries(int kind_, int M_) : kind(kind_), M(M_) {
+    const bool cosine = kind != KIND_DD && kind != KIND_DN, sine = !cosine || kind == KIND_PP;
+    for (int t = 0; t < 8 * M; ++t) {
+      if (cosine) c.push_back(2.0 * std::cos(M_PI * t / (4.0 * M)));
+      if (sine) s.push_back(2.0 * std::sin(M_PI * t / (4.0 * M)));
+    }
   }
-}
-double bwd_entry(int kind, int M, int m, int kap) {
-  const double f = fwd_entry(kind, M, kap, m);
-  const bool half = (kind == KIND_PP && (kap == 0 || kap == M / 2)) || ((kind == KIND_NN || kind == KIND_DD) && kap == 0);
-  return half ? 0.5 * f : f;
-}
+  double fwd(int kap, int m) const {
+    const long long T = 8LL * M;
+    switch (kind) {
+      case KIND_PP: return kap <= M / 2 ? c[8LL * kap * m % T] : -s[8LL * (M - kap) * m % T];
+      case KIND_NN: return c[2 * (2LL * m + 1) * kap % T];
+      case KIND_DD: return s[2 * (2LL * m + 1) * (M - kap) % T];
+      case KIND_ND: return c[(2LL * m + 1) * (2LL * kap + 1) % T];
+      default: return s[(2LL * m + 1) * (2LL * (M - 1 - kap) + 1) % T];
+    }
+  }
+  double bwd(int m, int kap) const {
+    const double f = fwd(kap, m);
+    const bool half = (kind == KIND_PP && (kap == 0 || kap == M / 2)) || ((kind == KIND_NN || kind == KIND_DD) && kap == 0);
+    return half ? 0.5 * f : f;
+  }
+};
 
 // The matrices between end values, jumps and fluxes.
 int build_iface(snac_plan* P, const Layout& L) {
@@ -533,6 +599,8 @@ int build_iface(snac_plan* P, const Layout& L) {
     if (D.pc[p].pin) I.sp[I.ns++] = (int)p;
   I.kk = I.k + I.ns;
   std::vector<double> Y((size_t)I.E * I.kk, 0.0), Z((size_t)I.kk * I.E, 0.0);
+  std::vector<Entries> en;
+  for (const DirectTab& T : D.pc) en.emplace_back(T.kind, T.cls == LINES_DENSE ? 0 : T.M);
   for (int j = 0; j < I.k; ++j) {
     const IfaceCell& c = L.cells[j];
     I.cells.push_back({{end_of[2 * c.pa + 1], end_of[2 * c.pb]}, {c.ma, c.mb}, {-c.ca, c.cb}});
@@ -541,8 +609,8 @@ int build_iface(snac_plan* P, const Layout& L) {
       const int u = end_of[2 * p + (side == 0 ? 1 : 0)];
       const DirectTab& T = D.pc[p];
       for (int k = 0; k < T.M; ++k) {
-        Y[(size_t)(I.eo[u] + k) * I.kk + j] = (side == 0 ? -1.0 : 1.0) * (T.cls == LINES_DENSE ? T.B[(size_t)m * T.M + k] : bwd_entry(T.kind, T.M, m, k));
-        Z[(size_t)j * I.E + I.eo[u] + k] = (side == 0 ? -c.ca : c.cb) * (T.cls == LINES_DENSE ? T.F[(size_t)k * T.M + m] : fwd_entry(T.kind, T.M, k, m));
+        Y[(size_t)(I.eo[u] + k) * I.kk + j] = (side == 0 ? -1.0 : 1.0) * (T.cls == LINES_DENSE ? T.B[(size_t)m * T.M + k] : en[p].bwd(m, k));
+        Z[(size_t)j * I.E + I.eo[u] + k] = (side == 0 ? -c.ca : c.cb) * (T.cls == LINES_DENSE ? T.F[(size_t)k * T.M + m] : en[p].fwd(k, m));
       }
     }
   }
