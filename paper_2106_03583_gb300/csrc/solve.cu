@@ -374,8 +374,8 @@ struct Job {
 
 // Mixed plans compute the residual of an intermediate defect-correction step in float-float
 // arithmetic (written in FP32, the precision the FP32 transform reads); the FP64 pass decides
-// convergence: it runs after a correction that aimed at the tolerance itself, and whenever the
-// float-float residual comes within 2x of the tolerance. (The float-float error, a few units of
+// convergence: it runs after a correction that aimed at the tolerance itself (or within 2x of it), and
+// whenever the float-float residual comes within 2x of the tolerance. (The float-float error, a few units of
 // 2^-47 of |f| + |A||p| per cell, is about 1e-11 ||f|| on the 2.7e8-cell channel: it steers an
 // intermediate correction well enough, but a convergence decision near tol takes the FP64 pass.)
 
@@ -449,9 +449,7 @@ cudaError_t job_resid_read(Job& J, cudaStream_t s) {
   J.late_wait = false;
   if (J.ff && !J.redo) {
     J.rn = std::sqrt(P->h_sums[0]);
-    // (NaN stays: reported by the decision). Direct plans take another step anyway above half the
-    // tolerance, where the float-float value decides as well
-    J.r32 = !(J.rn <= (P->direct.on && J.k < P->max_outer ? 0.5 : 2.0) * J.tol * J.fn);
+    J.r32 = !(J.rn <= 2.0 * J.tol * J.fn);  // (NaN stays: reported by the decision)
     if (J.r32) return cudaSuccess;
     J.redo = true;
     const bool need_vp = P->singular;
@@ -521,9 +519,11 @@ int job_decide(Job& J, cudaStream_t s) {
   if (P->direct.on && P->precision == SNAC_MIXED) {
     // a direct step reduces the residual to the FP32 floor whatever the target: from f to 1e-4 or so of it (6e-6
     // to 1.1e-4 measured on planes of 64^2 to 512^2 cells), by about 3e-7 from the rough residual that such a step
-    // leaves (6e-7 with interfaces between pieces). The FP64 pass comes directly where that reaches the
-    // tolerance (with the margin above): at 1e-3 one step and no float-float pass, as with V-cycles
-    J.aim_final = (J.k == 0 ? 2e-4 : P->direct.it.k ? 6e-7 : 3e-7) * rel <= 0.5 * J.tol;
+    // leaves (6e-7 with interfaces between pieces). The FP64 pass comes directly where that comes within 2x of
+    // the tolerance, from where it is needed in any case: to decide, or as the right-hand side of one more step
+    // (from a float-float residual that step ends at 5e-12 to 1e-11 of f, from the FP64 one at 2e-13: L of 512 x
+    // 512 x 128 cells, 1024 x 512 x 512 channel). At 1e-3 one step and no float-float pass, as with V-cycles
+    J.aim_final = (J.k == 0 ? 2e-4 : P->direct.it.k ? 6e-7 : 3e-7) * rel <= 2.0 * J.tol;
   }
   J.fused = fused_ready(P);
   if (J.fused) {  // the forward transform goes into the same launch as the wavenumber solves

@@ -272,3 +272,20 @@ def test_loose_tolerance_takes_one_residual_pass(case):
     assert st["field3d_ff"]["launches"] == 0 and st["field3d"]["launches"] == 2   # the statistics of f, the residual
     assert osv.rel_residual(blocks, f, host(p)) <= 1.01e-3
     pl.close()
+
+
+@pytest.mark.parametrize("case", [("1", 32, 768, 0.0, 2.0, "DDNN", "PP"), ("1", 64, 1024, 0.0, 2.0, "DDNN", "PP"),
+                                  ("L", 64, 544, 0.0, 1.0, "NNDN", "NN")], ids=lambda c: "-".join(map(str, c[:6])))
+def test_mixed_step_near_the_tolerance_starts_from_the_fp64_residual(case):
+    """A step from a residual within twice the tolerance 1e-10 reduces it by 6e-7 or more, to 1.2e-16, if it is the
+    FP64 residual: what is left is the FP64 rounding of the residual of these clustered axes, below 2e-12. From a
+    float-float residual it would be about 1e-11."""
+    import torch
+    layout, nx, ny, xf, yf, walls, zp = case
+    blocks = build(layout, nx, ny, xf, yf, walls, zp, nz=8)
+    f = inputs.divergence_rhs(blocks, 1)
+    pl = plan(blocks, precision="mixed")
+    p = torch.zeros(len(f), dtype=torch.float64, device="cuda")
+    info = pl.solve(dev(f), p, tol=1e-10)
+    assert info["status"] == 0 and info["outer_iters"] == 3 and info["rel_res"] <= 2e-12
+    pl.close()
