@@ -506,33 +506,39 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
   int st;
   if (!f64) {
     // the systems with the smallest -(lambda + sigma): up to LOW_SPAN times the smallest nonzero one, 1/64 of
-    // all at most (kern_direct.cu, k_tri_low; rows of longer systems do not fit its CTA)
+    // all at most (kern_direct.cu, k_tri_low; rows of longer systems do not fit its CTA). Of all wavenumbers of the
+    // problem, so that a plan that holds a range of them solves the same systems the same way
     constexpr double LOW_SPAN = 256.0;
     std::vector<std::pair<double, int>> by;
     std::vector<unsigned char> low((size_t)P->nz * M, 0);
     std::vector<int> smooth(M);  // slots from the smallest -lambda up
     for (int k = 0; k < M; ++k) smooth[k] = k;
     std::stable_sort(smooth.begin(), smooth.end(), [&](int a, int b) { return D.lam[a] > D.lam[b]; });
-    const auto value = [&](int l, int k) { return -(P->sigma[l] * D.cscale + D.lam[k]); };
+    std::vector<double> sigma(P->nzt);
+    for (int q = 0; q < P->nzt; ++q) sigma[q] = mode_lambda(P->kind, P->nzt, q) / (P->dz * P->dz) + P->shift;
+    std::copy(P->sigma.begin(), P->sigma.end(), sigma.begin() + P->q0);
+    const auto value = [&](int q, int k) { return -(sigma[q] * D.cscale + D.lam[k]); };
     double least = INFINITY;
-    for (int l = 0; l < P->nz; ++l)
+    for (int q = 0; q < P->nzt; ++q)
       for (int k : smooth)
-        if (value(l, k) > 0.0) {
-          least = std::min(least, value(l, k));
+        if (value(q, k) > 0.0) {
+          least = std::min(least, value(q, k));
           break;
         }
-    if (N <= 512 && !P->ranged)
-      for (int l = 0; l < P->nz; ++l)
+    if (N <= 512)
+      for (int q = 0; q < P->nzt; ++q)
         for (int k : smooth) {
-          if (value(l, k) > LOW_SPAN * least) break;
-          by.push_back({value(l, k), l * M + k});
+          if (value(q, k) > LOW_SPAN * least) break;
+          by.push_back({value(q, k), q * M + k});
         }
     std::sort(by.begin(), by.end());
-    by.resize(std::min(by.size(), low.size() / 64));
+    by.resize(std::min(by.size(), (size_t)P->nzt * M / 64));
     std::vector<int> list;
     for (const auto& v : by) {
-      list.push_back(v.second);
-      low[v.second] = 1;
+      const int l = v.second / M - P->q0;
+      if (l < 0 || l >= P->nz) continue;
+      list.push_back(l * M + v.second % M);
+      low[list.back()] = 1;
     }
     D.nlow = (int)list.size();
     if ((st = up_vec(P, &D.d_lam64, D.lam)) || (st = up_vec(P, &D.d_tri64, tri)) ||

@@ -289,3 +289,23 @@ def test_mixed_step_near_the_tolerance_starts_from_the_fp64_residual(case):
     info = pl.solve(dev(f), p, tol=1e-10)
     assert info["status"] == 0 and info["outer_iters"] == 3 and info["rel_res"] <= 2e-12
     pl.close()
+
+
+@pytest.mark.parametrize("case", [DIRECT[8], DIRECT[26], DIRECT[0]], ids=lambda c: "-".join(map(str, c[:6])))
+def test_mixed_range_plan_solves_as_the_whole_plan(case):
+    """A plan that holds some wavenumbers takes the smoothest systems of the whole problem in FP64, as the whole plan
+    does: the same solutions bit for bit."""
+    import torch
+    layout, nx, ny, xf, yf, walls, zp, per = case
+    blocks = build(layout, nx, ny, xf, yf, walls, zp, nz=12, per=per)
+    whole, n = plan(blocks, precision="mixed"), 12
+    F = torch.from_numpy(np.random.default_rng(7).standard_normal((n, whole.ncell)).astype(np.float32)).cuda()
+    u = torch.empty_like(F)
+    whole.mode_solve(F, u, target=0.0)
+    for a, b in ((0, 5), (5, 12)):
+        part = plan(blocks, precision="mixed", modes=(a, b))
+        v = torch.empty((b - a, whole.ncell), dtype=torch.float32, device="cuda")
+        part.mode_solve(F[a:b].contiguous(), v, target=0.0)
+        assert torch.equal(v, u[a:b])
+        part.close()
+    whole.close()
