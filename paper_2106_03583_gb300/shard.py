@@ -312,6 +312,7 @@ class ShardedSolver:
             info["rel_res"] = 0.0
             return info
         prev = math.inf
+        direct = False   # the last step solved every wavenumber directly (one cycle each)
         for k in range(self.max_outer + 1):
             rn = math.sqrt(sums[0])
             rel = rn / fn
@@ -319,10 +320,17 @@ class ShardedSolver:
             if not math.isfinite(rel):
                 info["status"] = -6
                 return info
-            if rel <= tol:
+            # direct FP32 solves stop at half the tolerance where they can, as an unsharded solve does: what
+            # a step leaves lies in the smoothest modes, where a residual just under the tolerance still
+            # means several times as much error in p
+            if rel <= (0.5 * tol if mixed and direct and k < self.max_outer else tol):
                 return info
             if k == self.max_outer or rel >= prev:
-                info["status"] = -5
+                if prev <= tol:   # the step beyond the tolerance did not help: take it back
+                    st.backward_update(modes.neg_(), p)
+                    info["rel_res"] = prev
+                else:
+                    info["status"] = -5
                 return info
             prev = rel
             target = 0.5 * tol * fn
@@ -330,7 +338,9 @@ class ShardedSolver:
                 target = max(target, self.inner_reduction * rn)
             st.forward(r, modes)                                   # Algorithm 3, first loop
             self.pencil_to_slab(modes, slab_rhs)                   # pencil -> slab
-            info["cycles"] += int(self._sum([st.mode_solve(slab_rhs, slab_sol, target)])[0])
+            cycles = int(self._sum([st.mode_solve(slab_rhs, slab_sol, target)])[0])
+            info["cycles"] += cycles
+            direct = cycles == nz
             if self.singular:
                 st.fix_mean(slab_sol, float(sums[2]))              # on the rank holding q = 0
             self.slab_to_pencil(slab_sol, modes)                   # slab -> pencil

@@ -120,3 +120,38 @@ def test_predicted_costs_fall_with_the_eigenvalue():
     blocks, _ = inputs.config("mb2x2", seed=0, scale=8)      # NN: |lambda_q| grows with q
     c = shard.predicted_mode_costs(blocks)
     assert c[0] >= c[-1] and np.all(np.diff(c) <= 0) and c.min() >= 1
+
+
+@pytest.mark.parametrize("delta,floor,steps,lo,hi", [
+    (8.9e-6, 0.0, 3, 0.0, 1e-12),    # 7.9e-11 after two steps: within the tolerance, not within half of it
+    (6e-6, 0.0, 2, 3e-11, 4e-11),    # 3.6e-11 after two: done
+    (8.9e-6, 1.0, 3, 7e-11, 9e-11)])  # a third step that does not help is taken back
+def test_direct_mixed_steps_stop_at_half_the_tolerance(delta, floor, steps, lo, hi):
+    """Solves of one cycle per wavenumber whose correction is off by a factor 1 + delta, so that every step reduces
+    the residual by delta; with ``floor`` the third one does not reduce it."""
+    sys.path.insert(0, os.path.join(ROOT, "tests"))
+    import torch
+    from oracle import grid as ogrid
+    from paper_2106_03583_gb300 import shard
+    from shard_stages import OracleStages, ThreadExchange
+
+    class Direct(OracleStages):
+        step = 0
+
+        def mode_solve(self, rhs, sol, target):
+            super().mode_solve(rhs, sol, target)
+            self.step += 1
+            sol.mul_(1.0 + (delta if self.step < 3 or not floor else -2.0))
+            return self.q1 - self.q0
+
+    blocks, f = _problem("L")
+    g = ogrid.Grid(blocks)
+    n = g.plane.n
+    sv = shard.ShardedSolver(blocks, Direct(blocks, 0, g.nz), ThreadExchange(ThreadExchange.Hub(1), 0), [(0, n)],
+                             [(0, g.nz)])
+    F, p = torch.from_numpy(g.to_planes(f)), torch.zeros((g.nz, n), dtype=torch.float64)
+    info = sv.solve(F, p, tol=1e-10, mixed=True)
+    r = (F.numpy() - g.apply(p.numpy()))
+    rel = float(np.linalg.norm(r) / np.linalg.norm(F.numpy()))
+    assert info["status"] == 0 and info["outer_iters"] == steps
+    assert lo <= info["rel_res"] <= hi and abs(rel - info["rel_res"]) <= 0.01 * hi
