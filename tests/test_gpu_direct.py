@@ -309,3 +309,16 @@ def test_mixed_range_plan_solves_as_the_whole_plan(case):
         assert torch.equal(v, u[a:b])
         part.close()
     whole.close()
+
+
+# two rows of blocks around a periodic axis whose rings are met at different blocks; interfaces of 1024 cells with two
+# pinned pieces (1026 unknowns: more than the threads of the interface kernel)
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("case", [("2x2", 48, 40, 0.0, 1.2, "NNDN", "NN", 6, (True, False)),
+                                  ("2x2", 160, 128, 0.0, 1.0, "NNNN", "PP", 6, (True, False)),
+                                  ("2x2", 40, 48, 1.1, 0.0, "DNNN", "DD", 6, (False, True)),
+                                  ("L", 2048, 2048, 0.0, 0.0, "NNNN", "NN", 4, (False, False))],
+                         ids=lambda c: "-".join(map(str, c[:6])))
+def test_direct_mode_solve_rings_and_long_interfaces(case, precision):
+    layout, nx, ny, xf, yf, walls, zp, nz, per = case
+    _check_modes(build(layout, nx, ny, xf, yf, walls, zp, nz=nz, per=per), precision)
