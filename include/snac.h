@@ -195,6 +195,12 @@ int snac_poisson_solve_batch(int32_t n, snac_plan *const *plans, const double *c
  * plan's internal work buffers, not the caller's arrays. */
 int snac_test_wait_timeout(snac_plan *plan, double wait_seconds, void *stream);
 
+/* The same within whole solves: snac_poisson_solve_batch (n = 1: snac_poisson_solve) with a chunk count that
+ * nothing can reach for plan `which` alone, and the limit of wait_seconds for every wait. That plan's status is
+ * SNAC_ERR_TIMEOUT and its d_p is left as it was; the others are solved. */
+int snac_test_solve_timeout(int32_t n, snac_plan *const *plans, const double *const *d_rhs, double *const *d_p,
+                            double tol, int32_t which, double wait_seconds, int32_t *h_status, void *stream);
+
 /* Statistics of the last solve. */
 int snac_plan_info(const snac_plan *plan, snac_solve_info *info);
 

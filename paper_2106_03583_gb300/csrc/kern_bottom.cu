@@ -928,8 +928,8 @@ size_t fwd_onchip_batch_scratch(int nplans, int nitems) {
 }
 
 template <typename T>
-cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs, const double* targets, int nplans,
-                               double wait_s, void* d_scratch, int sms, cudaStream_t s) {
+cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs, const double* targets,
+                               const int* extra, int nplans, double wait_s, void* d_scratch, int sms, cudaStream_t s) {
   constexpr int TC = fused_tc<T>();
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   char* base = static_cast<char*>(d_scratch);
@@ -950,7 +950,7 @@ cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs
     snac_plan* P = plans[k];
     const cudaError_t er = fused_reset(P, s);
     if (er != cudaSuccess) return er;
-    fargs[k] = fwd_args<T>(P, inputs[k].in3, inputs[k].in_f32, inputs[k].shift0, d_ctr + 1 + k, P->dh_wait, 0);
+    fargs[k] = fwd_args<T>(P, inputs[k].in3, inputs[k].in_f32, inputs[k].shift0, d_ctr + 1 + k, P->dh_wait, extra[k]);
     args[k] = onchip_args<T>(P, targets[k]);
     smem = std::max(smem, fused_smem<T>(P));
     KernelStat& ks = P->kstats[K_FWD_ONCHIP];  // each plan counts the shared launch once
@@ -974,13 +974,14 @@ cudaError_t fwd_onchip_batch_t(snac_plan* const* plans, const FusedInput* inputs
 }
 
 cudaError_t launch_fwd_onchip_batch(snac_plan* const* plans, const FusedInput* inputs, const double* targets,
-                                    int nplans, double wait_s, void* d_scratch, int sms, cudaStream_t s) {
+                                    const int* extra_need, int nplans, double wait_s, void* d_scratch, int sms,
+                                    cudaStream_t s) {
   if (nplans <= 0) return cudaSuccess;
   for (int k = 0; k < nplans; ++k)
     if (!fused_ready(plans[k]) || plans[k]->precision != plans[0]->precision) return cudaErrorInvalidValue;
   if (plans[0]->precision == SNAC_FP64)
-    return fwd_onchip_batch_t<double>(plans, inputs, targets, nplans, wait_s, d_scratch, sms, s);
-  return fwd_onchip_batch_t<float>(plans, inputs, targets, nplans, wait_s, d_scratch, sms, s);
+    return fwd_onchip_batch_t<double>(plans, inputs, targets, extra_need, nplans, wait_s, d_scratch, sms, s);
+  return fwd_onchip_batch_t<float>(plans, inputs, targets, extra_need, nplans, wait_s, d_scratch, sms, s);
 }
 
 // Many plans, one launch: the items (plan index, wavenumber) of plans of the same precision, every

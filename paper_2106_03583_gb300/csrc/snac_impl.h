@@ -483,7 +483,8 @@ struct FusedInput {
 };
 size_t fwd_onchip_batch_scratch(int nplans, int nitems);
 cudaError_t launch_fwd_onchip_batch(snac_plan* const* plans, const FusedInput* inputs, const double* targets,
-                                    int nplans, double wait_s, void* d_scratch, int sms, cudaStream_t s);
+                                    const int* extra_need, int nplans, double wait_s, void* d_scratch, int sms,
+                                    cudaStream_t s);
 constexpr double WAIT_LIMIT_S = 1.0;  // bound of every device-side wait of a solve
 cudaError_t launch_onchip_batch(snac_plan* const* plans, const double* targets, int nplans, const int2* h_items,
                                 int nitems, void* d_scratch, int sms, cudaStream_t s);

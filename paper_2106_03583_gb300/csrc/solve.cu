@@ -361,6 +361,7 @@ struct Job {
   bool p_zero = false, updated = false, aim_final = false, r32 = false, ff = false, redo = false;
   bool late_wait = false;  // the status of the step's bounded waits is read with the next residual
   bool fused = false;  // this step's forward transform runs inside the on-chip launch
+  int extra_need = 0;  // chunks more than there are that its solves wait for (the timeout self-test)
   FusedInput fin{};
   double fshift = 0.0, fn = 0.0, fn_pre = 0.0, prev_rel = INFINITY, rn = 0.0, target = 0.0;
   int k = 0;
@@ -612,7 +613,7 @@ struct SideStreams {
   }
 };
 
-int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
+int run_jobs(std::vector<Job>& jobs, cudaStream_t s, double wait_s = WAIT_LIMIT_S) {
   SideStreams ss(s, jobs.size() > 1 ? (int)std::min<size_t>(16, jobs.size()) : 0);
   auto js = [&](const Job& J) { return ss.of((size_t)(&J - jobs.data())); };
   auto sync = [&]() -> cudaError_t {
@@ -666,18 +667,20 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
       if (fusedj[g].empty()) continue;
       if (fusedj[g].size() == 1) {
         Job& J = *fusedj[g][0];
-        job_cuda(J, launch_fwd_onchip(J.P, J.fin.in3, J.fin.in_f32, J.fin.shift0, J.target, WAIT_LIMIT_S, 0, s),
+        job_cuda(J, launch_fwd_onchip(J.P, J.fin.in3, J.fin.in_f32, J.fin.shift0, J.target, wait_s, J.extra_need, s),
                  "forward transform and on-chip wavenumber solves");
         continue;
       }
       std::vector<snac_plan*> plans;
       std::vector<FusedInput> ins;
       std::vector<double> targets;
+      std::vector<int> extra;
       int nitems = 0;
       for (Job* J : fusedj[g]) {
         plans.push_back(J->P);
         ins.push_back(J->fin);
         targets.push_back(J->target);
+        extra.push_back(J->extra_need);
         nitems += J->P->nz + (int)std::max(J->P->chunks64.size(), J->P->chunks32.size());
       }
       const size_t need = fwd_onchip_batch_scratch((int)plans.size(), nitems);
@@ -688,8 +691,8 @@ int run_jobs(std::vector<Job>& jobs, cudaStream_t s) {
         if ((e = cudaMallocAsync(&scratch, need, s)) != cudaSuccess) { status = cuda_fail(e, "cudaMallocAsync"); break; }
         scratch_bytes = need;
       }
-      e = launch_fwd_onchip_batch(plans.data(), ins.data(), targets.data(), (int)plans.size(), WAIT_LIMIT_S, scratch,
-                                  sms, s);
+      e = launch_fwd_onchip_batch(plans.data(), ins.data(), targets.data(), extra.data(), (int)plans.size(), wait_s,
+                                  scratch, sms, s);
       if (e != cudaSuccess)
         for (Job* J : fusedj[g]) job_cuda(*J, e, "forward transform and on-chip wavenumber solves");
       // the next group reuses the scratch only after this launch has read it
@@ -820,8 +823,8 @@ int snac_poisson_solve(snac_plan* plan, const double* d_rhs, double* d_p, double
   return st;
 }
 
-int snac_poisson_solve_batch(int32_t n, snac_plan* const* plans, const double* const* d_rhs, double* const* d_p,
-                             double tol, int32_t* h_status, void* stream) {
+static int solve_batch(int32_t n, snac_plan* const* plans, const double* const* d_rhs, double* const* d_p, double tol,
+                       int32_t* h_status, int which, double wait_s, void* stream) {
   if (n < 1 || !plans || !d_rhs || !d_p || !h_status || !(tol > 0.0) || !std::isfinite(tol)) return SNAC_ERR_INVALID_ARG;
   std::vector<Job> jobs(n);
   for (int k = 0; k < n; ++k) {
@@ -837,8 +840,9 @@ int snac_poisson_solve_batch(int32_t n, snac_plan* const* plans, const double* c
     jobs[k].f = d_rhs[k];
     jobs[k].p = d_p[k];
     jobs[k].tol = tol;
+    jobs[k].extra_need = k == which ? 1 : 0;
   }
-  const int st = run_jobs(jobs, (cudaStream_t)stream);
+  const int st = run_jobs(jobs, (cudaStream_t)stream, wait_s);
   int worst = st;
   for (int k = 0; k < n; ++k) {
     h_status[k] = st ? st : jobs[k].st;
@@ -846,6 +850,17 @@ int snac_poisson_solve_batch(int32_t n, snac_plan* const* plans, const double* c
     if (!worst && h_status[k]) worst = h_status[k];
   }
   return worst;
+}
+
+int snac_poisson_solve_batch(int32_t n, snac_plan* const* plans, const double* const* d_rhs, double* const* d_p,
+                             double tol, int32_t* h_status, void* stream) {
+  return solve_batch(n, plans, d_rhs, d_p, tol, h_status, -1, WAIT_LIMIT_S, stream);
+}
+
+int snac_test_solve_timeout(int32_t n, snac_plan* const* plans, const double* const* d_rhs, double* const* d_p,
+                            double tol, int32_t which, double wait_seconds, int32_t* h_status, void* stream) {
+  if (which < 0 || which >= n || !(wait_seconds > 0.0) || wait_seconds > WAIT_LIMIT_S) return SNAC_ERR_INVALID_ARG;
+  return solve_batch(n, plans, d_rhs, d_p, tol, h_status, which, wait_seconds, stream);
 }
 
 int snac_test_wait_timeout(snac_plan* plan, double wait_seconds, void* stream) {

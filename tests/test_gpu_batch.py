@@ -10,6 +10,7 @@
 import numpy as np
 import pytest
 
+from oracle import grid as ogrid
 from oracle import solve as osv
 from paper_2106_03583_gb300 import inputs, snac
 
@@ -127,3 +128,42 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(precision):
     lvl = plan(blocks, precision=precision, onchip=False)   # level by level: no on-chip wait to test
     assert lvl.test_wait_timeout(0.05) == "INVALID_ARG"
     lvl.close()
+
+
+def _solve_with_timeout(plans, f, p, which):
+    import ctypes
+    import torch
+    n = len(plans)
+    vps = ctypes.c_void_p * n
+    st = (ctypes.c_int32 * n)()
+    rc = snac.lib().snac_test_solve_timeout(n, vps(*[pl._h for pl in plans]), vps(*[t.data_ptr() for t in f]),
+                                            vps(*[t.data_ptr() for t in p]), 1e-10, which, 0.02, st,
+                                            ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    return rc, [snac.STATUS[s] for s in st]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [1, 3])
+def test_a_solve_whose_wait_gives_up(n, precision):
+    """A whole solve, and one plan of a batch, whose device-side waits run out: that plan alone reports it, its p is
+    as it was bit for bit (the update behind the launch skips itself), and the next solve converges."""
+    probs = [make(lay, n=16, nz=nz, zpair=z, walls=w) for lay, nz, z, w in
+             (("1", 12, "PP", ("D", "D", "N", "N")), ("2x2", 8, "NN", ("N", "N", "N", "N")), ("L", 10, "DN", ("D", "N", "N", "N")))]
+    for which in range(n):
+        blocks = probs if n == 3 else [probs[1]]
+        f = [inputs.uniform_rhs(b, 3 + k, remove_mean=ogrid.Grid(b).singular) for k, b in enumerate(blocks)]
+        plans = [plan(b, precision=precision) for b in blocks]
+        df = [dev(x) for x in f]
+        rng = np.random.default_rng(1)
+        start = [rng.standard_normal(len(x)) for x in f]
+        p = [dev(x) for x in start]
+        rc, st = _solve_with_timeout(plans, df, p, which)
+        assert rc == -8 and st == ["TIMEOUT" if k == which else "OK" for k in range(n)]
+        assert np.array_equal(host(p[which]), start[which])
+        for k in range(n):
+            if k != which:
+                assert osv.rel_residual(blocks[k], f[k], host(p[k])) <= 1.01e-10
+        assert plans[which].solve(df[which], p[which], tol=1e-10)["status"] == 0
+        assert osv.rel_residual(blocks[which], f[which], host(p[which])) <= 1.01e-10
+        for pl in plans:
+            pl.close()
