@@ -221,7 +221,7 @@ def test_direct_solve_with_a_nearly_singular_piece(case, precision):
     blocks = build(*case)
     f = inputs.divergence_rhs(blocks, 8)
     steps = []
-    for shift in (0.0, -1e-13, -1e-8, -1e-4, -1e-2):
+    for shift in (0.0, -1e-13, -1e-8, -1e-4, -1e-2, -1.0, -10.0):
         pl = plan(blocks, precision=precision, shift=shift)
         p = torch.zeros(len(f), dtype=torch.float64, device="cuda")
         info = pl.solve(dev(f), p, tol=1e-10)
