@@ -361,7 +361,9 @@ static cudaError_t pencil_tables(snac_plan* P, long long ncols) {
     cudaError_t e = cudaMalloc((void**)d, bytes);
     if (e != cudaSuccess) return e;
     P->pen_tallocs.push_back(*d);
-    return copy_in(P, *d, src, bytes);
+    e = copy_in(P, *d, src, bytes);
+    setup_done(P);
+    return e;
   };
   cudaError_t e;
   if ((e = put(&P->d_pen_tblk, &b, sizeof b)) != cudaSuccess || (e = put(&P->d_pen_tcb, &c, sizeof c)) != cudaSuccess ||

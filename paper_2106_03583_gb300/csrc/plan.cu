@@ -502,7 +502,7 @@ void free_plan(snac_plan* P) {
   profile_release(P);
   for (auto& kv : P->round_graphs)
     if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
-  if (P->setup_stream) cudaStreamDestroy(P->setup_stream);
+  setup_done(P);
   if (P->capture_stream) cudaStreamDestroy(P->capture_stream);
   for (void* p : P->allocs) cudaFree(p);
   for (void* p : P->pen_tallocs) cudaFree(p);
@@ -990,6 +990,7 @@ int create(snac_plan** out, int32_t nblocks, const snac_block* blocks_in, int32_
     free_plan(P);
     return st;
   }
+  setup_done(P);
   P->mode_cycles.assign(P->nz, 0);
   P->info.levels = (int)P->lev.size();
   P->info.n_modes = P->nz;
@@ -1005,6 +1006,11 @@ cudaError_t copy_in(snac_plan* P, void* dst, const void* src, size_t bytes) {
   if (!P->setup_stream) e = cudaStreamCreateWithFlags(&P->setup_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, P->setup_stream);
   return e != cudaSuccess || !bytes ? e : cudaStreamSynchronize(P->setup_stream);
+}
+
+void setup_done(snac_plan* P) {
+  if (P->setup_stream) cudaStreamDestroy(P->setup_stream);
+  P->setup_stream = nullptr;
 }
 
 int plan_alloc(snac_plan* P, void** p, size_t bytes) {
@@ -1043,6 +1049,7 @@ int check_layout(int nblocks, const snac_block* blocks, int homog_axis) {
 }
 
 size_t interface_bytes(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt) {
+  if (nblocks == 1) return 0;
   const std::vector<snac_block> ib = internal_blocks(nblocks, blocks, homog_axis);
   std::vector<HBlock> hb;
   if (validate(nblocks, ib.data(), hb)) return 0;

@@ -215,7 +215,9 @@ int snac_pencil_setup(snac_plan* plan, int64_t c0, int64_t ncols, int64_t* h_hal
   plan->pen_allocs.push_back(plan->d_pen_cell);
   CK(cudaMalloc((void**)&plan->d_pen_part, (size_t)plan->pen_nparts * 8 * sizeof(double)));
   plan->pen_allocs.push_back(plan->d_pen_part);
-  CK(copy_in(plan, plan->d_pen_cell, cell.data(), cell.size() * sizeof(int)));
+  const cudaError_t e = copy_in(plan, plan->d_pen_cell, cell.data(), cell.size() * sizeof(int));
+  setup_done(plan);
+  CK(e);
   plan->pen_c0 = c0;
   plan->pen_ncols = ncols;
   plan->pen_nhalo = (long long)halo.size();

@@ -388,7 +388,7 @@ struct snac_plan {
   };
   std::map<int, RoundGraph> round_graphs;
   bool graphs = true;                   // off after a failed capture
-  cudaStream_t setup_stream = nullptr;    // private stream of the plan's uploads and setup kernels (copy_in)
+  cudaStream_t setup_stream = nullptr;    // private stream of the plan's uploads and setup kernels, while they run
   cudaStream_t capture_stream = nullptr;  // private stream the rounds are captured on
   snac::KernelStat kstats[snac::K_COUNT];
   std::vector<snac::PendingEvent> pending;
@@ -529,8 +529,10 @@ int plan_upload(snac_plan* P, void** p, const void* src, size_t bytes);
 // Host memory into device memory, there on return. A copy from pageable memory may return before the data
 // has reached the device and is ordered within its own stream only, so it goes through the plan's private
 // stream, which is waited for: kernels on any stream then read the copied tables, and no other stream's work
-// is waited for.
+// is waited for. The stream is made by the first copy and given back by setup_done: a stream per plan kept for
+// its lifetime shares the device's few queues with those of batched solves and engine workers.
 cudaError_t copy_in(snac_plan* P, void* dst, const void* src, size_t bytes);
+void setup_done(snac_plan* P);
 double mode_lambda(int kind, int n, int q);
 bool fft_tab(int n, int max_log2, FftTab& F);
 std::vector<int> fft_perm(const FftTab& F);
