@@ -36,6 +36,8 @@ struct PlanSlot {
   uint64_t bytes = 0;
   bool busy = false;
   uint64_t last_use = 0;
+  uint64_t estimate = 0;  // of its request: another request of the same problem reserves the same
+  bool direct = true;
 };
 
 enum class State { Queued, Ready, Running, Done };
@@ -286,7 +288,9 @@ int snac_engine::run(Request* r, cudaStream_t s) {
     account(-(int64_t)r->plan_estimate);
     if (r->tune) account(-(int64_t)r->tune_bytes);
     if (--building[r->key] == 0) building.erase(r->key);
-    PlanSlot* slot = st == SNAC_OK ? new (std::nothrow) PlanSlot{r->key, pl, (uint64_t)bytes, true, 0} : nullptr;
+    PlanSlot* slot = st == SNAC_OK ? new (std::nothrow)
+                                         PlanSlot{r->key, pl, (uint64_t)bytes, true, 0, r->plan_estimate, r->direct}
+                                   : nullptr;
     if (st == SNAC_OK && !slot) {
       snac_plan_destroy(pl);
       st = SNAC_ERR_OOM;
@@ -525,9 +529,22 @@ int snac_engine_submit(snac_engine* e, int32_t nblocks, const snac_block* blocks
   r->buf_bytes = 16ull * (uint64_t)n3;
   r->plan_estimate = plan_estimate(n3, !(opt && opt->precision == SNAC_MIXED));
   r->tune_bytes = e->opt.autotune ? 8ull * (uint64_t)n3 : 0;
-  const uint64_t iface = snac::interface_bytes(nblocks, r->blocks.data(), homog_axis, opt);
-  r->direct = r->buf_bytes + r->plan_estimate + iface + r->tune_bytes <= e->opt.hbm_budget;
-  if (r->direct) r->plan_estimate += iface;
+  bool known = false;  // (the interfaces take 30 us to describe, as much as a small solve's launches)
+  {
+    std::lock_guard<std::mutex> lk(e->mu);
+    for (const PlanSlot* s : e->plans)
+      if (s->key == r->key) {
+        r->plan_estimate = s->estimate;
+        r->direct = s->direct;
+        known = true;
+        break;
+      }
+  }
+  if (!known) {
+    const uint64_t iface = snac::interface_bytes(nblocks, r->blocks.data(), homog_axis, opt);
+    r->direct = r->buf_bytes + r->plan_estimate + iface + r->tune_bytes <= e->opt.hbm_budget;
+    if (r->direct) r->plan_estimate += iface;
+  }
   if (r->buf_bytes + r->plan_estimate + r->tune_bytes > e->opt.hbm_budget) {
     delete r;
     return SNAC_ERR_OOM;
