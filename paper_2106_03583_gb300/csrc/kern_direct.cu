@@ -577,6 +577,7 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
       x[(long long)(n0 + u) * M] = d;
     }
   }
+  if (A.pin && kap == 0) x[(long long)(N - 1) * M] = alpha[q * IFACE_MAX_ENDS];  // (zero so far: its f is zero)
   T y = 0;
   for (int n0 = (N - 1) / TRI_U * TRI_U; n0 >= 0; n0 -= TRI_U) {
     T v[TRI_U], f[TRI_U];
@@ -590,7 +591,6 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
     for (int u = TRI_U - 1; u >= 0; --u) {
       if (n0 + u >= N) continue;
       y = fma(A.tri[n0 + u].hi * f[u], y, v[u]);
-      if (n0 + u == N - 1 && A.pin && kap == 0) y = alpha[q * IFACE_MAX_ENDS];
       x[(long long)(n0 + u) * M] = y;
     }
   }
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(128, 8) k_tri_pre(const DirectArgs<T> A, const
 
 // FP32 plans: the field is read and written once (12 bytes per cell instead of k_tri_pre's 24; FP64 would pay the
 // 12 operations per row). Measured with the listed systems' k_tri_low: 512 x 512 x 256 cells 0.345 -> 0.262 ms,
-// 1024 x 512 x 512 1.14 -> 0.81 ms (4.0 TB/s; what is left is the barriers between its phases); 256 x 256 x 32 50 ->
+// 1024 x 512 x 512 1.14 -> 0.81 ms (4.0 TB/s; stalls: barriers 3.1, memory 2.6 per issue, 58 % of the issue slots); 256 x 256 x 32 50 ->
 // 47 us, 336 x 192 x 150 0.11 -> 0.085 ms against the segments eliminated without kept pivots. Two CTAs of 512
 // threads per multiprocessor: four of 256 (shorter rows of systems) take 0.31 ms, one of 1024 0.29 ms.
 // One thread per system and segment of TRI_R rows, which stay in its registers; with the pivots known, both
