@@ -92,7 +92,8 @@ typedef enum { SNAC_FP64 = 0, SNAC_MIXED = 1 } snac_precision;
  * uniform axis of an even number of cells, half or all of it a product of 2, 3, 5 and 7; the eigenvectors of the
  * axis otherwise, for planes that do not solve on chip, up to 384 (SNAC_MIXED) or about 200 (SNAC_FP64) cells along
  * it), tridiagonal systems run along the other axis (not periodic), and a dense system per wavenumber gives the
- * fluxes between rectangles. Setting any of these options asks for the multigrid. */
+ * fluxes between rectangles. Setting any of these options asks for the multigrid. A plan whose direct solve cannot be
+ * set up (device memory for its tables, couplings that are not finite) keeps its V-cycles. */
 typedef struct {
   int32_t precision;   /* SNAC_FP64 (default): every stage in FP64. SNAC_MIXED: transforms and
                           multigrid in FP32 inside the FP64 defect-correction loop; the outer
@@ -336,7 +337,11 @@ int snac_pencil_residual(snac_plan *plan, const double *d_f, const double *d_p_e
  * range of a wavenumber-range plan): d_rhs, d_sol [local q][plane cell] of the plan's inner type.
  * Each wavenumber runs V-cycles from zero until w_q ||r_q||^2 <= target^2 / n_z (w_q the transform's
  * Parseval weight), it stagnates, or max_cycles: the per-mode stopping rule of snac_poisson_solve,
- * which makes the 3-D residual after the update at most `target` over all ranks together. */
+ * which makes the 3-D residual after the update at most `target` over all ranks together where V-cycles of the
+ * inner type reach it. Plans with direct solves (snac_options) solve every wavenumber once, to the rounding of the
+ * inner type and whatever the target: measured 3e-6 to 1.4e-5 of the right-hand side in SNAC_MIXED on planes of 256 x
+ * 128 to 512 x 256 cells (V-cycles stagnate at 0.4 to 0.8 of that), 8e-15 to 3e-14 in SNAC_FP64 (V-cycles 3e-15 to
+ * 1.2e-14). SNAC_OK does not say that `target` was met: the caller's residual of the updated field does. */
 int snac_mode_solve(snac_plan *plan, const void *d_rhs, void *d_sol, double target, void *stream);
 
 /* Singular problems (see snac_poisson_solve): shift the wavenumber-0 plane of d_sol by a constant so
