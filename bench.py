@@ -60,7 +60,7 @@ FP64_IN_FP64_PLAN = {"smooth", "restrict", "prolong", "mode_resid", "mode_apply"
 _FUSED = {"src": "paper_2106_03583_gb300/csrc/kern_fused.cu",
           "sha256": "2b68f2b1fd20f060bc103825a18f00981660e81a8b8743649cd5d4ea215d0b23"}
 _LINES = {"src": "paper_2106_03583_gb300/csrc/kern_direct.cu",
-          "sha256": "1832384e88e19c3a8140116062612f72d8836fcf770a7029d709bfa33dfb88f9"}
+          "sha256": "6d76898e472d7e1e317fe7ea1d3d789af134b40ade8fec03c482894304598388"}
 _Z = {"src": "paper_2106_03583_gb300/csrc/ztrans_dev.cuh",
       "sha256": "679b1e33500a8b243667ab6f2b42e3757d317f4c597ba14d788b8b0b14d5ce08"}
 _FF = {"src": "paper_2106_03583_gb300/csrc/kern_ffresid.cu",
@@ -73,10 +73,10 @@ TRAFFIC = {
     ("chan", "backward_update", "mixed"): dict(_Z, ratio=641.9 / 671.1),      # 4 + 8 + 8 B per cell
     ("chan", "field3d_ff", "mixed"): dict(_FF, ratio=662.7 / 671.1),
     ("chan", "field3d", "mixed"): dict(_F64, ratio=1270.2 / 805.3),           # 24 B; edges of the tiles re-read
-    ("chan", "lines_forward", "mixed"): dict(_LINES, ratio=218.0 / 268.4),
-    ("chan", "lines_backward", "mixed"): dict(_LINES, ratio=221.4 / 268.4),
-    ("chan", "tridiagonal", "mixed"): dict(_LINES, ratio=332.1 / 268.4),      # the kept pivots beside the field
-    ("chan", "lines_forward", "fp64"): dict(_LINES, ratio=486.9 / 536.9),
+    ("chan", "lines_forward", "mixed"): dict(_LINES, ratio=217.8 / 268.4),
+    ("chan", "lines_backward", "mixed"): dict(_LINES, ratio=220.8 / 268.4),
+    ("chan", "tridiagonal", "mixed"): dict(_LINES, ratio=332.6 / 268.4),      # the kept pivots beside the field
+    ("chan", "lines_forward", "fp64"): dict(_LINES, ratio=486.3 / 536.9),
     ("chan", "lines_backward", "fp64"): dict(_LINES, ratio=487.8 / 536.9),
     ("chan", "forward_transform", "fp64"): dict(_Z, ratio=490.0 / 536.9),
     ("chan", "backward_update", "fp64"): dict(_Z, ratio=760.1 / 805.3),
