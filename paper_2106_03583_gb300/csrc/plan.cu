@@ -1050,16 +1050,20 @@ int check_layout(int nblocks, const snac_block* blocks, int homog_axis) {
 
 size_t interface_bytes(int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt) {
   if (nblocks == 1) return 0;
-  const std::vector<snac_block> ib = internal_blocks(nblocks, blocks, homog_axis);
-  std::vector<HBlock> hb;
-  if (validate(nblocks, ib.data(), hb)) return 0;
-  snac_plan P;
-  if (opt) take_options(&P, opt);
-  if (!default_schedule(&P)) return 0;
-  P.nz = P.nzt = hb[0].n[2];
-  P.kind = hb[0].bc[2][0] == SNAC_BC_PERIODIC ? KIND_PP : KIND_NN;
-  P.max_coarse = INT32_MAX;  // level 0 only
-  return build_levels(&P, hb) ? 0 : direct_interface_bytes(&P, face_kinds(hb));
+  try {
+    const std::vector<snac_block> ib = internal_blocks(nblocks, blocks, homog_axis);
+    std::vector<HBlock> hb;
+    if (validate(nblocks, ib.data(), hb)) return 0;
+    snac_plan P;
+    if (opt) take_options(&P, opt);
+    if (!default_schedule(&P)) return 0;
+    P.nz = P.nzt = hb[0].n[2];
+    P.kind = hb[0].bc[2][0] == SNAC_BC_PERIODIC ? KIND_PP : KIND_NN;
+    P.max_coarse = INT32_MAX;  // level 0 only
+    return build_levels(&P, hb) ? 0 : direct_interface_bytes(&P, face_kinds(hb));
+  } catch (const std::bad_alloc&) {  // (no room to describe the interfaces: none to build them either)
+    return 0;
+  }
 }
 
 int create_plan(snac_plan** out, int32_t nblocks, const snac_block* blocks, int32_t homog_axis, const snac_options* opt,
