@@ -30,8 +30,9 @@
 // sums (tau) instead of the diagonal, so that every operation adds or multiplies non-negative numbers:
 // no cancellation, the factors are accurate to a few units in the last place of the working type even
 // where the system is nearly singular, and an exactly singular one (all tau = 0) ends in an exactly zero
-// pivot, whose unknown is set to zero (the caller fixes the mean). A piece of several without a Dirichlet face
-// has the last unknown of its slot 0 given (pinned): its value alpha comes from the interface system.
+// pivot, whose unknown is set to zero (the caller fixes the mean). A piece of several without a Dirichlet face, in
+// a plan with small shifts, has the last unknown of its slot 0 given (pinned): its value alpha comes from the
+// interface system.
 #pragma once
 
 #include <algorithm>

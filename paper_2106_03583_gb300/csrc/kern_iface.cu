@@ -52,8 +52,8 @@ __global__ void __launch_bounds__(128) k_resp(const TriRow<double>* __restrict__
 // the entries of B R F depend on the difference and the sum of the two cells only, through
 //   C(d) = sum_kappa h_kappa R_kappa cos(pi a_kappa d / 2M),   d < 2M
 // (products of cosines or sines as sums; h: 1/2 for the first and, periodic, the last slot). One CTA per row of
-// wavenumbers and piece, for every pair of its ends: 2 M^2 terms in place of k^2 M multiply-adds (with k_build, L of
-// 512 x 512 x 128 cells).
+// wavenumbers and piece, for every pair of its ends: 2 M^2 terms in place of k^2 M multiply-adds. Bound by the FP64 pipe
+// (92 to 94 % busy); with k_build on the L of 512 x 512 x 128 cells 10.8 -> 1.0 ms.
 struct CsumArgs {
   int M, kind, slots, a0, da;    // a_kappa = a0 + kappa da, kappa < slots
   int ne, u[2], ee[2];           // ends of the piece
@@ -182,7 +182,9 @@ __global__ void __launch_bounds__(256) k_build(const BuildArgs A, double* __rest
 }
 
 // In-place Gauss-Jordan inverse of every K, one CTA each. No pivoting: K is the identity plus a product
-// of positive operators, and the pinned unknowns come last.
+// of positive operators, and the pinned unknowns come last. Bound by the FP64 pipe (128 systems of 256: 5.4 ms, 91 %
+// busy) or, for smaller systems, by the latency of a step: 1024 threads from 64 unknowns on (96 systems of 160 with
+// 256 threads 5.7 ms, 49 with 1024 2.1 ms).
 __global__ void __launch_bounds__(1024) k_invert(double* __restrict__ Kq, int n) {
   extern __shared__ double sh[];
   double* rp = sh;        // pivot row / pivot
