@@ -483,9 +483,9 @@ int build_piece(snac_plan* P, const Piece& p, int ax, int soff, DirectTab& D) {
     tri[4 * n + 2] = D.cscale * tau;
     tri[4 * n + 3] = c.hi > 0.0 ? c.lo / c.hi : 0.0;
   }
-  // slot 0 of an all-Neumann or periodic piece is nearly singular for shifts well below the next slot's eigenvalue
-  // (mixed 256 x 160 x 16, T of 48 x 32: one step more from a tenth of it on); above, its response is like theirs and
-  // the interface system stays one unknown smaller (32 cells instead of 33: 3 % of a batch of small problems)
+  // slot 0 of an all-Neumann or periodic piece is nearly singular for shifts well below the next slot's eigenvalue:
+  // not pinned, a mixed L of 256 x 160 cells took a third step at a tenth of it, a fourth at a thousandth. Above a
+  // quarter its response is like theirs, and the interface systems stay one unknown smaller
   D.pin = (p.iface[0] || p.iface[1]) && (p.kind == KIND_PP || p.kind == KIND_NN) && p.side[0] != SNAC_BC_DIRICHLET &&
           p.side[1] != SNAC_BC_DIRICHLET;
   if (D.pin) {

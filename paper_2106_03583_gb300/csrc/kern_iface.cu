@@ -6,9 +6,10 @@
 // rows, Y takes end values to jumps. A piece without a Dirichlet face is singular for a zero shift, and nearly
 // so for a small one: R of its slot 0 then grows like 1 / shift and swamps the system (with shift -1e-8 of a
 // unit box no step reduced the residual in FP64, with -1e-4 none in FP32). So where some wavenumber's shift is
-// small (build_piece) that slot's system is pinned, for every wavenumber: its last unknown alpha is an unknown of the interface system, all others follow from it by
-// h (1 at a zero shift) and its last row, eliminated, is the extra equation den alpha = num. The inverse of
-// every system is kept with the plan, one for all wavenumbers of equal shift (a row of DirectPlan::d_qrow).
+// small (build_piece) that slot's system is pinned, for every wavenumber: its last unknown alpha is an unknown of
+// the interface system, all others follow from it by h (1 at a zero shift) and its last row, eliminated, is the
+// extra equation den alpha = num. The inverse of every system is kept with the plan, one for all wavenumbers of
+// equal shift (a row of DirectPlan::d_qrow).
 #include <cmath>
 #include <vector>
 
